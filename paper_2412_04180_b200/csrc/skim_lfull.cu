@@ -6,7 +6,10 @@
 //                             same midpoint rule as the packer.  Streaming: 2 B in, 2 B out per element.
 //   skim_lfull_gemm_kernel    Y = D H (H = X X^T, symmetric, binary16) on the tensor cores and, fused into the
 //                             epilogue, the row-wise dot  sum_n Y_in D_in  of every output tile, so Y never
-//                             leaves the SM.  This is the one dense contraction of the method.
+//                             leaves the SM.  This is the one dense contraction of the method.  Where only the errors are
+//                             asked for it runs over the upper half of H with weight 2 (half the products; the kernel's
+//                             spare warps check that H is symmetric, and the full contraction follows if not):
+//                             bound by the tensor pipe, 4096 x 11008 x 11008 0.374 ms per width against 0.709 ms in full.
 //   skim_lfull_reduce_kernel  adds the per-tile partial sums of a row in a fixed order, divides 4^e out.
 //
 // GEMM kernel: persistent, one CTA per SM, tile 128 x 256 x 64, tcgen05.mma (kind::f16, binary32 accumulators
@@ -18,6 +21,8 @@
 // sets SKIM_STATUS_TIMEOUT, and all roles leave their loops; tensor memory is freed on every path.
 #include <cuda.h>
 #include <cudaTypedefs.h>
+
+#include <vector>
 
 #include "skim_internal.cuh"
 
@@ -127,7 +132,10 @@ constexpr int STAGES = 4;
 constexpr int UMMA_K = 16;
 constexpr int A_BYTES = BM * BK * 2, B_BYTES = BN * BK * 2, STAGE_BYTES = A_BYTES + B_BYTES;
 constexpr int GEMM_THREADS = 192;
+constexpr int CHECK_WARPS = 4;                  // further warps of the half contraction: they compare H with its transpose
 constexpr int SPLIT_MAX = 8;                    // ranges of K a tile of the last round is cut into, at most
+constexpr int HALF_MIN_ROWS = 768, HALF_MIN_NT = 4;
+constexpr size_t HALF_FLAG_BYTES = 4096;         // symmetry flags of up to 1024 blocks
 constexpr int TMEM_COLS = 512;                  // two accumulator stages of BN binary32 columns
 constexpr long long WAIT_LIMIT_CYCLES = 400000000ll;   // about 0.2 s; a whole launch takes milliseconds
 constexpr size_t GEMM_SMEM = (size_t)STAGES * STAGE_BYTES + 1024 /* alignment slack */ + 256 /* barriers */;
@@ -139,6 +147,7 @@ struct GemmSync {
     uint64_t tmem_empty[2];
     uint32_t tmem_base;
     int abort;
+    int asym;
 };
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -209,6 +218,13 @@ __device__ __forceinline__ void umma_f16(uint32_t tmem_d, uint64_t adesc, uint64
                  "l"(adesc), "l"(bdesc), "r"(IDESC), "r"(accumulate)
                  : "memory");
 }
+// D = A B + D / 2
+__device__ __forceinline__ void umma_f16_halve(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc)
+{
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.eq.b32 p, 0, 0;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p, 1;\n\t}" ::"r"(tmem_d),
+                 "l"(adesc), "l"(bdesc), "r"(IDESC)
+                 : "memory");
+}
 __device__ __forceinline__ void umma_commit(uint64_t *bar)
 {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
@@ -240,6 +256,9 @@ struct GemmArgs {
     float *partial;          // [mt * BM][split][nt]
     float *Y;                // optional [rows][ldy]: the product D H itself (the scaling-vector update needs it)
     int64_t ldy;
+    int *asym;               // [asym_n] per block of the half contraction: H is not symmetric in the part it compared
+    int asym_n;
+    int piece_kb;            // half contraction: a tile's list of K blocks is cut into pieces of about this length
     unsigned long long *status;
 };
 
@@ -265,8 +284,89 @@ __device__ __forceinline__ GemmUnit unit_of(const GemmArgs &a, int u, int nkb)
     return w;
 }
 
-__global__ void __launch_bounds__(GEMM_THREADS, 1)
-skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, GemmArgs a)
+// The quadratic form of a symmetric H needs half of its products:  d H d^T = sum_n d_n (H_nn d_n + 2 sum_{k>n} H_nk d_k).
+// In tiles: column tile nb takes the K blocks of its own diagonal block with weight 1 and those beyond it (k >= n0 + BN)
+// with weight 2, so its K list is simply n0/BK .. nkb-1.  The diagonal part comes first and is halved by the first MMA
+// of the rest (the tensor core's own scaling of the accumulator input, exact); the epilogue doubles the dot.  (The
+// upper half, not the lower: a large residual then meets as many later roundings of the accumulator as in the full
+// contraction.)  Lists shrink from nkb blocks to one: tiles are taken in descending length, every other round of blocks
+// in reverse order, so that the blocks end together; a list may be cut into pieces (their dots add up).  Row tiles vary
+// fastest, so the blocks of a round share the panels of H.
+struct HalfList {
+    int nb, base, pieces;    // cursor: units base .. base + mt * pieces - 1 belong to column tile nb
+};
+constexpr int HALF_DIAG = BN / BK;                  // K blocks of a diagonal block (the last one may have fewer)
+__host__ __device__ __forceinline__ int half_len(int nb, int nkb) { return nkb - nb * HALF_DIAG; }
+__host__ __device__ __forceinline__ int half_pieces(int nb, int nkb, int piece_kb)
+{
+    const int p = (half_len(nb, nkb) + piece_kb - 1) / piece_kb;
+    return p < SPLIT_MAX ? p : SPLIT_MAX;
+}
+// The GemmUnit of unit u (kb0, kb1 are list positions); units are asked for in ascending order.
+__device__ __forceinline__ GemmUnit half_unit(const GemmArgs &a, HalfList &h, int u, int nkb)
+{
+    while (u >= h.base + a.mt * h.pieces) {
+        h.base += a.mt * h.pieces;
+        ++h.nb;
+        h.pieces = half_pieces(h.nb, nkb, a.piece_kb);
+    }
+    const int r = u - h.base, len = half_len(h.nb, nkb);
+    GemmUnit w;
+    w.slice = r / a.mt;
+    w.tile = h.nb * a.mt + r % a.mt;
+    w.kb0 = len * w.slice / h.pieces;
+    w.kb1 = len * (w.slice + 1) / h.pieces;
+    return w;
+}
+
+// Unit of this block in round t, or -1: round-robin (HALF: every other round reversed).
+template <bool HALF>
+__device__ __forceinline__ int unit_index(int t, int nunits)
+{
+    const int u = t * (int)gridDim.x + ((HALF && (t & 1)) ? (int)gridDim.x - 1 - (int)blockIdx.x : (int)blockIdx.x);
+    return u < nunits ? u : -1;
+}
+
+// Compares H with its transpose, one warp per pair of blocks H[32 I .. +32][64 J .. +64] and H[64 J ..][32 I ..] at or
+// above the diagonal.  A lane compares an 8 x 8 sub-block against its mirror image in registers; whole sectors on either side.
+// The ragged end (fewer than 8 rows or columns cannot occur: cols is a multiple of 8).  Returns nonzero on a difference.
+__device__ __forceinline__ uint32_t compare_transpose(const uint16_t *H, int64_t ldh, int cols, int first, int step)
+{
+    const int lane = threadIdx.x & 31;
+    const int ni = (cols + 31) / 32, nj = (cols + 63) / 64;
+    uint32_t diff = 0u;
+    for (long long t = first; t < (long long)ni * nj; t += step) {
+        const int I = (int)(t % ni), J = (int)(t / ni);
+        if (64 * J + 64 <= 32 * I) continue;                  // below the diagonal: the mirror pair is compared
+        const int r0 = 32 * I + (lane >> 3) * 8, c0 = 64 * J + (lane & 7) * 8;
+        if (r0 < cols && c0 < cols) {
+            uint4 x[8], y[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) x[u] = __ldg(reinterpret_cast<const uint4 *>(H + (int64_t)(r0 + u) * ldh + c0));
+#pragma unroll
+            for (int u = 0; u < 8; ++u) y[u] = __ldg(reinterpret_cast<const uint4 *>(H + (int64_t)(c0 + u) * ldh + r0));
+#pragma unroll
+            for (int r = 0; r < 8; r += 2) {
+                const uint32_t a0[4] = {x[r].x, x[r].y, x[r].z, x[r].w}, a1[4] = {x[r + 1].x, x[r + 1].y, x[r + 1].z, x[r + 1].w};
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const uint4 b0 = y[2 * q], b1 = y[2 * q + 1];
+                    const uint32_t v0 = r == 0 ? b0.x : r == 2 ? b0.y : r == 4 ? b0.z : b0.w;
+                    const uint32_t v1 = r == 0 ? b1.x : r == 2 ? b1.y : r == 4 ? b1.z : b1.w;
+                    diff |= __byte_perm(a0[q], a1[q], 0x5410) ^ v0;
+                    diff |= __byte_perm(a0[q], a1[q], 0x7632) ^ v1;
+                }
+            }
+        }
+    }
+    return diff;
+}
+
+// HALF: the half contraction for a symmetric H, launched first; it leaves in a.asym whether H was.  Otherwise the full
+// contraction; with a.asym given it is the fallback of a half launch and leaves at once unless H was not symmetric.
+template <bool HALF>
+__global__ void __launch_bounds__(GEMM_THREADS + (HALF ? CHECK_WARPS * 32 : 0), 1)
+skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, GemmArgs a, const uint16_t *H, int64_t ldh)
 {
     extern __shared__ unsigned char smem_raw[];
     unsigned char *tiles = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -275,12 +375,22 @@ skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nkb = (a.cols + BK - 1) / BK;
     const int ntiles = a.mt * a.nt;
-    const int nunits = a.full_tiles + (ntiles - a.full_tiles) * a.split;
+    int nunits = a.full_tiles + (ntiles - a.full_tiles) * a.split;
+    HalfList half = {0, 0, HALF ? half_pieces(0, nkb, a.piece_kb) : 1};
+    if (HALF) {
+        nunits = 0;
+        for (int nb = 0; nb < a.nt; ++nb) nunits += a.mt * half_pieces(nb, nkb, a.piece_kb);
+    } else if (a.asym) {
+        int any = 0;
+        for (int i = threadIdx.x; i < a.asym_n; i += GEMM_THREADS) any |= a.asym[i];
+        if (!__syncthreads_or(any)) return;
+    }
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) { mbar_init(&sy.full[s], 1); mbar_init(&sy.empty[s], 1); }
         for (int s = 0; s < 2; ++s) { mbar_init(&sy.tmem_full[s], 1); mbar_init(&sy.tmem_empty[s], 4); }
         sy.abort = 0;
+        sy.asym = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
@@ -298,10 +408,13 @@ skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
             int stage = 0;
             uint32_t phase = 0;
             bool ok = true;
-            for (int u = blockIdx.x; u < nunits && ok; u += gridDim.x) {
-                const GemmUnit w = unit_of(a, u, nkb);
+            for (int t = 0; t * (int)gridDim.x < nunits && ok; ++t) {
+                const int u = unit_index<HALF>(t, nunits);
+                if (u < 0) continue;
+                const GemmUnit w = HALF ? half_unit(a, half, u, nkb) : unit_of(a, u, nkb);
                 const int m0 = (w.tile % a.mt) * BM, n0 = (w.tile / a.mt) * BN;
-                for (int kb = w.kb0; kb < w.kb1; ++kb) {
+                for (int l = w.kb0; l < w.kb1; ++l) {
+                    const int kb = HALF ? n0 / BK + l : l;
                     if (!(ok = mbar_wait(&sy.empty[stage], phase ^ 1u, abort_flag))) break;
                     unsigned char *sa = tiles + (size_t)stage * STAGE_BYTES;
                     mbar_expect_tx(&sy.full[stage], STAGE_BYTES);
@@ -318,32 +431,42 @@ skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
             uint32_t phase = 0;
             bool ok = true;
             int it = 0;
-            for (int u = blockIdx.x; u < nunits && ok; u += gridDim.x, ++it) {
-                const GemmUnit w = unit_of(a, u, nkb);
+            for (int t = 0; t * (int)gridDim.x < nunits && ok; ++t) {
+                const int u = unit_index<HALF>(t, nunits);
+                if (u < 0) continue;
+                const GemmUnit w = HALF ? half_unit(a, half, u, nkb) : unit_of(a, u, nkb);
                 const int as = it & 1;
                 if (!(ok = mbar_wait(&sy.tmem_empty[as], (((uint32_t)it >> 1) & 1u) ^ 1u, abort_flag))) break;
                 tc_fence_after();
                 const uint32_t tmem_d = tmem_base + (uint32_t)(as * BN);
-                for (int kb = w.kb0; kb < w.kb1; ++kb) {
+                for (int kb = w.kb0; kb < w.kb1; ++kb) {          // HALF: list positions
                     if (!(ok = mbar_wait(&sy.full[stage], phase, abort_flag))) break;
                     tc_fence_after();
                     const uint32_t sa = smem_u32(tiles + (size_t)stage * STAGE_BYTES), sb = sa + A_BYTES;
 #pragma unroll
                     for (int k = 0; k < BK / UMMA_K; ++k)
-                        umma_f16(tmem_d, umma_desc(sa + k * UMMA_K * 2), umma_desc(sb + k * UMMA_K * 2), (kb > w.kb0 || k) ? 1u : 0u);
+                        if (HALF && k == 0 && kb == HALF_DIAG && kb > w.kb0) umma_f16_halve(tmem_d, umma_desc(sa), umma_desc(sb));
+                        else umma_f16(tmem_d, umma_desc(sa + k * UMMA_K * 2), umma_desc(sb + k * UMMA_K * 2), (kb > w.kb0 || k) ? 1u : 0u);
                     umma_commit(&sy.empty[stage]);           // the stage is free once these MMAs have read it
                     if (++stage == STAGES) { stage = 0; phase ^= 1u; }
                 }
                 if (ok) umma_commit(&sy.tmem_full[as]);      // the accumulator is complete once all MMAs are
+                ++it;
             }
         }
+    } else if (HALF && warp >= GEMM_THREADS / 32) {
+        // ------------------------------------------------------------ H against its transpose, under the contraction
+        const uint32_t diff = compare_transpose(H, ldh, a.cols, (int)blockIdx.x * CHECK_WARPS + warp - GEMM_THREADS / 32, (int)gridDim.x * CHECK_WARPS);
+        if (diff) sy.asym = 1;
     } else {
         // ------------------------------------------------------------ epilogue: 4 warps, one row per thread
         const int q = warp & 3;                               // the tensor-memory lane quarter this warp may read
         bool ok = true;
         int it = 0;
-        for (int u = blockIdx.x; u < nunits && ok; u += gridDim.x, ++it) {
-            const GemmUnit w = unit_of(a, u, nkb);
+        for (int t = 0; t * (int)gridDim.x < nunits && ok; ++t) {
+            const int u = unit_index<HALF>(t, nunits);
+            if (u < 0) continue;
+            const GemmUnit w = HALF ? half_unit(a, half, u, nkb) : unit_of(a, u, nkb);
             const int as = it & 1;
             const int mb = w.tile % a.mt, nb = w.tile / a.mt;
             const int row = mb * BM + q * 32 + lane;
@@ -365,7 +488,7 @@ skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
                 }
                 uint32_t v[32];
                 tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(as * BN + c * 32), v);
-                if (a.Y && row < a.rows) {
+                if (!HALF && a.Y && row < a.rows) {
                     float *yrow = a.Y + (int64_t)row * a.ldy + col;
 #pragma unroll
                     for (int u = 0; u < 8; ++u)
@@ -386,12 +509,16 @@ skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&sy.tmem_empty[as]);
-            if (row < a.rows) a.partial[((int64_t)row * a.split + w.slice) * a.nt + nb] = acc;
+            // a piece that reaches past its diagonal blocks holds half the dot (the diagonal blocks' part was halved)
+            if (HALF && w.kb1 > HALF_DIAG) acc *= 2.0f;
+            if (row < a.rows) a.partial[((int64_t)row * (HALF ? SPLIT_MAX : a.split) + w.slice) * a.nt + nb] = acc;
+            ++it;
         }
     }
     // ---------------------------------------------------------------- teardown (every path comes here)
     tc_fence_before();
     __syncthreads();
+    if (HALF && threadIdx.x == 0) a.asym[blockIdx.x] = sy.asym;
     if (sy.abort) {
         // a wait ran out: give the bulk copies that may still be in flight time to land before the block's
         // shared memory is released (about a millisecond), and report
@@ -404,21 +531,55 @@ skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
     }
 }
 
-// Adds a row's partial dots in a fixed order: slice 0 of every column tile, then the further slices of the tiles
-// that were cut along K (only those entries were written).
-__global__ void skim_lfull_reduce_kernel(const float *__restrict__ partial, int rows, int mt, int nt, int full_tiles, int split,
-                                         int exp2, float *__restrict__ err, int64_t err_stride, double *__restrict__ err64)
+constexpr int RED_WARPS = 8;
+
+// Adds a row's partial dots in a fixed order, one warp per row: a lane takes every 32nd column tile, then a tree.  After a
+// half contraction whose H was symmetric a tile has half_pieces() dots; after a full one slice 0 of every tile was
+// written, and the further slices of the tiles that were cut along K.
+__global__ void __launch_bounds__(RED_WARPS * 32)
+skim_lfull_reduce_kernel(GemmArgs a, int exp2, float *__restrict__ err, int64_t err_stride, double *__restrict__ err64)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= rows) return;
-    const int mb = i / BM;
+    bool half = false;
+    if (a.asym) {
+        int any = 0;
+        for (int i = threadIdx.x; i < a.asym_n; i += RED_WARPS * 32) any |= a.asym[i];
+        half = !__syncthreads_or(any);
+    }
+    const int i = blockIdx.x * RED_WARPS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (i >= a.rows) return;
+    const int mb = i / BM, nkb = (a.cols + BK - 1) / BK;
     double s = 0.0;
-    for (int t = 0; t < nt; ++t) s += (double)partial[((int64_t)i * split) * nt + t];
-    for (int sl = 1; sl < split; ++sl)
-        for (int t = 0; t < nt; ++t)
-            if (t * mt + mb >= full_tiles) s += (double)partial[((int64_t)i * split + sl) * nt + t];
-    if (err) err[(int64_t)i * err_stride] = (float)ldexp(s, -2 * exp2);
-    if (err64) err64[i] = ldexp(s, -2 * exp2);
+    for (int t = lane; t < a.nt; t += 32) {
+        const int split = half ? SPLIT_MAX : a.split;
+        const int pieces = half ? half_pieces(t, nkb, a.piece_kb) : t * a.mt + mb >= a.full_tiles ? a.split : 1;
+        for (int sl = 0; sl < pieces; ++sl) s += (double)a.partial[((int64_t)i * split + sl) * a.nt + t];
+    }
+#pragma unroll
+    for (int off = 16; off; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    if (lane == 0) {
+        if (err) err[(int64_t)i * err_stride] = (float)ldexp(s, -2 * exp2);
+        if (err64) err64[i] = ldexp(s, -2 * exp2);
+    }
+}
+
+// Length of the longest block of a half contraction, in K blocks, if lists are cut into pieces of about piece_kb: a
+// piece also costs its epilogue, which hides under the next piece's MMAs unless that one is shorter.
+double half_makespan(int mt, int nt, int nkb, int piece_kb, int blocks)
+{
+    constexpr double EPILOGUE = 10.0;          // K blocks' worth of MMA time (256 columns read back and multiplied)
+    std::vector<double> load(blocks, 0.0);
+    int u = 0;
+    for (int nb = 0; nb < nt; ++nb) {
+        const int p = half_pieces(nb, nkb, piece_kb);
+        const double len = (double)half_len(nb, nkb) / p;
+        for (int r = 0; r < p * mt; ++r, ++u) {
+            const int t = u / blocks, b = u % blocks;
+            load[(t & 1) ? blocks - 1 - b : b] += len > EPILOGUE ? len : EPILOGUE;
+        }
+    }
+    double most = 0.0;
+    for (double v : load) most = v > most ? v : most;
+    return most + EPILOGUE;
 }
 
 int encode_map(CUtensorMap *map, const uint16_t *base, int64_t rows, int64_t cols, int64_t ld, int box_rows)
@@ -474,7 +635,7 @@ int skim_launch_residual(skim_ctx *ctx, const uint16_t *W, int64_t rows, int64_t
 size_t skim_lfull_scratch_bytes(int64_t rows, int64_t cols)
 {
     const int64_t mt = (rows + BM - 1) / BM, nt = (cols + BN - 1) / BN;
-    return skim_align256((size_t)(mt * BM) * (size_t)nt * SPLIT_MAX * sizeof(float));
+    return skim_align256((size_t)(mt * BM) * (size_t)nt * SPLIT_MAX * sizeof(float)) + HALF_FLAG_BYTES;
 }
 
 int skim_launch_err_lfull(skim_ctx *ctx, const uint16_t *D, int64_t rows, int64_t cols, int64_t ldd, const uint16_t *H,
@@ -498,7 +659,7 @@ int skim_launch_err_lfull(skim_ctx *ctx, const uint16_t *D, int64_t rows, int64_
     a.Y = Y;
     a.ldy = ldy;
     a.status = (unsigned long long *)ctx->ws;
-    SKIM_CUDA_OK(cudaFuncSetAttribute(skim_lfull_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GEMM_SMEM));
+    SKIM_CUDA_OK(cudaFuncSetAttribute(skim_lfull_gemm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GEMM_SMEM));
     const int tiles = a.mt * a.nt;
     // the tiles of the last round, if it is not full, are cut along K into as many ranges as fit the SMs
     const int nkb = (int)((cols + BK - 1) / BK);
@@ -518,12 +679,35 @@ int skim_launch_err_lfull(skim_ctx *ctx, const uint16_t *D, int64_t rows, int64_
             a.split = sp;
         }
     }
+    // Half the contraction where H turns out symmetric, as a Gram matrix is.  The comparison of H with its transpose
+    // reads all of H (2 B per entry) under a contraction of rows MACs per entry: at the measured rates the two take equally long
+    // near 700 rows; below that, or with so few column tiles that the diagonal blocks are most of the work, the full
+    // contraction is no slower.
+    a.asym = nullptr;
+    a.asym_n = 0;
+    a.piece_kb = nkb;
+    if (!Y && rows >= HALF_MIN_ROWS && a.nt >= HALF_MIN_NT && ctx->sm_count * sizeof(int) <= HALF_FLAG_BYTES) {
+        // pieces of about the full contraction's length (the accumulator's rounding errors grow with it), or half of that
+        // where it balances the blocks clearly better
+        double best = 0.0;
+        const int c0 = a.full_tiles == 0 ? a.split : 1;
+        for (int c = c0; c <= 2 * c0 && c <= SPLIT_MAX; ++c) {
+            const int piece = (nkb + c - 1) / c;
+            const double v = half_makespan(a.mt, a.nt, nkb, piece, ctx->sm_count);
+            if (c == c0 || v < best * 0.95) { best = v; a.piece_kb = piece; }
+        }
+        a.asym = (int *)((char *)scratch + skim_lfull_scratch_bytes(rows, cols) - HALF_FLAG_BYTES);
+        a.asym_n = ctx->sm_count;
+        SKIM_CUDA_OK(cudaFuncSetAttribute(skim_lfull_gemm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GEMM_SMEM));
+        skim_lfull_gemm_kernel<true><<<(unsigned)ctx->sm_count, GEMM_THREADS + CHECK_WARPS * 32, GEMM_SMEM, ctx->stream>>>(map_a, map_b, a, H, ldh);
+        SKIM_CUDA_OK(cudaGetLastError());
+        ctx->launches += 1;
+    }
     const int units = a.full_tiles + (tiles - a.full_tiles) * a.split;
     const unsigned blocks = (unsigned)(units < ctx->sm_count ? units : ctx->sm_count);    // persistent: one CTA per SM
-    skim_lfull_gemm_kernel<<<blocks, GEMM_THREADS, GEMM_SMEM, ctx->stream>>>(map_a, map_b, a);
+    skim_lfull_gemm_kernel<false><<<blocks, GEMM_THREADS, GEMM_SMEM, ctx->stream>>>(map_a, map_b, a, H, ldh);
     SKIM_CUDA_OK(cudaGetLastError());
-    skim_lfull_reduce_kernel<<<(unsigned)((rows + 255) / 256), 256, 0, ctx->stream>>>(a.partial, (int)rows, a.mt, a.nt, a.full_tiles, a.split, exp2, err,
-                                                                                      err_stride, err64);
+    skim_lfull_reduce_kernel<<<(unsigned)((rows + RED_WARPS - 1) / RED_WARPS), RED_WARPS * 32, 0, ctx->stream>>>(a, exp2, err, err_stride, err64);
     SKIM_CUDA_OK(cudaGetLastError());
     ctx->launches += 2;
     return SKIM_OK;

@@ -166,3 +166,18 @@ def test_lfull_argument_errors(ctx, skimlib):
         ctx.err_lfull(D, H, exp2=40)
     assert e.value.code == -2
     assert float(ctx.err_lfull(D, H).abs().max().item()) == 0.0
+
+
+@pytest.mark.parametrize("rows,cols,symmetric", [(768, 776, True), (1000, 1096, True), (770, 2056, True), (4100, 1024, True), (897, 4104, True),
+                                                 (1000, 1096, False), (770, 2056, False), (767, 1096, True)])
+def test_lfull_half_contraction_of_a_symmetric_matrix(ctx, oracle, rows, cols, symmetric):
+    """Enough rows and columns for the half contraction: symmetric H, and one that differs from its transpose in a
+    single corner entry (the full contraction must take over)."""
+    ctx.reserve(rows, cols)
+    rng = np.random.default_rng(rows + cols)
+    D = (rng.standard_normal((rows, cols)) * 2).astype(np.float16)
+    H = inputs.make_gram(cols, 90 + cols)
+    if not symmetric:
+        H[cols - 1, 0] += np.float16(3.0)
+    sel = np.unique(np.concatenate([[0, 127, 128, rows - 1], rng.choice(rows, 20)]))
+    _check_err(ctx, oracle, D, H, 8, rows=sel, label=f"{rows}x{cols} {symmetric}")
