@@ -51,7 +51,8 @@ struct SkimWorkspace {
     double *grad_part;           // [SKIM_SCALE_MAX_CTAS][cols]  partial gradients of the row ranges
     double *scale_const;         // [rows][16][2]  scale update: per-cluster constants (sum g, sum g w^2)
     double *scale_cq;            // [rows][16][2]  scale update: per-cluster centroid and gradient factor
-    unsigned char *cluster_scratch;  // [min(rows, SKIM_CLUSTER_CHUNK_ROWS)] row records of the clustering
+    uint16_t *scale_ord_end;     // [rows][16]  scale update: steps of the clusters in the label-ordered rows
+    unsigned char *cluster_scratch;  // [min(rows, SKIM_CLUSTER_CHUNK_ROWS)] row records of the clustering; during a scale update the label-ordered matrix
     size_t bytes;
 };
 
@@ -64,6 +65,15 @@ __host__ __device__ static inline size_t skim_cluster_record_bytes(int64_t cols)
 {
     const size_t m8 = ((size_t)cols + 7) & ~(size_t)7;
     return (13 * m8 + 1024 + 127) & ~(size_t)127;
+}
+
+// The label-ordered matrix of the scale update (skim_scale.cu): elements (8 bytes each) of a row, at most, with 16
+// clusters padded to whole units of 64; and the bytes behind the last row that its readers may fetch.
+#define SKIM_ORDER_UNIT 64
+#define SKIM_ORDER_SLACK 8192
+__host__ __device__ static inline int64_t skim_ordered_stride(int64_t cols)
+{
+    return (cols + SKIM_ORDER_UNIT - 1) / SKIM_ORDER_UNIT * SKIM_ORDER_UNIT + 16 * SKIM_ORDER_UNIT;
 }
 
 static inline size_t skim_align256(size_t v) { return (v + 255) & ~(size_t)255; }
@@ -85,8 +95,10 @@ static inline SkimWorkspace skim_carve(void *base, int64_t rows, int64_t cols)
     w.grad_part = (double *)take((size_t)SKIM_SCALE_MAX_CTAS * (size_t)cols * 8);
     w.scale_const = (double *)take((size_t)rows * 16 * 2 * 8);
     w.scale_cq = (double *)take((size_t)rows * 16 * 2 * 8);
-    w.cluster_scratch = (unsigned char *)take((size_t)(rows < SKIM_CLUSTER_CHUNK_ROWS ? rows : SKIM_CLUSTER_CHUNK_ROWS) *
-                                              skim_cluster_record_bytes(cols));
+    w.scale_ord_end = (uint16_t *)take((size_t)rows * 16 * 2);
+    const size_t records = (size_t)(rows < SKIM_CLUSTER_CHUNK_ROWS ? rows : SKIM_CLUSTER_CHUNK_ROWS) * skim_cluster_record_bytes(cols);
+    const size_t ordered = (size_t)rows * (size_t)skim_ordered_stride(cols) * 8 + SKIM_ORDER_SLACK;
+    w.cluster_scratch = (unsigned char *)take(records > ordered ? records : ordered);
     w.bytes = off;
     return w;
 }

@@ -4,18 +4,17 @@
 //   loss(alpha) = sum_ij g_ij (W_ij - alpha_j c_{i,l_ij})^2,
 //   c_ik        = sum_{j in k} g_ij W_ij / alpha_j  /  sum_{j in k} g_ij   (re-fitted each step)
 //
-// Per Adam step the matrix is read twice, by two kernels:
-//   skim_scale_sums_kernel  one warp per row.  Per cluster k of the row it forms, in binary64,
+// Once per call skim_scale_order_kernel writes every row in label order.  Per Adam step the matrix is then read twice:
+//   skim_scale_sums_kernel  one warp per row, on the label-ordered copy.  Per cluster k of the row it forms, in binary64,
 //       S_k = sum g w / alpha,  A_k = sum g w alpha,  B_k = sum g alpha^2  (sums over the members).
 //       With the per-call constants G_k = sum g and D_k = sum g w^2 (the same kernel, run once in
 //       its INIT form) these give the centroid c_k = S_k / G_k, the row's loss
 //       sum_k D_k - 2 c_k A_k + c_k^2 B_k, and the factor q_k = 2 (A_k - c_k B_k) / G_k through which the
-//       re-fitted centroid enters the gradient -- without a second pass over the row.  A lane adds
-//       its elements into accumulator slots of its own in shared memory (one per cluster and
-//       sum), so no atomics are needed and every sum has a fixed order.
+//       re-fitted centroid enters the gradient -- without a second pass over the row.  No atomics: every sum has a
+//       fixed order.
 //   skim_scale_grad_kernel  a thread owns four columns and walks a range of rows:
 //       d loss / d alpha_j = sum_i  -2 g c (w - alpha_j c) + q g w / alpha_j^2   (c, q of the element's
-//       cluster, read from the 512-byte table the first kernel left for the row), accumulated in
+//       cluster, from the 256-byte table the first kernel left for the row), accumulated in
 //       registers; the row ranges leave partial gradients that the Adam kernel adds in a fixed order.
 //   skim_scale_adam_kernel  sums the partials and the rows' losses (deterministic), applies the
 //       Adam update to the binary64 master copy of alpha and to its lane-interleaved copy, the
@@ -26,8 +25,6 @@ namespace {
 
 constexpr int KC = 16;      // clusters per row at most (4 bits)
 constexpr int SW = 4;       // warps (rows) per block of the sums kernel
-constexpr int NSUM = 3;
-constexpr int GW = 2;       // elements whose slot updates of the sums kernel go together
 constexpr int GT = 256;     // threads of a gradient block
 constexpr int GC = 4;       // columns per thread
 
@@ -40,6 +37,8 @@ struct ScaleArgs {
     int64_t rows, ld;
     int cols;
     int vec;                // rows of W, G and labels allow the vector loads of both kernels
+    uint2 *ord;             // [rows][skim_ordered_stride(cols)]  the matrix in label order
+    uint16_t *ord_end;      // [rows][KC]  units of the clusters up to and including each
     double2 *tconst;        // [rows][KC]  (G_k, D_k)
     double2 *tq;            // [rows][KC]  (c_k, q_k)
     double *loss_row;       // [rows]
@@ -57,258 +56,494 @@ __host__ __device__ __forceinline__ int alpha_il_pos(int j)
     return (j & ~255) + 64 * ((r >> 1) & 3) + 2 * (r >> 3) + (r & 1);
 }
 
+// Every kernel of an Adam step is launched as a programmatic dependent of the one before it: it may start while that
+// one drains, fetches what no kernel of the loop writes (the matrix), and waits here before it touches anything else.
+__device__ __forceinline__ void wait_for_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void let_next_kernel_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // 1 / a for a positive, normal binary64 a (the scale vector is checked to be that): the hardware's approximate
-// reciprocal (about 23 bits) and two Newton steps, within one unit in the last place.  Five instructions where the
-// correctly rounded division-free reciprocal takes about twelve; the sums kernel needs one per element.
+// reciprocal (better than 20 bits, error e) and one step of the series 1 + e + e^2, within one unit in the last place.  Four
+// instructions where the correctly rounded division-free reciprocal takes about twelve; the sums kernel needs one per element.
 __device__ __forceinline__ double rcp_pos(double a)
 {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
-    r = fma(r, fma(-a, r, 1.0), r);
-    return fma(r, fma(-a, r, 1.0), r);
+    const double e = fma(-a, r, 1.0);
+    return fma(r, fma(e, e, e), r);
 }
 
-// Eight consecutive elements of a row starting at e0 (a multiple of 8), as loaded; entries at or
-// beyond cols come back with zero importance, label 0 and alpha 1.
-struct Raw8 {
-    uint4 w;            // 8 binary16 weights
-    float4 ga, gb;      // 8 importances
-    uint2 l;            // 8 labels
-    double2 al[4];      // 8 alphas
-};
+// ---------------------------------------------------------------- the label-ordered copy of the matrix
+//
+// Labels are fixed during a call, so every row is put in label order once: element = (importance, weight, column) in
+// 8 bytes, the members of a cluster padded to whole units of 64.  The sums of a unit then belong to one cluster and
+// stay in registers (in column order every element costs three binary64 read-modify-writes of an accumulator slot in
+// shared memory, 96 wavefronts of the L1 data path per 256 elements, which bound the kernel), and the price is one
+// gather of alpha from shared memory per element.  Inside a cluster the elements are dealt by column modulo 16, the
+// bank pair of alpha's entry, so that the 16 lanes of a half-warp mostly hit 16 different bank pairs: the i-th
+// elements of all 16 classes come first for i = 0, then for i = 1, and so on.
+constexpr int OT = 512;                    // threads per block of the ordering kernel
+constexpr int OW = OT / 32;
+constexpr int OB = 6;                      // chunks of 32 columns whose loads a warp has in flight
+constexpr int UNIT = SKIM_ORDER_UNIT;
+static_assert(UNIT == 64 && KC == 16 && OW == KC, "a lane takes two elements of a unit; the ordering kernel has a warp per label");
 
-template <bool VEC>
-__device__ __forceinline__ void load8(const ScaleArgs &a, int64_t row, int e0, Raw8 &r)
+// entries of the ordering kernel's place tables: sum over the labels of the largest class, about cols / 12 when
+// columns and labels are unrelated; rows that need more take the slow branch
+__host__ __device__ __forceinline__ int order_table_entries(int cols) { return cols / 6 + 256; }
+
+__host__ __device__ __forceinline__ size_t order_smem_bytes(int cols)
 {
+    return (size_t)skim_ordered_stride(cols) * sizeof(uint2) + (size_t)OW * KC * 32 * sizeof(uint16_t) + KC * 16 * sizeof(uint16_t) +
+           (size_t)order_table_entries(cols) * 4 + (3 * KC + 1) * sizeof(int);
+}
+
+// Of the 16 classes' counts (packed in tw): how many elements come before element i of class `cls`, i.e. the first
+// min(count, i) of every class and the i-th of the classes before it.
+__device__ __forceinline__ int order_place(const uint16_t *tot, uint32_t i, int cls)
+{
+    int before = 0;
+    for (int c = 0; c < 16; ++c) before += min((int)tot[c], (int)i) + ((c < cls && tot[c] > i) ? 1 : 0);
+    return before;
+}
+
+__global__ void __launch_bounds__(OT) skim_scale_order_kernel(ScaleArgs a)
+{
+    extern __shared__ __align__(16) unsigned char osmem[];
+    uint2 *row_out = reinterpret_cast<uint2 *>(osmem);                                              // the ordered row
+    uint16_t *cnt = reinterpret_cast<uint16_t *>(row_out + skim_ordered_stride(a.cols));           // [OW][KC][32] per lane and label
+    uint16_t *tot = cnt + OW * KC * 32;                                                              // [KC][16] per label and class
+    uint32_t *table = reinterpret_cast<uint32_t *>(tot + KC * 16);                                   // per label and i: elements before | classes with an i-th
+    int *base = reinterpret_cast<int *>(table + order_table_entries(a.cols));                        // [KC] first element of a label
+    int *members = base + KC;                                                                        // [KC]
+    int *tbase = members + KC;                                                                       // [KC] its table; [KC] all units
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t row = blockIdx.x;
     const uint16_t *Wr = a.W + row * a.ld;
     const float *Gr = a.G + row * a.ld;
     const uint8_t *Lr = a.labels + row * (int64_t)a.cols;
-    if (VEC && e0 + 8 <= a.cols) {
-        // the matrix streams through once per kernel: keep it from evicting alpha
-        r.w = __ldcs(reinterpret_cast<const uint4 *>(Wr + e0));
-        r.ga = __ldcs(reinterpret_cast<const float4 *>(Gr + e0));
-        r.gb = __ldcs(reinterpret_cast<const float4 *>(Gr + e0 + 4));
-        r.l = __ldcs(reinterpret_cast<const uint2 *>(Lr + e0));
+    uint16_t *mine = cnt + warp * KC * 32 + lane;                                                    // entry l at mine[l * 32]
 #pragma unroll
-        for (int u = 0; u < 4; ++u) r.al[u] = __ldg(reinterpret_cast<const double2 *>(a.alpha_il + alpha_il_pos(e0 + 2 * u)));
-    } else {
-        uint32_t ww[4] = {0u, 0u, 0u, 0u}, ll[2] = {0u, 0u};
-        float gg[8];
-        double aa[8];
+    for (int l = 0; l < KC; ++l) mine[l * 32] = 0;
+    __syncwarp();
+    // a warp takes 32 consecutive columns at a time, so a lane's columns are all of class lane % 16
+    const int chunks = (a.cols + 31) / 32;
+    for (int c0 = warp; c0 < chunks; c0 += OW * OB) {
+        int l[OB];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const bool in = e0 + u < a.cols;
-            ww[u >> 1] |= (in ? (uint32_t)Wr[e0 + u] : 0u) << (16 * (u & 1));
-            ll[u >> 2] |= (in ? (uint32_t)(Lr[e0 + u] & (KC - 1)) : 0u) << (8 * (u & 3));
-            gg[u] = in ? Gr[e0 + u] : 0.0f;
-            aa[u] = in ? a.alpha[e0 + u] : 1.0;
-        }
-        r.w = make_uint4(ww[0], ww[1], ww[2], ww[3]);
-        r.ga = make_float4(gg[0], gg[1], gg[2], gg[3]);
-        r.gb = make_float4(gg[4], gg[5], gg[6], gg[7]);
-        r.l = make_uint2(ll[0], ll[1]);
+        for (int u = 0; u < OB; ++u) l[u] = Lr[min((c0 + u * OW) * 32 + lane, a.cols - 1)] & (KC - 1);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) r.al[u] = make_double2(aa[2 * u], aa[2 * u + 1]);
+        for (int u = 0; u < OB; ++u)
+            if ((c0 + u * OW) * 32 + lane < a.cols) mine[l[u] * 32] += 1;
     }
-}
-
-// Adds W (2 or 4) elements' terms to the lane's accumulator slots.  The slots of a sum are read together and the
-// additions then run in element order in registers, an element whose cluster matches an earlier one of the
-// group continuing from that one's result: the same sums in the same order as one read-modify-write after
-// another, without the round trips through shared memory in a row.
-template <int NS, int W>
-__device__ __forceinline__ void add_group(double *slot, const int (&l)[8], const double (&cs)[NS][8], int u0)
-{
-    double v[NS][W];
-#pragma unroll
-    for (int s = 0; s < NS; ++s)
-#pragma unroll
-        for (int u = 0; u < W; ++u) v[s][u] = slot[(s * KC + l[u0 + u]) * 32];
-#pragma unroll
-    for (int s = 0; s < NS; ++s) {
-        double n[W];
-#pragma unroll
-        for (int u = 0; u < W; ++u) {
-            double base = v[s][u];
-#pragma unroll
-            for (int t = 0; t < u; ++t)
-                if (l[u0 + t] == l[u0 + u]) base = n[t];          // the latest earlier element of the cluster wins
-            n[u] = base + cs[s][u0 + u];
-        }
-        // in element order: where clusters repeat, the last store holds the full sum
-#pragma unroll
-        for (int u = 0; u < W; ++u) slot[(s * KC + l[u0 + u]) * 32] = n[u];
+    __syncthreads();
+    // thread (label, class): the counts of the class's 2 OW lanes become exclusive prefixes
+    if (tid < KC * 16) {
+        const int l = tid >> 4, cls = tid & 15;
+        int run = 0;
+        for (int w = 0; w < OW; ++w)
+            for (int h = 0; h < 2; ++h) {
+                uint16_t *p = cnt + (w * KC + l) * 32 + h * 16 + cls;
+                const int v = *p;
+                *p = (uint16_t)run;
+                run += v;
+            }
+        tot[tid] = (uint16_t)run;
     }
-}
-
-// INIT: the per-call constants (G_k, D_k) of every row.  Otherwise: (c_k, q_k) and the row's loss.
-template <bool INIT, bool VEC>
-__global__ void __launch_bounds__(SW * 32) skim_scale_sums_kernel(ScaleArgs a)
-{
-    extern __shared__ __align__(16) double slots_all[];       // [SW][NSUM * KC][32]
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t row = (int64_t)blockIdx.x * SW + warp;
-    if (row >= a.rows) return;
-    double *slot = slots_all + (size_t)warp * (NSUM * KC * 32) + lane;   // entry (s, k) at slot[(s * KC + k) * 32]
+    __syncthreads();
+    if (warp == 0) {
+        // units of every label, where its elements start, and where its place table does
+        int n = 0, most = 0;
+        if (lane < KC)
+            for (int c = 0; c < 16; ++c) {
+                n += tot[lane * 16 + c];
+                most = max(most, (int)tot[lane * 16 + c]);
+            }
+        const int units = (n + UNIT - 1) / UNIT;
+        int inc = units, tinc = most;
 #pragma unroll
-    for (int q = 0; q < NSUM * KC; ++q) slot[q * 32] = 0.0;
-    // the loads of the next step are issued before the current one is worked on
-    Raw8 cur, nxt;
-    if (lane * 8 < a.cols) load8<VEC>(a, row, lane * 8, cur);
-    for (int e0 = lane * 8; e0 < a.cols; e0 += 256) {
-        if (e0 + 256 < a.cols) load8<VEC>(a, row, e0 + 256, nxt);
-        const uint32_t ww[4] = {cur.w.x, cur.w.y, cur.w.z, cur.w.w};
-        const float g[8] = {cur.ga.x, cur.ga.y, cur.ga.z, cur.ga.w, cur.gb.x, cur.gb.y, cur.gb.z, cur.gb.w};
-        const double al[8] = {cur.al[0].x, cur.al[0].y, cur.al[1].x, cur.al[1].y, cur.al[2].x, cur.al[2].y, cur.al[3].x, cur.al[3].y};
-        int l[8];
-        double cs[INIT ? 2 : NSUM][8];
+        for (int off = 1; off < KC; off <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, inc, off), tt = __shfl_up_sync(0xffffffffu, tinc, off);
+            if (lane >= off) { inc += t; tinc += tt; }
+        }
+        if (lane < KC) {
+            base[lane] = (inc - units) * UNIT;
+            members[lane] = n;
+            tbase[lane] = tinc <= order_table_entries(a.cols) ? tinc - most : -1;      // -1: no room, the slow branch
+            a.ord_end[row * KC + lane] = (uint16_t)inc;
+        }
+        if (lane == KC - 1) tbase[KC] = inc;
+    }
+    __syncthreads();
+    const int total = tbase[KC] * UNIT;
+    // slot of position p: the two 32-element halves of a unit are interleaved, so that a lane's two elements are one
+    // 16-byte load and the warp's first (second) elements are 32 consecutive positions
+    auto slot = [](int p) { return (p & ~(UNIT - 1)) + 2 * (p & 31) + ((p >> 5) & 1); };
+    {
+        // warp l: the padding behind label l's elements, and its place table
+        const int l = warp, n = members[l];
+        for (int q = n + lane; q < (n + UNIT - 1) / UNIT * UNIT; q += 32) row_out[slot(base[l] + q)] = make_uint2(0u, 0u);
+        if (tbase[l] >= 0) {
+            int most = lane < 16 ? (int)tot[l * 16 + lane] : 0;
+            const int own = most;
+            most = __reduce_max_sync(0xffffffffu, most);
+            int run = 0;
+            for (int i0 = 0; i0 < most; i0 += 32) {
+                uint32_t have = 0u;
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const float wf = __half2float(__ushort_as_half((uint16_t)((u & 1) ? (ww[u >> 1] >> 16) : (ww[u >> 1] & 0xffffu))));
-            l[u] = (int)(((u < 4 ? cur.l.x : cur.l.y) >> (8 * (u & 3))) & (KC - 1));
-            const double gd = (double)g[u], wd = (double)wf;
-            const double gw = gd * wd;
-            if (INIT) {
-                cs[0][u] = gd;
-                cs[1][u] = gw * wd;
-            } else {
-                cs[0][u] = gw * rcp_pos(al[u]);
-                cs[1][u] = gw * al[u];
-                cs[2][u] = gd * al[u] * al[u];
+                for (int c = 0; c < 16; ++c) have |= (__shfl_sync(0xffffffffu, own, c) > i0 + lane ? 1u : 0u) << c;
+                const int pc = __popc(have);
+                int inc = pc;
+#pragma unroll
+                for (int off = 1; off < 32; off <<= 1) {
+                    const int t = __shfl_up_sync(0xffffffffu, inc, off);
+                    if (lane >= off) inc += t;
+                }
+                if (i0 + lane < most) table[tbase[l] + i0 + lane] = ((uint32_t)(run + inc - pc) << 16) | have;
+                run += __shfl_sync(0xffffffffu, inc, 31);
             }
         }
+    }
+    __syncthreads();
+    const uint32_t below = (1u << (lane & 15)) - 1u;           // classes before mine
+    for (int c0 = warp; c0 < chunks; c0 += OW * OB) {
+        int l[OB];
+        uint32_t w[OB];
+        float g[OB];
 #pragma unroll
-        for (int u0 = 0; u0 < 8; u0 += GW) add_group<INIT ? 2 : NSUM, GW>(slot, l, cs, u0);
-        cur = nxt;
+        for (int u = 0; u < OB; ++u) {
+            const int j = min((c0 + u * OW) * 32 + lane, a.cols - 1);
+            l[u] = Lr[j] & (KC - 1);
+            w[u] = Wr[j];
+            g[u] = Gr[j];
+        }
+#pragma unroll
+        for (int u = 0; u < OB; ++u) {
+            const int j = (c0 + u * OW) * 32 + lane;
+            if (j < a.cols) {
+                const uint32_t i = mine[l[u] * 32];
+                mine[l[u] * 32] = (uint16_t)(i + 1);
+                const int tb = tbase[l[u]];
+                int place;
+                if (tb >= 0) {
+                    const uint32_t e = table[tb + i];
+                    place = (int)(e >> 16) + __popc(e & below);
+                } else {
+                    place = order_place(tot + l[u] * 16, i, lane & 15);
+                }
+                const int pos = slot(base[l[u]] + place);
+                if (SKIM_IDX(pos, total, nullptr)) row_out[pos] = make_uint2(__float_as_uint(g[u]), (w[u] << 16) | (uint32_t)j);
+            }
+        }
     }
-    __syncwarp();
-    // lane L adds up entry L (and L + 32) over the 32 lanes' slots, starting at its own (no bank conflicts)
-    const double *base = slots_all + (size_t)warp * (NSUM * KC * 32);
-    double v0 = 0.0, v1 = 0.0;
-    for (int t = 0; t < 32; ++t) {
-        const int src = (t + lane) & 31;
-        v0 += base[lane * 32 + src];
-        if (lane < NSUM * KC - 32) v1 += base[(lane + 32) * 32 + src];
+    __syncthreads();
+    uint4 *dst = reinterpret_cast<uint4 *>(a.ord + row * skim_ordered_stride(a.cols));
+    const uint4 *src = reinterpret_cast<const uint4 *>(row_out);
+    for (int q = tid; q < total / 2; q += OT) dst[q] = src[q];
+}
+
+// ---------------------------------------------------------------- the sums of a step
+
+constexpr int SUM_T = 768;                 // threads per block of the sums kernel, one block per SM (80 registers)
+constexpr int SUM_W = SUM_T / 32;
+constexpr int AHEAD = 4;                   // units fetched together; two such batches take turns
+static_assert(AHEAD * 3 * UNIT * 8 <= SKIM_ORDER_SLACK, "a warp fetches up to three batches past its last unit");
+
+enum SumsMode { SUMS_INIT, SUMS_STEP, SUMS_CENTROIDS };
+
+// shared memory: alpha (not for INIT), then the warps' partial sums
+__host__ __device__ __forceinline__ size_t sums_smem_bytes(int cols, bool init)
+{
+    return (init ? 0 : ((size_t)cols + 1) / 2 * 16) + (size_t)SUM_W * 2 * 32 * sizeof(double);
+}
+
+// The two elements a lane has of a unit, added to its accumulators.
+template <int MODE>
+__device__ __forceinline__ void add_element(uint32_t gbits, uint32_t wcol, const double *alpha, double (&acc)[3])
+{
+    const double g = (double)__uint_as_float(gbits);
+    const double w = (double)__half2float(__ushort_as_half((uint16_t)(wcol >> 16)));
+    const double gw = g * w;
+    if (MODE == SUMS_INIT) {
+        acc[0] += g;
+        acc[1] = fma(gw, w, acc[1]);
+    } else {
+        const double al = alpha[wcol & 0xffffu];
+        acc[0] = fma(gw, rcp_pos(al), acc[0]);
+        if (MODE == SUMS_STEP) {
+            const double ga = g * al;
+            acc[1] = fma(ga, w, acc[1]);
+            acc[2] = fma(ga, al, acc[2]);
+        }
     }
-    // sums 0 and 1 of cluster k sit in lanes k and 16 + k (v0), sum 2 in lane k (v1)
-    const double s0 = v0, s1 = __shfl_sync(0xffffffffu, v0, (lane & 15) + 16), s2 = v1;
+}
+
+// One row's share of one warp: units [t0, t1) of its label-ordered elements.  The sums of cluster k come back in
+// lanes k (sum 0) and 16 + k (sum 1) of vx, and in lane k of vb (sum 2).
+template <int MODE>
+__device__ __forceinline__ void sum_units(const uint4 *src, int end, int t0, int t1, const double *alpha, double &vx, double &vb)
+{
+    const int lane = threadIdx.x & 31;
+    double acc[3] = {0.0, 0.0, 0.0};
+    vx = 0.0;
+    vb = 0.0;
+    int k = 0;
+    while (k < KC - 1 && __shfl_sync(0xffffffffu, end, k) <= t0) ++k;
+    int stop = min(__shfl_sync(0xffffffffu, end, k), t1);
+    src += (int64_t)t0 * (UNIT / 2) + lane;
+    uint4 buf[2][AHEAD];
+#pragma unroll
+    for (int u = 0; u < AHEAD; ++u) buf[0][u] = __ldcs(src + u * (UNIT / 2));
+    // Batches of AHEAD units take turns in two register buffers; the reads past the last unit stay inside the
+    // ordered matrix and its slack, and are not used.
+    for (int t = t0; t < t1; t += 2 * AHEAD) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+#pragma unroll
+            for (int u = 0; u < AHEAD; ++u) buf[h ^ 1][u] = __ldcs(src + ((h + 1) * AHEAD + u) * (UNIT / 2));
+#pragma unroll
+            for (int u = 0; u < AHEAD; ++u) {
+                if (t + h * AHEAD + u < t1) {
+                    add_element<MODE>(buf[h][u].x, buf[h][u].y, alpha, acc);
+                    add_element<MODE>(buf[h][u].z, buf[h][u].w, alpha, acc);
+                    if (t + h * AHEAD + u + 1 == stop) {
+                        // the cluster (or the share) ends here: sum 0 goes to the lower half-warp, sum 1 to the upper
+                        double x = lane < 16 ? acc[0] : acc[1];
+                        if (MODE != SUMS_CENTROIDS) x += __shfl_xor_sync(0xffffffffu, lane < 16 ? acc[1] : acc[0], 16);
+                        else x = acc[0] + __shfl_xor_sync(0xffffffffu, acc[0], 16);
+                        double b = acc[2];
+                        if (MODE == SUMS_STEP) b += __shfl_xor_sync(0xffffffffu, b, 16);
+#pragma unroll
+                        for (int off = 8; off; off >>= 1) {
+                            x += __shfl_xor_sync(0xffffffffu, x, off);
+                            if (MODE == SUMS_STEP) b += __shfl_xor_sync(0xffffffffu, b, off);
+                        }
+                        if ((lane & 15) == k) { vx = x; vb = b; }
+                        acc[0] = acc[1] = acc[2] = 0.0;
+                        const int done = stop;
+                        while (k < KC - 1 && __shfl_sync(0xffffffffu, end, k) <= done) ++k;
+                        stop = min(__shfl_sync(0xffffffffu, end, k), t1);
+                    }
+                }
+            }
+        }
+        src += 2 * AHEAD * (UNIT / 2);
+    }
+}
+
+// What the sums of a row are turned into (lanes as sum_units leaves them).
+//   SUMS_INIT       the per-call constants (G_k, D_k)
+//   SUMS_STEP       (c_k, q_k) and the row's loss
+//   SUMS_CENTROIDS  (c_k, 0)
+template <int MODE>
+__device__ __forceinline__ void finish_row(const ScaleArgs &a, int64_t row, double vx, double vb)
+{
+    const int lane = threadIdx.x & 31;
+    const double s1 = __shfl_down_sync(0xffffffffu, vx, 16);
     double loss_k = 0.0;
     if (lane < KC) {
-        if (INIT) {
-            a.tconst[row * KC + lane] = make_double2(s0, s1);
+        if (MODE == SUMS_INIT) {
+            a.tconst[row * KC + lane] = make_double2(vx, s1);
         } else {
             const double2 gdk = a.tconst[row * KC + lane];
             double c = 0.0, q = 0.0;
             if (gdk.x > 0.0) {
-                c = s0 / gdk.x;
-                q = 2.0 * (s1 - c * s2) / gdk.x;
-                loss_k = gdk.y - 2.0 * c * s1 + c * c * s2;
+                c = vx / gdk.x;
+                if (MODE == SUMS_STEP) {
+                    q = 2.0 * (s1 - c * vb) / gdk.x;
+                    loss_k = gdk.y - 2.0 * c * s1 + c * c * vb;
+                }
             }
             a.tq[row * KC + lane] = make_double2(c, q);
         }
     }
-    if (!INIT) {
+    if (MODE == SUMS_STEP) {
 #pragma unroll
         for (int off = 8; off; off >>= 1) loss_k += __shfl_down_sync(0xffffffffu, loss_k, off);
         if (lane == 0) a.loss_row[row] = loss_k;
     }
 }
 
-// The W, G and label entries of one thread's four columns in RB consecutive rows, as loaded.
-template <int RB>
-struct GradRows {
-    uint2 wv[RB];
-    float4 gv[RB];
-    uint32_t lv[RB];
-};
-
-template <bool VEC, int RB>
-__device__ __forceinline__ void grad_load(const ScaleArgs &a, int64_t rb, int64_t r1, int j0, bool full, GradRows<RB> &r)
+// One block per SM, rows dealt round-robin to the blocks.  A warp takes whole rows while there are rows for all of the
+// block's warps; the rows that are left are shared by the warps in equal stretches, whose sums meet in shared memory in a
+// fixed order.  Bound by HBM: 8 B an element.
+template <int MODE>
+__global__ void __launch_bounds__(SUM_T, 1) skim_scale_sums_kernel(ScaleArgs a)
 {
-#pragma unroll
-    for (int q = 0; q < RB; ++q) {
-        const int64_t row = rb + q;
-        r.wv[q] = make_uint2(0u, 0u); r.gv[q] = make_float4(0.f, 0.f, 0.f, 0.f); r.lv[q] = 0u;
-        if (row < r1 && j0 < a.cols) {
-            const uint16_t *Wr = a.W + row * a.ld + j0;
-            const float *Gr = a.G + row * a.ld + j0;
-            const uint8_t *Lr = a.labels + row * (int64_t)a.cols + j0;
-            if (full) {
-                r.wv[q] = __ldcs(reinterpret_cast<const uint2 *>(Wr));
-                r.gv[q] = __ldcs(reinterpret_cast<const float4 *>(Gr));
-                r.lv[q] = __ldcs(reinterpret_cast<const uint32_t *>(Lr));
-            } else {
-                uint32_t ww[2] = {0u, 0u};
-                float gg[GC];
-#pragma unroll
-                for (int u = 0; u < GC; ++u) {
-                    const bool in = j0 + u < a.cols;
-                    ww[u >> 1] |= (in ? (uint32_t)Wr[u] : 0u) << (16 * (u & 1));
-                    r.lv[q] |= (in ? (uint32_t)(Lr[u] & (KC - 1)) : 0u) << (8 * u);
-                    gg[u] = in ? Gr[u] : 0.0f;
-                }
-                r.wv[q] = make_uint2(ww[0], ww[1]);
-                r.gv[q] = make_float4(gg[0], gg[1], gg[2], gg[3]);
-            }
+    extern __shared__ __align__(16) double ssmem[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double *alpha = ssmem;
+    double2 *part = reinterpret_cast<double2 *>(ssmem + (MODE == SUMS_INIT ? 0 : (a.cols + 1) / 2 * 2));     // [SUM_W][32]
+    let_next_kernel_start();
+    wait_for_previous_kernel();
+    if (MODE != SUMS_INIT) {
+        for (int q = threadIdx.x; q < a.cols / 2; q += SUM_T)
+            reinterpret_cast<double2 *>(alpha)[q] = __ldg(reinterpret_cast<const double2 *>(a.alpha) + q);
+        if ((a.cols & 1) && threadIdx.x == 0) alpha[a.cols - 1] = a.alpha[a.cols - 1];
+        __syncthreads();
+    }
+    const int64_t stride = skim_ordered_stride(a.cols) / 2;
+    const int mine = (int)((a.rows - blockIdx.x + gridDim.x - 1) / gridDim.x);       // rows of this block (at least one)
+    const int whole = mine / SUM_W * SUM_W, rest = mine - whole;
+    double vx, vb;
+    for (int r = warp; r < whole; r += SUM_W) {
+        const int64_t row = blockIdx.x + (int64_t)gridDim.x * r;
+        const int end = a.ord_end[row * KC + (lane & 15)];
+        sum_units<MODE>(reinterpret_cast<const uint4 *>(a.ord) + row * stride, end, 0, __shfl_sync(0xffffffffu, end, KC - 1), alpha, vx, vb);
+        finish_row<MODE>(a, row, vx, vb);
+    }
+    if (rest == 0) return;
+    const int per_row = SUM_W / rest, idx = warp / per_row, sub = warp - idx * per_row;
+    const int64_t row = blockIdx.x + (int64_t)gridDim.x * (whole + idx);
+    if (idx < rest) {
+        const int end = a.ord_end[row * KC + (lane & 15)];
+        const int total = __shfl_sync(0xffffffffu, end, KC - 1);
+        const int t0 = total * sub / per_row, t1 = total * (sub + 1) / per_row;
+        sum_units<MODE>(reinterpret_cast<const uint4 *>(a.ord) + row * stride, end, t0, t1, alpha, vx, vb);
+        part[threadIdx.x] = make_double2(vx, vb);
+    }
+    __syncthreads();
+    if (idx < rest && sub == 0) {
+        for (int q = 1; q < per_row; ++q) {
+            const double2 o = part[threadIdx.x + 32 * q];
+            vx += o.x;
+            vb += o.y;
         }
+        finish_row<MODE>(a, row, vx, vb);
     }
 }
 
+// ---------------------------------------------------------------- the gradient of a step
+//
+// A thread owns four columns and walks a range of rows.  The (c_k, q_k) entry of an element comes by four 32-bit
+// shuffles from the row's table, which sits in the lanes (reading 16-byte entries from shared memory by label costs
+// about nine wavefronts a warp, and a barrier per batch of rows); warps do not wait for one another.  Two blocks are resident
+// per SM and the grid is one wave of them.  HBM traffic: 7 B an element.
 template <bool VEC>
-__global__ void __launch_bounds__(GT) skim_scale_grad_kernel(ScaleArgs a)
+struct GradCols {
+    int j[VEC ? 1 : GC];          // columns as loaded: clamped to the matrix, so that no load needs a guard
+    bool in[VEC ? 1 : GC];
+    // VEC: four consecutive columns (cols % 4 == 0: all inside or all outside).  Otherwise four columns a block width
+    // apart, so that scalar loads are contiguous across a warp.
+    __device__ __forceinline__ GradCols(int tile, int cols)
+    {
+        if constexpr (VEC) {
+            const int c = (tile * GT + threadIdx.x) * GC;
+            in[0] = c < cols;
+            j[0] = min(c, cols - GC);
+        } else {
+#pragma unroll
+            for (int u = 0; u < GC; ++u) {
+                const int c = (tile * GC + u) * GT + threadIdx.x;
+                in[u] = c < cols;
+                j[u] = min(c, cols - 1);
+            }
+        }
+    }
+    __device__ __forceinline__ int col(int u) const { return VEC ? j[0] + u : j[VEC ? 0 : u]; }
+    __device__ __forceinline__ bool inside(int u) const { return in[VEC ? 0 : u]; }
+};
+
+// One row's entries at a thread's columns.
+struct GradRow {
+    uint2 w;
+    float4 g;
+    uint32_t l;
+};
+
+template <bool VEC>
+__device__ __forceinline__ void grad_load(const ScaleArgs &a, int64_t row, const GradCols<VEC> &c, GradRow &r)
 {
-    // Rows go by in batches of RB.  While a batch is worked on, the next batch's loads are in flight and its
-    // (c_k, q_k) tables wait in a register of the first RB * KC threads; the tables alternate between two buffers,
-    // so one barrier per batch is enough.
-    constexpr int RB = 4;
-    __shared__ double2 tq_s[2][RB * KC];
-    const int j0 = (blockIdx.x * GT + threadIdx.x) * GC;
+    const uint16_t *Wr = a.W + row * a.ld;
+    const float *Gr = a.G + row * a.ld;
+    const uint8_t *Lr = a.labels + row * (int64_t)a.cols;
+    if constexpr (VEC) {
+        r.w = __ldcs(reinterpret_cast<const uint2 *>(Wr + c.j[0]));
+        r.g = __ldcs(reinterpret_cast<const float4 *>(Gr + c.j[0]));
+        r.l = __ldcs(reinterpret_cast<const uint32_t *>(Lr + c.j[0]));
+    } else {
+        r.w = make_uint2((uint32_t)__ldcs(Wr + c.j[0]) | ((uint32_t)__ldcs(Wr + c.j[1]) << 16),
+                         (uint32_t)__ldcs(Wr + c.j[2]) | ((uint32_t)__ldcs(Wr + c.j[3]) << 16));
+        r.g = make_float4(__ldcs(Gr + c.j[0]), __ldcs(Gr + c.j[1]), __ldcs(Gr + c.j[2]), __ldcs(Gr + c.j[3]));
+        r.l = (uint32_t)__ldcs(Lr + c.j[0]) | ((uint32_t)__ldcs(Lr + c.j[1]) << 8) | ((uint32_t)__ldcs(Lr + c.j[2]) << 16) |
+              ((uint32_t)__ldcs(Lr + c.j[3]) << 24);
+    }
+}
+
+__device__ __forceinline__ double weight_of(const uint2 &w, int u)
+{
+    const uint32_t x = u < 2 ? w.x : w.y;
+    return (double)__half2float(__ushort_as_half((uint16_t)((u & 1) ? (x >> 16) : (x & 0xffffu))));
+}
+
+// The tables of two rows in one register pair: lane L holds entry L % 16 of row `row` + L / 16.
+__device__ __forceinline__ double2 table_load(const ScaleArgs &a, int64_t row, int64_t last)
+{
+    const int lane = threadIdx.x & 31;
+    return a.tq[min(row + (lane >> 4), last) * KC + (lane & 15)];
+}
+// Shuffle indices of four labels: byte u holds label u, plus 16 for the second row of the pair (a shuffle takes the
+// low five bits of its index, so `>> 8 u` is all an element needs).
+__device__ __forceinline__ uint32_t table_index(uint32_t l, int second) { return (l & 0x0f0f0f0fu) | (second ? 0x10101010u : 0u); }
+__device__ __forceinline__ double2 table_get(const double2 &t, uint32_t index, int u)
+{
+    const int src = (int)(index >> (8 * u));
+    return make_double2(__shfl_sync(0xffffffffu, t.x, src), __shfl_sync(0xffffffffu, t.y, src));
+}
+
+template <bool VEC>
+__global__ void __launch_bounds__(GT, 2) skim_scale_grad_kernel(ScaleArgs a)
+{
+    constexpr int RB = VEC ? 4 : 2;   // rows of a batch (four column addresses leave fewer registers); two batches take turns in registers, one of them in flight
+    const GradCols<VEC> c(blockIdx.x, a.cols);
     const int64_t r0 = (int64_t)blockIdx.y * a.rows_per_range;
-    const int64_t r1 = min(a.rows, r0 + a.rows_per_range);
-    double al[GC], rr[GC], acc[GC];
+    const int64_t r1 = min(a.rows, r0 + a.rows_per_range), last = r1 - 1;
+    GradRow row[2][RB];
+    double2 tab[2][RB / 2];
+    auto fetch_rows = [&](int h, int64_t rb) {
+#pragma unroll
+        for (int q = 0; q < RB; ++q) grad_load<VEC>(a, min(rb + q, last), c, row[h][q]);
+    };
+    auto fetch_tables = [&](int h, int64_t rb) {
+#pragma unroll
+        for (int q = 0; q < RB / 2; ++q) tab[h][q] = table_load(a, rb + 2 * q, last);
+    };
+    let_next_kernel_start();
+    fetch_rows(0, r0);
+    wait_for_previous_kernel();
+    fetch_tables(0, r0);
+    double ah[GC], rr[GC], acc[GC];   // alpha / 2, alpha^-2
 #pragma unroll
     for (int u = 0; u < GC; ++u) {
-        al[u] = j0 + u < a.cols ? a.alpha[j0 + u] : 1.0;
-        const double r = __drcp_rn(al[u]);
+        const double al = a.alpha[c.col(u)], r = __drcp_rn(al);
+        ah[u] = 0.5 * al;
         rr[u] = r * r;
         acc[u] = 0.0;
     }
-    const bool full = VEC && j0 + GC <= a.cols;
-    const bool tq_thread = threadIdx.x < RB * KC;
-    GradRows<RB> cur, nxt;
-    grad_load<VEC, RB>(a, r0, r1, j0, full, cur);
-    if (tq_thread && r0 + threadIdx.x / KC < r1) tq_s[0][threadIdx.x] = a.tq[r0 * KC + threadIdx.x];
-    int buf = 0;
-    for (int64_t rb = r0; rb < r1; rb += RB, buf ^= 1) {
-        const int64_t rn = rb + RB;
-        double2 tnext = make_double2(0.0, 0.0);
-        if (rn < r1) {
-            grad_load<VEC, RB>(a, rn, r1, j0, full, nxt);
-            if (tq_thread && rn + threadIdx.x / KC < r1) tnext = a.tq[rn * KC + threadIdx.x];
-        }
-        __syncthreads();                        // this batch's tables are in place; the other buffer is no longer read
+    for (int64_t rb = r0; rb < r1; rb += 2 * RB) {
 #pragma unroll
-        for (int q = 0; q < RB; ++q) {
-            const int64_t row = rb + q;
-            if (row >= r1) break;
-            const double2 *tq = tq_s[buf] + q * KC;
-            const uint32_t ww[2] = {cur.wv[q].x, cur.wv[q].y};
-            const float g[GC] = {cur.gv[q].x, cur.gv[q].y, cur.gv[q].z, cur.gv[q].w};
+        for (int h = 0; h < 2; ++h) {
+            fetch_rows(h ^ 1, rb + (h + 1) * RB);
+            fetch_tables(h ^ 1, rb + (h + 1) * RB);
 #pragma unroll
-            for (int u = 0; u < GC; ++u) {
-                const double2 cq = tq[(cur.lv[q] >> (8 * u)) & (KC - 1)];
-                const double gd = (double)g[u];
-                const double wd = (double)__half2float(__ushort_as_half((uint16_t)((u & 1) ? (ww[u >> 1] >> 16) : (ww[u >> 1] & 0xffffu))));
-                const double res = wd - al[u] * cq.x;
-                acc[u] += gd * (cq.y * wd * rr[u] - 2.0 * cq.x * res);
+            for (int q = 0; q < RB; ++q) {
+                if (rb + h * RB + q < r1) {
+                    const float g[GC] = {row[h][q].g.x, row[h][q].g.y, row[h][q].g.z, row[h][q].g.w};
+                    const uint32_t index = table_index(row[h][q].l, q & 1);
+#pragma unroll
+                    for (int u = 0; u < GC; ++u) {
+                        // g (q w / alpha^2 - 2 c (w - alpha c)) with d = 2 c:  g (w (q / alpha^2 - d) + d (d alpha / 2))
+                        const double2 cq = table_get(tab[h][q >> 1], index, u);
+                        const double d = cq.x + cq.x;
+                        const double t = fma(weight_of(row[h][q].w, u), fma(cq.y, rr[u], -d), d * (d * ah[u]));
+                        acc[u] = fma((double)g[u], t, acc[u]);
+                    }
+                }
             }
         }
-        if (tq_thread) tq_s[buf ^ 1][threadIdx.x] = tnext;
-        cur = nxt;
     }
 #pragma unroll
     for (int u = 0; u < GC; ++u)
-        if (j0 + u < a.cols) a.grad_part[(int64_t)blockIdx.y * a.cols + j0 + u] = acc[u];
+        if (c.inside(u)) a.grad_part[(int64_t)blockIdx.y * a.cols + c.col(u)] = acc[u];
 }
 
 __global__ void __launch_bounds__(256) skim_scale_adam_kernel(const double *__restrict__ grad_part,
@@ -318,6 +553,8 @@ __global__ void __launch_bounds__(256) skim_scale_adam_kernel(const double *__re
                                                                double bc1, double bc2, double eps, double *loss_out)
 {
     __shared__ double red[256];
+    let_next_kernel_start();
+    wait_for_previous_kernel();
     if (blockIdx.x == gridDim.x - 1) {
         // the last block adds the rows' losses: strided partial sums, then a fixed tree
         double s = 0.0;
@@ -388,51 +625,30 @@ struct ScaleLfArgs {
     int exp2;
 };
 
-// One warp per row: S_k = sum g w / alpha per cluster, c_k = S_k / G_k, then the row of D.
+// The residual as the operand of the contraction: one warp per stretch of RES_COLS columns of a row.
+constexpr int RES_COLS = 2048;
+
 __global__ void __launch_bounds__(SW * 32) skim_scale_lf_residual_kernel(ScaleLfArgs b)
 {
-    extern __shared__ __align__(16) double slots_all[];       // [SW][KC][32], then [SW][KC] centroids
+    __shared__ double cs_all[SW][KC];
     const ScaleArgs &a = b.s;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t row = (int64_t)blockIdx.x * SW + warp;
+    const int parts = (a.cols + RES_COLS - 1) / RES_COLS;
+    const int64_t unit = (int64_t)blockIdx.x * SW + warp, row = unit / parts;
     if (row >= a.rows) return;
-    double *slot = slots_all + (size_t)warp * (KC * 32) + lane;
-    double *cs = slots_all + (size_t)SW * (KC * 32) + warp * KC;
-#pragma unroll
-    for (int q = 0; q < KC; ++q) slot[q * 32] = 0.0;
-    Raw8 cur, nxt;
-    if (lane * 8 < a.cols) load8<true>(a, row, lane * 8, cur);
-    for (int e0 = lane * 8; e0 < a.cols; e0 += 256) {
-        if (e0 + 256 < a.cols) load8<true>(a, row, e0 + 256, nxt);
-        const uint32_t ww[4] = {cur.w.x, cur.w.y, cur.w.z, cur.w.w};
-        const float g[8] = {cur.ga.x, cur.ga.y, cur.ga.z, cur.ga.w, cur.gb.x, cur.gb.y, cur.gb.z, cur.gb.w};
-        const double al[8] = {cur.al[0].x, cur.al[0].y, cur.al[1].x, cur.al[1].y, cur.al[2].x, cur.al[2].y, cur.al[3].x, cur.al[3].y};
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const float wf = __half2float(__ushort_as_half((uint16_t)((u & 1) ? (ww[u >> 1] >> 16) : (ww[u >> 1] & 0xffffu))));
-            const int l = (int)(((u < 4 ? cur.l.x : cur.l.y) >> (8 * (u & 3))) & (KC - 1));
-            slot[l * 32] += ((double)g[u] * (double)wf) * rcp_pos(al[u]);
-        }
-        cur = nxt;
-    }
-    __syncwarp();
-    if (lane < KC) {
-        const double *base = slots_all + (size_t)warp * (KC * 32) + lane * 32;
-        double v = 0.0;
-        for (int t = 0; t < 32; ++t) v += base[(t + lane) & 31];
-        const double gk = a.tconst[row * KC + lane].x;
-        const double c = gk > 0.0 ? v / gk : 0.0;
-        cs[lane] = c;
-        a.tq[row * KC + lane] = make_double2(c, 0.0);
-    }
+    const int j0 = (int)(unit % parts) * RES_COLS, j1 = min(j0 + RES_COLS, a.cols);
+    double *cs = cs_all[warp];
+    let_next_kernel_start();
+    wait_for_previous_kernel();
+    if (lane < KC) cs[lane] = a.tq[row * KC + lane].x;
     __syncwarp();
     const float scale = __int_as_float((127 + b.exp2) << 23);
     const uint16_t *Wr = a.W + row * a.ld;
     const uint8_t *Lr = a.labels + row * (int64_t)a.cols;
     uint16_t *Dr = b.D + row * (int64_t)a.cols;
-    for (int e0 = lane * 8; e0 < a.cols; e0 += 256) {
-        const uint4 wv = *reinterpret_cast<const uint4 *>(Wr + e0);
-        const uint2 lv = *reinterpret_cast<const uint2 *>(Lr + e0);
+    for (int e0 = j0 + lane * 8; e0 < j1; e0 += 256) {
+        const uint4 wv = __ldcs(reinterpret_cast<const uint4 *>(Wr + e0));
+        const uint2 lv = __ldcs(reinterpret_cast<const uint2 *>(Lr + e0));
         double al[8];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
@@ -461,6 +677,8 @@ __global__ void __launch_bounds__(SW * 32) skim_scale_lf_r_kernel(ScaleLfArgs b)
     const ScaleArgs &a = b.s;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t row = (int64_t)blockIdx.x * SW + warp;
+    let_next_kernel_start();
+    wait_for_previous_kernel();
     if (row >= a.rows) return;
     double *slot = slots_all + (size_t)warp * (KC * 32) + lane;
 #pragma unroll
@@ -496,84 +714,62 @@ __global__ void __launch_bounds__(SW * 32) skim_scale_lf_r_kernel(ScaleLfArgs b)
     }
 }
 
-// A thread owns four columns and walks a range of rows: sum_i -2 Y_ij c + q g w / alpha_j^2.  Batches of RB rows,
-// the next batch's loads in flight and its tables parked in registers, as in skim_scale_grad_kernel.
-template <int RB>
-struct GradRowsLf {
-    uint2 wv[RB];
-    float4 gv[RB], yv[RB];
-    uint32_t lv[RB];
-};
-
-template <int RB>
-__device__ __forceinline__ void grad_load_lf(const ScaleLfArgs &b, int64_t rb, int64_t r1, int j0, bool in, GradRowsLf<RB> &r)
-{
-    const ScaleArgs &a = b.s;
-#pragma unroll
-    for (int q = 0; q < RB; ++q) {
-        const int64_t row = rb + q;
-        r.wv[q] = make_uint2(0u, 0u); r.gv[q] = make_float4(0.f, 0.f, 0.f, 0.f); r.yv[q] = r.gv[q]; r.lv[q] = 0u;
-        if (row < r1 && in) {
-            r.wv[q] = __ldcs(reinterpret_cast<const uint2 *>(a.W + row * a.ld + j0));
-            r.gv[q] = __ldcs(reinterpret_cast<const float4 *>(a.G + row * a.ld + j0));
-            r.yv[q] = __ldcs(reinterpret_cast<const float4 *>(b.Y + row * (int64_t)a.cols + j0));
-            r.lv[q] = __ldcs(reinterpret_cast<const uint32_t *>(a.labels + row * (int64_t)a.cols + j0));
-        }
-    }
-}
-
+// A thread owns four columns and walks a range of rows: sum_i -2 Y_ij c + q g w / alpha_j^2; as skim_scale_grad_kernel
+// (cols is a multiple of 8 and the rows are aligned: vector loads always).
 __global__ void __launch_bounds__(GT, 2) skim_scale_lf_grad_kernel(ScaleLfArgs b)
 {
     constexpr int RB = 2;
-    __shared__ double2 tq_s[2][RB * KC];
     const ScaleArgs &a = b.s;
-    const int j0 = (blockIdx.x * GT + threadIdx.x) * GC;
+    const GradCols<true> c(blockIdx.x, a.cols);
     const int64_t r0 = (int64_t)blockIdx.y * a.rows_per_range;
-    const int64_t r1 = min(a.rows, r0 + a.rows_per_range);
-    const double yscale = ldexp(1.0, -b.exp2);
+    const int64_t r1 = min(a.rows, r0 + a.rows_per_range), last = r1 - 1;
+    const double ys = ldexp(-2.0, -b.exp2);
+    let_next_kernel_start();
+    wait_for_previous_kernel();
     double rr[GC], acc[GC];
 #pragma unroll
     for (int u = 0; u < GC; ++u) {
-        const double al = j0 + u < a.cols ? a.alpha[j0 + u] : 1.0;
-        const double r = __drcp_rn(al);
+        const double r = __drcp_rn(a.alpha[c.col(u)]);
         rr[u] = r * r;
         acc[u] = 0.0;
     }
-    const bool in = j0 + GC <= a.cols;           // cols is a multiple of 8: a thread's columns are all inside or all outside
-    const bool tq_thread = threadIdx.x < RB * KC;
-    GradRowsLf<RB> cur, nxt;
-    grad_load_lf<RB>(b, r0, r1, j0, in, cur);
-    if (tq_thread && r0 + threadIdx.x / KC < r1) tq_s[0][threadIdx.x] = a.tq[r0 * KC + threadIdx.x];
-    int buf = 0;
-    for (int64_t rb = r0; rb < r1; rb += RB, buf ^= 1) {
-        const int64_t rn = rb + RB;
-        double2 tnext = make_double2(0.0, 0.0);
-        if (rn < r1) {
-            grad_load_lf<RB>(b, rn, r1, j0, in, nxt);
-            if (tq_thread && rn + threadIdx.x / KC < r1) tnext = a.tq[rn * KC + threadIdx.x];
-        }
-        __syncthreads();                        // this batch's tables are in place; the other buffer is no longer read
+    GradRow row[2][RB];
+    float4 yv[2][RB];
+    double2 tab[2];
+    auto fetch = [&](int h, int64_t rb) {
 #pragma unroll
         for (int q = 0; q < RB; ++q) {
-            if (rb + q >= r1) break;
-            const double2 *tq = tq_s[buf] + q * KC;
-            const uint32_t ww[2] = {cur.wv[q].x, cur.wv[q].y};
-            const float g[GC] = {cur.gv[q].x, cur.gv[q].y, cur.gv[q].z, cur.gv[q].w};
-            const float y[GC] = {cur.yv[q].x, cur.yv[q].y, cur.yv[q].z, cur.yv[q].w};
+            const int64_t i = min(rb + q, last);
+            grad_load<true>(a, i, c, row[h][q]);
+            yv[h][q] = __ldcs(reinterpret_cast<const float4 *>(b.Y + i * (int64_t)a.cols + c.j[0]));
+        }
+        tab[h] = table_load(a, rb, last);
+        tab[h].x *= ys;                 // -2 c / 2^exp2
+    };
+    fetch(0, r0);
+    for (int64_t rb = r0; rb < r1; rb += 2 * RB) {
 #pragma unroll
-            for (int u = 0; u < GC; ++u) {
-                const double2 cq = tq[(cur.lv[q] >> (8 * u)) & (KC - 1)];
-                const double wd = (double)__half2float(__ushort_as_half((uint16_t)((u & 1) ? (ww[u >> 1] >> 16) : (ww[u >> 1] & 0xffffu))));
-                acc[u] += cq.y * (double)g[u] * wd * rr[u] - 2.0 * ((double)y[u] * yscale) * cq.x;
+        for (int h = 0; h < 2; ++h) {
+            fetch(h ^ 1, rb + (h + 1) * RB);
+#pragma unroll
+            for (int q = 0; q < RB; ++q) {
+                if (rb + h * RB + q < r1) {
+                    const float g[GC] = {row[h][q].g.x, row[h][q].g.y, row[h][q].g.z, row[h][q].g.w};
+                    const float y[GC] = {yv[h][q].x, yv[h][q].y, yv[h][q].z, yv[h][q].w};
+                    const uint32_t index = table_index(row[h][q].l, q & 1);
+#pragma unroll
+                    for (int u = 0; u < GC; ++u) {
+                        const double2 cq = table_get(tab[h], index, u);
+                        acc[u] = fma((double)y[u], cq.x, acc[u]);
+                        acc[u] = fma((cq.y * rr[u]) * (double)g[u], weight_of(row[h][q].w, u), acc[u]);
+                    }
+                }
             }
         }
-        if (tq_thread) tq_s[buf ^ 1][threadIdx.x] = tnext;
-        cur = nxt;
     }
-    if (in) {
 #pragma unroll
-        for (int u = 0; u < GC; ++u) a.grad_part[(int64_t)blockIdx.y * a.cols + j0 + u] = acc[u];
-    }
+    for (int u = 0; u < GC; ++u)
+        if (c.inside(u)) a.grad_part[(int64_t)blockIdx.y * a.cols + c.col(u)] = acc[u];
 }
 
 }  // namespace
@@ -583,18 +779,42 @@ size_t skim_scale_lfull_scratch_bytes(int64_t rows, int64_t cols)
     return skim_align256((size_t)rows * cols * 2) + skim_align256((size_t)rows * cols * 4) + skim_lfull_scratch_bytes(rows, cols);
 }
 
-int skim_launch_scale_update_lfull(skim_ctx *ctx, const uint16_t *W, const float *importance, int64_t rows, int64_t cols,
-                                   int64_t ld, const uint8_t *labels, const uint16_t *H, int64_t ldh, float *alpha,
-                                   int steps, float lr0, float decay, int decay_every, int exp2, void *scratch,
-                                   double *loss_trace)
+namespace {
+
+// What both updates do first: alpha's master copies, the label-ordered matrix, the per-call constants (G_k, D_k).
+// Launches `kernel` as a programmatic dependent of the kernel before it on the stream.
+template <typename... Params, typename... Args>
+int launch_dependent(skim_ctx *ctx, void (*kernel)(Params...), dim3 grid, unsigned threads, size_t smem, Args... args)
 {
-    SkimWorkspace ws = skim_carve(ctx->ws, rows, cols);
-    const unsigned cb = (unsigned)((cols + 255) / 256), ab = (unsigned)((cols + 31) / 32);   // Adam: 32 columns a block
-    skim_scale_init_kernel<<<cb, 256, 0, ctx->stream>>>(alpha, (int)cols, ws.alpha64, ws.alpha_il, ws.adam_m, ws.adam_v, ws.status);
-    SKIM_CUDA_OK(cudaGetLastError());
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = ctx->stream;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    SKIM_CUDA_OK(cudaLaunchKernelEx(&cfg, kernel, args...));
     ctx->launches += 1;
-    ScaleLfArgs b;
-    ScaleArgs &a = b.s;
+    return SKIM_OK;
+}
+
+struct ScalePlan {
+    ScaleArgs a;
+    unsigned cb, ab;                 // blocks over the columns; Adam: 32 columns a block
+    dim3 grad_grid;
+    int ranges;
+    unsigned sum_blocks;
+};
+
+int scale_begin(skim_ctx *ctx, const SkimWorkspace &ws, const uint16_t *W, const float *importance, int64_t rows, int64_t cols,
+                int64_t ld, const uint8_t *labels, const float *alpha, ScalePlan *p)
+{
+    p->cb = (unsigned)((cols + 255) / 256);
+    p->ab = (unsigned)((cols + 31) / 32);
+    ScaleArgs &a = p->a;
     a.W = W;
     a.G = importance;
     a.labels = labels;
@@ -603,11 +823,83 @@ int skim_launch_scale_update_lfull(skim_ctx *ctx, const uint16_t *W, const float
     a.rows = rows;
     a.ld = ld;
     a.cols = (int)cols;
-    a.vec = 1;
+    a.vec = ((reinterpret_cast<uintptr_t>(W) & 7u) == 0 && (reinterpret_cast<uintptr_t>(importance) & 15u) == 0 &&
+             (reinterpret_cast<uintptr_t>(labels) & 3u) == 0 && ld % 4 == 0 && cols % 4 == 0) ? 1 : 0;
+    a.ord = reinterpret_cast<uint2 *>(ws.cluster_scratch);
+    a.ord_end = ws.scale_ord_end;
     a.tconst = reinterpret_cast<double2 *>(ws.scale_const);
     a.tq = reinterpret_cast<double2 *>(ws.scale_cq);
     a.loss_row = ws.loss_part;
     a.grad_part = ws.grad_part;
+    // gradient kernels: column tiles x row ranges, one wave of two blocks per SM
+    const int tiles = (int)((cols + GT * GC - 1) / (GT * GC));
+    int ranges = 2 * ctx->sm_count / tiles;
+    if (ranges > SKIM_SCALE_MAX_CTAS) ranges = SKIM_SCALE_MAX_CTAS;
+    if (ranges > rows) ranges = (int)rows;
+    if (ranges < 1) ranges = 1;
+    a.rows_per_range = (int)((rows + ranges - 1) / ranges);
+    p->ranges = (int)((rows + a.rows_per_range - 1) / a.rows_per_range);
+    p->grad_grid = dim3((unsigned)tiles, (unsigned)p->ranges);
+    // sums kernel: one block per SM
+    p->sum_blocks = (unsigned)(rows < ctx->sm_count ? rows : ctx->sm_count);
+    // set on every launch: host-side calls of microseconds, and no state shared between contexts
+    const int sm_order = (int)order_smem_bytes((int)cols), sm_init = (int)sums_smem_bytes((int)cols, true), sm_sums = (int)sums_smem_bytes((int)cols, false);
+    SKIM_CUDA_OK(cudaFuncSetAttribute(skim_scale_order_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sm_order));
+    SKIM_CUDA_OK(cudaFuncSetAttribute(skim_scale_sums_kernel<SUMS_INIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm_init));
+    SKIM_CUDA_OK(cudaFuncSetAttribute(skim_scale_sums_kernel<SUMS_STEP>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm_sums));
+    SKIM_CUDA_OK(cudaFuncSetAttribute(skim_scale_sums_kernel<SUMS_CENTROIDS>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm_sums));
+    skim_scale_init_kernel<<<p->cb, 256, 0, ctx->stream>>>(alpha, (int)cols, ws.alpha64, ws.alpha_il, ws.adam_m, ws.adam_v, ws.status);
+    SKIM_CUDA_OK(cudaGetLastError());
+    skim_scale_order_kernel<<<(unsigned)rows, OT, sm_order, ctx->stream>>>(a);
+    SKIM_CUDA_OK(cudaGetLastError());
+    skim_scale_sums_kernel<SUMS_INIT><<<p->sum_blocks, SUM_T, sm_init, ctx->stream>>>(a);
+    SKIM_CUDA_OK(cudaGetLastError());
+    ctx->launches += 3;
+    return SKIM_OK;
+}
+
+// The learning rate and bias corrections of the Adam steps (Section 5.1: betas 0.9 / 0.999, eps 1e-8).
+struct AdamSchedule {
+    double lr, p1 = 1.0, p2 = 1.0, decay;
+    int every, t = 0;
+    AdamSchedule(float lr0, float d, int e) : lr((double)lr0), decay((double)d), every(e) {}
+    void next()
+    {
+        if (t > 0 && t % every == 0) lr *= decay;
+        p1 *= 0.9;
+        p2 *= 0.999;
+        ++t;
+    }
+};
+
+int scale_adam(skim_ctx *ctx, const SkimWorkspace &ws, const ScalePlan &p, const AdamSchedule &s, double *loss_trace)
+{
+    return launch_dependent(ctx, skim_scale_adam_kernel, dim3(p.ab + 1), 256, 0, (const double *)ws.grad_part, (const double *)ws.loss_part, p.ranges,
+                            p.a.rows, p.a.cols, ws.alpha64, ws.alpha_il, ws.adam_m, ws.adam_v, s.lr, 0.9, 0.999, 1.0 - s.p1, 1.0 - s.p2,
+                            1e-8, loss_trace ? loss_trace + (s.t - 1) : nullptr);
+}
+
+int scale_finish(skim_ctx *ctx, const SkimWorkspace &ws, const ScalePlan &p, float *alpha)
+{
+    skim_scale_finish_kernel<<<p.cb, 256, 0, ctx->stream>>>(ws.alpha64, p.a.cols, alpha);
+    SKIM_CUDA_OK(cudaGetLastError());
+    ctx->launches += 1;
+    return SKIM_OK;
+}
+
+}  // namespace
+
+int skim_launch_scale_update_lfull(skim_ctx *ctx, const uint16_t *W, const float *importance, int64_t rows, int64_t cols,
+                                   int64_t ld, const uint8_t *labels, const uint16_t *H, int64_t ldh, float *alpha,
+                                   int steps, float lr0, float decay, int decay_every, int exp2, void *scratch,
+                                   double *loss_trace)
+{
+    SkimWorkspace ws = skim_carve(ctx->ws, rows, cols);
+    ScalePlan p;
+    int rc = scale_begin(ctx, ws, W, importance, rows, cols, ld, labels, alpha, &p);
+    if (rc) return rc;
+    ScaleLfArgs b;
+    b.s = p.a;
     unsigned char *sp = (unsigned char *)scratch;
     b.D = (uint16_t *)sp;
     sp += skim_align256((size_t)rows * cols * 2);
@@ -616,47 +908,26 @@ int skim_launch_scale_update_lfull(skim_ctx *ctx, const uint16_t *W, const float
     void *gemm_scratch = sp;
     b.Y = Y;
     b.exp2 = exp2;
-    const int tiles = (int)((cols + GT * GC - 1) / (GT * GC));
-    int ranges = (4 * ctx->sm_count + tiles - 1) / tiles;
-    if (ranges > SKIM_SCALE_MAX_CTAS) ranges = SKIM_SCALE_MAX_CTAS;
-    if (ranges > rows) ranges = (int)rows;
-    a.rows_per_range = (int)((rows + ranges - 1) / ranges);
-    ranges = (int)((rows + a.rows_per_range - 1) / a.rows_per_range);
-    const size_t smem_init = (size_t)SW * NSUM * KC * 32 * sizeof(double);
-    const size_t smem_res = (size_t)SW * KC * 32 * sizeof(double) + (size_t)SW * KC * sizeof(double);
     const size_t smem_r = (size_t)SW * KC * 32 * sizeof(double);
-    const unsigned sum_blocks = (unsigned)((rows + SW - 1) / SW);
-    SKIM_CUDA_OK(cudaFuncSetAttribute(skim_scale_sums_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_init));
-    skim_scale_sums_kernel<true, true><<<sum_blocks, SW * 32, smem_init, ctx->stream>>>(a);
-    SKIM_CUDA_OK(cudaGetLastError());
-    ctx->launches += 1;
-    const double beta1 = 0.9, beta2 = 0.999, eps = 1e-8;
-    double p1 = 1.0, p2 = 1.0, lr = (double)lr0;
+    const unsigned row_blocks = (unsigned)((rows + SW - 1) / SW);
+    const unsigned res_blocks = (unsigned)((rows * ((cols + RES_COLS - 1) / RES_COLS) + SW - 1) / SW);
+    AdamSchedule sched(lr0, decay, decay_every);
     for (int t = 0; t < steps; ++t) {
-        if (t > 0 && t % decay_every == 0) lr *= (double)decay;
-        p1 *= beta1;
-        p2 *= beta2;
-        skim_scale_lf_residual_kernel<<<sum_blocks, SW * 32, smem_res, ctx->stream>>>(b);
-        SKIM_CUDA_OK(cudaGetLastError());
-        ctx->launches += 1;
-        const int rc = skim_launch_err_lfull(ctx, b.D, rows, cols, cols, H, ldh, exp2, gemm_scratch, nullptr, 1, Y, cols, ws.loss_part);
+        sched.next();
+        rc = launch_dependent(ctx, skim_scale_sums_kernel<SUMS_CENTROIDS>, dim3(p.sum_blocks), SUM_T, sums_smem_bytes((int)cols, false), p.a);
         if (rc) return rc;
-        skim_scale_lf_r_kernel<<<sum_blocks, SW * 32, smem_r, ctx->stream>>>(b);
-        SKIM_CUDA_OK(cudaGetLastError());
-        skim_scale_lf_grad_kernel<<<dim3((unsigned)tiles, (unsigned)ranges), GT, 0, ctx->stream>>>(b);
-        SKIM_CUDA_OK(cudaGetLastError());
-        skim_scale_adam_kernel<<<ab + 1, 256, 0, ctx->stream>>>(ws.grad_part, ws.loss_part, ranges, rows, (int)cols,
-                                                                ws.alpha64, ws.alpha_il, ws.adam_m, ws.adam_v, lr, beta1,
-                                                                beta2,
-                                                                1.0 - p1, 1.0 - p2, eps,
-                                                                loss_trace ? loss_trace + t : nullptr);
-        SKIM_CUDA_OK(cudaGetLastError());
-        ctx->launches += 3;
+        rc = launch_dependent(ctx, skim_scale_lf_residual_kernel, dim3(res_blocks), SW * 32, 0, b);
+        if (rc) return rc;
+        rc = skim_launch_err_lfull(ctx, b.D, rows, cols, cols, H, ldh, exp2, gemm_scratch, nullptr, 1, Y, cols, ws.loss_part);
+        if (rc) return rc;
+        rc = launch_dependent(ctx, skim_scale_lf_r_kernel, dim3(row_blocks), SW * 32, smem_r, b);
+        if (rc) return rc;
+        rc = launch_dependent(ctx, skim_scale_lf_grad_kernel, p.grad_grid, GT, 0, b);
+        if (rc) return rc;
+        rc = scale_adam(ctx, ws, p, sched, loss_trace);
+        if (rc) return rc;
     }
-    skim_scale_finish_kernel<<<cb, 256, 0, ctx->stream>>>(ws.alpha64, (int)cols, alpha);
-    SKIM_CUDA_OK(cudaGetLastError());
-    ctx->launches += 1;
-    return SKIM_OK;
+    return scale_finish(ctx, ws, p, alpha);
 }
 
 int skim_launch_scale_update(skim_ctx *ctx, const uint16_t *W, const float *importance, int64_t rows, int64_t cols,
@@ -664,62 +935,19 @@ int skim_launch_scale_update(skim_ctx *ctx, const uint16_t *W, const float *impo
                              int decay_every, double *loss_trace)
 {
     SkimWorkspace ws = skim_carve(ctx->ws, rows, cols);
-    const unsigned cb = (unsigned)((cols + 255) / 256), ab = (unsigned)((cols + 31) / 32);   // Adam: 32 columns a block
-    skim_scale_init_kernel<<<cb, 256, 0, ctx->stream>>>(alpha, (int)cols, ws.alpha64, ws.alpha_il, ws.adam_m, ws.adam_v, ws.status);
-    SKIM_CUDA_OK(cudaGetLastError());
-    ctx->launches += 1;
-    ScaleArgs a;
-    a.W = W;
-    a.G = importance;
-    a.labels = labels;
-    a.alpha = ws.alpha64;
-    a.alpha_il = ws.alpha_il;
-    a.rows = rows;
-    a.ld = ld;
-    a.cols = (int)cols;
-    a.vec = ((reinterpret_cast<uintptr_t>(W) & 15u) == 0 && (reinterpret_cast<uintptr_t>(importance) & 15u) == 0 &&
-             (reinterpret_cast<uintptr_t>(labels) & 7u) == 0 && ld % 8 == 0 && cols % 8 == 0) ? 1 : 0;
-    a.tconst = reinterpret_cast<double2 *>(ws.scale_const);
-    a.tq = reinterpret_cast<double2 *>(ws.scale_cq);
-    a.loss_row = ws.loss_part;
-    a.grad_part = ws.grad_part;
-    // gradient kernel: column tiles x row ranges, about four blocks per SM in all
-    const int tiles = (int)((cols + GT * GC - 1) / (GT * GC));
-    int ranges = (4 * ctx->sm_count + tiles - 1) / tiles;
-    if (ranges > SKIM_SCALE_MAX_CTAS) ranges = SKIM_SCALE_MAX_CTAS;
-    if (ranges > rows) ranges = (int)rows;
-    a.rows_per_range = (int)((rows + ranges - 1) / ranges);
-    ranges = (int)((rows + a.rows_per_range - 1) / a.rows_per_range);
-    const size_t smem = (size_t)SW * NSUM * KC * 32 * sizeof(double);
-    const unsigned sum_blocks = (unsigned)((rows + SW - 1) / SW);
-    auto sums_init = a.vec ? skim_scale_sums_kernel<true, true> : skim_scale_sums_kernel<true, false>;
-    auto sums_step = a.vec ? skim_scale_sums_kernel<false, true> : skim_scale_sums_kernel<false, false>;
-    auto grad = a.vec ? skim_scale_grad_kernel<true> : skim_scale_grad_kernel<false>;
-    SKIM_CUDA_OK(cudaFuncSetAttribute(sums_init, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    SKIM_CUDA_OK(cudaFuncSetAttribute(sums_step, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    sums_init<<<sum_blocks, SW * 32, smem, ctx->stream>>>(a);
-    SKIM_CUDA_OK(cudaGetLastError());
-    ctx->launches += 1;
-    const double beta1 = 0.9, beta2 = 0.999, eps = 1e-8;
-    double p1 = 1.0, p2 = 1.0, lr = (double)lr0;
+    ScalePlan p;
+    int rc = scale_begin(ctx, ws, W, importance, rows, cols, ld, labels, alpha, &p);
+    if (rc) return rc;
+    auto grad = p.a.vec ? skim_scale_grad_kernel<true> : skim_scale_grad_kernel<false>;
+    AdamSchedule sched(lr0, decay, decay_every);
     for (int t = 0; t < steps; ++t) {
-        if (t > 0 && t % decay_every == 0) lr *= (double)decay;
-        p1 *= beta1;
-        p2 *= beta2;
-        sums_step<<<sum_blocks, SW * 32, smem, ctx->stream>>>(a);
-        SKIM_CUDA_OK(cudaGetLastError());
-        grad<<<dim3((unsigned)tiles, (unsigned)ranges), GT, 0, ctx->stream>>>(a);
-        SKIM_CUDA_OK(cudaGetLastError());
-        skim_scale_adam_kernel<<<ab + 1, 256, 0, ctx->stream>>>(ws.grad_part, ws.loss_part, ranges, rows, (int)cols,
-                                                                ws.alpha64, ws.alpha_il, ws.adam_m, ws.adam_v, lr, beta1,
-                                                                beta2,
-                                                                1.0 - p1, 1.0 - p2, eps,
-                                                                loss_trace ? loss_trace + t : nullptr);
-        SKIM_CUDA_OK(cudaGetLastError());
-        ctx->launches += 3;
+        sched.next();
+        rc = launch_dependent(ctx, skim_scale_sums_kernel<SUMS_STEP>, dim3(p.sum_blocks), SUM_T, sums_smem_bytes((int)cols, false), p.a);
+        if (rc) return rc;
+        rc = launch_dependent(ctx, grad, p.grad_grid, GT, 0, p.a);
+        if (rc) return rc;
+        rc = scale_adam(ctx, ws, p, sched, loss_trace);
+        if (rc) return rc;
     }
-    skim_scale_finish_kernel<<<cb, 256, 0, ctx->stream>>>(ws.alpha64, (int)cols, alpha);
-    SKIM_CUDA_OK(cudaGetLastError());
-    ctx->launches += 1;
-    return SKIM_OK;
+    return scale_finish(ctx, ws, p, alpha);
 }

@@ -34,6 +34,29 @@ def test_scale_update_matches_oracle(ctx, oracle, rows, cols, steps):
     np.testing.assert_allclose(alpha.cpu().numpy().astype(np.float64), want, rtol=1e-6, atol=0)
 
 
+@pytest.mark.parametrize("rows,cols,kind", [(1, 8, "mixed"), (3, 63, "mixed"), (25, 65, "mixed"), (149, 33, "mixed"), (3560, 68, "mixed"),
+                                            (7, 1024, "one"), (5, 2050, "column"), (9, 700, "runs"), (4, 4100, "rare")])
+def test_scale_update_label_layouts(ctx, oracle, rows, cols, kind):
+    """The label-ordered copy at its edges: rows that are shared by several warps, taken whole, or both; clusters that
+    are empty, a single one, one per column class, contiguous, or a few elements beside a large one."""
+    rng = np.random.default_rng(rows + cols)
+    w, g = inputs.make_rows(rows, cols, 60 + cols)
+    j = np.arange(cols)
+    labels = {"mixed": lambda: rng.integers(0, np.array([2, 4, 8, 16])[np.arange(rows) % 4][:, None], size=(rows, cols)),
+              "one": lambda: np.full((rows, cols), 15), "column": lambda: np.broadcast_to(j % 16, (rows, cols)),
+              "runs": lambda: np.broadcast_to(j * 16 // cols, (rows, cols)),
+              "rare": lambda: np.where(rng.random((rows, cols)) < 0.002, rng.integers(0, 16, size=(rows, cols)), 7)}[kind]().astype(np.uint8)
+    a0 = inputs.make_scale(cols, 5, spread=0.05)
+    want, trace = oracle.scale_update(w, g, labels, a0.astype(np.float64), steps=2)
+    ctx.reserve(rows, cols)
+    alpha = torch.from_numpy(a0.copy()).cuda()
+    got = ctx.scale_update(torch.from_numpy(w).cuda(), torch.from_numpy(g).cuda(), torch.from_numpy(np.ascontiguousarray(labels)).cuda(), alpha, steps=2)
+    torch.cuda.synchronize()
+    assert ctx.get_status() == 0
+    np.testing.assert_allclose(got.cpu().numpy(), trace, rtol=1e-7, atol=1e-12)
+    np.testing.assert_allclose(alpha.cpu().numpy().astype(np.float64), want, rtol=1e-6, atol=0)
+
+
 def test_scale_update_wide_rows(ctx, oracle):
     rows, cols = 6, 22016
     w, g = inputs.make_rows(8192, cols, 5001, 0, rows, importance_sigma=2.0)
@@ -90,3 +113,9 @@ def test_scale_update_lfull_argument_errors(ctx, skimlib):
         ctx.scale_update_lfull(W[:, :60].contiguous(), G[:, :60].contiguous(), L[:, :60].contiguous(), a[:60].contiguous(),
                                H[:60, :60].contiguous(), steps=1)
     assert e.value.code == -2
+
+
+@pytest.mark.parametrize("rows,cols,steps", [(257, 776, 4), (3560, 264, 2)])
+def test_scale_update_lfull_tiles_and_shared_rows(ctx, oracle, rows, cols, steps):
+    """More than one tile of the contraction either way, its last tiles halved; rows taken whole and rows shared by warps."""
+    test_scale_update_lfull_matches_oracle(ctx, oracle, rows, cols, steps)
