@@ -12,11 +12,13 @@
 //                             bound by the tensor pipe, 4096 x 11008 x 11008 0.374 ms per width against 0.709 ms in full.
 //   skim_lfull_reduce_kernel  adds the per-tile partial sums of a row in a fixed order, divides 4^e out.
 //
-// GEMM kernel: persistent, one CTA per SM, tile 128 x 256 x 64, tcgen05.mma (kind::f16, binary32 accumulators
-// in tensor memory, two accumulator stages of 256 columns), operands brought in by TMA
-// (cp.async.bulk.tensor, 128-byte swizzle) through a 4-stage shared-memory ring.  Warp 0 issues the TMA loads,
-// warp 1 allocates tensor memory and issues the MMAs, warps 2-5 read the accumulators back (tcgen05.ld) and do
-// the dot product with the matching D tile.  No cluster launch and no multicast: every CTA fetches its own tiles.
+// GEMM kernel: persistent, one CTA per SM, CTAs in pairs (cluster of two, tcgen05 cta_group::2), tile 256 x 256 x 64
+// per pair, tcgen05.mma (kind::f16, binary32 accumulators in tensor memory, two accumulator stages of 256 columns),
+// operands brought in by TMA (cp.async.bulk.tensor, 128-byte swizzle) through a 6-stage shared-memory ring.  A CTA
+// fetches its 128 rows of D and half of the tile's rows of H (32 KB per K block of 64; a tile of its own of 128 x 256
+// took 48 KB for the same MMA time, more than the L2 delivers to an SM meanwhile).  Warp 0 issues the TMA loads, warp 1
+// allocates tensor memory and, in the first CTA, issues the MMAs of both, warps 2-5 read the accumulators back
+// (tcgen05.ld) and do the dot product with the matching D tile.  No TMA multicast: every CTA fetches its own operands.
 // Every wait on an mbarrier is bounded: after WAIT_LIMIT_CYCLES the waiting role raises the block's abort flag,
 // sets SKIM_STATUS_TIMEOUT, and all roles leave their loops; tensor memory is freed on every path.
 #include <cuda.h>
@@ -127,10 +129,12 @@ __global__ void __launch_bounds__(RES_T) skim_residual_kernel(ResidualArgs a)
 
 // ---------------------------------------------------------------- GEMM with fused row-wise dot
 
-constexpr int BM = 128, BN = 256, BK = 64;
-constexpr int STAGES = 4;
+constexpr int BM = 256, BN = 256, BK = 64;      // a tile belongs to a pair of CTAs: each has half of its rows
+constexpr int CM = BM / 2;                      // rows of D (and of the accumulator) in a CTA
+constexpr int CB = 64;                          // rows of H in a TMA box; a CTA holds BN / 2 = two boxes
+constexpr int STAGES = 6;
 constexpr int UMMA_K = 16;
-constexpr int A_BYTES = BM * BK * 2, B_BYTES = BN * BK * 2, STAGE_BYTES = A_BYTES + B_BYTES;
+constexpr int A_BYTES = CM * BK * 2, BOX_BYTES = CB * BK * 2, STAGE_BYTES = A_BYTES + 2 * BOX_BYTES;     // per CTA
 constexpr int GEMM_THREADS = 192;
 constexpr int CHECK_WARPS = 4;                  // further warps of the half contraction: they compare H with its transpose
 constexpr int SPLIT_MAX = 8;                    // ranges of K a tile of the last round is cut into, at most
@@ -160,9 +164,27 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, uint32_t bytes)
 {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
 }
-__device__ __forceinline__ void mbar_arrive(uint64_t *bar)
+// Address of `p` (this CTA's shared memory) in the pair's CTA of rank `rank`.
+__device__ __forceinline__ uint32_t cluster_addr(const void *p, uint32_t rank)
 {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ uint32_t cluster_rank()
+{
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t addr)
+{
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
 }
 __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity)
 {
@@ -187,11 +209,12 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, volati
     return true;
 }
 
-__device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, uint64_t *bar, int x, int y)
+// Into this CTA's shared memory; the bytes are counted by the mbarrier at `bar` (an address in either CTA of the pair).
+__device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, uint32_t bar, int x, int y)
 {
-    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];" ::"r"(
+    asm volatile("cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];" ::"r"(
                      smem_u32(dst)),
-                 "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(x), "r"(y)
+                 "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(y)
                  : "memory");
 }
 
@@ -209,25 +232,30 @@ __device__ __forceinline__ uint64_t umma_desc(uint32_t smem_addr)
     return d;
 }
 
-// Instruction descriptor of kind::f16: D binary32, A and B binary16, both K-major, M = 128, N = 256.
-constexpr uint32_t IDESC = (1u << 4) | (0u << 7) | (0u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+// Instruction descriptor of kind::f16: D binary32, A and B binary16, both K-major, M = 256 (a pair of CTAs), N columns.
+__host__ __device__ constexpr uint32_t umma_idesc(int n) { return (1u << 4) | (0u << 7) | (0u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(BM >> 4) << 24); }
 
-__device__ __forceinline__ void umma_f16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t accumulate)
+// One lane of the pair's first CTA issues for both: each contributes its rows of A and its half of the rows of B from
+// its own shared memory (same offsets) and accumulates its rows of D in its own tensor memory.
+__device__ __forceinline__ void umma_f16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate)
 {
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-                 "l"(adesc), "l"(bdesc), "r"(IDESC), "r"(accumulate)
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
+                 "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
                  : "memory");
 }
 // D = A B + D / 2
-__device__ __forceinline__ void umma_f16_halve(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc)
+__device__ __forceinline__ void umma_f16_halve(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc)
 {
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.eq.b32 p, 0, 0;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p, 1;\n\t}" ::"r"(tmem_d),
-                 "l"(adesc), "l"(bdesc), "r"(IDESC)
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.eq.b32 p, 0, 0;\n\ttcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p, 1;\n\t}" ::"r"(tmem_d),
+                 "l"(adesc), "l"(bdesc), "r"(idesc)
                  : "memory");
 }
+// Arrives on the mbarrier at this offset in both CTAs once the MMAs issued so far are done.
 __device__ __forceinline__ void umma_commit(uint64_t *bar)
 {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(smem_u32(bar)),
+                 "h"((uint16_t)3)
+                 : "memory");
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -252,7 +280,7 @@ struct GemmArgs {
     int64_t ldd;
     int rows, cols;
     int mt, nt;              // tiles along rows and along columns
-    int full_tiles, split;   // tiles [full_tiles, mt * nt) are cut into `split` ranges of K (see unit_of)
+    int full_tiles, split;   // tiles [full_tiles, mt * nt) are cut into `split` parts (see unit_of)
     float *partial;          // [mt * BM][split][nt]
     float *Y;                // optional [rows][ldy]: the product D H itself (the scaling-vector update needs it)
     int64_t ldy;
@@ -262,24 +290,29 @@ struct GemmArgs {
     unsigned long long *status;
 };
 
-// Work units.  Tiles are taken round-robin by the persistent CTAs; the tiles of the last, partly filled round
-// would leave most SMs idle for a whole tile time, so each of them is cut into `split` ranges of K that run
-// side by side.  The fused row-wise dot is linear in the accumulator, so a range simply leaves one more partial
-// dot per row (column `slice` of the partial array); the product Y itself is only written by unsplit launches.
+// Work units.  Tiles are taken round-robin by the persistent pairs of CTAs; the tiles of the last, partly filled round
+// would leave most pairs idle for a whole tile time, so each of them is cut into `split` parts that run side by side:
+// ranges of K (the fused row-wise dot is linear in the accumulator, so a range simply leaves one more partial dot per
+// row), or, where the product Y itself is asked for, the two halves of its columns.
 struct GemmUnit {
     int tile, slice, kb0, kb1;
+    int n_off, n;            // columns of the tile
 };
 __device__ __forceinline__ GemmUnit unit_of(const GemmArgs &a, int u, int nkb)
 {
     GemmUnit w;
-    if (u < a.full_tiles) {
-        w.tile = u; w.slice = 0; w.kb0 = 0; w.kb1 = nkb;
-    } else {
+    w.tile = u; w.slice = 0; w.kb0 = 0; w.kb1 = nkb; w.n_off = 0; w.n = BN;
+    if (u >= a.full_tiles) {
         const int r = u - a.full_tiles;
         w.tile = a.full_tiles + r / a.split;
         w.slice = r % a.split;
-        w.kb0 = (int)((long long)nkb * w.slice / a.split);
-        w.kb1 = (int)((long long)nkb * (w.slice + 1) / a.split);
+        if (a.Y) {
+            w.n = BN / a.split;
+            w.n_off = w.slice * w.n;
+        } else {
+            w.kb0 = (int)((long long)nkb * w.slice / a.split);
+            w.kb1 = (int)((long long)nkb * (w.slice + 1) / a.split);
+        }
     }
     return w;
 }
@@ -316,14 +349,17 @@ __device__ __forceinline__ GemmUnit half_unit(const GemmArgs &a, HalfList &h, in
     w.tile = h.nb * a.mt + r % a.mt;
     w.kb0 = len * w.slice / h.pieces;
     w.kb1 = len * (w.slice + 1) / h.pieces;
+    w.n_off = 0;
+    w.n = BN;
     return w;
 }
 
-// Unit of this block in round t, or -1: round-robin (HALF: every other round reversed).
+// Unit of this pair in round t, or -1: round-robin (HALF: every other round reversed).
 template <bool HALF>
 __device__ __forceinline__ int unit_index(int t, int nunits)
 {
-    const int u = t * (int)gridDim.x + ((HALF && (t & 1)) ? (int)gridDim.x - 1 - (int)blockIdx.x : (int)blockIdx.x);
+    const int pairs = (int)gridDim.x / 2, pair = (int)blockIdx.x / 2;
+    const int u = t * pairs + ((HALF && (t & 1)) ? pairs - 1 - pair : pair);
     return u < nunits ? u : -1;
 }
 
@@ -365,7 +401,7 @@ __device__ __forceinline__ uint32_t compare_transpose(const uint16_t *H, int64_t
 // HALF: the half contraction for a symmetric H, launched first; it leaves in a.asym whether H was.  Otherwise the full
 // contraction; with a.asym given it is the fallback of a half launch and leaves at once unless H was not symmetric.
 template <bool HALF>
-__global__ void __launch_bounds__(GEMM_THREADS + (HALF ? CHECK_WARPS * 32 : 0), 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS + (HALF ? CHECK_WARPS * 32 : 0), 1)
 skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, GemmArgs a, const uint16_t *H, int64_t ldh)
 {
     extern __shared__ unsigned char smem_raw[];
@@ -386,68 +422,73 @@ skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
         if (!__syncthreads_or(any)) return;
     }
 
+    const uint32_t rank = cluster_rank();
     if (threadIdx.x == 0) {
+        // full and tmem_empty are used in the first CTA only; the other two in both
         for (int s = 0; s < STAGES; ++s) { mbar_init(&sy.full[s], 1); mbar_init(&sy.empty[s], 1); }
-        for (int s = 0; s < 2; ++s) { mbar_init(&sy.tmem_full[s], 1); mbar_init(&sy.tmem_empty[s], 4); }
+        for (int s = 0; s < 2; ++s) { mbar_init(&sy.tmem_full[s], 1); mbar_init(&sy.tmem_empty[s], 8); }
         sy.abort = 0;
         sy.asym = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sy.tmem_base)), "r"(TMEM_COLS));
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sy.tmem_base)), "r"(TMEM_COLS));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;");
     }
     tc_fence_before();
     __syncthreads();
+    cluster_sync();
     tc_fence_after();
     const uint32_t tmem_base = sy.tmem_base;
 
     if (warp == 0) {
-        // ------------------------------------------------------------ TMA producer (one lane)
+        // ------------------------------------------------------------ TMA producer (one lane): this CTA's half of either operand
         if (lane == 0) {
             int stage = 0;
             uint32_t phase = 0;
             bool ok = true;
-            for (int t = 0; t * (int)gridDim.x < nunits && ok; ++t) {
+            for (int t = 0; t * ((int)gridDim.x / 2) < nunits && ok; ++t) {
                 const int u = unit_index<HALF>(t, nunits);
                 if (u < 0) continue;
                 const GemmUnit w = HALF ? half_unit(a, half, u, nkb) : unit_of(a, u, nkb);
-                const int m0 = (w.tile % a.mt) * BM, n0 = (w.tile / a.mt) * BN;
+                const int m0 = (w.tile % a.mt) * BM + (int)rank * CM, n0 = (w.tile / a.mt) * BN;
+                const int boxes = w.n / (2 * CB), b0 = n0 + w.n_off + (int)rank * (w.n / 2);
                 for (int l = w.kb0; l < w.kb1; ++l) {
                     const int kb = HALF ? n0 / BK + l : l;
                     if (!(ok = mbar_wait(&sy.empty[stage], phase ^ 1u, abort_flag))) break;
                     unsigned char *sa = tiles + (size_t)stage * STAGE_BYTES;
-                    mbar_expect_tx(&sy.full[stage], STAGE_BYTES);
-                    tma_load_2d(sa, &map_a, &sy.full[stage], kb * BK, m0);
-                    tma_load_2d(sa + A_BYTES, &map_b, &sy.full[stage], kb * BK, n0);
+                    if (rank == 0) mbar_expect_tx(&sy.full[stage], 2 * (A_BYTES + boxes * BOX_BYTES));
+                    const uint32_t bar = cluster_addr(&sy.full[stage], 0);
+                    tma_load_2d(sa, &map_a, bar, kb * BK, m0);
+                    for (int b = 0; b < boxes; ++b) tma_load_2d(sa + A_BYTES + b * BOX_BYTES, &map_b, bar, kb * BK, b0 + b * CB);
                     if (++stage == STAGES) { stage = 0; phase ^= 1u; }
                 }
             }
         }
     } else if (warp == 1) {
-        // ------------------------------------------------------------ MMA issuer (one lane)
-        if (lane == 0) {
+        // ------------------------------------------------------------ MMA issuer (one lane of the first CTA)
+        if (lane == 0 && rank == 0) {
             int stage = 0;
             uint32_t phase = 0;
             bool ok = true;
             int it = 0;
-            for (int t = 0; t * (int)gridDim.x < nunits && ok; ++t) {
+            for (int t = 0; t * ((int)gridDim.x / 2) < nunits && ok; ++t) {
                 const int u = unit_index<HALF>(t, nunits);
                 if (u < 0) continue;
                 const GemmUnit w = HALF ? half_unit(a, half, u, nkb) : unit_of(a, u, nkb);
                 const int as = it & 1;
                 if (!(ok = mbar_wait(&sy.tmem_empty[as], (((uint32_t)it >> 1) & 1u) ^ 1u, abort_flag))) break;
                 tc_fence_after();
-                const uint32_t tmem_d = tmem_base + (uint32_t)(as * BN);
+                const uint32_t tmem_d = tmem_base + (uint32_t)(as * BN), idesc = umma_idesc(w.n);
                 for (int kb = w.kb0; kb < w.kb1; ++kb) {          // HALF: list positions
                     if (!(ok = mbar_wait(&sy.full[stage], phase, abort_flag))) break;
                     tc_fence_after();
                     const uint32_t sa = smem_u32(tiles + (size_t)stage * STAGE_BYTES), sb = sa + A_BYTES;
 #pragma unroll
                     for (int k = 0; k < BK / UMMA_K; ++k)
-                        if (HALF && k == 0 && kb == HALF_DIAG && kb > w.kb0) umma_f16_halve(tmem_d, umma_desc(sa), umma_desc(sb));
-                        else umma_f16(tmem_d, umma_desc(sa + k * UMMA_K * 2), umma_desc(sb + k * UMMA_K * 2), (kb > w.kb0 || k) ? 1u : 0u);
-                    umma_commit(&sy.empty[stage]);           // the stage is free once these MMAs have read it
+                        if (HALF && k == 0 && kb == HALF_DIAG && kb > w.kb0) umma_f16_halve(tmem_d, umma_desc(sa), umma_desc(sb), idesc);
+                        else umma_f16(tmem_d, umma_desc(sa + k * UMMA_K * 2), umma_desc(sb + k * UMMA_K * 2), idesc, (kb > w.kb0 || k) ? 1u : 0u);
+                    umma_commit(&sy.empty[stage]);           // the stage is free, in both CTAs, once these MMAs have read it
                     if (++stage == STAGES) { stage = 0; phase ^= 1u; }
                 }
                 if (ok) umma_commit(&sy.tmem_full[as]);      // the accumulator is complete once all MMAs are
@@ -463,14 +504,14 @@ skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
         const int q = warp & 3;                               // the tensor-memory lane quarter this warp may read
         bool ok = true;
         int it = 0;
-        for (int t = 0; t * (int)gridDim.x < nunits && ok; ++t) {
+        for (int t = 0; t * ((int)gridDim.x / 2) < nunits && ok; ++t) {
             const int u = unit_index<HALF>(t, nunits);
             if (u < 0) continue;
             const GemmUnit w = HALF ? half_unit(a, half, u, nkb) : unit_of(a, u, nkb);
             const int as = it & 1;
             const int mb = w.tile % a.mt, nb = w.tile / a.mt;
-            const int row = mb * BM + q * 32 + lane;
-            const int n0 = nb * BN;
+            const int row = mb * BM + (int)rank * CM + q * 32 + lane;
+            const int n0 = nb * BN + w.n_off;
             const uint16_t *drow = a.D + (int64_t)min(row, a.rows - 1) * a.ldd;
             ok = mbar_wait(&sy.tmem_full[as], ((uint32_t)it >> 1) & 1u, abort_flag);
             ok = __all_sync(0xffffffffu, ok);
@@ -478,7 +519,7 @@ skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
             tc_fence_after();
             float acc = 0.0f;
 #pragma unroll 1
-            for (int c = 0; c < BN / 32; ++c) {
+            for (int c = 0; c < w.n / 32; ++c) {
                 const int col = n0 + c * 32;
                 uint4 dv[4];
 #pragma unroll
@@ -508,7 +549,7 @@ skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&sy.tmem_empty[as]);
+            if (lane == 0) mbar_arrive_cluster(cluster_addr(&sy.tmem_empty[as], 0));
             // a piece that reaches past its diagonal blocks holds half the dot (the diagonal blocks' part was halved)
             if (HALF && w.kb1 > HALF_DIAG) acc *= 2.0f;
             if (row < a.rows) a.partial[((int64_t)row * (HALF ? SPLIT_MAX : a.split) + w.slice) * a.nt + nb] = acc;
@@ -525,9 +566,10 @@ skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
         for (int i = 0; i < 1000; ++i) __nanosleep(1000);
         if (threadIdx.x == 0) atomicOr(a.status, (unsigned long long)SKIM_STATUS_TIMEOUT);
     }
+    cluster_sync();                    // the other CTA may still read this one's shared memory, or arrive on its mbarriers
     if (warp == 1) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS));
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS));
     }
 }
 
@@ -562,19 +604,19 @@ skim_lfull_reduce_kernel(GemmArgs a, int exp2, float *__restrict__ err, int64_t 
     }
 }
 
-// Length of the longest block of a half contraction, in K blocks, if lists are cut into pieces of about piece_kb: a
+// Length of the busiest pair of CTAs in a half contraction, in K blocks, if lists are cut into pieces of about piece_kb: a
 // piece also costs its epilogue, which hides under the next piece's MMAs unless that one is shorter.
-double half_makespan(int mt, int nt, int nkb, int piece_kb, int blocks)
+double half_makespan(int mt, int nt, int nkb, int piece_kb, int pairs)
 {
     constexpr double EPILOGUE = 10.0;          // K blocks' worth of MMA time (256 columns read back and multiplied)
-    std::vector<double> load(blocks, 0.0);
+    std::vector<double> load(pairs, 0.0);
     int u = 0;
     for (int nb = 0; nb < nt; ++nb) {
         const int p = half_pieces(nb, nkb, piece_kb);
         const double len = (double)half_len(nb, nkb) / p;
         for (int r = 0; r < p * mt; ++r, ++u) {
-            const int t = u / blocks, b = u % blocks;
-            load[(t & 1) ? blocks - 1 - b : b] += len > EPILOGUE ? len : EPILOGUE;
+            const int t = u / pairs, b = u % pairs;
+            load[(t & 1) ? pairs - 1 - b : b] += len > EPILOGUE ? len : EPILOGUE;
         }
     }
     double most = 0.0;
@@ -644,9 +686,9 @@ int skim_launch_err_lfull(skim_ctx *ctx, const uint16_t *D, int64_t rows, int64_
 {
     if (rows == 0) return SKIM_OK;
     CUtensorMap map_a, map_b;
-    int rc = encode_map(&map_a, D, rows, cols, ldd, BM);
+    int rc = encode_map(&map_a, D, rows, cols, ldd, CM);
     if (rc) return rc;
-    rc = encode_map(&map_b, H, cols, cols, ldh, BN);
+    rc = encode_map(&map_b, H, cols, cols, ldh, CB);
     if (rc) return rc;
     GemmArgs a;
     a.D = D;
@@ -663,15 +705,19 @@ int skim_launch_err_lfull(skim_ctx *ctx, const uint16_t *D, int64_t rows, int64_
     const int tiles = a.mt * a.nt;
     // the tiles of the last round, if it is not full, are cut along K into as many ranges as fit the SMs
     const int nkb = (int)((cols + BK - 1) / BK);
-    const int rest = tiles % ctx->sm_count;
+    const int pairs = ctx->sm_count / 2;
+    const int rest = tiles % pairs;
     a.full_tiles = tiles;
     a.split = 1;
-    if (!Y && rest > 0) {
-        // `rest` tiles in s ranges each take ceil(rest s / SMs) sub-rounds of 1/s tile time: the least, the smaller s on a tie
+    if (Y && rest > 0 && 2 * rest <= pairs) {
+        a.full_tiles = tiles - rest;
+        a.split = 2;
+    } else if (!Y && rest > 0) {
+        // `rest` tiles in s ranges each take ceil(rest s / pairs) sub-rounds of 1/s tile time: the least, the smaller s on a tie
         int sp = 1;
         double best = 1.0;
         for (int c = 2; c <= SPLIT_MAX && c <= nkb; ++c) {
-            const double cost = (double)((rest * c + ctx->sm_count - 1) / ctx->sm_count) / c;
+            const double cost = (double)((rest * c + pairs - 1) / pairs) / c;
             if (cost < best - 1e-9) { best = cost; sp = c; }
         }
         if (sp > 1) {
@@ -693,18 +739,18 @@ int skim_launch_err_lfull(skim_ctx *ctx, const uint16_t *D, int64_t rows, int64_
         const int c0 = a.full_tiles == 0 ? a.split : 1;
         for (int c = c0; c <= 2 * c0 && c <= SPLIT_MAX; ++c) {
             const int piece = (nkb + c - 1) / c;
-            const double v = half_makespan(a.mt, a.nt, nkb, piece, ctx->sm_count);
+            const double v = half_makespan(a.mt, a.nt, nkb, piece, pairs);
             if (c == c0 || v < best * 0.95) { best = v; a.piece_kb = piece; }
         }
         a.asym = (int *)((char *)scratch + skim_lfull_scratch_bytes(rows, cols) - HALF_FLAG_BYTES);
-        a.asym_n = ctx->sm_count;
+        a.asym_n = 2 * pairs;
         SKIM_CUDA_OK(cudaFuncSetAttribute(skim_lfull_gemm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GEMM_SMEM));
-        skim_lfull_gemm_kernel<true><<<(unsigned)ctx->sm_count, GEMM_THREADS + CHECK_WARPS * 32, GEMM_SMEM, ctx->stream>>>(map_a, map_b, a, H, ldh);
+        skim_lfull_gemm_kernel<true><<<(unsigned)(2 * pairs), GEMM_THREADS + CHECK_WARPS * 32, GEMM_SMEM, ctx->stream>>>(map_a, map_b, a, H, ldh);
         SKIM_CUDA_OK(cudaGetLastError());
         ctx->launches += 1;
     }
     const int units = a.full_tiles + (tiles - a.full_tiles) * a.split;
-    const unsigned blocks = (unsigned)(units < ctx->sm_count ? units : ctx->sm_count);    // persistent: one CTA per SM
+    const unsigned blocks = (unsigned)(2 * (units < pairs ? units : pairs));    // persistent: one CTA per SM
     skim_lfull_gemm_kernel<false><<<blocks, GEMM_THREADS, GEMM_SMEM, ctx->stream>>>(map_a, map_b, a, H, ldh);
     SKIM_CUDA_OK(cudaGetLastError());
     skim_lfull_reduce_kernel<<<(unsigned)((rows + RED_WARPS - 1) / RED_WARPS), RED_WARPS * 32, 0, ctx->stream>>>(a, exp2, err, err_stride, err64);
