@@ -44,7 +44,6 @@ struct SkimWorkspace {
     float *rscale;               // [cols]     reciprocal of the installed scale vector
     int32_t *row_pos;            // [rows]     packed-row index of every source row
     double *alpha64;             // [cols]     scale-update master copy of alpha
-    double *alpha_il;            // [cols rounded up to 256]  the same values in the order the row-wise kernels load them
     double *adam_m;              // [cols]
     double *adam_v;              // [cols]
     double *loss_part;           // [rows]     scale update: loss of every row
@@ -88,7 +87,6 @@ static inline SkimWorkspace skim_carve(void *base, int64_t rows, int64_t cols)
     w.rscale = (float *)take((size_t)cols * 4);
     w.row_pos = (int32_t *)take((size_t)rows * 4);
     w.alpha64 = (double *)take((size_t)cols * 8);
-    w.alpha_il = (double *)take((((size_t)cols + 255) & ~(size_t)255) * 8);
     w.adam_m = (double *)take((size_t)cols * 8);
     w.adam_v = (double *)take((size_t)cols * 8);
     w.loss_part = (double *)take((size_t)(rows > SKIM_SCALE_MAX_CTAS ? rows : SKIM_SCALE_MAX_CTAS) * 8);
@@ -167,10 +165,19 @@ int skim_launch_residual(skim_ctx *ctx, const uint16_t *W, int64_t rows, int64_t
                          const uint8_t *row_bits, int width, const SkimBits &bs, const float *s, int exp2, uint16_t *D,
                          int64_t ldd);
 size_t skim_lfull_scratch_bytes(int64_t rows, int64_t cols);
+// Sums of Y alpha by cluster, R_ik = sum_{j in k} Y_ij alpha_j, formed in the contraction's epilogue for the scale update.
+struct SkimLfullClusters {
+    const uint8_t *labels;   // [rows][cols]
+    const double *alpha;     // [cols]
+    double *rpart;           // skim_lfull_cluster_bytes(): per row, column tile and half of it
+    const double2 *tconst;   // [rows][16]  (G_k, .)
+    double2 *tq;             // [rows][16]  y <- 2 R_k / (2^exp2 G_k)
+};
+size_t skim_lfull_cluster_bytes(int64_t rows, int64_t cols);
 // Y (optional): the product D H itself, [rows][ldy] binary32; err64 (optional): the row errors in binary64
 int skim_launch_err_lfull(skim_ctx *ctx, const uint16_t *D, int64_t rows, int64_t cols, int64_t ldd, const uint16_t *H,
                           int64_t ldh, int exp2, void *scratch, float *err, int64_t err_stride, float *Y = nullptr,
-                          int64_t ldy = 0, double *err64 = nullptr);
+                          int64_t ldy = 0, double *err64 = nullptr, const SkimLfullClusters *clusters = nullptr);
 size_t skim_scale_lfull_scratch_bytes(int64_t rows, int64_t cols);
 int skim_launch_scale_update_lfull(skim_ctx *ctx, const uint16_t *W, const float *importance, int64_t rows, int64_t cols,
                                    int64_t ld, const uint8_t *labels, const uint16_t *H, int64_t ldh, float *alpha,

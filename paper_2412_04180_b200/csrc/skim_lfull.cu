@@ -132,17 +132,29 @@ __global__ void __launch_bounds__(RES_T) skim_residual_kernel(ResidualArgs a)
 constexpr int BM = 256, BN = 256, BK = 64;      // a tile belongs to a pair of CTAs: each has half of its rows
 constexpr int CM = BM / 2;                      // rows of D (and of the accumulator) in a CTA
 constexpr int CB = 64;                          // rows of H in a TMA box; a CTA holds BN / 2 = two boxes
-constexpr int STAGES = 6;
+constexpr int STAGES = 6;                       // ring of the half contraction; the full one gives a stage up for EpilogueSmem
 constexpr int UMMA_K = 16;
 constexpr int A_BYTES = CM * BK * 2, BOX_BYTES = CB * BK * 2, STAGE_BYTES = A_BYTES + 2 * BOX_BYTES;     // per CTA
-constexpr int GEMM_THREADS = 192;
+constexpr int EPI_WARPS = 8;                    // two for every quarter of the accumulator's rows, each with half of the columns
+constexpr int GEMM_THREADS = (2 + EPI_WARPS) * 32;
 constexpr int CHECK_WARPS = 4;                  // further warps of the half contraction: they compare H with its transpose
 constexpr int SPLIT_MAX = 8;                    // ranges of K a tile of the last round is cut into, at most
 constexpr int HALF_MIN_ROWS = 768, HALF_MIN_NT = 4;
 constexpr size_t HALF_FLAG_BYTES = 4096;         // symmetry flags of up to 1024 blocks
 constexpr int TMEM_COLS = 512;                  // two accumulator stages of BN binary32 columns
 constexpr long long WAIT_LIMIT_CYCLES = 400000000ll;   // about 0.2 s; a whole launch takes milliseconds
-constexpr size_t GEMM_SMEM = (size_t)STAGES * STAGE_BYTES + 1024 /* alignment slack */ + 256 /* barriers */;
+constexpr int KC = 16;                          // clusters of a row at most
+
+// What the epilogue warps of a CTA exchange.
+struct EpilogueSmem {
+    double slot[2][KC][CM];      // per half of the columns and row: sums of y alpha by cluster (full contraction with Y only)
+    double alpha[BN];
+};
+__host__ __device__ constexpr int ring_stages(bool half) { return half ? STAGES : STAGES - 1; }
+__host__ __device__ constexpr size_t gemm_smem(bool half)
+{
+    return (size_t)ring_stages(half) * STAGE_BYTES + 1024 /* alignment slack */ + 256 /* barriers */ + CM * sizeof(float) + (half ? 0 : sizeof(EpilogueSmem));
+}
 
 struct GemmSync {
     uint64_t full[STAGES];
@@ -284,6 +296,7 @@ struct GemmArgs {
     float *partial;          // [mt * BM][split][nt]
     float *Y;                // optional [rows][ldy]: the product D H itself (the scaling-vector update needs it)
     int64_t ldy;
+    SkimLfullClusters cl;    // with Y, optional: sums of Y alpha by cluster
     int *asym;               // [asym_n] per block of the half contraction: H is not symmetric in the part it compared
     int asym_n;
     int piece_kb;            // half contraction: a tile's list of K blocks is cut into pieces of about this length
@@ -398,6 +411,48 @@ __device__ __forceinline__ uint32_t compare_transpose(const uint16_t *H, int64_t
     return diff;
 }
 
+// Adds y_j alpha_j of 32 consecutive columns to the row's sums by cluster (slot k of this thread at slot[k * CM]).  The
+// slots of four elements are read together and the additions run in element order in registers, an element whose
+// cluster matches an earlier one of the four continuing from that one's result, so that the round trips through shared
+// memory do not follow one another.
+__device__ __forceinline__ void add_by_cluster(double *slot, const uint32_t *y, const uint2 *labels, const double *alpha)
+{
+#pragma unroll
+    for (int u0 = 0; u0 < 32; u0 += 4) {
+        const uint32_t l4 = (u0 & 4) ? labels[u0 / 8].y : labels[u0 / 8].x;
+        const double2 a0 = *reinterpret_cast<const double2 *>(alpha + u0), a1 = *reinterpret_cast<const double2 *>(alpha + u0 + 2);
+        const double al[4] = {a0.x, a0.y, a1.x, a1.y};
+        int l[4];
+        double v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            l[u] = (int)((l4 >> (8 * u)) & (KC - 1));
+            v[u] = slot[l[u] * CM];
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            double base = v[u];
+#pragma unroll
+            for (int t = 0; t < u; ++t)
+                if (l[t] == l[u]) base = v[t];
+            v[u] = fma((double)__uint_as_float(y[u0 + u]), al[u], base);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) slot[l[u] * CM] = v[u];      // where clusters repeat the last store holds the full sum
+    }
+}
+
+__device__ __forceinline__ bool epilogue_barrier_or(bool v)
+{
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbar.red.or.pred q, 1, %2, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+                 : "=r"(r)
+                 : "r"((uint32_t)v), "n"(EPI_WARPS * 32)
+                 : "memory");
+    return r != 0;
+}
+__device__ __forceinline__ void epilogue_barrier() { asm volatile("bar.sync 1, %0;" ::"n"(EPI_WARPS * 32) : "memory"); }
+
 // HALF: the half contraction for a symmetric H, launched first; it leaves in a.asym whether H was.  Otherwise the full
 // contraction; with a.asym given it is the fallback of a half launch and leaves at once unless H was not symmetric.
 template <bool HALF>
@@ -406,7 +461,10 @@ skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
 {
     extern __shared__ unsigned char smem_raw[];
     unsigned char *tiles = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    GemmSync &sy = *reinterpret_cast<GemmSync *>(tiles + (size_t)STAGES * STAGE_BYTES);
+    constexpr int NST = ring_stages(HALF);
+    GemmSync &sy = *reinterpret_cast<GemmSync *>(tiles + (size_t)NST * STAGE_BYTES);
+    float *dot_s = reinterpret_cast<float *>(tiles + (size_t)NST * STAGE_BYTES + 256);                           // [CM]
+    EpilogueSmem &ep = *reinterpret_cast<EpilogueSmem *>(tiles + (size_t)NST * STAGE_BYTES + 256 + CM * sizeof(float));   // not for HALF
     volatile int *abort_flag = &sy.abort;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nkb = (a.cols + BK - 1) / BK;
@@ -425,8 +483,8 @@ skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
     const uint32_t rank = cluster_rank();
     if (threadIdx.x == 0) {
         // full and tmem_empty are used in the first CTA only; the other two in both
-        for (int s = 0; s < STAGES; ++s) { mbar_init(&sy.full[s], 1); mbar_init(&sy.empty[s], 1); }
-        for (int s = 0; s < 2; ++s) { mbar_init(&sy.tmem_full[s], 1); mbar_init(&sy.tmem_empty[s], 8); }
+        for (int s = 0; s < NST; ++s) { mbar_init(&sy.full[s], 1); mbar_init(&sy.empty[s], 1); }
+        for (int s = 0; s < 2; ++s) { mbar_init(&sy.tmem_full[s], 1); mbar_init(&sy.tmem_empty[s], 2 * EPI_WARPS); }
         sy.abort = 0;
         sy.asym = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -461,7 +519,7 @@ skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
                     const uint32_t bar = cluster_addr(&sy.full[stage], 0);
                     tma_load_2d(sa, &map_a, bar, kb * BK, m0);
                     for (int b = 0; b < boxes; ++b) tma_load_2d(sa + A_BYTES + b * BOX_BYTES, &map_b, bar, kb * BK, b0 + b * CB);
-                    if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+                    if (++stage == NST) { stage = 0; phase ^= 1u; }
                 }
             }
         }
@@ -489,7 +547,7 @@ skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
                         if (HALF && k == 0 && kb == HALF_DIAG && kb > w.kb0) umma_f16_halve(tmem_d, umma_desc(sa), umma_desc(sb), idesc);
                         else umma_f16(tmem_d, umma_desc(sa + k * UMMA_K * 2), umma_desc(sb + k * UMMA_K * 2), idesc, (kb > w.kb0 || k) ? 1u : 0u);
                     umma_commit(&sy.empty[stage]);           // the stage is free, in both CTAs, once these MMAs have read it
-                    if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+                    if (++stage == NST) { stage = 0; phase ^= 1u; }
                 }
                 if (ok) umma_commit(&sy.tmem_full[as]);      // the accumulator is complete once all MMAs are
                 ++it;
@@ -500,59 +558,99 @@ skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
         const uint32_t diff = compare_transpose(H, ldh, a.cols, (int)blockIdx.x * CHECK_WARPS + warp - GEMM_THREADS / 32, (int)gridDim.x * CHECK_WARPS);
         if (diff) sy.asym = 1;
     } else {
-        // ------------------------------------------------------------ epilogue: 4 warps, one row per thread
+        // ------------------------------------------------------------ epilogue: one row per thread, half of the tile's columns
         const int q = warp & 3;                               // the tensor-memory lane quarter this warp may read
+        const int ch = (warp - 2) >> 2, r = q * 32 + lane;    // half of the columns, row of the CTA
+        const bool by_cluster = !HALF && a.cl.labels != nullptr;
+        double *slot = &ep.slot[ch][0][r];
         bool ok = true;
         int it = 0;
-        for (int t = 0; t * ((int)gridDim.x / 2) < nunits && ok; ++t) {
+        for (int t = 0; t * ((int)gridDim.x / 2) < nunits; ++t) {
             const int u = unit_index<HALF>(t, nunits);
             if (u < 0) continue;
             const GemmUnit w = HALF ? half_unit(a, half, u, nkb) : unit_of(a, u, nkb);
             const int as = it & 1;
             const int mb = w.tile % a.mt, nb = w.tile / a.mt;
-            const int row = mb * BM + (int)rank * CM + q * 32 + lane;
-            const int n0 = nb * BN + w.n_off;
-            const uint16_t *drow = a.D + (int64_t)min(row, a.rows - 1) * a.ldd;
+            const int row = mb * BM + (int)rank * CM + r;
+            const int n0 = nb * BN + w.n_off, c0 = ch * (w.n / 2);
+            const int64_t lrow = min(row, a.rows - 1);
+            const uint16_t *drow = a.D + lrow * a.ldd;
+            if (by_cluster) {
+                const int j = threadIdx.x - 64;
+                if (j < w.n) ep.alpha[j] = n0 + j < a.cols ? a.cl.alpha[n0 + j] : 0.0;
+#pragma unroll
+                for (int k = 0; k < KC; ++k) slot[k * CM] = 0.0;
+            }
+            // the operands of the dot (and the labels) do not depend on the accumulator: the next 32 columns' are in flight
+            uint4 dv[4], dn[4];
+            uint2 lv[4], ln[4];
+            auto fetch = [&](int c, uint4 (&d)[4], uint2 (&l)[4]) {
+#pragma unroll
+                for (int v = 0; v < 4; ++v) {
+                    const int col = n0 + c + v * 8;
+                    const bool in = c < c0 + w.n / 2 && col < a.cols;             // cols is a multiple of 8
+                    d[v] = in ? __ldg(reinterpret_cast<const uint4 *>(drow + col)) : make_uint4(0u, 0u, 0u, 0u);
+                    if (by_cluster) l[v] = in ? __ldg(reinterpret_cast<const uint2 *>(a.cl.labels + lrow * a.cols + col)) : make_uint2(0u, 0u);
+                }
+            };
+            fetch(c0, dv, lv);
+            epilogue_barrier();                               // alpha is in place
             ok = mbar_wait(&sy.tmem_full[as], ((uint32_t)it >> 1) & 1u, abort_flag);
             ok = __all_sync(0xffffffffu, ok);
-            if (!ok) break;
-            tc_fence_after();
             float acc = 0.0f;
+            if (ok) {
+                tc_fence_after();
 #pragma unroll 1
-            for (int c = 0; c < w.n / 32; ++c) {
-                const int col = n0 + c * 32;
-                uint4 dv[4];
+                for (int c = c0; c < c0 + w.n / 2; c += 32) {
+                    const int col = n0 + c;
+                    fetch(c + 32, dn, ln);
+                    uint32_t v[32];
+                    tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(as * BN + c), v);
+                    if (!HALF && a.Y && row < a.rows) {
+                        float *yrow = a.Y + (int64_t)row * a.ldy + col;
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    dv[u] = make_uint4(0u, 0u, 0u, 0u);
-                    if (col + u * 8 + 8 <= a.cols) dv[u] = __ldg(reinterpret_cast<const uint4 *>(drow + col + u * 8));
-                }
-                uint32_t v[32];
-                tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(as * BN + c * 32), v);
-                if (!HALF && a.Y && row < a.rows) {
-                    float *yrow = a.Y + (int64_t)row * a.ldy + col;
-#pragma unroll
-                    for (int u = 0; u < 8; ++u)
-                        if (col + u * 4 + 4 <= a.cols)
-                            *reinterpret_cast<uint4 *>(yrow + u * 4) = make_uint4(v[u * 4], v[u * 4 + 1], v[u * 4 + 2], v[u * 4 + 3]);
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const uint32_t w4[4] = {dv[u].x, dv[u].y, dv[u].z, dv[u].w};
-#pragma unroll
-                    for (int h = 0; h < 4; ++h) {
-                        const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&w4[h]));
-                        acc = fmaf(__uint_as_float(v[u * 8 + 2 * h]), f.x, acc);
-                        acc = fmaf(__uint_as_float(v[u * 8 + 2 * h + 1]), f.y, acc);
+                        for (int g = 0; g < 8; ++g)
+                            if (col + g * 4 + 4 <= a.cols)
+                                *reinterpret_cast<uint4 *>(yrow + g * 4) = make_uint4(v[g * 4], v[g * 4 + 1], v[g * 4 + 2], v[g * 4 + 3]);
                     }
+                    // columns past the matrix have a zero accumulator and a zero alpha
+                    if (by_cluster) add_by_cluster(slot, v, lv, ep.alpha + c);
+#pragma unroll
+                    for (int g = 0; g < 4; ++g) {
+                        const uint32_t w4[4] = {dv[g].x, dv[g].y, dv[g].z, dv[g].w};
+#pragma unroll
+                        for (int h = 0; h < 4; ++h) {
+                            const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&w4[h]));
+                            acc = fmaf(__uint_as_float(v[g * 8 + 2 * h]), f.x, acc);
+                            acc = fmaf(__uint_as_float(v[g * 8 + 2 * h + 1]), f.y, acc);
+                        }
+                    }
+#pragma unroll
+                    for (int g = 0; g < 4; ++g) { dv[g] = dn[g]; lv[g] = ln[g]; }
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cluster(cluster_addr(&sy.tmem_empty[as], 0));
+            }
+            if (ch) dot_s[r] = acc;
+            // the other half's dots and sums are in place; a warp whose wait ran out takes all of them out of the loop
+            if (epilogue_barrier_or(!ok)) break;
+            if (ch == 0 && row < a.rows) {
+                acc += dot_s[r];
+                // a piece that reaches past its diagonal blocks holds half the dot (the diagonal blocks' part was halved)
+                if (HALF && w.kb1 > HALF_DIAG) acc *= 2.0f;
+                a.partial[((int64_t)row * (HALF ? SPLIT_MAX : a.split) + w.slice) * a.nt + nb] = acc;
+            }
+            if (by_cluster && row < a.rows) {
+                // this thread's half of the row's clusters
+                double2 *rp = reinterpret_cast<double2 *>(a.cl.rpart + (((int64_t)row * a.nt + nb) * 2 + w.slice) * KC) + ch * (KC / 4);
+#pragma unroll
+                for (int k = 0; k < KC / 2; k += 2) {
+                    const int kk = ch * (KC / 2) + k;
+                    rp[k / 2] = make_double2(ep.slot[0][kk][r] + ep.slot[1][kk][r], ep.slot[0][kk + 1][r] + ep.slot[1][kk + 1][r]);
                 }
             }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(cluster_addr(&sy.tmem_empty[as], 0));
-            // a piece that reaches past its diagonal blocks holds half the dot (the diagonal blocks' part was halved)
-            if (HALF && w.kb1 > HALF_DIAG) acc *= 2.0f;
-            if (row < a.rows) a.partial[((int64_t)row * (HALF ? SPLIT_MAX : a.split) + w.slice) * a.nt + nb] = acc;
+            epilogue_barrier();                               // before the slots, alpha and dots are written again
             ++it;
         }
     }
@@ -595,6 +693,21 @@ skim_lfull_reduce_kernel(GemmArgs a, int exp2, float *__restrict__ err, int64_t 
         const int split = half ? SPLIT_MAX : a.split;
         const int pieces = half ? half_pieces(t, nkb, a.piece_kb) : t * a.mt + mb >= a.full_tiles ? a.split : 1;
         for (int sl = 0; sl < pieces; ++sl) s += (double)a.partial[((int64_t)i * split + sl) * a.nt + t];
+    }
+    if (a.cl.labels) {
+        // R_k = sum_{j in k} Y_ij alpha_j over the column tiles, q_k = 2 R_k / (2^exp2 G_k) into the row's table
+        const int k = lane & (KC - 1);
+        double r = 0.0;
+        for (int t = lane / KC; t < a.nt; t += 32 / KC) {
+            const double *p = a.cl.rpart + ((int64_t)i * a.nt + t) * 2 * KC + k;
+            r += p[0];
+            if (a.split == 2 && t * a.mt + mb >= a.full_tiles) r += p[KC];
+        }
+        r += __shfl_down_sync(0xffffffffu, r, KC);
+        if (lane < KC) {
+            const double gk = a.cl.tconst[(int64_t)i * KC + lane].x;
+            a.cl.tq[(int64_t)i * KC + lane].y = gk > 0.0 ? ldexp(2.0 * r, -exp2) / gk : 0.0;
+        }
     }
 #pragma unroll
     for (int off = 16; off; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
@@ -674,6 +787,11 @@ int skim_launch_residual(skim_ctx *ctx, const uint16_t *W, int64_t rows, int64_t
     return SKIM_OK;
 }
 
+size_t skim_lfull_cluster_bytes(int64_t rows, int64_t cols)
+{
+    return skim_align256((size_t)rows * ((cols + BN - 1) / BN) * 2 * KC * sizeof(double));
+}
+
 size_t skim_lfull_scratch_bytes(int64_t rows, int64_t cols)
 {
     const int64_t mt = (rows + BM - 1) / BM, nt = (cols + BN - 1) / BN;
@@ -682,7 +800,7 @@ size_t skim_lfull_scratch_bytes(int64_t rows, int64_t cols)
 
 int skim_launch_err_lfull(skim_ctx *ctx, const uint16_t *D, int64_t rows, int64_t cols, int64_t ldd, const uint16_t *H,
                           int64_t ldh, int exp2, void *scratch, float *err, int64_t err_stride, float *Y, int64_t ldy,
-                          double *err64)
+                          double *err64, const SkimLfullClusters *clusters)
 {
     if (rows == 0) return SKIM_OK;
     CUtensorMap map_a, map_b;
@@ -700,8 +818,10 @@ int skim_launch_err_lfull(skim_ctx *ctx, const uint16_t *D, int64_t rows, int64_
     a.partial = (float *)scratch;
     a.Y = Y;
     a.ldy = ldy;
+    a.cl = clusters ? *clusters : SkimLfullClusters{};
+    const size_t smem = gemm_smem(false);
     a.status = (unsigned long long *)ctx->ws;
-    SKIM_CUDA_OK(cudaFuncSetAttribute(skim_lfull_gemm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GEMM_SMEM));
+    SKIM_CUDA_OK(cudaFuncSetAttribute(skim_lfull_gemm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const int tiles = a.mt * a.nt;
     // the tiles of the last round, if it is not full, are cut along K into as many ranges as fit the SMs
     const int nkb = (int)((cols + BK - 1) / BK);
@@ -744,14 +864,14 @@ int skim_launch_err_lfull(skim_ctx *ctx, const uint16_t *D, int64_t rows, int64_
         }
         a.asym = (int *)((char *)scratch + skim_lfull_scratch_bytes(rows, cols) - HALF_FLAG_BYTES);
         a.asym_n = 2 * pairs;
-        SKIM_CUDA_OK(cudaFuncSetAttribute(skim_lfull_gemm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GEMM_SMEM));
-        skim_lfull_gemm_kernel<true><<<(unsigned)(2 * pairs), GEMM_THREADS + CHECK_WARPS * 32, GEMM_SMEM, ctx->stream>>>(map_a, map_b, a, H, ldh);
+        SKIM_CUDA_OK(cudaFuncSetAttribute(skim_lfull_gemm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem(true)));
+        skim_lfull_gemm_kernel<true><<<(unsigned)(2 * pairs), GEMM_THREADS + CHECK_WARPS * 32, gemm_smem(true), ctx->stream>>>(map_a, map_b, a, H, ldh);
         SKIM_CUDA_OK(cudaGetLastError());
         ctx->launches += 1;
     }
     const int units = a.full_tiles + (tiles - a.full_tiles) * a.split;
     const unsigned blocks = (unsigned)(2 * (units < pairs ? units : pairs));    // persistent: one CTA per SM
-    skim_lfull_gemm_kernel<false><<<blocks, GEMM_THREADS, GEMM_SMEM, ctx->stream>>>(map_a, map_b, a, H, ldh);
+    skim_lfull_gemm_kernel<false><<<blocks, GEMM_THREADS, smem, ctx->stream>>>(map_a, map_b, a, H, ldh);
     SKIM_CUDA_OK(cudaGetLastError());
     skim_lfull_reduce_kernel<<<(unsigned)((rows + RED_WARPS - 1) / RED_WARPS), RED_WARPS * 32, 0, ctx->stream>>>(a, exp2, err, err_stride, err64);
     SKIM_CUDA_OK(cudaGetLastError());

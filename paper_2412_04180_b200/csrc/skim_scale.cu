@@ -17,14 +17,12 @@
 //       cluster, from the 256-byte table the first kernel left for the row), accumulated in
 //       registers; the row ranges leave partial gradients that the Adam kernel adds in a fixed order.
 //   skim_scale_adam_kernel  sums the partials and the rows' losses (deterministic), applies the
-//       Adam update to the binary64 master copy of alpha and to its lane-interleaved copy, the
-//       one the row-wise kernels read (alpha_il_pos).
+//       Adam update to the binary64 master copy of alpha.
 #include "skim_internal.cuh"
 
 namespace {
 
 constexpr int KC = 16;      // clusters per row at most (4 bits)
-constexpr int SW = 4;       // warps (rows) per block of the sums kernel
 constexpr int GT = 256;     // threads of a gradient block
 constexpr int GC = 4;       // columns per thread
 
@@ -33,7 +31,6 @@ struct ScaleArgs {
     const float *G;
     const uint8_t *labels;
     const double *alpha;
-    const double *alpha_il; // alpha in the lane-interleaved order of alpha_il_pos()
     int64_t rows, ld;
     int cols;
     int vec;                // rows of W, G and labels allow the vector loads of both kernels
@@ -43,18 +40,10 @@ struct ScaleArgs {
     double2 *tq;            // [rows][KC]  (c_k, q_k)
     double *loss_row;       // [rows]
     double *grad_part;      // [row ranges][cols]
+    uint16_t *D;            // L-full loss: [rows][cols] binary16 residual * 2^exp2
+    int exp2;
     int rows_per_range;
 };
-
-// A lane of the row-wise kernels owns eight consecutive columns of every 256 and reads their alphas two at a
-// time.  From the plain array those reads are 64 bytes apart across the lanes (sixteen 128-byte wavefronts of the
-// L1 data path for 512 useful bytes, and that path is what bounds the sums kernel); from this order -- the u-th
-// pair of lane L at 64 u + 2 L of its block of 256 -- a warp's read is one contiguous 512 bytes.
-__host__ __device__ __forceinline__ int alpha_il_pos(int j)
-{
-    const int r = j & 255;
-    return (j & ~255) + 64 * ((r >> 1) & 3) + 2 * (r >> 3) + (r & 1);
-}
 
 // Every kernel of an Adam step is launched as a programmatic dependent of the one before it: it may start while that
 // one drains, fetches what no kernel of the loop writes (the matrix), and waits here before it touches anything else.
@@ -256,6 +245,27 @@ __host__ __device__ __forceinline__ size_t sums_smem_bytes(int cols, bool init)
     return (init ? 0 : ((size_t)cols + 1) / 2 * 16) + (size_t)SUM_W * 2 * 32 * sizeof(double);
 }
 
+__device__ __forceinline__ double weight_of(const uint2 &w, int u)
+{
+    const uint32_t x = u < 2 ? w.x : w.y;
+    return (double)__half2float(__ushort_as_half((uint16_t)((u & 1) ? (x >> 16) : (x & 0xffffu))));
+}
+
+// The tables of two rows in one register pair: lane L holds entry L % 16 of row `row` + L / 16.
+__device__ __forceinline__ double2 table_load(const ScaleArgs &a, int64_t row, int64_t last)
+{
+    const int lane = threadIdx.x & 31;
+    return a.tq[min(row + (lane >> 4), last) * KC + (lane & 15)];
+}
+// Shuffle indices of four labels: byte u holds label u, plus 16 for the second row of the pair (a shuffle takes the
+// low five bits of its index, so `>> 8 u` is all an element needs).
+__device__ __forceinline__ uint32_t table_index(uint32_t l, int second) { return (l & 0x0f0f0f0fu) | (second ? 0x10101010u : 0u); }
+__device__ __forceinline__ double2 table_get(const double2 &t, uint32_t index, int u)
+{
+    const int src = (int)(index >> (8 * u));
+    return make_double2(__shfl_sync(0xffffffffu, t.x, src), __shfl_sync(0xffffffffu, t.y, src));
+}
+
 // The two elements a lane has of a unit, added to its accumulators.
 template <int MODE>
 __device__ __forceinline__ void add_element(uint32_t gbits, uint32_t wcol, const double *alpha, double (&acc)[3])
@@ -333,19 +343,19 @@ __device__ __forceinline__ void sum_units(const uint4 *src, int end, int t0, int
 // What the sums of a row are turned into (lanes as sum_units leaves them).
 //   SUMS_INIT       the per-call constants (G_k, D_k)
 //   SUMS_STEP       (c_k, q_k) and the row's loss
-//   SUMS_CENTROIDS  (c_k, 0)
+//   SUMS_CENTROIDS  (c_k, 0); the kernel then writes the row's residual
 template <int MODE>
-__device__ __forceinline__ void finish_row(const ScaleArgs &a, int64_t row, double vx, double vb)
+__device__ __forceinline__ double finish_row(const ScaleArgs &a, int64_t row, double vx, double vb)
 {
     const int lane = threadIdx.x & 31;
     const double s1 = __shfl_down_sync(0xffffffffu, vx, 16);
-    double loss_k = 0.0;
+    double loss_k = 0.0, c = 0.0;
     if (lane < KC) {
         if (MODE == SUMS_INIT) {
             a.tconst[row * KC + lane] = make_double2(vx, s1);
         } else {
             const double2 gdk = a.tconst[row * KC + lane];
-            double c = 0.0, q = 0.0;
+            double q = 0.0;
             if (gdk.x > 0.0) {
                 c = vx / gdk.x;
                 if (MODE == SUMS_STEP) {
@@ -361,6 +371,43 @@ __device__ __forceinline__ void finish_row(const ScaleArgs &a, int64_t row, doub
         for (int off = 8; off; off >>= 1) loss_k += __shfl_down_sync(0xffffffffu, loss_k, off);
         if (lane == 0) a.loss_row[row] = loss_k;
     }
+    return c;
+}
+
+// L-full loss: the residual of columns [j0, j1) of a row as the binary16 operand of the contraction; c: the centroid of
+// cluster lane % 16.  Four consecutive columns per lane and step.
+__device__ __forceinline__ void residual_columns(const ScaleArgs &a, int64_t row, int j0, int j1, const double *alpha, double c)
+{
+    constexpr int RU = 4;                                     // steps whose loads are in flight
+    const int lane = threadIdx.x & 31;
+    const float scale = __int_as_float((127 + a.exp2) << 23);
+    const uint16_t *Wr = a.W + row * a.ld;
+    const uint8_t *Lr = a.labels + row * (int64_t)a.cols;
+    uint16_t *Dr = a.D + row * (int64_t)a.cols;
+    for (int jb = j0; jb < j1; jb += RU * 128) {
+        uint2 w[RU];
+        uint32_t l[RU];
+#pragma unroll
+        for (int u = 0; u < RU; ++u) {
+            const int j = min(jb + u * 128 + lane * 4, j1 - 4);
+            w[u] = __ldcs(reinterpret_cast<const uint2 *>(Wr + j));
+            l[u] = __ldcs(reinterpret_cast<const uint32_t *>(Lr + j));
+        }
+#pragma unroll
+        for (int u = 0; u < RU; ++u) {
+            const int j = min(jb + u * 128 + lane * 4, j1 - 4);      // lanes past the end repeat the last columns
+            const double2 a0 = *reinterpret_cast<const double2 *>(alpha + j), a1 = *reinterpret_cast<const double2 *>(alpha + j + 2);
+            const double al[4] = {a0.x, a0.y, a1.x, a1.y};
+            const uint32_t index = table_index(l[u], 0);
+            uint32_t h[4];
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                const double d = weight_of(w[u], v) - al[v] * __shfl_sync(0xffffffffu, c, (int)(index >> (8 * v)));
+                h[v] = __half_as_ushort(__float2half_rn(__fmul_rn((float)d, scale)));
+            }
+            *reinterpret_cast<uint2 *>(Dr + j) = make_uint2(h[0] | (h[1] << 16), h[2] | (h[3] << 16));
+        }
+    }
 }
 
 // One block per SM, rows dealt round-robin to the blocks.  A warp takes whole rows while there are rows for all of the
@@ -374,6 +421,18 @@ __global__ void __launch_bounds__(SUM_T, 1) skim_scale_sums_kernel(ScaleArgs a)
     double *alpha = ssmem;
     double2 *part = reinterpret_cast<double2 *>(ssmem + (MODE == SUMS_INIT ? 0 : (a.cols + 1) / 2 * 2));     // [SUM_W][32]
     let_next_kernel_start();
+    const int64_t stride = skim_ordered_stride(a.cols) / 2;
+    const int mine = (int)((a.rows - blockIdx.x + gridDim.x - 1) / gridDim.x);       // rows of this block (at least one)
+    const int whole = mine / SUM_W * SUM_W, rest = mine - whole;
+    if (MODE != SUMS_INIT) {
+        // the start of this warp's first row, while the previous kernel ends
+        const int r = whole ? warp : warp / (SUM_W / rest);
+        if (r < mine) {
+            const uint4 *p = reinterpret_cast<const uint4 *>(a.ord) + (blockIdx.x + (int64_t)gridDim.x * r) * stride;
+#pragma unroll
+            for (int u = 0; u < 2 * AHEAD; ++u) asm volatile("prefetch.global.L2 [%0];" ::"l"(p + u * (UNIT / 2) + lane));
+        }
+    }
     wait_for_previous_kernel();
     if (MODE != SUMS_INIT) {
         for (int q = threadIdx.x; q < a.cols / 2; q += SUM_T)
@@ -381,15 +440,13 @@ __global__ void __launch_bounds__(SUM_T, 1) skim_scale_sums_kernel(ScaleArgs a)
         if ((a.cols & 1) && threadIdx.x == 0) alpha[a.cols - 1] = a.alpha[a.cols - 1];
         __syncthreads();
     }
-    const int64_t stride = skim_ordered_stride(a.cols) / 2;
-    const int mine = (int)((a.rows - blockIdx.x + gridDim.x - 1) / gridDim.x);       // rows of this block (at least one)
-    const int whole = mine / SUM_W * SUM_W, rest = mine - whole;
     double vx, vb;
     for (int r = warp; r < whole; r += SUM_W) {
         const int64_t row = blockIdx.x + (int64_t)gridDim.x * r;
         const int end = a.ord_end[row * KC + (lane & 15)];
         sum_units<MODE>(reinterpret_cast<const uint4 *>(a.ord) + row * stride, end, 0, __shfl_sync(0xffffffffu, end, KC - 1), alpha, vx, vb);
-        finish_row<MODE>(a, row, vx, vb);
+        const double c = finish_row<MODE>(a, row, vx, vb);
+        if (MODE == SUMS_CENTROIDS) residual_columns(a, row, 0, a.cols, alpha, c);
     }
     if (rest == 0) return;
     const int per_row = SUM_W / rest, idx = warp / per_row, sub = warp - idx * per_row;
@@ -408,7 +465,14 @@ __global__ void __launch_bounds__(SUM_T, 1) skim_scale_sums_kernel(ScaleArgs a)
             vx += o.x;
             vb += o.y;
         }
-        finish_row<MODE>(a, row, vx, vb);
+        const double c = finish_row<MODE>(a, row, vx, vb);
+        if (MODE == SUMS_CENTROIDS) part[threadIdx.x].x = c;
+    }
+    if (MODE == SUMS_CENTROIDS) {
+        // the row's columns are shared by the same warps (in fours: cols is a multiple of 8 on this path)
+        __syncthreads();
+        const int quads = a.cols / 4, q0 = quads * sub / per_row, q1 = quads * (sub + 1) / per_row;
+        if (idx < rest && q0 < q1) residual_columns(a, row, q0 * 4, q1 * 4, alpha, part[idx * per_row * 32 + lane].x);
     }
 }
 
@@ -469,27 +533,6 @@ __device__ __forceinline__ void grad_load(const ScaleArgs &a, int64_t row, const
     }
 }
 
-__device__ __forceinline__ double weight_of(const uint2 &w, int u)
-{
-    const uint32_t x = u < 2 ? w.x : w.y;
-    return (double)__half2float(__ushort_as_half((uint16_t)((u & 1) ? (x >> 16) : (x & 0xffffu))));
-}
-
-// The tables of two rows in one register pair: lane L holds entry L % 16 of row `row` + L / 16.
-__device__ __forceinline__ double2 table_load(const ScaleArgs &a, int64_t row, int64_t last)
-{
-    const int lane = threadIdx.x & 31;
-    return a.tq[min(row + (lane >> 4), last) * KC + (lane & 15)];
-}
-// Shuffle indices of four labels: byte u holds label u, plus 16 for the second row of the pair (a shuffle takes the
-// low five bits of its index, so `>> 8 u` is all an element needs).
-__device__ __forceinline__ uint32_t table_index(uint32_t l, int second) { return (l & 0x0f0f0f0fu) | (second ? 0x10101010u : 0u); }
-__device__ __forceinline__ double2 table_get(const double2 &t, uint32_t index, int u)
-{
-    const int src = (int)(index >> (8 * u));
-    return make_double2(__shfl_sync(0xffffffffu, t.x, src), __shfl_sync(0xffffffffu, t.y, src));
-}
-
 template <bool VEC>
 __global__ void __launch_bounds__(GT, 2) skim_scale_grad_kernel(ScaleArgs a)
 {
@@ -548,7 +591,7 @@ __global__ void __launch_bounds__(GT, 2) skim_scale_grad_kernel(ScaleArgs a)
 
 __global__ void __launch_bounds__(256) skim_scale_adam_kernel(const double *__restrict__ grad_part,
                                                                const double *__restrict__ loss_row, int nranges,
-                                                               int64_t rows, int cols, double *alpha, double *alpha_il,
+                                                               int64_t rows, int cols, double *alpha,
                                                                double *m1, double *m2, double lr, double beta1, double beta2,
                                                                double bc1, double bc2, double eps, double *loss_out)
 {
@@ -587,10 +630,9 @@ __global__ void __launch_bounds__(256) skim_scale_adam_kernel(const double *__re
     m2[j] = a2;
     const double an = alpha[j] - lr * (a1 / bc1) / (sqrt(a2 / bc2) + eps);
     alpha[j] = an;
-    alpha_il[alpha_il_pos(j)] = an;
 }
 
-__global__ void skim_scale_init_kernel(const float *__restrict__ alpha32, int cols, double *alpha, double *alpha_il,
+__global__ void skim_scale_init_kernel(const float *__restrict__ alpha32, int cols, double *alpha,
                                        double *m1, double *m2, unsigned long long *status)
 {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
@@ -598,7 +640,6 @@ __global__ void skim_scale_init_kernel(const float *__restrict__ alpha32, int co
     const float v = alpha32[j];
     if (!(v > 0.0f) || v > 3.0e38f) atomicOr(status, (unsigned long long)SKIM_STATUS_BAD_SCALE);
     alpha[j] = (double)v;
-    alpha_il[alpha_il_pos(j)] = (double)v;
     m1[j] = 0.0;
     m2[j] = 0.0;
 }
@@ -614,116 +655,19 @@ __global__ void skim_scale_finish_kernel(const double *__restrict__ alpha, int c
 //   loss(alpha) = sum_i d_i H d_i^T,  d_ij = W_ij - alpha_j c_{i,l_ij},  H = X X^T   (Section 4.3 with the L-full form of
 //   Section 3.4).  With Y = D H:  d loss / d alpha_j = sum_i -2 Y_ij c_{i,l} + q_{i,l} g_ij W_ij / alpha_j^2,
 //   q_ik = 2 R_ik / G_ik,  R_ik = sum_{j in k} Y_ij alpha_j.
-// Per Adam step: skim_scale_lf_residual_kernel (centroids of the step, residual as the binary16 operand of the
-// contraction), the tcgen05 GEMM of skim_lfull.cu (Y = D H stored, row-wise dot = the loss), skim_scale_lf_r_kernel
-// (R_ik, q_ik), skim_scale_lf_grad_kernel (column sums), and the Adam kernel above.
-
-struct ScaleLfArgs {
-    ScaleArgs s;
-    uint16_t *D;         // [rows][cols] binary16 residual * 2^exp2
-    const float *Y;      // [rows][cols] binary32, D H
-    int exp2;
-};
-
-// The residual as the operand of the contraction: one warp per stretch of RES_COLS columns of a row.
-constexpr int RES_COLS = 2048;
-
-__global__ void __launch_bounds__(SW * 32) skim_scale_lf_residual_kernel(ScaleLfArgs b)
-{
-    __shared__ double cs_all[SW][KC];
-    const ScaleArgs &a = b.s;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int parts = (a.cols + RES_COLS - 1) / RES_COLS;
-    const int64_t unit = (int64_t)blockIdx.x * SW + warp, row = unit / parts;
-    if (row >= a.rows) return;
-    const int j0 = (int)(unit % parts) * RES_COLS, j1 = min(j0 + RES_COLS, a.cols);
-    double *cs = cs_all[warp];
-    let_next_kernel_start();
-    wait_for_previous_kernel();
-    if (lane < KC) cs[lane] = a.tq[row * KC + lane].x;
-    __syncwarp();
-    const float scale = __int_as_float((127 + b.exp2) << 23);
-    const uint16_t *Wr = a.W + row * a.ld;
-    const uint8_t *Lr = a.labels + row * (int64_t)a.cols;
-    uint16_t *Dr = b.D + row * (int64_t)a.cols;
-    for (int e0 = j0 + lane * 8; e0 < j1; e0 += 256) {
-        const uint4 wv = __ldcs(reinterpret_cast<const uint4 *>(Wr + e0));
-        const uint2 lv = __ldcs(reinterpret_cast<const uint2 *>(Lr + e0));
-        double al[8];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const double2 t = __ldg(reinterpret_cast<const double2 *>(a.alpha_il + alpha_il_pos(e0 + 2 * u)));
-            al[2 * u] = t.x;
-            al[2 * u + 1] = t.y;
-        }
-        const uint32_t ww[4] = {wv.x, wv.y, wv.z, wv.w};
-        uint32_t out[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const float wf = __half2float(__ushort_as_half((uint16_t)((u & 1) ? (ww[u >> 1] >> 16) : (ww[u >> 1] & 0xffffu))));
-            const int l = (int)(((u < 4 ? lv.x : lv.y) >> (8 * (u & 3))) & (KC - 1));
-            const double d = (double)wf - al[u] * cs[l];
-            const uint32_t h = __half_as_ushort(__float2half_rn(__fmul_rn((float)d, scale)));
-            out[u >> 1] |= h << (16 * (u & 1));
-        }
-        *reinterpret_cast<uint4 *>(Dr + e0) = make_uint4(out[0], out[1], out[2], out[3]);
-    }
-}
-
-// One warp per row: R_k = sum_{j in k} Y_ij alpha_j, q_k = 2 R_k / (2^exp2 G_k) into the row's table.
-__global__ void __launch_bounds__(SW * 32) skim_scale_lf_r_kernel(ScaleLfArgs b)
-{
-    extern __shared__ __align__(16) double slots_all[];       // [SW][KC][32]
-    const ScaleArgs &a = b.s;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t row = (int64_t)blockIdx.x * SW + warp;
-    let_next_kernel_start();
-    wait_for_previous_kernel();
-    if (row >= a.rows) return;
-    double *slot = slots_all + (size_t)warp * (KC * 32) + lane;
-#pragma unroll
-    for (int q = 0; q < KC; ++q) slot[q * 32] = 0.0;
-    const float *Yr = b.Y + row * (int64_t)a.cols;
-    const uint8_t *Lr = a.labels + row * (int64_t)a.cols;
-    for (int e0 = lane * 8; e0 < a.cols; e0 += 256) {
-        const float4 ya = __ldcs(reinterpret_cast<const float4 *>(Yr + e0)), yb = __ldcs(reinterpret_cast<const float4 *>(Yr + e0 + 4));
-        const uint2 lv = __ldcs(reinterpret_cast<const uint2 *>(Lr + e0));
-        const float y[8] = {ya.x, ya.y, ya.z, ya.w, yb.x, yb.y, yb.z, yb.w};
-        double al[8];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const double2 t = __ldg(reinterpret_cast<const double2 *>(a.alpha_il + alpha_il_pos(e0 + 2 * u)));
-            al[2 * u] = t.x;
-            al[2 * u + 1] = t.y;
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int l = (int)(((u < 4 ? lv.x : lv.y) >> (8 * (u & 3))) & (KC - 1));
-            slot[l * 32] += (double)y[u] * al[u];
-        }
-    }
-    __syncwarp();
-    if (lane < KC) {
-        const double *base = slots_all + (size_t)warp * (KC * 32) + lane * 32;
-        double v = 0.0;
-        for (int t = 0; t < 32; ++t) v += base[(t + lane) & 31];
-        const double gk = a.tconst[row * KC + lane].x;
-        double2 cq = a.tq[row * KC + lane];
-        cq.y = gk > 0.0 ? ldexp(2.0 * v, -b.exp2) / gk : 0.0;
-        a.tq[row * KC + lane] = cq;
-    }
-}
+// Per Adam step: skim_scale_sums_kernel (centroids of the step, and the residual as the binary16 operand of the
+// contraction), the tcgen05 GEMM of skim_lfull.cu (Y = D H stored, row-wise dot = the loss, R_ik summed in its epilogue
+// and q_ik in its reduction), skim_scale_lf_grad_kernel (column sums), and the Adam kernel above.
 
 // A thread owns four columns and walks a range of rows: sum_i -2 Y_ij c + q g w / alpha_j^2; as skim_scale_grad_kernel
 // (cols is a multiple of 8 and the rows are aligned: vector loads always).
-__global__ void __launch_bounds__(GT, 2) skim_scale_lf_grad_kernel(ScaleLfArgs b)
+__global__ void __launch_bounds__(GT, 2) skim_scale_lf_grad_kernel(ScaleArgs a, const float *Y)
 {
     constexpr int RB = 2;
-    const ScaleArgs &a = b.s;
     const GradCols<true> c(blockIdx.x, a.cols);
     const int64_t r0 = (int64_t)blockIdx.y * a.rows_per_range;
     const int64_t r1 = min(a.rows, r0 + a.rows_per_range), last = r1 - 1;
-    const double ys = ldexp(-2.0, -b.exp2);
+    const double ys = ldexp(-2.0, -a.exp2);
     let_next_kernel_start();
     wait_for_previous_kernel();
     double rr[GC], acc[GC];
@@ -741,7 +685,7 @@ __global__ void __launch_bounds__(GT, 2) skim_scale_lf_grad_kernel(ScaleLfArgs b
         for (int q = 0; q < RB; ++q) {
             const int64_t i = min(rb + q, last);
             grad_load<true>(a, i, c, row[h][q]);
-            yv[h][q] = __ldcs(reinterpret_cast<const float4 *>(b.Y + i * (int64_t)a.cols + c.j[0]));
+            yv[h][q] = __ldcs(reinterpret_cast<const float4 *>(Y + i * (int64_t)a.cols + c.j[0]));
         }
         tab[h] = table_load(a, rb, last);
         tab[h].x *= ys;                 // -2 c / 2^exp2
@@ -776,7 +720,8 @@ __global__ void __launch_bounds__(GT, 2) skim_scale_lf_grad_kernel(ScaleLfArgs b
 
 size_t skim_scale_lfull_scratch_bytes(int64_t rows, int64_t cols)
 {
-    return skim_align256((size_t)rows * cols * 2) + skim_align256((size_t)rows * cols * 4) + skim_lfull_scratch_bytes(rows, cols);
+    return skim_align256((size_t)rows * cols * 2) + skim_align256((size_t)rows * cols * 4) + skim_lfull_cluster_bytes(rows, cols) +
+           skim_lfull_scratch_bytes(rows, cols);
 }
 
 namespace {
@@ -819,7 +764,6 @@ int scale_begin(skim_ctx *ctx, const SkimWorkspace &ws, const uint16_t *W, const
     a.G = importance;
     a.labels = labels;
     a.alpha = ws.alpha64;
-    a.alpha_il = ws.alpha_il;
     a.rows = rows;
     a.ld = ld;
     a.cols = (int)cols;
@@ -831,6 +775,8 @@ int scale_begin(skim_ctx *ctx, const SkimWorkspace &ws, const uint16_t *W, const
     a.tq = reinterpret_cast<double2 *>(ws.scale_cq);
     a.loss_row = ws.loss_part;
     a.grad_part = ws.grad_part;
+    a.D = nullptr;
+    a.exp2 = 0;
     // gradient kernels: column tiles x row ranges, one wave of two blocks per SM
     const int tiles = (int)((cols + GT * GC - 1) / (GT * GC));
     int ranges = 2 * ctx->sm_count / tiles;
@@ -848,7 +794,7 @@ int scale_begin(skim_ctx *ctx, const SkimWorkspace &ws, const uint16_t *W, const
     SKIM_CUDA_OK(cudaFuncSetAttribute(skim_scale_sums_kernel<SUMS_INIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm_init));
     SKIM_CUDA_OK(cudaFuncSetAttribute(skim_scale_sums_kernel<SUMS_STEP>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm_sums));
     SKIM_CUDA_OK(cudaFuncSetAttribute(skim_scale_sums_kernel<SUMS_CENTROIDS>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm_sums));
-    skim_scale_init_kernel<<<p->cb, 256, 0, ctx->stream>>>(alpha, (int)cols, ws.alpha64, ws.alpha_il, ws.adam_m, ws.adam_v, ws.status);
+    skim_scale_init_kernel<<<p->cb, 256, 0, ctx->stream>>>(alpha, (int)cols, ws.alpha64, ws.adam_m, ws.adam_v, ws.status);
     SKIM_CUDA_OK(cudaGetLastError());
     skim_scale_order_kernel<<<(unsigned)rows, OT, sm_order, ctx->stream>>>(a);
     SKIM_CUDA_OK(cudaGetLastError());
@@ -875,7 +821,7 @@ struct AdamSchedule {
 int scale_adam(skim_ctx *ctx, const SkimWorkspace &ws, const ScalePlan &p, const AdamSchedule &s, double *loss_trace)
 {
     return launch_dependent(ctx, skim_scale_adam_kernel, dim3(p.ab + 1), 256, 0, (const double *)ws.grad_part, (const double *)ws.loss_part, p.ranges,
-                            p.a.rows, p.a.cols, ws.alpha64, ws.alpha_il, ws.adam_m, ws.adam_v, s.lr, 0.9, 0.999, 1.0 - s.p1, 1.0 - s.p2,
+                            p.a.rows, p.a.cols, ws.alpha64, ws.adam_m, ws.adam_v, s.lr, 0.9, 0.999, 1.0 - s.p1, 1.0 - s.p2,
                             1e-8, loss_trace ? loss_trace + (s.t - 1) : nullptr);
 }
 
@@ -898,31 +844,27 @@ int skim_launch_scale_update_lfull(skim_ctx *ctx, const uint16_t *W, const float
     ScalePlan p;
     int rc = scale_begin(ctx, ws, W, importance, rows, cols, ld, labels, alpha, &p);
     if (rc) return rc;
-    ScaleLfArgs b;
-    b.s = p.a;
     unsigned char *sp = (unsigned char *)scratch;
-    b.D = (uint16_t *)sp;
+    p.a.D = (uint16_t *)sp;
     sp += skim_align256((size_t)rows * cols * 2);
     float *Y = (float *)sp;
     sp += skim_align256((size_t)rows * cols * 4);
-    void *gemm_scratch = sp;
-    b.Y = Y;
-    b.exp2 = exp2;
-    const size_t smem_r = (size_t)SW * KC * 32 * sizeof(double);
-    const unsigned row_blocks = (unsigned)((rows + SW - 1) / SW);
-    const unsigned res_blocks = (unsigned)((rows * ((cols + RES_COLS - 1) / RES_COLS) + SW - 1) / SW);
+    SkimLfullClusters cl;
+    cl.labels = labels;
+    cl.alpha = ws.alpha64;
+    cl.rpart = (double *)sp;
+    cl.tconst = p.a.tconst;
+    cl.tq = p.a.tq;
+    sp += skim_lfull_cluster_bytes(rows, cols);
+    p.a.exp2 = exp2;
     AdamSchedule sched(lr0, decay, decay_every);
     for (int t = 0; t < steps; ++t) {
         sched.next();
         rc = launch_dependent(ctx, skim_scale_sums_kernel<SUMS_CENTROIDS>, dim3(p.sum_blocks), SUM_T, sums_smem_bytes((int)cols, false), p.a);
         if (rc) return rc;
-        rc = launch_dependent(ctx, skim_scale_lf_residual_kernel, dim3(res_blocks), SW * 32, 0, b);
+        rc = skim_launch_err_lfull(ctx, p.a.D, rows, cols, cols, H, ldh, exp2, sp, nullptr, 1, Y, cols, ws.loss_part, &cl);
         if (rc) return rc;
-        rc = skim_launch_err_lfull(ctx, b.D, rows, cols, cols, H, ldh, exp2, gemm_scratch, nullptr, 1, Y, cols, ws.loss_part);
-        if (rc) return rc;
-        rc = launch_dependent(ctx, skim_scale_lf_r_kernel, dim3(row_blocks), SW * 32, smem_r, b);
-        if (rc) return rc;
-        rc = launch_dependent(ctx, skim_scale_lf_grad_kernel, p.grad_grid, GT, 0, b);
+        rc = launch_dependent(ctx, skim_scale_lf_grad_kernel, p.grad_grid, GT, 0, p.a, (const float *)Y);
         if (rc) return rc;
         rc = scale_adam(ctx, ws, p, sched, loss_trace);
         if (rc) return rc;
