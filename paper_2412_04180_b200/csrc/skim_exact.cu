@@ -8,13 +8,17 @@
 // evaluations.  One block owns a row and reads the row record the sort kernels leave (sorted values and
 // importances by groups of 8 with their binary64 prefix sums).
 //
-//   prefix   the record's two-level prefix sums become one flat array Q[t] = (P0, P1, P2, F_{j-1})(t): a cost
-//            evaluation is one 32-byte load.
+//   prefix   the record's two-level prefix sums become flat arrays P0, P1, P2 (sums of g, g x, g x^2) and
+//            A = F_{j-1} - P2: the cost of a candidate is A(t) - S1^2 / S0 up to a term of i alone, so a candidate needs
+//            (P0, P1, A)(t), 24 bytes.  They sit in shared memory where the row fits, else in global memory.
 //   layer    positions are visited like the in-order nodes of a perfect binary tree, level by level: a node's
 //            search range is bounded by the minimisers of its two nearest finished neighbours.  The ranges of
-//            a level tile the span of split points; the span is dealt to the threads in equal stretches and
-//            the candidates of a node meet in one atomic minimum, because the ranges themselves are very
-//            unequal (the minimiser jumps where an outlier enters the prefix).
+//            a level tile the span of split points, sharing their end points, so candidate number x of node q in
+//            the level's list of all candidates is known without a scan: P(q) = tlo(q) - tlo(0) + q come before it.  The list is
+//            dealt to the threads in equal stretches -- by candidates, not by nodes or by split points: one range can be a
+//            thousand times another (the minimiser jumps where an outlier enters the prefix), and a thousand nodes
+//            can share one split point (it stays put while the elements behind it weigh nothing).  Nodes that end inside a
+//            thread's stretch are written at once; the rest meet in a segmented minimum over the lanes, then over the warps.
 //   result   for every width the split points are walked back from the row's end; centroid = weighted mean of
 //            its interval (an interval without weight: mean of its first and last value), error = F_k(m).
 // All widths share the layers: F_2, F_4, F_8, F_16 are read off on the way.
@@ -24,11 +28,10 @@ namespace {
 
 using namespace skimk;
 
-constexpr int XT = 256;                       // threads per block
 constexpr int X_MAX_K = 1 << SKIM_MAX_BIT;    // 16 layers at most
 
 struct ExactSlot {
-    size_t q, fc, t, total;                   // byte offsets inside a block's scratch slot
+    size_t q, t, total;                       // byte offsets inside a block's scratch slot
 };
 
 __host__ __device__ inline ExactSlot exact_slot(int m)
@@ -37,61 +40,111 @@ __host__ __device__ inline ExactSlot exact_slot(int m)
     const size_t mpad = ((size_t)m + 7) & ~(size_t)7;
     size_t off = 0;
     auto take = [&](size_t b) { size_t o = off; off += (b + 255) & ~(size_t)255; return o; };
-    S.q = take((mpad + 8) * 32);                                  // double4 per position 0 .. mpad
-    S.fc = take(((size_t)m + 1) * 8);                             // the layer being filled
+    S.q = take((mpad + 8) * 32);                                  // (P0, P1, P2, A) of position 0 .. mpad; only P2 where the rest is in shared memory
     S.t = take((size_t)(X_MAX_K + 1) * ((size_t)m + 1) * 2);      // minimisers of every layer, 16-bit
     S.total = off;
     return S;
 }
 
-// shared memory: the minimisers by tree position (2^L + 8 entries, 2^L - 1 >= m), then one key per node of a level
+// A candidate: the node it belongs to, its cost, its split point.
+struct Cand {
+    double v;
+    int q, t;
+};
+__device__ __forceinline__ bool better(const Cand &x, const Cand &y) { return x.v < y.v || (x.v == y.v && x.t < y.t); }
+__device__ __forceinline__ Cand shfl_up(const Cand &c, int off)
+{
+    Cand r;
+    r.v = __shfl_up_sync(0xffffffffu, c.v, off);
+    r.q = __shfl_up_sync(0xffffffffu, c.q, off);
+    r.t = __shfl_up_sync(0xffffffffu, c.t, off);
+    return r;
+}
+// Every lane's candidate becomes the best of its node's candidates in this and the lower lanes (nodes ascend).
+__device__ __forceinline__ void segmented_min(Cand &c)
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const Cand o = shfl_up(c, off);
+        if (lane >= off && o.q == c.q && better(o, c)) c = o;
+    }
+}
+
+constexpr int X_NONE = 0x7fffffff;            // node of an idle lane (above every node)
+
+struct ExactShared {
+    Cand head[32], tail[32];                  // per warp: its first node, if that ends inside the warp, and its last
+    int first[32];                            // per warp: its first node
+    float dvals[16];
+};
+
+// shared memory: the minimisers by tree position, ExactShared, and (SM) P0, P1, A
 __host__ __device__ inline size_t exact_optarr_bytes(int m)
 {
-    int L = 1;
-    while ((1 << L) - 1 < m) ++L;
-    return ((((size_t)1 << L) + 8) * sizeof(uint16_t) + 15) & ~(size_t)15;
+    return (((size_t)m + 8) * sizeof(uint16_t) + 15) & ~(size_t)15;
 }
-__host__ __device__ inline size_t exact_smem_bytes(int m) { return exact_optarr_bytes(m) + ((size_t)m / 2 + 8) * sizeof(unsigned long long); }
-
-__device__ __forceinline__ double4 ld_q(const double4 *p)
+__host__ __device__ inline size_t exact_smem_bytes(int m, bool sm)
 {
-    double4 v;
-    asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(v.x), "=d"(v.y), "=d"(v.z), "=d"(v.w) : "l"(p));
-    return v;
+    const size_t mpad = ((size_t)m + 7) & ~(size_t)7;
+    return exact_optarr_bytes(m) + ((sizeof(ExactShared) + 15) & ~(size_t)15) + (sm ? (mpad + 8) * 24 : 0);
 }
 
-// Candidates of one node compete through a 64-bit atomic minimum: the order-preserving image of the cost with
-// its 16 lowest mantissa bits replaced by the split point, so that costs equal to 2^-36 relative go to the
-// smaller split point.
-__device__ __forceinline__ unsigned long long candidate_key(double v, int t)
+// The per-position sums, either way.
+template <bool SM> struct Sums;
+template <> struct Sums<true> {
+    double *p0, *p1, *a, *p2;                 // p2 in global memory
+    __device__ __forceinline__ void init(unsigned char *smem, unsigned char *slot, int m)
+    {
+        const int n = ((m + 7) & ~7) + 8;
+        p0 = reinterpret_cast<double *>(smem);
+        p1 = p0 + n;
+        a = p1 + n;
+        p2 = reinterpret_cast<double *>(slot);
+    }
+    __device__ __forceinline__ void set(int t, double s0, double s1, double s2) { p0[t] = s0; p1[t] = s1; p2[t] = s2; }
+    __device__ __forceinline__ void load(int t, double &s0, double &s1, double &av) const { s0 = p0[t]; s1 = p1[t]; av = a[t]; }
+    __device__ __forceinline__ double get_p2(int t) const { return p2[t]; }
+    __device__ __forceinline__ void set_a(int t, double v) { a[t] = v; }
+};
+template <> struct Sums<false> {
+    double4 *q;
+    __device__ __forceinline__ void init(unsigned char *, unsigned char *slot, int) { q = reinterpret_cast<double4 *>(slot); }
+    __device__ __forceinline__ void set(int t, double s0, double s1, double s2) { q[t] = make_double4(s0, s1, s2, 0.0); }
+    __device__ __forceinline__ void load(int t, double &s0, double &s1, double &av) const
+    {
+        double s2;
+        asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(s0), "=d"(s1), "=d"(s2), "=d"(av) : "l"(q + t));
+    }
+    __device__ __forceinline__ double get_p2(int t) const { return q[t].z; }
+    __device__ __forceinline__ void set_a(int t, double v) { reinterpret_cast<double *>(q + t)[3] = v; }
+};
+
+// S1^2 / S0 of the candidates: the hardware's approximate reciprocal (better than 20 bits) and one step of the series
+// 1 + e + e^2, within one unit in the last place.  What is kept (the layer's F, the result) uses the division.
+__device__ __forceinline__ double square_over(double s1, double s0)
 {
-    if (v == 0.0) v = 0.0;
-    const unsigned long long u = (unsigned long long)__double_as_longlong(v);
-    const unsigned long long ob = (u >> 63) ? ~u : (u | 0x8000000000000000ull);
-    return (ob & ~0xffffull) | (unsigned long long)(unsigned)t;
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(s0));
+    const double e = fma(-s0, r, 1.0);
+    return s1 * s1 * fma(r, fma(e, e, e), r);
 }
 
-// cost of the interval [t, i) given Q[t] and Q[i]
-__device__ __forceinline__ double interval_cost(const double4 &qt, const double4 &qi)
-{
-    const double s0 = qi.x - qt.x, s1 = qi.y - qt.y, s2 = qi.z - qt.z;
-    return s0 > 0.0 ? s2 - s1 * s1 / s0 : 0.0;
-}
-
-__global__ void __launch_bounds__(XT) skim_exact_kernel(ClusterArgs a, int rows_in_chunk, unsigned char *scratch, size_t slot_bytes)
+template <bool SM, int XT>
+__global__ void __launch_bounds__(XT, 1024 / XT) skim_exact_kernel(ClusterArgs a, int rows_in_chunk, unsigned char *scratch, size_t slot_bytes)
 {
     extern __shared__ __align__(16) unsigned char xsmem[];
-    __shared__ float s_dvals[16];
-    const int tid = threadIdx.x;
+    constexpr int NW = XT / 32;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int m = a.m;
     const RowRecord R = row_record(m);
     const ExactSlot S = exact_slot(m);
     unsigned char *slot = scratch + (size_t)blockIdx.x * slot_bytes;
-    double4 *Q = reinterpret_cast<double4 *>(slot + S.q);
-    double *Fc = reinterpret_cast<double *>(slot + S.fc);
     uint16_t *T = reinterpret_cast<uint16_t *>(slot + S.t);
     uint16_t *optarr = reinterpret_cast<uint16_t *>(xsmem);           // minimisers of the current layer by node position
-    unsigned long long *keys = reinterpret_cast<unsigned long long *>(xsmem + exact_optarr_bytes(m));   // per node of a level
+    ExactShared &sh = *reinterpret_cast<ExactShared *>(xsmem + exact_optarr_bytes(m));
+    Sums<SM> Q;
+    Q.init(xsmem + exact_optarr_bytes(m) + ((sizeof(ExactShared) + 15) & ~(size_t)15), slot + S.q, m);
     const int kmax = 1 << (a.bmin + a.nb - 1);
 
     for (int local = blockIdx.x; local < rows_in_chunk; local += gridDim.x) {
@@ -100,7 +153,7 @@ __global__ void __launch_bounds__(XT) skim_exact_kernel(ClusterArgs a, int rows_
         const int nd_rec = *reinterpret_cast<const int *>(rec);
         if (nd_rec < 0) continue;                                   // the sort kernel gave the row up
         const int nd = max(nd_rec, 1);
-        if (tid < 16) s_dvals[tid] = reinterpret_cast<const float *>(rec + 64)[tid];
+        if (tid < 16) sh.dvals[tid] = reinterpret_cast<const float *>(rec + 64)[tid];
         const unsigned char *groups = rec + R.groups;
         const double4 *seg = reinterpret_cast<const double4 *>(rec + R.seg);
 
@@ -116,22 +169,24 @@ __global__ void __launch_bounds__(XT) skim_exact_kernel(ClusterArgs a, int rows_
             const float gs[8] = {ga.x, ga.y, ga.z, ga.w, gb.x, gb.y, gb.z, gb.w};
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
-                Q[q * 8 + u] = make_double4(p0, p1, p2, 0.0);
+                Q.set(q * 8 + u, p0, p1, p2);
                 const double g = (double)gs[u], x = (double)xs[u];      // padding: g = 0
                 p0 += g;
                 p1 += g * x;
                 p2 += g * x * x;
             }
-            if (q == R.ngrp - 1) Q[q * 8 + 8] = make_double4(p0, p1, p2, 0.0);
+            if (q == R.ngrp - 1) Q.set(q * 8 + 8, p0, p1, p2);
         }
         __syncthreads();
 
-        // ------------------------------------------------------------ layer 1
-        const double4 q0 = ld_q(Q);
+        // ------------------------------------------------------------ layer 1: F_1(i) - P2(i) = -S1^2 / S0 over [0, i)
+        double z0, z1, za;
+        Q.load(0, z0, z1, za);
         for (int i = 1 + tid; i <= m; i += XT) {
-            double4 qi = ld_q(Q + i);
-            qi.w = interval_cost(q0, qi);
-            Q[i] = qi;
+            double p0, p1, pa;
+            Q.load(i, p0, p1, pa);
+            const double s0 = p0 - z0, s1 = p1 - z1;
+            Q.set_a(i, s0 > 0.0 ? -(s1 * s1 / s0) : -Q.get_p2(i));
         }
         __syncthreads();
 
@@ -144,91 +199,125 @@ __global__ void __launch_bounds__(XT) skim_exact_kernel(ClusterArgs a, int rows_
             if (tid == 0) optarr[0] = (uint16_t)(j - 1);
             __syncthreads();
             for (int lev = 0; lev < L; ++lev) {
-                const int h = 1 << (L - 1 - lev);
+                const int sh_h = L - 1 - lev, h = 1 << sh_h;
                 const int nvalid = (n / h + 1) >> 1;                 // nodes (2q + 1) h <= n of this level
                 // a node's position, and the range of split points its two finished neighbours leave it
-                auto node_i = [&](int q) { return j + (2 * q + 1) * h - 1; };
-                auto node_tlo = [&](int q) { return (int)optarr[2 * q * h]; };
+                auto node_i = [&](int q) { return j + ((2 * q + 1) << sh_h) - 1; };
+                auto node_tlo = [&](int q) { return (int)optarr[(2 * q) << sh_h]; };
                 auto node_thi = [&](int q) {
-                    const int i = node_i(q);
-                    int thi = i - 1;
-                    if ((2 * q + 2) * h <= n) thi = min(thi, (int)optarr[(2 * q + 2) * h]);
-                    return max(thi, node_tlo(q));                   // rounding may break the order of two near-tied minimisers
+                    const int thi = node_i(q) - 1, right = (2 * q + 2) << sh_h;
+                    return right <= n ? min(thi, (int)optarr[right]) : thi;
                 };
-                for (int q = tid; q < nvalid; q += XT) keys[q] = ~0ull;
-                __syncthreads();
-                // The ranges of a level's nodes tile the span of split points, sharing their end points.  The
-                // span, not the nodes, is dealt to the threads in equal stretches (a node's range can be a
-                // thousand times another's); a thread walks its stretch node by node and commits each node's
-                // best candidate with one atomic minimum on (cost rounded to 2^-36 relative, split point).
-                const int tmin = (int)optarr[0], tmax = node_thi(nvalid - 1);
-                const int chunk = (tmax - tmin + XT) / XT;
-                const int ta = tmin + tid * chunk, tb = min(ta + chunk, tmax + 1);
-                if (ta < tb) {
-                    int lo = 0, hi = nvalid - 1;
+                // the list of candidates: node q has P(q) = tlo(q) - tlo(0) + q before its own tlo(q) .. thi(q) (where the limit
+                // t < i cuts a range short of its right neighbour's minimiser, the missing split points are skipped)
+                const int tmin = (int)optarr[0], total = node_thi(nvalid - 1) - tmin + nvalid;
+                const int chunk = ((total + XT - 1) / XT) | 1;       // odd: neighbouring lanes' reads fall into different banks
+                const int xa = min(tid * chunk, total), xb = min(xa + chunk, total);
+                Cand head{__longlong_as_double(0x7ff0000000000000ll), -1, 0}, cur{head.v, X_NONE, 0};
+                int first = X_NONE;
+                if (xa < xb) {
+                    int lo = 0, hi = nvalid - 1;                     // the last node with P(q) <= xa
                     while (lo < hi) {
-                        const int mid = (lo + hi) >> 1;
-                        if (node_thi(mid) < ta) lo = mid + 1; else hi = mid;
+                        const int mid = (lo + hi + 1) >> 1;
+                        if (node_tlo(mid) - tmin + mid <= xa) lo = mid; else hi = mid - 1;
                     }
-                    for (int q = lo; q < nvalid; ++q) {
-                        const int tlo = node_tlo(q), thi = node_thi(q);
-                        if (tlo >= tb) break;
-                        const int t0 = max(ta, tlo), t1 = min(tb - 1, thi);
-                        if (t0 <= t1) {
-                            const double4 qi = ld_q(Q + node_i(q));
-                            double best = __longlong_as_double(0x7ff0000000000000ll);     // +inf
-                            int bt = t0;
-                            int t = t0;
-                            for (; t + 3 <= t1; t += 4) {            // four loads in flight
-                                const double4 qa = ld_q(Q + t), qb = ld_q(Q + t + 1), qc = ld_q(Q + t + 2), qd = ld_q(Q + t + 3);
-                                const double va = qa.w + interval_cost(qa, qi), vb = qb.w + interval_cost(qb, qi);
-                                const double vc = qc.w + interval_cost(qc, qi), vd = qd.w + interval_cost(qd, qi);
-                                if (va < best) { best = va; bt = t; }
-                                if (vb < best) { best = vb; bt = t + 1; }
-                                if (vc < best) { best = vc; bt = t + 2; }
-                                if (vd < best) { best = vd; bt = t + 3; }
-                            }
-                            for (; t <= t1; ++t) {
-                                const double4 qt = ld_q(Q + t);
-                                const double v = qt.w + interval_cost(qt, qi);
-                                if (v < best) { best = v; bt = t; }
-                            }
-                            atomicMin(&keys[q], candidate_key(best, bt));
+                    int q = lo;
+                    first = q;
+                    int t = xa - q + tmin, thi = node_thi(q);
+                    int end = (q + 1 < nvalid) ? node_tlo(q + 1) : thi;      // last split point that is counted as this node's
+                    double i0, i1, ia;
+                    Q.load(node_i(q), i0, i1, ia);
+                    cur.q = q;
+                    cur.t = min(t, thi);
+                    for (int x = xa; x < xb; ++x, ++t) {
+                        if (t > end) {
+                            // node q ends inside the stretch: its minimiser is known, unless it began in an earlier one
+                            if (q == first) head = cur; else optarr[(2 * q + 1) << sh_h] = (uint16_t)cur.t;
+                            ++q;
+                            t = node_tlo(q);
+                            thi = node_thi(q);
+                            end = (q + 1 < nvalid) ? node_tlo(q + 1) : thi;
+                            Q.load(node_i(q), i0, i1, ia);
+                            cur.v = __longlong_as_double(0x7ff0000000000000ll);
+                            cur.q = q;
+                            cur.t = t;
                         }
-                        if (thi >= tb) break;                        // the rest of this node, and all later ones, are other threads'
+                        double t0, t1, av;
+                        Q.load(min(t, thi), t0, t1, av);             // past the cut: thi once more
+                        const double s0 = i0 - t0, s1 = i1 - t1;
+                        const double v = s0 > 0.0 ? av - square_over(s1, s0) : av;
+                        if (v < cur.v) { cur.v = v; cur.t = min(t, thi); }
                     }
                 }
-                __syncthreads();
-                for (int q = tid; q < nvalid; q += XT) {
-                    const int i = node_i(q);
-                    const double4 qi = ld_q(Q + i);
-                    const unsigned long long key = keys[q];
-                    int bt = (int)(key & 0xffffull);
-                    double best;
-                    if (key != ~0ull) {
-                        const double4 qt = ld_q(Q + bt);
-                        best = qt.w + interval_cost(qt, qi);
-                    } else {
-                        // no stretch met the node (possible only where rounding broke the order of the ranges)
-                        best = __longlong_as_double(0x7ff0000000000000ll);
-                        bt = node_tlo(q);
-                        for (int t = node_tlo(q); t <= node_thi(q); ++t) {
-                            const double4 qt = ld_q(Q + t);
-                            const double v = qt.w + interval_cost(qt, qi);
-                            if (v < best) { best = v; bt = t; }
-                        }
-                    }
-                    Fc[i] = best;
-                    T[(size_t)j * (m + 1) + i] = (uint16_t)bt;
+                // ---- over the lanes
+                segmented_min(cur);
+                const Cand below = shfl_up(cur, 1);
+                if (lane > 0 && head.q >= 0 && below.q == head.q && better(below, head)) head = below;
+                const int wfirst = __shfl_sync(0xffffffffu, first, 0), nfirst = __shfl_down_sync(0xffffffffu, first, 1);
+                if (lane == 0) {
+                    sh.first[warp] = wfirst;
+                    sh.head[warp].q = -1;
+                }
+                __syncwarp();
+                if (head.q >= 0) {
+                    if (head.q == wfirst) sh.head[warp] = head; else optarr[(2 * head.q + 1) << sh_h] = (uint16_t)head.t;
+                }
+                const bool last = lane == 31 || nfirst == X_NONE;     // no lane behind this one has candidates
+                if (lane == 0) sh.tail[warp].q = X_NONE;
+                __syncwarp();
+                if (first == X_NONE) {
+                    // idle
+                } else if (last) {
+                    sh.tail[warp] = cur;
+                } else if (nfirst != cur.q) {
+                    // the node ends exactly where the stretch does
+                    if (cur.q == wfirst) sh.head[warp] = cur; else optarr[(2 * cur.q + 1) << sh_h] = (uint16_t)cur.t;
                 }
                 __syncthreads();
-                for (int q = tid; q < nvalid; q += XT) optarr[(2 * q + 1) * h] = T[(size_t)j * (m + 1) + node_i(q)];
+                // ---- over the warps
+                if (warp == 0) {
+                    Cand tl{0.0, X_NONE, 0}, hd{0.0, -1, 0};
+                    int nf = X_NONE;
+                    if (lane < NW) {
+                        tl = sh.tail[lane];
+                        hd = sh.head[lane];
+                        if (lane + 1 < NW) nf = sh.first[lane + 1];
+                    }
+                    segmented_min(tl);
+                    const Cand bl = shfl_up(tl, 1);
+                    if (hd.q >= 0) {
+                        if (lane > 0 && bl.q == hd.q && better(bl, hd)) hd = bl;
+                        optarr[(2 * hd.q + 1) << sh_h] = (uint16_t)hd.t;
+                    }
+                    if (tl.q != X_NONE && nf != tl.q) optarr[(2 * tl.q + 1) << sh_h] = (uint16_t)tl.t;
+                }
                 __syncthreads();
             }
-            // F_j becomes the previous layer
-            for (int i = j + tid; i <= m; i += XT) {
-                const double f = Fc[i];
-                reinterpret_cast<double *>(Q + i)[3] = f;
+            // F_j - P2 becomes the previous layer.  A position needs the old values of lower ones only: stretches of positions
+            // go by from the top, each read in full before it is written.
+            uint16_t *Tj = T + (size_t)j * (m + 1);
+            constexpr int PER = 4;
+            for (int base = j + (n - 1) / (PER * XT) * (PER * XT); base >= j; base -= PER * XT) {
+                double an[PER];
+#pragma unroll
+                for (int u = 0; u < PER; ++u) {
+                    const int i = base + tid + u * XT;
+                    if (i <= m) {
+                        const int t = optarr[i - j + 1];
+                        Tj[i] = (uint16_t)t;
+                        double t0, t1, av, i0, i1, ia;
+                        Q.load(t, t0, t1, av);
+                        Q.load(i, i0, i1, ia);
+                        const double s0 = i0 - t0, s1 = i1 - t1;
+                        an[u] = s0 > 0.0 ? av - s1 * s1 / s0 : av;
+                    }
+                }
+                __syncthreads();
+#pragma unroll
+                for (int u = 0; u < PER; ++u) {
+                    const int i = base + tid + u * XT;
+                    if (i <= m) Q.set_a(i, an[u]);
+                }
             }
             __syncthreads();
         }
@@ -241,27 +330,31 @@ __global__ void __launch_bounds__(XT) skim_exact_kernel(ClusterArgs a, int rows_
             for (int u = 0; u < tid; ++u) off += 1 << (a.bmin + u);
             float *cout = a.centroids + row * a.sumk + off;
             if (nd <= k) {
-                for (int u = 0; u < k; ++u) cout[u] = s_dvals[min(u, nd - 1)];
+                for (int u = 0; u < k; ++u) cout[u] = sh.dvals[min(u, nd - 1)];
                 a.err[row * a.nb + tid] = 0.0f;
             } else {
-                // F_k(m) was overwritten by later layers in Q; walk the minimisers back and add the interval costs up
+                // walk the minimisers back and add the interval costs up
                 int i = m;
-                double total = 0.0;
+                double total = 0.0, i0, i1, ia;
+                Q.load(m, i0, i1, ia);
                 for (int jj = k; jj >= 1; --jj) {
                     const int t = (jj == 1) ? 0 : (int)T[(size_t)jj * (m + 1) + i];
-                    const double4 qi = ld_q(Q + i), qt = ld_q(Q + t);
-                    const double s0 = qi.x - qt.x;
+                    double t0, t1, ta;
+                    Q.load(t, t0, t1, ta);
+                    const double s0 = i0 - t0, s1 = i1 - t1;
                     float c;
                     if (s0 > 0.0) {
-                        c = (float)((qi.y - qt.y) / s0);
+                        c = (float)(s1 / s0);
+                        total += (Q.get_p2(i) - Q.get_p2(t)) - s1 * s1 / s0;
                     } else {
                         const float xf = *(reinterpret_cast<const float *>(groups + (size_t)(t >> 3) * SKIM_GROUP_BYTES) + (t & 7));
                         const float xl = *(reinterpret_cast<const float *>(groups + (size_t)((i - 1) >> 3) * SKIM_GROUP_BYTES) + ((i - 1) & 7));
                         c = (float)(0.5 * ((double)xf + (double)xl));
                     }
                     cout[jj - 1] = c;
-                    total += interval_cost(qt, qi);
                     i = t;
+                    i0 = t0;
+                    i1 = t1;
                 }
                 a.err[row * a.nb + tid] = (float)fmax(total, 0.0);
             }
@@ -269,7 +362,6 @@ __global__ void __launch_bounds__(XT) skim_exact_kernel(ClusterArgs a, int rows_
         __syncthreads();
     }
 }
-
 }  // namespace
 
 size_t skim_exact_slot_bytes(int64_t cols) { return exact_slot((int)cols).total; }
@@ -280,19 +372,38 @@ int skim_exact_slots(const skim_ctx *ctx, int64_t rows)
     return (int)(rows < want ? rows : want);
 }
 
+namespace {
+struct ExactVariant {
+    void (*kernel)(ClusterArgs, int, unsigned char *, size_t);
+    int threads;
+    bool sm;
+    int blocks;              // per SM, what the shared memory has to allow
+};
+// Rows whose sums fit shared memory twice per SM (to about 4300 columns) run with two blocks of 512 threads per SM,
+// rows that fit once (to about 9200) with one of 1024, longer ones from global memory.
+const ExactVariant kExact[] = {
+    {skim_exact_kernel<true, 512>, 512, true, 2},
+    {skim_exact_kernel<true, 1024>, 1024, true, 1},
+    {skim_exact_kernel<false, 512>, 512, false, 1},
+};
+}  // namespace
+
 int skim_launch_exact(skim_ctx *ctx, const ClusterArgs &args, int64_t rows, void *scratch, int slots)
 {
-    const size_t smem = exact_smem_bytes(args.m);
-    if (smem > (size_t)ctx->max_smem_optin) return SKIM_ERR_SHAPE;
-    SKIM_CUDA_OK(cudaFuncSetAttribute(skim_exact_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    // as many blocks as are resident at once (each owns a scratch slot), at most `slots`
-    int per_sm = 1;
-    SKIM_CUDA_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, skim_exact_kernel, XT, smem));
-    int64_t resident = (int64_t)(per_sm > 0 ? per_sm : 1) * ctx->sm_count;
-    if (resident > slots) resident = slots;
-    const unsigned blocks = (unsigned)(rows < resident ? rows : resident);
-    skim_exact_kernel<<<blocks, XT, smem, ctx->stream>>>(args, (int)rows, (unsigned char *)scratch, exact_slot(args.m).total);
-    SKIM_CUDA_OK(cudaGetLastError());
-    ctx->launches += 1;
-    return SKIM_OK;
+    for (const ExactVariant &v : kExact) {
+        const size_t smem = exact_smem_bytes(args.m, v.sm);
+        if (smem + 1024 > ((size_t)ctx->max_smem_optin + 1024) / v.blocks) continue;      // 1 KB of an SM's shared memory goes to each block
+        SKIM_CUDA_OK(cudaFuncSetAttribute(v.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        // as many blocks as are resident at once (each owns a scratch slot), at most `slots`
+        int per_sm = 1;
+        SKIM_CUDA_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, v.kernel, v.threads, smem));
+        int64_t resident = (int64_t)(per_sm > 0 ? per_sm : 1) * ctx->sm_count;
+        if (resident > slots) resident = slots;
+        const unsigned blocks = (unsigned)(rows < resident ? rows : resident);
+        v.kernel<<<blocks, v.threads, smem, ctx->stream>>>(args, (int)rows, (unsigned char *)scratch, exact_slot(args.m).total);
+        SKIM_CUDA_OK(cudaGetLastError());
+        ctx->launches += 1;
+        return SKIM_OK;
+    }
+    return SKIM_ERR_SHAPE;
 }
