@@ -139,7 +139,7 @@ int skim_cluster_rows_at(skim_ctx *ctx, const uint16_t *W, const float *importan
  * Rows with at most 2^b distinct values get those values and error 0, as in skim_cluster_rows.  Where two
  * partitions cost the same up to rounding either may be returned.  An installed scale vector applies.
  *   scratch    device, 256-byte aligned, at least skim_cluster_exact_bytes(ctx, rows, cols) bytes
- *              (about 74 bytes per column for each of min(rows, 3 x SM count) rows in flight)
+ *              (about 66 bytes per column for each of min(rows, n x SM count) rows in flight; n = 8 for short rows, 1 for long)
  */
 int skim_cluster_exact_bytes(const skim_ctx *ctx, int64_t rows, int64_t cols, size_t *out);
 int skim_cluster_rows_exact(skim_ctx *ctx, const uint16_t *W, const float *importance, int64_t rows, int64_t cols,

@@ -192,7 +192,7 @@ int skim_cluster_exact_bytes(const skim_ctx *ctx, int64_t rows, int64_t cols, si
     if (!ctx || !out) return SKIM_ERR_NULL;
     int rc = check_matrix(ctx, rows, cols, cols);
     if (rc) return rc;
-    *out = skim_align256((size_t)skim_exact_slots(ctx, rows > 0 ? rows : 1) * skim_exact_slot_bytes(cols));
+    *out = skim_align256((size_t)skim_exact_slots(ctx, rows > 0 ? rows : 1, cols) * skim_exact_slot_bytes(cols));
     return SKIM_OK;
 }
 
@@ -210,7 +210,7 @@ int skim_cluster_rows_exact(skim_ctx *ctx, const uint16_t *W, const float *impor
     if (rc) return rc;
     if (ctx->scaled && ctx->scale_cols != cols) return SKIM_ERR_SCALE;
     if ((reinterpret_cast<uintptr_t>(scratch) & 255u) != 0 ||
-        scratch_bytes < (size_t)skim_exact_slots(ctx, rows > 0 ? rows : 1) * skim_exact_slot_bytes(cols))
+        scratch_bytes < (size_t)skim_exact_slots(ctx, rows > 0 ? rows : 1, cols) * skim_exact_slot_bytes(cols))
         return SKIM_ERR_WORKSPACE;
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return SKIM_ERR_CUDA;

@@ -290,7 +290,7 @@ int skim_launch_cluster(skim_ctx *ctx, const uint16_t *W, const float *importanc
             ctx->launches += 1;
         }
         if (tev) SKIM_CUDA_OK(cudaEventRecord(tev[1], ctx->stream));
-        const int rc = exact_scratch ? skim_launch_exact(ctx, a, n, exact_scratch, skim_exact_slots(ctx, rows))
+        const int rc = exact_scratch ? skim_launch_exact(ctx, a, n, exact_scratch, skim_exact_slots(ctx, rows, cols))
                                      : skim_launch_lloyd(ctx, a, n);
         if (rc) return rc;
         if (tev) {

@@ -79,43 +79,47 @@ struct ExactShared {
     float dvals[16];
 };
 
-// shared memory: the minimisers by tree position, ExactShared, and (SM) P0, P1, A
+// Where P0, P1 and A of a row live: all in shared memory, P0 and P1 there and A in global memory, or all in global memory.
+enum SumsPlace { SUMS_SHARED, SUMS_MIXED, SUMS_GLOBAL };
+
+// shared memory: the minimisers by tree position, ExactShared, and the sums
 __host__ __device__ inline size_t exact_optarr_bytes(int m)
 {
     return (((size_t)m + 8) * sizeof(uint16_t) + 15) & ~(size_t)15;
 }
-__host__ __device__ inline size_t exact_smem_bytes(int m, bool sm)
+__host__ __device__ inline size_t exact_smem_bytes(int m, int place)
 {
     const size_t mpad = ((size_t)m + 7) & ~(size_t)7;
-    return exact_optarr_bytes(m) + ((sizeof(ExactShared) + 15) & ~(size_t)15) + (sm ? (mpad + 8) * 24 : 0);
+    return exact_optarr_bytes(m) + ((sizeof(ExactShared) + 15) & ~(size_t)15) + (mpad + 8) * (place == SUMS_SHARED ? 24 : place == SUMS_MIXED ? 16 : 0);
 }
 
 // The per-position sums, either way.
-template <bool SM> struct Sums;
-template <> struct Sums<true> {
+template <int PLACE> struct Sums {
     double *p0, *p1, *a, *p2;                 // p2 in global memory
     __device__ __forceinline__ void init(unsigned char *smem, unsigned char *slot, int m)
     {
         const int n = ((m + 7) & ~7) + 8;
         p0 = reinterpret_cast<double *>(smem);
         p1 = p0 + n;
-        a = p1 + n;
         p2 = reinterpret_cast<double *>(slot);
+        a = PLACE == SUMS_SHARED ? p1 + n : p2 + n;
     }
     __device__ __forceinline__ void set(int t, double s0, double s1, double s2) { p0[t] = s0; p1[t] = s1; p2[t] = s2; }
     __device__ __forceinline__ void load(int t, double &s0, double &s1, double &av) const { s0 = p0[t]; s1 = p1[t]; av = a[t]; }
+    __device__ __forceinline__ void load_i(int t, double &s0, double &s1) const { s0 = p0[t]; s1 = p1[t]; }
     __device__ __forceinline__ double get_p2(int t) const { return p2[t]; }
     __device__ __forceinline__ void set_a(int t, double v) { a[t] = v; }
 };
-template <> struct Sums<false> {
+template <> struct Sums<SUMS_GLOBAL> {
     double4 *q;
     __device__ __forceinline__ void init(unsigned char *, unsigned char *slot, int) { q = reinterpret_cast<double4 *>(slot); }
     __device__ __forceinline__ void set(int t, double s0, double s1, double s2) { q[t] = make_double4(s0, s1, s2, 0.0); }
     __device__ __forceinline__ void load(int t, double &s0, double &s1, double &av) const
     {
-        double s2;
-        asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(s0), "=d"(s1), "=d"(s2), "=d"(av) : "l"(q + t));
+        [[maybe_unused]] double unused;
+        asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(s0), "=d"(s1), "=d"(unused), "=d"(av) : "l"(q + t));
     }
+    __device__ __forceinline__ void load_i(int t, double &s0, double &s1) const { const double2 v = *reinterpret_cast<const double2 *>(q + t); s0 = v.x; s1 = v.y; }
     __device__ __forceinline__ double get_p2(int t) const { return q[t].z; }
     __device__ __forceinline__ void set_a(int t, double v) { reinterpret_cast<double *>(q + t)[3] = v; }
 };
@@ -130,7 +134,7 @@ __device__ __forceinline__ double square_over(double s1, double s0)
     return s1 * s1 * fma(r, fma(e, e, e), r);
 }
 
-template <bool SM, int XT>
+template <int PLACE, int XT>
 __global__ void __launch_bounds__(XT, 1024 / XT) skim_exact_kernel(ClusterArgs a, int rows_in_chunk, unsigned char *scratch, size_t slot_bytes)
 {
     extern __shared__ __align__(16) unsigned char xsmem[];
@@ -143,7 +147,7 @@ __global__ void __launch_bounds__(XT, 1024 / XT) skim_exact_kernel(ClusterArgs a
     uint16_t *T = reinterpret_cast<uint16_t *>(slot + S.t);
     uint16_t *optarr = reinterpret_cast<uint16_t *>(xsmem);           // minimisers of the current layer by node position
     ExactShared &sh = *reinterpret_cast<ExactShared *>(xsmem + exact_optarr_bytes(m));
-    Sums<SM> Q;
+    Sums<PLACE> Q;
     Q.init(xsmem + exact_optarr_bytes(m) + ((sizeof(ExactShared) + 15) & ~(size_t)15), slot + S.q, m);
     const int kmax = 1 << (a.bmin + a.nb - 1);
 
@@ -221,33 +225,38 @@ __global__ void __launch_bounds__(XT, 1024 / XT) skim_exact_kernel(ClusterArgs a
                         const int mid = (lo + hi + 1) >> 1;
                         if (node_tlo(mid) - tmin + mid <= xa) lo = mid; else hi = mid - 1;
                     }
-                    int q = lo;
+                    int q = lo, i = node_i(q), t = xa - q + tmin;
                     first = q;
-                    int t = xa - q + tmin, thi = node_thi(q);
-                    int end = (q + 1 < nvalid) ? node_tlo(q + 1) : thi;      // last split point that is counted as this node's
+                    // `end`: the last split point that is counted as the node's (a split point past its limit i - 1 is replaced by that)
+                    int end = (q + 1 < nvalid) ? node_tlo(q + 1) : node_thi(q);
                     double i0, i1, ia;
-                    Q.load(node_i(q), i0, i1, ia);
-                    cur.q = q;
-                    cur.t = min(t, thi);
-                    for (int x = xa; x < xb; ++x, ++t) {
-                        if (t > end) {
-                            // node q ends inside the stretch: its minimiser is known, unless it began in an earlier one
-                            if (q == first) head = cur; else optarr[(2 * q + 1) << sh_h] = (uint16_t)cur.t;
-                            ++q;
-                            t = node_tlo(q);
-                            thi = node_thi(q);
-                            end = (q + 1 < nvalid) ? node_tlo(q + 1) : thi;
-                            Q.load(node_i(q), i0, i1, ia);
-                            cur.v = __longlong_as_double(0x7ff0000000000000ll);
-                            cur.q = q;
-                            cur.t = t;
-                        }
+                    Q.load(i, i0, i1, ia);
+                    double best = __longlong_as_double(0x7ff0000000000000ll);
+                    int bt = min(t, i - 1);
+                    for (int x = xa;;) {
+                        const int te = min(t, i - 1);
                         double t0, t1, av;
-                        Q.load(min(t, thi), t0, t1, av);             // past the cut: thi once more
+                        Q.load(te, t0, t1, av);
                         const double s0 = i0 - t0, s1 = i1 - t1;
                         const double v = s0 > 0.0 ? av - square_over(s1, s0) : av;
-                        if (v < cur.v) { cur.v = v; cur.t = min(t, thi); }
+                        if (v < best) { best = v; bt = te; }
+                        if (++x == xb) break;
+                        const bool fin = t == end;
+                        ++t;
+                        if (fin) {
+                            // node q ends inside the stretch: its minimiser is known, unless it began in an earlier one
+                            if (q == first) head = Cand{best, q, bt}; else optarr[(2 * q + 1) << sh_h] = (uint16_t)bt;
+                            ++q;
+                            t = end;
+                            i += 2 << sh_h;
+                            const int right = (2 * q + 2) << sh_h;
+                            end = right <= n ? (int)optarr[right] : i - 1;
+                            Q.load_i(i, i0, i1);
+                            best = __longlong_as_double(0x7ff0000000000000ll);
+                            bt = min(t, i - 1);
+                        }
                     }
+                    cur = Cand{best, q, bt};
                 }
                 // ---- over the lanes
                 segmented_min(cur);
@@ -364,46 +373,56 @@ __global__ void __launch_bounds__(XT, 1024 / XT) skim_exact_kernel(ClusterArgs a
 }
 }  // namespace
 
-size_t skim_exact_slot_bytes(int64_t cols) { return exact_slot((int)cols).total; }
-
-int skim_exact_slots(const skim_ctx *ctx, int64_t rows)
-{
-    const int64_t want = (int64_t)ctx->sm_count * 3;
-    return (int)(rows < want ? rows : want);
-}
-
 namespace {
 struct ExactVariant {
     void (*kernel)(ClusterArgs, int, unsigned char *, size_t);
     int threads;
-    bool sm;
-    int blocks;              // per SM, what the shared memory has to allow
+    int place;
+    int cap;                 // columns up to which it is taken
 };
-// Rows whose sums fit shared memory twice per SM (to about 4300 columns) run with two blocks of 512 threads per SM,
-// rows that fit once (to about 9200) with one of 1024, longer ones from global memory.
-const ExactVariant kExact[] = {
-    {skim_exact_kernel<true, 512>, 512, true, 2},
-    {skim_exact_kernel<true, 1024>, 1024, true, 1},
-    {skim_exact_kernel<false, 512>, 512, false, 1},
+#define SKIM_XV(P, T, CAP) {skim_exact_kernel<P, T>, T, P, CAP}
+// Few threads for short rows: a level then has some ten candidates per thread, and its search and reductions (about
+// half of the instructions) are not paid by threads with nothing to do; 64 to 512 threads at 512 columns take 1.00, 0.98, 1.54
+// and 2.57 ms for 2048 rows.  With no more rows than SMs nothing else fills the SM: twice the threads (32 x 1000: 473 ->
+// 416 us).  The largest cap of a place is what one of its blocks (two of those of 512 threads) finds in an SM's shared memory.
+const ExactVariant kVariantsExact[] = {
+    SKIM_XV(SUMS_SHARED, 64, 384),   SKIM_XV(SUMS_SHARED, 128, 1024),  SKIM_XV(SUMS_SHARED, 256, 2304), SKIM_XV(SUMS_SHARED, 512, 4300),
+    SKIM_XV(SUMS_SHARED, 1024, 8700), SKIM_XV(SUMS_MIXED, 1024, 12500), SKIM_XV(SUMS_GLOBAL, 512, 1 << 30),
 };
+const ExactVariant *exact_variant(const skim_ctx *ctx, int64_t rows, int64_t cols)
+{
+    for (const ExactVariant &v : kVariantsExact)
+        if (cols * (v.threads < 512 && rows <= ctx->sm_count ? 2 : 1) <= v.cap && exact_smem_bytes((int)cols, v.place) <= (size_t)ctx->max_smem_optin) return &v;
+    return nullptr;
+}
 }  // namespace
+
+size_t skim_exact_slot_bytes(int64_t cols) { return exact_slot((int)cols).total; }
+
+// Blocks in flight, each with a scratch slot: what 1024 threads of an SM hold, at most eight per SM.
+int skim_exact_slots(const skim_ctx *ctx, int64_t rows, int64_t cols)
+{
+    const ExactVariant *v = exact_variant(ctx, rows, cols);
+    int per_sm = v ? 1024 / v->threads : 1;
+    if (per_sm > 8) per_sm = 8;
+    const int64_t want = (int64_t)ctx->sm_count * per_sm;
+    return (int)(rows < want ? rows : want);
+}
 
 int skim_launch_exact(skim_ctx *ctx, const ClusterArgs &args, int64_t rows, void *scratch, int slots)
 {
-    for (const ExactVariant &v : kExact) {
-        const size_t smem = exact_smem_bytes(args.m, v.sm);
-        if (smem + 1024 > ((size_t)ctx->max_smem_optin + 1024) / v.blocks) continue;      // 1 KB of an SM's shared memory goes to each block
-        SKIM_CUDA_OK(cudaFuncSetAttribute(v.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        // as many blocks as are resident at once (each owns a scratch slot), at most `slots`
-        int per_sm = 1;
-        SKIM_CUDA_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, v.kernel, v.threads, smem));
-        int64_t resident = (int64_t)(per_sm > 0 ? per_sm : 1) * ctx->sm_count;
-        if (resident > slots) resident = slots;
-        const unsigned blocks = (unsigned)(rows < resident ? rows : resident);
-        v.kernel<<<blocks, v.threads, smem, ctx->stream>>>(args, (int)rows, (unsigned char *)scratch, exact_slot(args.m).total);
-        SKIM_CUDA_OK(cudaGetLastError());
-        ctx->launches += 1;
-        return SKIM_OK;
-    }
-    return SKIM_ERR_SHAPE;
+    const ExactVariant *v = exact_variant(ctx, rows, args.m);
+    if (!v) return SKIM_ERR_SHAPE;
+    const size_t smem = exact_smem_bytes(args.m, v->place);
+    SKIM_CUDA_OK(cudaFuncSetAttribute(v->kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // as many blocks as are resident at once (each owns a scratch slot), at most `slots`
+    int per_sm = 1;
+    SKIM_CUDA_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, v->kernel, v->threads, smem));
+    int64_t resident = (int64_t)(per_sm > 0 ? per_sm : 1) * ctx->sm_count;
+    if (resident > slots) resident = slots;
+    const unsigned blocks = (unsigned)(rows < resident ? rows : resident);
+    v->kernel<<<blocks, v->threads, smem, ctx->stream>>>(args, (int)rows, (unsigned char *)scratch, exact_slot(args.m).total);
+    SKIM_CUDA_OK(cudaGetLastError());
+    ctx->launches += 1;
+    return SKIM_OK;
 }

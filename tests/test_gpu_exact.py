@@ -87,3 +87,17 @@ def test_exact_argument_errors(ctx, skimlib):
     with pytest.raises(skimlib.SkimError) as e:
         ctx.cluster_rows_exact(W, G, [1, 3])
     assert e.value.code == -3
+
+
+@pytest.mark.parametrize("rows,cols", [(3, 192), (160, 193), (150, 384), (2, 513), (160, 1025), (2, 2305), (1, 4301), (1, 8701), (1, 12501)])
+def test_exact_block_sizes(ctx, oracle, rows, cols):
+    """Every block size and place of the sums, at the row lengths where the choice changes (the rule also looks at the row count)."""
+    n = min(rows, 3)
+    w, g = inputs.make_rows(rows, cols, 950 + cols)
+    ctx.reserve(rows, cols)
+    ctx.apply_scale(None)
+    cent, err = ctx.cluster_rows_exact(torch.from_numpy(w).cuda(), torch.from_numpy(g).cuda(), BITS)
+    assert ctx.get_status() == 0
+    ora = oracle.cluster_rows_exact(w[-n:], g[-n:], BITS)
+    np.testing.assert_allclose(err.cpu().numpy()[-n:], ora["err"], rtol=1e-6)
+    assert bool((torch.diff(cent[:, 14:], dim=1) >= 0).all())
