@@ -1,0 +1,295 @@
+// Row-sorting kernel, the first half of the row clustering (SKIM Algorithm 3, error pre-recording loop; objective of
+// Section 3.2, diagonal form).  One block per row: every element's bucket is a monotone function of its value, chosen so that a bucket holds about one
+// element of a bell-shaped row; one counting pass orders the row up to the order inside the buckets.
+//
+//   load     values (binary32 products where a scale vector is installed, else the binary16 weights) and the sum of |x|,
+//            which sets the buckets' scale.
+//   count    one shared-memory atomic per element; its return value is the element's slot inside its bucket.
+//   scatter  bucket base + slot: value and importance (read from global memory here) go to their bucket's place.
+//   order    the buckets that reach from one group of 8 into the next are sorted (groups ascend; inside a group the Lloyd
+//            kernel compares every element with its boundary, so its order does not matter).
+//   then     one pass over the row (skim_cluster_phases.cuh) writes the row record -- group records with
+//            prefix sums, group index, segment table -- to global memory, from which the Lloyd kernel
+//            (skim_lloyd.cu) iterates with one warp per row.
+//
+// Buckets: v = 1 + |x| / s with s half a standard deviation (from the mean of |x|).  The bits of v grow with |x|: the
+// first three octaves, v in [1, 8), i.e. |x| up to 3.5 deviations, have N/8 buckets each on either side of zero, the next
+// eight share N/8 (N = 32 per thread).  A row whose values this cannot spread (some bucket with BUCKET_LIMIT elements or
+// more: few distinct values, a clump) is put on a list and sorted by the radix kernel of skim_cluster.cu.
+//
+// Why not a radix sort: rows of 32-bit keys took four passes, each with ballots or random shared-memory traffic of all
+// elements (1.17 ms for 4096 x 11008); 16-bit keys two (0.284 ms).  What bounds this kernel is the same resource,
+// shared-memory wavefronts of random accesses, but there is one counting atomic and one scatter per element.
+#include "skim_cluster_phases.cuh"
+
+namespace {
+
+using namespace skimk;
+
+constexpr int BUCKET_LIMIT = 48;
+
+template <int THREADS> struct Buckets {
+    static constexpr int N = 32 * THREADS;
+    static constexpr int HALF = N / 2;
+    static constexpr int LOG = (THREADS == 128 ? 9 : THREADS == 256 ? 10 : THREADS == 512 ? 11 : 12);      // log2(N / 8)
+    static_assert((8 << LOG) == N, "eight octave blocks");
+    float inv_s;
+    // ascends with x; any bit pattern of x gives an index inside [0, N)
+    __device__ __forceinline__ int operator()(float x) const
+    {
+        const uint32_t b = __float_as_uint(__fadd_rn(1.0f, __fmul_rn(fabsf(x), inv_s))) - 0x3f800000u;
+        const uint32_t fine = b >> (23 - LOG), coarse = 3u * (N / 8) + ((b - (3u << 23)) >> (26 - LOG));
+        const int i = (int)min(b < (3u << 23) ? fine : coarse, (uint32_t)HALF - 1u);
+        return x < 0.0f ? HALF - 1 - i : HALF + i;
+    }
+};
+
+// keys, gs: values and importances in bucket order
+// uni:      the bucket counters (8-bit) and the bases of every four of them (16-bit)
+struct BucketLayout {
+    size_t keys, gs, uni, phase, total;
+};
+__host__ __device__ inline BucketLayout bucket_layout(int m, int threads)
+{
+    BucketLayout L;
+    size_t off = 0;
+    auto take = [&](size_t b) { size_t o = off; off += (b + 15) & ~(size_t)15; return o; };
+    const size_t mpad = ((size_t)m + 7) & ~(size_t)7;
+    L.keys = take(mpad * 4);
+    L.gs = take(mpad * 4);
+    L.uni = take((size_t)threads * 48);
+    L.phase = take(sizeof(PhaseSmem));
+    L.total = off;
+    return L;
+}
+
+// Insertion sort of n elements by one thread.
+__device__ __forceinline__ void sort_bucket(float *keys, float *gs, int lo, int n)
+{
+    for (int i = lo + 1; i < lo + n; ++i) {
+        const float k = keys[i], g = gs[i];
+        int j = i;
+        for (float y; j > lo && (y = keys[j - 1]) > k; --j) {
+            keys[j] = y;
+            gs[j] = gs[j - 1];
+        }
+        if (j != i) {
+            keys[j] = k;
+            gs[j] = g;
+        }
+    }
+}
+
+template <int THREADS, int ITEMS>
+__global__ void __launch_bounds__(THREADS, 1024 / THREADS) skim_sort_bucket_kernel(ClusterArgs a)
+{
+    using Bk = Buckets<THREADS>;
+    constexpr int NW = THREADS / 32;
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int m = a.m;
+    const BucketLayout L = bucket_layout(m, THREADS);
+    float *keys = reinterpret_cast<float *>(smem + L.keys);
+    float *gs = reinterpret_cast<float *>(smem + L.gs);
+    uint32_t *cnt = reinterpret_cast<uint32_t *>(smem + L.uni);         // four counters a word
+    uint16_t *wbase = reinterpret_cast<uint16_t *>(cnt + Bk::N / 4);    // elements before a word's buckets
+    PhaseSmem &ps = *reinterpret_cast<PhaseSmem *>(smem + L.phase);
+    float *red = reinterpret_cast<float *>(ps.segtot);                  // free until the record pass
+    uint32_t *wsum = reinterpret_cast<uint32_t *>(ps.segtot) + 32;
+
+    const int64_t row = a.row0 + blockIdx.x;
+    const uint16_t *Wr = a.W + row * a.ld;
+    const float *Gr = a.G + row * a.ld;
+    for (int j = tid * 32; j < m; j += THREADS * 32) asm volatile("prefetch.global.L2 [%0];" ::"l"(Gr + j));      // for the scatter
+
+    // ---------------------------------------------------------------- load
+    float x[ITEMS];
+    unsigned bad = 0u;
+    float sum = 0.0f;
+    {
+        uint16_t h[ITEMS];
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) h[i] = (i * THREADS + tid < m) ? Wr[i * THREADS + tid] : (uint16_t)0;
+        if (tid == 0) {
+            ps.misc[0] = 0;
+            ps.misc[1] = 0;
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) reinterpret_cast<uint4 *>(cnt)[u * THREADS + tid] = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) {
+            if ((h[i] & 0x7c00u) == 0x7c00u) bad |= 1u;
+            x[i] = __half2float(__ushort_as_half(h[i]));
+            x[i] = __fmul_rn(x[i], (i * THREADS + tid < m) ? a.rscale[i * THREADS + tid] : 1.0f);
+            x[i] += 0.0f;                                               // -0 and +0 are one value
+            sum += fabsf(x[i]);
+        }
+    }
+#pragma unroll
+    for (int off = 16; off; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+    if (lane == 0) red[warp] = sum;
+    __syncthreads();
+    sum = 0.0f;
+    for (int w = 0; w < NW; ++w) sum += red[w];
+    // s = half a standard deviation of a normal row: 0.5 sqrt(pi / 2) mean |x|
+    const Bk bucket{(sum > 0.0f && sum < 3.0e38f) ? fminf(__fdividef((float)m, 0.6267f * sum), 1.0e38f) : 0.0f};
+
+    // ---------------------------------------------------------------- count: slots inside the buckets
+    uint32_t slot[(ITEMS + 3) / 4];
+    bool over = false;
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i) {
+        if ((i & 3) == 0) slot[i >> 2] = 0u;
+        if (i * THREADS + tid < m) {
+            const int b = bucket(x[i]);
+            const uint32_t s = (atomicAdd(&cnt[b >> 2], 1u << (8 * (b & 3))) >> (8 * (b & 3))) & 0xffu;
+            over |= s >= (uint32_t)BUCKET_LIMIT;
+            slot[i >> 2] |= s << (8 * (i & 3));
+        }
+    }
+    if (__syncthreads_or(over ? 1 : 0)) {
+        // not a row for buckets: the radix kernel takes it
+        if (bad) atomicOr(a.status, (unsigned long long)bad);
+        if (tid == 0) {
+            const int at = atomicAdd(a.sort_count, 1);
+            if (SKIM_IDX(at, a.chunk_rows, a.status)) a.sort_list[at] = (int)blockIdx.x;
+        }
+        return;
+    }
+
+    // ---------------------------------------------------------------- counters -> bases
+    {
+        uint4 v[2];
+        uint32_t t[8], s = 0u, occupied = 0u;
+#pragma unroll
+        for (int u = 0; u < 2; ++u) v[u] = reinterpret_cast<const uint4 *>(cnt)[2 * tid + u];
+        const uint32_t *w = reinterpret_cast<const uint32_t *>(v);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            t[u] = s;
+            s = __dp4a(w[u], 0x01010101u, s);
+            occupied += w[u] ? 1u : 0u;
+        }
+        // occupied words: a lower bound of the number of distinct values
+        occupied = __reduce_add_sync(0xffffffffu, occupied);
+        if (lane == 0 && occupied) atomicAdd(&ps.misc[0], (int)occupied);
+        uint32_t inc = s;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const uint32_t x = __shfl_up_sync(0xffffffffu, inc, off);
+            if (lane >= off) inc += x;
+        }
+        if (lane == 31) wsum[warp] = inc;
+        __syncthreads();
+        uint32_t run = inc - s;
+        for (int q = 0; q < warp; ++q) run += wsum[q];
+        reinterpret_cast<uint4 *>(wbase)[tid] = make_uint4((run + t[0]) | ((run + t[1]) << 16), (run + t[2]) | ((run + t[3]) << 16),
+                                                           (run + t[4]) | ((run + t[5]) << 16), (run + t[6]) | ((run + t[7]) << 16));
+    }
+    __syncthreads();
+    // first position of bucket b, and (in n) its elements
+    auto bucket_base = [&](int b, int &n) {
+        const uint32_t w = cnt[b >> 2];
+        const int sh = 8 * (b & 3);
+        n = (int)((w >> sh) & 0xffu);
+        return (int)__dp4a(w & ((1u << sh) - 1u), 0x01010101u, (uint32_t)wbase[b >> 2]);
+    };
+
+    // ---------------------------------------------------------------- scatter to the buckets
+    constexpr int GB = 8;                                               // importances in flight
+#pragma unroll
+    for (int i0 = 0; i0 < ITEMS; i0 += GB) {
+        float g[GB];
+#pragma unroll
+        for (int u = 0; u < GB; ++u) g[u] = (i0 + u < ITEMS && (i0 + u) * THREADS + tid < m) ? Gr[(i0 + u) * THREADS + tid] : 0.0f;
+#pragma unroll
+        for (int u = 0; u < GB; ++u) {
+            const int i = i0 + u;
+            if (i < ITEMS && i * THREADS + tid < m) {
+                if (!(g[u] >= 0.0f) || g[u] > 3.0e38f) bad |= 2u;
+                int n;
+                const int pos = bucket_base(bucket(x[i < ITEMS ? i : 0]), n) + (int)((slot[i < ITEMS ? i >> 2 : 0] >> (8 * (i & 3))) & 0xffu);
+                if (SKIM_IDX(pos, m, a.status)) {
+                    keys[pos] = x[i < ITEMS ? i : 0];
+                    gs[pos] = g[u];
+                }
+            }
+        }
+    }
+    if (bad) atomicOr(a.status, (unsigned long long)bad);
+    __syncthreads();
+
+    // ---------------------------------------------------------------- order where it matters
+    // The Lloyd kernel asks for groups of 8 in order, not for order inside a group: only a bucket that reaches from one
+    // group into the next has to be sorted.  A row with few distinct values is sorted in full (they are counted below), and so
+    // are all rows for the exact kernel.
+    int nd = ps.misc[0];                     // more than 16 occupied words: more than 16 distinct values
+    const bool full = a.full_order || nd <= 16;
+    for (int p0 = tid * 8; p0 < m; p0 += THREADS * 8) {
+        if (!full) {
+            if (p0 == 0) continue;
+            int n;
+            const int lo = bucket_base(bucket(keys[p0]), n);
+            if (lo < p0 && lo >= p0 - 8) sort_bucket(keys, gs, lo, n);          // (an earlier start: an earlier border's thread does it)
+        } else {
+            // every bucket that starts in these 8 positions (a bucket's other places hold elements of the bucket all along)
+            for (int p = p0; p < min(p0 + 8, m);) {
+                int n;
+                const int lo = bucket_base(bucket(keys[p]), n);
+                if (lo >= p0) sort_bucket(keys, gs, lo, n);
+                p = lo + n;
+            }
+        }
+    }
+    __syncthreads();
+
+    // ---------------------------------------------------------------- row record
+    const SortedArrays<float> src{keys, gs};
+    if (nd <= 16) {
+        // few occupied words: count the distinct values themselves
+        if (tid == 0) ps.misc[0] = 0;
+        __syncthreads();
+        int dcount = 0;
+        for (int p = tid; p < m; p += THREADS) dcount += (p == 0 || src.key_at(p) != src.key_at(p - 1)) ? 1 : 0;
+        dcount = __reduce_add_sync(0xffffffffu, dcount);
+        if (lane == 0 && dcount) atomicAdd(&ps.misc[0], dcount);
+        __syncthreads();
+        nd = ps.misc[0];
+    }
+    write_row_record<float, THREADS, false>(a, src, ps, nd, (int)blockIdx.x);
+    if (nd <= 16) {
+        collect_distinct<float, THREADS>(src, m, nd, ps);
+        write_distinct_values(a, nd, ps.dvals, (int)blockIdx.x);
+    }
+}
+
+struct BucketVariant {
+    int cap;
+    int threads;
+    void (*kernel)(ClusterArgs);
+};
+
+#define SKIM_BV(T, I) {T * I, T, skim_sort_bucket_kernel<T, I>}
+
+// About eight elements a thread for short rows; two blocks of 512 threads per SM up to 11 264 columns, one of 1024 beyond.
+const BucketVariant kVariantsBucket[] = {
+    SKIM_BV(128, 4), SKIM_BV(128, 8), SKIM_BV(256, 8), SKIM_BV(512, 8), SKIM_BV(512, 16), SKIM_BV(512, 22), SKIM_BV(1024, 16), SKIM_BV(1024, 22),
+};
+
+}  // namespace
+
+int skim_launch_sort_bucket(skim_ctx *ctx, const ClusterArgs &args, int64_t rows)
+{
+    for (const BucketVariant &v : kVariantsBucket) {
+        if (v.cap < args.m) continue;
+        const BucketLayout L = bucket_layout(args.m, v.threads);
+        if (L.total > (size_t)ctx->max_smem_optin) return SKIM_ERR_SHAPE;
+        // set on every launch: a host-side call of microseconds, and no state shared between contexts
+        SKIM_CUDA_OK(cudaFuncSetAttribute(v.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total));
+        v.kernel<<<(unsigned)rows, v.threads, L.total, ctx->stream>>>(args);
+        SKIM_CUDA_OK(cudaGetLastError());
+        ctx->launches += 1;
+        return SKIM_OK;
+    }
+    return SKIM_ERR_SHAPE;
+}

@@ -7,11 +7,11 @@
 // on one warp while two rows filled an SM's shared memory; from global memory (the hot lines stay in
 // L1) every SM keeps 28 rows in flight.
 //
-// This file: the generic sort kernel, which handles every case -- scaled rows (32-bit keys of the
-// binary32 product) and rows whose layout rules out the vectorised fp16-key kernel of
-// skim_cluster16.cu -- and the host-side launcher of the whole clustering.
+// Unscaled rows are sorted by skim_cluster16.cu, rows with a scale vector installed by skim_bucket.cu.  This file: the radix
+// sort kernel for the scaled rows the bucket kernel cannot spread (few distinct values, clumps), and the host-side
+// launcher of the whole clustering.
 //
-// One thread block owns one row.
+// One thread block owns one row at a time.
 //   1. load   the row's (value, importance) pairs into registers; the value is turned into an
 //             order-preserving unsigned key.
 //   2. sort   block-wide LSD radix sort (8-bit digits, warp-private digit counters, ballot-based
@@ -29,7 +29,6 @@ constexpr int RADIX = 1 << RADIX_BITS;
 
 template <typename KeyT> struct Passes;
 template <> struct Passes<uint32_t> { static constexpr int N = 4; };
-template <> struct Passes<uint16_t> { static constexpr int N = 2; };
 
 // Shared-memory layout, computed identically on host and device.
 struct SmemLayout {
@@ -50,6 +49,7 @@ __host__ __device__ inline SmemLayout smem_layout(int cap, int key_bytes, int nw
     return L;
 }
 
+// Takes the rows of a.sort_list (blocks leave at once when it is empty, the usual case).
 template <typename KeyT, int THREADS, int ITEMS>
 __global__ void __launch_bounds__(THREADS) skim_sort_kernel(ClusterArgs a)
 {
@@ -69,7 +69,10 @@ __global__ void __launch_bounds__(THREADS) skim_sort_kernel(ClusterArgs a)
     const int lane = tid & 31;
     const int warp = tid >> 5;
     const int m = a.m;
-    const int64_t row = a.row0 + blockIdx.x;
+    const int listed = min(*a.sort_count, a.chunk_rows);
+    for (int at = blockIdx.x; at < listed; at += gridDim.x) {
+    const int local = a.sort_list[at];
+    const int64_t row = a.row0 + local;
     const uint16_t *Wr = a.W + row * a.ld;
     const float *Gr = a.G + row * a.ld;
 
@@ -85,14 +88,10 @@ __global__ void __launch_bounds__(THREADS) skim_sort_kernel(ClusterArgs a)
             const float g = Gr[e];
             if ((h & 0x7c00u) == 0x7c00u) bad |= 1u;
             if (!(g >= 0.0f) || g > 3.0e38f) bad |= 2u;
-            if constexpr (sizeof(KeyT) == 2) {
-                key[i] = KeyOps<uint16_t>::from_half_bits(h == 0x8000u ? (uint16_t)0 : h);
-            } else {
-                float x = __half2float(__ushort_as_half(h));
-                if (a.rscale) x = __fmul_rn(x, a.rscale[e]);
-                if (x == 0.0f) x = 0.0f;
-                key[i] = KeyOps<uint32_t>::from_float(x);
-            }
+            float x = __half2float(__ushort_as_half(h));
+            if (a.rscale) x = __fmul_rn(x, a.rscale[e]);
+            if (x == 0.0f) x = 0.0f;
+            key[i] = K::from_float(x);
             val[i] = g;
         } else {
             key[i] = K::PAD;
@@ -180,10 +179,12 @@ __global__ void __launch_bounds__(THREADS) skim_sort_kernel(ClusterArgs a)
     if (tid == 0) { ps.misc[0] = 0; ps.misc[1] = 0; }
     __syncthreads();
     const SortedArrays<KeyT> src{skeys, sg};
-    const int nd = write_row_record<KeyT, THREADS, true>(a, src, ps, 0, (int)blockIdx.x);
+    const int nd = write_row_record<KeyT, THREADS, true>(a, src, ps, 0, local);
     if (nd <= 16) {
         collect_distinct<KeyT, THREADS>(src, m, nd, ps);
-        write_distinct_values(a, nd, ps.dvals, (int)blockIdx.x);
+        write_distinct_values(a, nd, ps.dvals, local);
+    }
+    __syncthreads();
     }
 }
 
@@ -194,19 +195,10 @@ struct Variant {
     void (*kernel)(ClusterArgs);
 };
 
-#define SKIM_VARIANT(KeyT, T, I) {T * I, T, (int)sizeof(KeyT), skim_sort_kernel<KeyT, T, I>}
+#define SKIM_VARIANT(T, I) {T * I, T, 4, skim_sort_kernel<uint32_t, T, I>}
 
-const Variant kVariants32[] = {
-    SKIM_VARIANT(uint32_t, 128, 4),  SKIM_VARIANT(uint32_t, 256, 8),  SKIM_VARIANT(uint32_t, 512, 8),
-    SKIM_VARIANT(uint32_t, 512, 16), SKIM_VARIANT(uint32_t, 512, 22), SKIM_VARIANT(uint32_t, 512, 32),
-    SKIM_VARIANT(uint32_t, 512, 44),
-};
-const Variant kVariants16[] = {
-    SKIM_VARIANT(uint16_t, 128, 4),  SKIM_VARIANT(uint16_t, 256, 8),  SKIM_VARIANT(uint16_t, 512, 8),
-    SKIM_VARIANT(uint16_t, 512, 16), SKIM_VARIANT(uint16_t, 512, 22), SKIM_VARIANT(uint16_t, 512, 32),
-    SKIM_VARIANT(uint16_t, 512, 44),
-};
-constexpr int kNumVariants = 7;
+const Variant kVariants32[] = {SKIM_VARIANT(512, 8), SKIM_VARIANT(512, 22), SKIM_VARIANT(512, 44)};
+constexpr int kNumVariants = 3;
 
 // Picks the smallest variant that holds `cols` and fits shared memory.
 const Variant *pick_variant(const Variant *table, int64_t cols, int max_smem, size_t *smem)
@@ -256,22 +248,21 @@ int skim_launch_cluster(skim_ctx *ctx, const uint16_t *W, const float *importanc
     a.err = err;
     a.status = ws.status;
     a.scratch = ws.cluster_scratch;
-    a.rec_stride = 0;
     a.row0 = 0;
-    a.rec_half = 0;
     a.early_exit = ctx->early_exit ? 1 : 0;
     a.iter_stats = ctx->timing ? ws.status + 1 : nullptr;
 
-    // plan: the fp16-key sort kernel when it applies, else the generic one
-    // (the exact kernel reads the full records with their g*x^2 prefixes, which only the generic kernel writes)
-    bool fast = !scaled && !exact_scratch && skim_launch_sort16(ctx, a, 0, false) == SKIM_OK;
-    const Variant *v = nullptr;
+    // unscaled rows get compact records (the exact kernel reads the full ones with their g*x^2 prefixes)
+    a.rec_half = (!scaled && !exact_scratch) ? 1 : 0;
+    a.rec_stride = (long long)row_record(a.m, a.rec_half != 0).total;
+    a.full_order = exact_scratch ? 1 : 0;
+    a.sort_list = ws.sort_list;
+    a.sort_count = (int *)(ws.status + 4);
     size_t smem = 0;
-    if (!fast) {
-        v = pick_variant(scaled ? kVariants32 : kVariants16, cols, ctx->max_smem_optin, &smem);
+    const Variant *v = nullptr;
+    if (scaled) {
+        v = pick_variant(kVariants32, cols, ctx->max_smem_optin, &smem);
         if (!v) return SKIM_ERR_SHAPE;
-        a.rec_stride = (long long)row_record(a.m).total;
-        a.rec_half = 0;
         SKIM_CUDA_OK(cudaFuncSetAttribute(v->kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     }
     if ((size_t)a.rec_stride > skim_cluster_record_bytes(cols)) return SKIM_ERR_WORKSPACE;
@@ -281,16 +272,17 @@ int skim_launch_cluster(skim_ctx *ctx, const uint16_t *W, const float *importanc
         a.row0 = row0;
         cudaEvent_t *tev = (ctx->timing && ctx->timing_used < SKIM_TIMING_SLOTS) ? ctx->timing_ev[ctx->timing_used] : nullptr;
         if (tev) SKIM_CUDA_OK(cudaEventRecord(tev[0], ctx->stream));
-        if (fast) {
-            const int rc = skim_launch_sort16(ctx, a, n, true);
-            if (rc) return rc < 0 ? rc : SKIM_ERR_SHAPE;
-        } else {
-            v->kernel<<<(unsigned)n, v->threads, smem, ctx->stream>>>(a);
+        a.chunk_rows = (int)n;
+        int rc = scaled ? skim_launch_sort_bucket(ctx, a, n) : skim_launch_sort16(ctx, a, n);
+        if (rc) return rc;
+        if (scaled) {
+            // the rows the buckets could not spread: usually none
+            v->kernel<<<(unsigned)(n < 2 * ctx->sm_count ? n : 2 * ctx->sm_count), v->threads, smem, ctx->stream>>>(a);
             SKIM_CUDA_OK(cudaGetLastError());
             ctx->launches += 1;
         }
         if (tev) SKIM_CUDA_OK(cudaEventRecord(tev[1], ctx->stream));
-        const int rc = exact_scratch ? skim_launch_exact(ctx, a, n, exact_scratch, skim_exact_slots(ctx, rows, cols))
+        rc = exact_scratch ? skim_launch_exact(ctx, a, n, exact_scratch, skim_exact_slots(ctx, rows, cols))
                                      : skim_launch_lloyd(ctx, a, n);
         if (rc) return rc;
         if (tev) {

@@ -1,10 +1,10 @@
 // fp16-key row-sorting kernel, the first half of the row clustering (SKIM Algorithm 3, error pre-recording loop; objective of
-// Section 3.2, diagonal form) for the common case: no scale vector installed, rows 16-byte aligned.
+// Section 3.2, diagonal form) where no scale vector is installed.
 //
 // With no scale the clustered value IS the fp16 weight, so a 16-bit order-preserving key is exact
 // and the sort moves one 32-bit word per element: (key << 16) | column.
 //
-//   load    128-bit loads of the fp16 row straight into keys.
+//   load    128-bit loads of the fp16 row (16-bit ones where rows are not 16-byte aligned) straight into keys.
 //   pass 0  low 12 key bits, 4096 block-wide counters; the counting atomic already hands every item
 //           its slot inside its bin.
 //           The first pass of an LSD sort need not be stable, so no ranking is needed.  The
@@ -51,7 +51,7 @@ __host__ __device__ inline Layout16 layout16(int m, int threads)
     auto take = [&](size_t b) { size_t o = off; off += (b + 15) & ~(size_t)15; return o; };
     const size_t row = ((size_t)m + 7) / 8 * 8 * 4;
     L.buf = take(row);
-    L.graw = take(row > (size_t)D0 * 4 ? row : (size_t)D0 * 4);
+    L.graw = take(row + 16 > (size_t)D0 * 4 ? row + 16 : (size_t)D0 * 4);      // 16: up to three floats before an unaligned row
     L.cnt1 = take((size_t)D1 * threads * 2);
     L.dbase1 = take(D1 * 4);
     L.phase = take(sizeof(PhaseSmem));
@@ -71,6 +71,11 @@ __device__ __forceinline__ void mbar_init(uint64_t *bar, int count)
 __device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, uint32_t bytes)
 {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
+}
+
+__device__ __forceinline__ void mbar_arrive(uint64_t *bar)
+{
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
 }
 
 __device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t bytes, uint64_t *bar)
@@ -122,7 +127,8 @@ struct SortedItems16 {
     __device__ __forceinline__ uint16_t key_at(int p) const { return (uint16_t)(items[p] >> 16); }
 };
 
-template <int THREADS, int VEC>
+// HALF_RECORD: the compact row record, for the Lloyd kernel; else the full one, for the exact kernel.
+template <bool HALF_RECORD, int THREADS, int VEC>
 __global__ void __launch_bounds__(THREADS, (THREADS <= 512 ? 2 : 1)) skim_sort16_kernel(ClusterArgs a)
 {
     using K = KeyOps<uint16_t>;
@@ -137,7 +143,6 @@ __global__ void __launch_bounds__(THREADS, (THREADS <= 512 ? 2 : 1)) skim_sort16
     const int mpad = (m + 7) & ~7;
     const Layout16 L = layout16(m, THREADS);
     uint32_t *buf = reinterpret_cast<uint32_t *>(smem + L.buf);
-    float *graw = reinterpret_cast<float *>(smem + L.graw);
     uint32_t *C0 = reinterpret_cast<uint32_t *>(smem + L.graw);
     uint32_t *cnt1w = reinterpret_cast<uint32_t *>(smem + L.cnt1);
     uint16_t *cnt1 = reinterpret_cast<uint16_t *>(smem + L.cnt1);
@@ -149,6 +154,10 @@ __global__ void __launch_bounds__(THREADS, (THREADS <= 512 ? 2 : 1)) skim_sort16
     const int64_t row = a.row0 + blockIdx.x;
     const uint16_t *Wr = a.W + row * a.ld;
     const float *Gr = a.G + row * a.ld;
+    // the importance row lands at the place in its 16-byte block that it has in global memory
+    const int gshift = (int)((reinterpret_cast<uintptr_t>(Gr) & 15u) / 4u);
+    float *graw = reinterpret_cast<float *>(smem + L.graw) + gshift;
+    const bool wvec = ((reinterpret_cast<uintptr_t>(Wr) & 15u) == 0);
 
     // ---------------------------------------------------------------- set-up
     if (tid == 0) {
@@ -168,7 +177,7 @@ __global__ void __launch_bounds__(THREADS, (THREADS <= 512 ? 2 : 1)) skim_sort16
     for (int j = 0; j < VEC; ++j) {
         const int e0 = (j * THREADS + tid) * 8;
         uint32_t w[4];
-        if (e0 + 8 <= m) {
+        if (wvec && e0 + 8 <= m) {
             const uint4 raw = *reinterpret_cast<const uint4 *>(Wr + e0);
             w[0] = raw.x; w[1] = raw.y; w[2] = raw.z; w[3] = raw.w;
         } else {
@@ -247,11 +256,16 @@ __global__ void __launch_bounds__(THREADS, (THREADS <= 512 ? 2 : 1)) skim_sort16
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
     if (tid == 0) {
-        const uint32_t bytes = (uint32_t)m * 4u;
-        mbar_expect_tx(mbar, bytes);
+        // whole 16-byte blocks, from the one that holds the row's first element to the last that ends inside the row
+        const uint32_t bytes = ((uint32_t)(m + gshift) * 4u) & ~15u;
+        if (bytes) mbar_expect_tx(mbar, bytes); else mbar_arrive(mbar);
         for (uint32_t o = 0; o < bytes; o += 32768u)
-            bulk_load(reinterpret_cast<unsigned char *>(graw) + o, reinterpret_cast<const unsigned char *>(Gr) + o,
+            bulk_load(reinterpret_cast<unsigned char *>(graw - gshift) + o, reinterpret_cast<const unsigned char *>(Gr - gshift) + o,
                       min(32768u, bytes - o), mbar);
+    }
+    {
+        const int done = ((m + gshift) & ~3) - gshift;      // the elements behind it (up to three), by plain loads
+        if (tid < m - max(done, 0)) graw[max(done, 0) + tid] = Gr[max(done, 0) + tid];
     }
 
     // ---------------------------------------------------------------- pass 1: counters -> positions
@@ -299,7 +313,7 @@ __global__ void __launch_bounds__(THREADS, (THREADS <= 512 ? 2 : 1)) skim_sort16
     for (int i = 0; i < ITEMS; i += 4) {
         const int p = tid * ITEMS + i;
         uint4 v = make_uint4(NO_ITEM, NO_ITEM, NO_ITEM, NO_ITEM);
-        if (p < m) v = *reinterpret_cast<const uint4 *>(buf + p);     // m is a multiple of 4 here
+        if (p < m) v = *reinterpret_cast<const uint4 *>(buf + p);     // past m: padding items, or the NO_ITEM of a later word
         item[i] = v.x; item[i + 1] = v.y; item[i + 2] = v.z; item[i + 3] = v.w;
     }
     __syncthreads();
@@ -358,7 +372,8 @@ __global__ void __launch_bounds__(THREADS, (THREADS <= 512 ? 2 : 1)) skim_sort16
         __syncthreads();
         nd = ps.misc[0];
     }
-    write_row_record_half<THREADS>(a, src, ps, nd, (int)blockIdx.x);
+    if constexpr (HALF_RECORD) write_row_record_half<THREADS>(a, src, ps, nd, (int)blockIdx.x);
+    else write_row_record<uint16_t, THREADS, false>(a, src, ps, nd, (int)blockIdx.x);
     if (nd <= 16) {
         collect_distinct<uint16_t, THREADS>(src, m, nd, ps);
         write_distinct_values(a, nd, ps.dvals, (int)blockIdx.x);
@@ -368,38 +383,31 @@ __global__ void __launch_bounds__(THREADS, (THREADS <= 512 ? 2 : 1)) skim_sort16
 struct Variant16 {
     int cap;
     int threads;
-    void (*kernel)(ClusterArgs);
+    void (*kernel[2])(ClusterArgs);      // full record, compact record
 };
 
-#define SKIM_V16(T, V) {T * V * 8, T, skim_sort16_kernel<T, V>}
+#define SKIM_V16(T, V) {T * V * 8, T, {skim_sort16_kernel<false, T, V>, skim_sort16_kernel<true, T, V>}}
 
-const Variant16 kVariants[] = {
+const Variant16 kVariants16[] = {
     SKIM_V16(128, 1), SKIM_V16(256, 1), SKIM_V16(512, 1), SKIM_V16(512, 2), SKIM_V16(512, 3), SKIM_V16(1024, 2),
     SKIM_V16(1024, 3),
 };
 
 }  // namespace
 
-int skim_launch_sort16(skim_ctx *ctx, ClusterArgs &args, int64_t rows, bool launch)
+int skim_launch_sort16(skim_ctx *ctx, const ClusterArgs &args, int64_t rows)
 {
-    const int64_t cols = args.m;
-    // 128-bit loads of W rows and the bulk copy of importance rows need 16-byte aligned rows
-    if ((reinterpret_cast<uintptr_t>(args.W) & 15u) || (args.ld % 8) != 0) return 1;
-    if ((reinterpret_cast<uintptr_t>(args.G) & 15u) || (cols % 4) != 0) return 1;
-    for (const Variant16 &v : kVariants) {
-        if (v.cap < cols) continue;
-        const Layout16 L = layout16((int)cols, v.threads);
+    for (const Variant16 &v : kVariants16) {
+        if (v.cap < args.m) continue;
+        const Layout16 L = layout16(args.m, v.threads);
         if (L.total > (size_t)ctx->max_smem_optin) continue;
-        args.rec_stride = (long long)row_record(args.m, true).total;
-        args.rec_half = 1;
-        if (!launch) return SKIM_OK;
-        const ClusterArgs a = args;
+        void (*kernel)(ClusterArgs) = v.kernel[args.rec_half ? 1 : 0];
         // set on every launch: a host-side call of microseconds, and no state shared between contexts
-        SKIM_CUDA_OK(cudaFuncSetAttribute(v.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total));
-        v.kernel<<<(unsigned)rows, v.threads, L.total, ctx->stream>>>(a);
+        SKIM_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total));
+        kernel<<<(unsigned)rows, v.threads, L.total, ctx->stream>>>(args);
         SKIM_CUDA_OK(cudaGetLastError());
         ctx->launches += 1;
         return SKIM_OK;
     }
-    return 1;
+    return SKIM_ERR_SHAPE;
 }

@@ -2,7 +2,8 @@
 // diagonal form): order-preserving keys, the phases the sort kernels run once a row is sorted
 // (distinct-value count, group index, binary64 block prefix sums, the row record), and the one-warp
 // Lloyd iteration with the error table entry and the optional labels that the Lloyd kernel runs on
-// a row record.  Used by skim_cluster.cu, skim_cluster16.cu and skim_lloyd.cu.
+// a row record.  Used by skim_cluster.cu, skim_cluster16.cu, skim_bucket.cu, skim_lloyd.cu
+// and skim_exact.cu.
 #pragma once
 
 #include "skim_internal.cuh"
@@ -64,6 +65,17 @@ template <> struct KeyOps<uint16_t> {
     }
 };
 
+// The binary32 value itself (the bucket sort kernel's scaled rows).
+template <> struct KeyOps<float> {
+    __device__ static __forceinline__ float to_float(float k) { return k; }
+    __device__ static __forceinline__ void load8(const float *p, float *k)
+    {
+        const float4 a = *reinterpret_cast<const float4 *>(p), b = *reinterpret_cast<const float4 *>(p + 4);
+        k[0] = a.x; k[1] = a.y; k[2] = a.z; k[3] = a.w;
+        k[4] = b.x; k[5] = b.y; k[6] = b.z; k[7] = b.w;
+    }
+};
+
 struct ClusterArgs {
     const uint16_t *W;
     const float *G;
@@ -81,7 +93,11 @@ struct ClusterArgs {
     unsigned char *scratch;   // row records of the current chunk (written by the sort kernel, read by the Lloyd kernel)
     long long rec_stride;     // bytes between row records
     int64_t row0;             // first row of the current chunk
-    int rec_half;             // the records are in the compact format of the fp16-key sort kernel
+    int rec_half;             // compact records (no scale installed: every value is a binary16 number)
+    int full_order;           // the reader wants order inside the groups too (exact kernel)
+    int chunk_rows;           // rows of the current chunk
+    int *sort_list;           // rows (indexes inside the chunk) the bucket kernel left to the radix kernel, and how many; the
+    int *sort_count;          // count is zero between chunks: whoever reads the records clears it
     int early_exit;           // stop a row once no boundary moved
     unsigned long long *iter_stats;   // nullptr, or two counters: iterations run, rows counted
 };
@@ -91,20 +107,21 @@ struct ClusterArgs {
 //   hdr     int nd (number of distinct values) at byte 0; float dvals[16] at byte 64
 //   seg     one 32-byte entry per segment of 32 groups (256 elements): the binary64 sums of g,
 //           g*x and g*x^2 over all earlier segments; entry nseg holds the row totals
-//   groups  one 96-byte record per group of 8 sorted elements, three whole 32-byte sectors: the 8
+//   groups  one 96-byte record per group of 8 elements (no value of a group above one of the next; inside a
+//           group the radix kernels leave order, the bucket kernel need not), three whole 32-byte sectors: the 8
 //           values | the 8 importances | the binary64 sums of g, g*x and g*x^2 from the start of
 //           the group's segment to the group's first element (and 8 bytes of padding).  With the
 //           segment entry that is everything a boundary needs in one Lloyd iteration.  The last
 //           group is padded with the largest finite value and zero importance.  Every sector is
 //           written by one 32-byte store and never touched again.
-//   gi      group index: first value of every group, sk_entries(m) floats (padded likewise)
+//   gi      group index: smallest value of every group, sk_entries(m) floats (padded likewise)
 struct RowRecord {
     size_t seg, groups, gi, total;
     size_t gi_bytes;
     int ngrp, nseg;
 };
 constexpr int SKIM_GROUP_BYTES = 96;                // three 32-byte sectors
-// Compact record of the fp16-key sort kernel (no scale installed, so a value IS a binary16 number): a group is
+// Compact record (no scale installed, so a value IS a binary16 number): a group is
 // two sectors, 8 binary16 values | the binary64 sums of g and g*x from the segment start | the 8 importances.
 // The g*x^2 sums are not kept per group: the error of a width is  sum g x^2 (row total, last segment entry)
 // minus  sum_j c_j (2 S1_j - c_j S0_j),  which needs the interval sums of g and g*x only.
@@ -157,12 +174,17 @@ __device__ __forceinline__ void st_sector(void *p, double a, double b, double c)
 template <typename KeyT> struct SortedArrays {
     const KeyT *skeys;
     const float *sg;
-    __device__ __forceinline__ unsigned group(int e, int, KeyT *ks, float *gs) const
+    __device__ __forceinline__ unsigned group(int e, int m, KeyT *ks, float *gs) const
     {
         KeyOps<KeyT>::load8(skeys + e, ks);
         const float4 ga = *reinterpret_cast<const float4 *>(sg + e), gb = *reinterpret_cast<const float4 *>(sg + e + 4);
         gs[0] = ga.x; gs[1] = ga.y; gs[2] = ga.z; gs[3] = ga.w;
         gs[4] = gb.x; gs[5] = gb.y; gs[6] = gb.z; gs[7] = gb.w;
+        if (e + 8 > m) {
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (e + u >= m) gs[u] = 0.0f;
+        }
         return 0u;
     }
     __device__ __forceinline__ KeyT key_at(int p) const { return skeys[p]; }
@@ -247,7 +269,8 @@ __device__ __forceinline__ int write_row_record(const ClusterArgs &a, const Src 
                 unsigned char *gr = rec + R.groups + (size_t)q * SKIM_GROUP_BYTES;
                 st_sector(gr, x);
                 st_sector(gr + 32, gs);
-                first[h] = x[0];
+                // the smallest value: inside a group a row of the bucket kernel is in no order
+                first[h] = fminf(fminf(fminf(x[0], x[1]), fminf(x[2], x[3])), fminf(fminf(x[4], x[5]), fminf(x[6], x[7])));
                 double t0[8], t1[8], t2[8];
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
@@ -345,7 +368,7 @@ __device__ __forceinline__ void st_sector(void *p, unsigned long long a, unsigne
 }
 
 // The compact row record (see SKIM_GROUP_BYTES_HALF) from a row sorted by 16-bit keys; the counterpart of
-// write_row_record for the fp16-key sort kernel.  One pass, one group per lane; only the sums of g and g*x are
+// write_row_record for unscaled rows.  One pass, one group per lane; only the sums of g and g*x are
 // scanned, the g*x^2 terms are added up per warp and meet in the row total.  nd: the distinct-value count
 // (any number above 16 stands for "more than 16").  Call with all threads.
 template <int THREADS, typename Src>
@@ -462,10 +485,10 @@ __device__ __forceinline__ void write_distinct_values(const ClusterArgs &a, int 
 
 }  // namespace skimk
 
-// fp16-key sort kernel (skim_cluster16.cu).  Fills args.rec_stride when `launch`
-// is false (planning) and launches over `rows` rows otherwise.  Returns SKIM_OK, or 1 when the
-// call does not meet the kernel's requirements (then the generic sort kernel must be used).
-int skim_launch_sort16(skim_ctx *ctx, skimk::ClusterArgs &args, int64_t rows, bool launch);
+// Bucket sort kernel (skim_bucket.cu), a scale vector installed: writes the row records of a chunk, or puts rows on args.sort_list.
+int skim_launch_sort_bucket(skim_ctx *ctx, const skimk::ClusterArgs &args, int64_t rows);
+// fp16-key sort kernel (skim_cluster16.cu): writes the row records of a chunk; no scale vector installed.
+int skim_launch_sort16(skim_ctx *ctx, const skimk::ClusterArgs &args, int64_t rows);
 // Exact clustering kernel (skim_exact.cu): one block per row record; `scratch` holds `slots` slots of
 // skim_exact_slot_bytes(cols) bytes.
 int skim_launch_exact(skim_ctx *ctx, const skimk::ClusterArgs &args, int64_t rows, void *scratch, int slots);

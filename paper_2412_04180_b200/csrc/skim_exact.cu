@@ -150,6 +150,7 @@ __global__ void __launch_bounds__(XT, 1024 / XT) skim_exact_kernel(ClusterArgs a
     Sums<PLACE> Q;
     Q.init(xsmem + exact_optarr_bytes(m) + ((sizeof(ExactShared) + 15) & ~(size_t)15), slot + S.q, m);
     const int kmax = 1 << (a.bmin + a.nb - 1);
+    if (blockIdx.x == 0 && tid == 0) *a.sort_count = 0;
 
     for (int local = blockIdx.x; local < rows_in_chunk; local += gridDim.x) {
         const int64_t row = a.row0 + local;

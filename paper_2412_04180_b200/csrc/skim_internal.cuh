@@ -40,7 +40,7 @@ struct skim_ctx {
 // Workspace layout (all offsets 256-byte aligned), carved per call for the call's (rows, cols).
 // The status word and the reciprocal scale sit at fixed offsets, so they persist across calls.
 struct SkimWorkspace {
-    unsigned long long *status;  // word 0: status bits; words 1, 2: Lloyd iterations run and rows counted (skim_lloyd_iterations)
+    unsigned long long *status;  // word 0: status bits; words 1, 2: Lloyd iterations run and rows counted (skim_lloyd_iterations); word 4: length of sort_list
     float *rscale;               // [cols]     reciprocal of the installed scale vector
     int32_t *row_pos;            // [rows]     packed-row index of every source row
     double *alpha64;             // [cols]     scale-update master copy of alpha
@@ -51,6 +51,7 @@ struct SkimWorkspace {
     double *scale_const;         // [rows][16][2]  scale update: per-cluster constants (sum g, sum g w^2)
     double *scale_cq;            // [rows][16][2]  scale update: per-cluster centroid and gradient factor
     uint16_t *scale_ord_end;     // [rows][16]  scale update: steps of the clusters in the label-ordered rows
+    int *sort_list;              // [min(rows, SKIM_CLUSTER_CHUNK_ROWS)] rows the bucket sort kernel leaves to the radix kernel
     unsigned char *cluster_scratch;  // [min(rows, SKIM_CLUSTER_CHUNK_ROWS)] row records of the clustering; during a scale update the label-ordered matrix
     size_t bytes;
 };
@@ -94,6 +95,7 @@ static inline SkimWorkspace skim_carve(void *base, int64_t rows, int64_t cols)
     w.scale_const = (double *)take((size_t)rows * 16 * 2 * 8);
     w.scale_cq = (double *)take((size_t)rows * 16 * 2 * 8);
     w.scale_ord_end = (uint16_t *)take((size_t)rows * 16 * 2);
+    w.sort_list = (int *)take((size_t)(rows < SKIM_CLUSTER_CHUNK_ROWS ? rows : SKIM_CLUSTER_CHUNK_ROWS) * 4);
     const size_t records = (size_t)(rows < SKIM_CLUSTER_CHUNK_ROWS ? rows : SKIM_CLUSTER_CHUNK_ROWS) * skim_cluster_record_bytes(cols);
     const size_t ordered = (size_t)rows * (size_t)skim_ordered_stride(cols) * 8 + SKIM_ORDER_SLACK;
     w.cluster_scratch = (unsigned char *)take(records > ordered ? records : ordered);

@@ -42,7 +42,7 @@ __device__ __forceinline__ void ld_sector(const unsigned char *p, float4 &a, flo
 }
 
 // One group record in registers.  HALF = false: the full record (three sectors: binary32 values | importances |
-// sums incl. g*x^2); HALF = true: the compact record of the fp16-key sort kernel (two sectors: binary16 values
+// sums incl. g*x^2); HALF = true: the compact record of unscaled rows (two sectors: binary16 values
 // and the sums of g and g*x | importances).
 template <bool HALF> struct Group;
 
@@ -57,7 +57,7 @@ template <> struct Group<false> {
         ld_sector(gr + 32, ga, gb);
         p = __ldg(reinterpret_cast<const double2 *>(gr + 64));   // the g*x^2 sum at +80 is read once, for the error
     }
-    // number of values <= t (values ascend; the padding is the largest finite value)
+    // number of values <= t (in any order; the padding is the largest finite value)
     __device__ __forceinline__ int count_le(float t) const
     {
         return (xa.x <= t) + (xa.y <= t) + (xa.z <= t) + (xa.w <= t) + (xb.x <= t) + (xb.y <= t) + (xb.z <= t) + (xb.w <= t);
@@ -67,9 +67,26 @@ template <> struct Group<false> {
         x[0] = (double)xa.x; x[1] = (double)xa.y; x[2] = (double)xa.z; x[3] = (double)xa.w;
         x[4] = (double)xb.x; x[5] = (double)xb.y; x[6] = (double)xb.z; x[7] = (double)xb.w;
     }
+    // the sorted row's value at idx: the (idx % 8)-th smallest of its group
     static __device__ __forceinline__ float value_at(const unsigned char *groups, int idx)
     {
-        return __ldg(reinterpret_cast<const float *>(groups + (size_t)(idx >> 3) * BYTES) + (idx & 7));
+        float4 a, b;
+        ld_sector(groups + (size_t)(idx >> 3) * BYTES, a, b);
+        const float x[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+        float v = x[0];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            int rank = 0;
+#pragma unroll
+            for (int w = 0; w < 8; ++w) rank += (w < u ? x[w] <= x[u] : x[w] < x[u]) ? 1 : 0;
+            if (rank == (idx & 7)) v = x[u];
+        }
+        return v;
+    }
+    __device__ __forceinline__ void in_prefix(int, float t, bool (&in)[8]) const
+    {
+        in[0] = xa.x <= t; in[1] = xa.y <= t; in[2] = xa.z <= t; in[3] = xa.w <= t;
+        in[4] = xb.x <= t; in[5] = xb.y <= t; in[6] = xb.z <= t; in[7] = xb.w <= t;
     }
 };
 
@@ -105,25 +122,32 @@ template <> struct Group<true> {
             x[2 * u + 1] = (double)f.y;
         }
     }
+    // values ascend
+    __device__ __forceinline__ void in_prefix(int n, float, bool (&in)[8]) const
+    {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) in[u] = u < n;
+    }
     static __device__ __forceinline__ float value_at(const unsigned char *groups, int idx)
     {
         return __half2float(__ushort_as_half(__ldg(reinterpret_cast<const unsigned short *>(groups + (size_t)(idx >> 3) * BYTES) + (idx & 7))));
     }
 };
 
-// Adds the first n (0..8) elements of a group to (s0, s1[, s2]): the eight terms are summed pairwise,
-// a fixed order with a short dependency chain.  Elements past n are masked before any arithmetic.
+// Adds the elements <= t of a group (n of them) to (s0, s1[, s2]): the eight terms are summed pairwise,
+// a fixed order with a short dependency chain.  The others are masked before any arithmetic.
 template <bool WANT_C, typename G>
-__device__ __forceinline__ void add_group(const G &grp, int n, double &s0, double &s1, double &s2)
+__device__ __forceinline__ void add_group(const G &grp, int n, float t, double &s0, double &s1, double &s2)
 {
     double xs[8];
+    bool in[8];
     grp.values(xs);
+    grp.in_prefix(n, t, in);
     const float gs[8] = {grp.ga.x, grp.ga.y, grp.ga.z, grp.ga.w, grp.gb.x, grp.gb.y, grp.gb.z, grp.gb.w};
     double t0[8], t1[8], t2[8];
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-        const bool in = u < n;
-        const double g = (double)(in ? gs[u] : 0.0f), x = xs[u];   // padding values are finite, so 0 * x = 0
+        const double g = (double)(in[u] ? gs[u] : 0.0f), x = xs[u];   // padding values are finite, so 0 * x = 0
         t0[u] = g;
         t1[u] = g * x;
         if (WANT_C) t2[u] = t1[u] * x;
@@ -296,9 +320,9 @@ __device__ __forceinline__ void lloyd_warp(const unsigned char *rec, const typen
                 P1 = sb.y + grp.p.y;
                 if (final && !HALF) {
                     Pc = __ldg(&seg[grp_i >> SKIM_SEG_SHIFT].z) + __ldg(reinterpret_cast<const double *>(groups + (size_t)grp_i * SKIM_GROUP_BYTES + 80));
-                    add_group<true>(grp, cntk, P0, P1, Pc);
+                    add_group<true>(grp, cntk, tf, P0, P1, Pc);
                 } else {
-                    add_group<false>(grp, cntk, P0, P1, Pc);
+                    add_group<false>(grp, cntk, tf, P0, P1, Pc);
                 }
             } else {
                 // the last centroid of a width has no boundary above it: its prefix is the row total
@@ -380,6 +404,7 @@ __global__ void __launch_bounds__(LLOYD_WARPS * 32, 7) skim_lloyd_kernel(Cluster
     extern __shared__ __align__(16) unsigned char gi_all[];      // [LLOYD_WARPS][sk_entries(m)] index entries (binary32, or binary16 with compact records)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int local = blockIdx.x * LLOYD_WARPS + warp;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *a.sort_count = 0;
     if (local >= rows_in_chunk) return;
     LloydSmem &sm = sm_all[warp];
     const int64_t row = a.row0 + local;
