@@ -14,8 +14,8 @@
 //
 // Buckets: v = 1 + |x| / s with s half a standard deviation (from the mean of |x|).  The bits of v grow with |x|: the
 // first three octaves, v in [1, 8), i.e. |x| up to 3.5 deviations, have N/8 buckets each on either side of zero, the next
-// eight share N/8 (N = 32 per thread).  A row whose values this cannot spread (some bucket with BUCKET_LIMIT elements or
-// more: few distinct values, a clump) is put on a list and sorted by the radix kernel of skim_cluster.cu.
+// eight share N/8 (N = 32 per thread).  A row whose values this cannot spread (a bucket with BUCKET_LIMIT elements, or 32
+// in three neighbouring ones: few distinct values, a clump) is put on a list and sorted by the radix kernel of skim_cluster.cu.
 //
 // Why not a radix sort: rows of 32-bit keys took four passes, each with ballots or random shared-memory traffic of all
 // elements (1.17 ms for 4096 x 11008); 16-bit keys two (0.284 ms).  What bounds this kernel is the same resource,
@@ -34,18 +34,19 @@ template <int THREADS> struct Buckets {
     static constexpr int LOG = (THREADS == 128 ? 9 : THREADS == 256 ? 10 : THREADS == 512 ? 11 : 12);      // log2(N / 8)
     static_assert((8 << LOG) == N, "eight octave blocks");
     float inv_s;
-    // ascends with x; any bit pattern of x gives an index inside [0, N)
+    // ascends with x (not -0); any bit pattern of x gives an index inside [0, N)
     __device__ __forceinline__ int operator()(float x) const
     {
-        const uint32_t b = __float_as_uint(__fadd_rn(1.0f, __fmul_rn(fabsf(x), inv_s))) - 0x3f800000u;
-        const uint32_t fine = b >> (23 - LOG), coarse = 3u * (N / 8) + ((b - (3u << 23)) >> (26 - LOG));
-        const int i = (int)min(b < (3u << 23) ? fine : coarse, (uint32_t)HALF - 1u);
-        return x < 0.0f ? HALF - 1 - i : HALF + i;
+        const uint32_t b = __float_as_uint(__fmaf_rn(fabsf(x), inv_s, 1.0f)) - 0x3f800000u;
+        // below three octaves the second term wraps round to a large number, beyond them it is the smaller one
+        const uint32_t i = min(min(b >> (23 - LOG), ((b - (3u << 23)) >> (26 - LOG)) + 3u * (N / 8)), (uint32_t)HALF - 1u);
+        return HALF + (int)(i ^ (uint32_t)(__float_as_int(x) >> 31));          // negative: HALF - 1 - i
     }
 };
 
 // keys, gs: values and importances in bucket order
-// uni:      the bucket counters (8-bit) and the bases of every four of them (16-bit)
+// uni:      the bucket counters, four 8-bit ones a word; then, in their place, the positions of the four buckets: the first
+//           one's in bits 15.., the elements between it and each of the others in three 5-bit fields
 struct BucketLayout {
     size_t keys, gs, uni, phase, total;
 };
@@ -57,7 +58,7 @@ __host__ __device__ inline BucketLayout bucket_layout(int m, int threads)
     const size_t mpad = ((size_t)m + 7) & ~(size_t)7;
     L.keys = take(mpad * 4);
     L.gs = take(mpad * 4);
-    L.uni = take((size_t)threads * 48);
+    L.uni = take((size_t)threads * 32);
     L.phase = take(sizeof(PhaseSmem));
     L.total = off;
     return L;
@@ -92,7 +93,6 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) skim_sort_bucket_kern
     float *keys = reinterpret_cast<float *>(smem + L.keys);
     float *gs = reinterpret_cast<float *>(smem + L.gs);
     uint32_t *cnt = reinterpret_cast<uint32_t *>(smem + L.uni);         // four counters a word
-    uint16_t *wbase = reinterpret_cast<uint16_t *>(cnt + Bk::N / 4);    // elements before a word's buckets
     PhaseSmem &ps = *reinterpret_cast<PhaseSmem *>(smem + L.phase);
     float *red = reinterpret_cast<float *>(ps.segtot);                  // free until the record pass
     uint32_t *wsum = reinterpret_cast<uint32_t *>(ps.segtot) + 32;
@@ -147,6 +147,43 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) skim_sort_bucket_kern
             slot[i >> 2] |= s << (8 * (i & 3));
         }
     }
+    __syncthreads();
+
+    // ---------------------------------------------------------------- counters -> bases
+    {
+        uint4 v[2];
+        uint32_t s = 0u, occupied = 0u;
+#pragma unroll
+        for (int u = 0; u < 2; ++u) v[u] = reinterpret_cast<const uint4 *>(cnt)[2 * tid + u];
+        uint32_t *w = reinterpret_cast<uint32_t *>(v);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            s = __dp4a(w[u], 0x01010101u, s);
+            occupied += w[u] ? 1u : 0u;
+        }
+        // occupied words: a lower bound of the number of distinct values
+        occupied = __reduce_add_sync(0xffffffffu, occupied);
+        if (lane == 0 && occupied) atomicAdd(&ps.misc[0], (int)occupied);
+        uint32_t inc = s;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const uint32_t t = __shfl_up_sync(0xffffffffu, inc, off);
+            if (lane >= off) inc += t;
+        }
+        if (lane == 31) wsum[warp] = inc;
+        __syncthreads();
+        uint32_t run = inc - s;
+        for (int q = 0; q < warp; ++q) run += wsum[q];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const uint32_t c0 = w[u] & 0xffu, c1 = c0 + ((w[u] >> 8) & 0xffu), c2 = c1 + ((w[u] >> 16) & 0xffu), c3 = c2 + (w[u] >> 24);
+            over |= c2 > 31u;
+            w[u] = (run << 15) | c0 | (c1 << 5) | (c2 << 10);
+            run += c3;
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) reinterpret_cast<uint4 *>(cnt)[2 * tid + u] = v[u];
+    }
     if (__syncthreads_or(over ? 1 : 0)) {
         // not a row for buckets: the radix kernel takes it
         if (bad) atomicOr(a.status, (unsigned long long)bad);
@@ -157,42 +194,10 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) skim_sort_bucket_kern
         return;
     }
 
-    // ---------------------------------------------------------------- counters -> bases
-    {
-        uint4 v[2];
-        uint32_t t[8], s = 0u, occupied = 0u;
-#pragma unroll
-        for (int u = 0; u < 2; ++u) v[u] = reinterpret_cast<const uint4 *>(cnt)[2 * tid + u];
-        const uint32_t *w = reinterpret_cast<const uint32_t *>(v);
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            t[u] = s;
-            s = __dp4a(w[u], 0x01010101u, s);
-            occupied += w[u] ? 1u : 0u;
-        }
-        // occupied words: a lower bound of the number of distinct values
-        occupied = __reduce_add_sync(0xffffffffu, occupied);
-        if (lane == 0 && occupied) atomicAdd(&ps.misc[0], (int)occupied);
-        uint32_t inc = s;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const uint32_t x = __shfl_up_sync(0xffffffffu, inc, off);
-            if (lane >= off) inc += x;
-        }
-        if (lane == 31) wsum[warp] = inc;
-        __syncthreads();
-        uint32_t run = inc - s;
-        for (int q = 0; q < warp; ++q) run += wsum[q];
-        reinterpret_cast<uint4 *>(wbase)[tid] = make_uint4((run + t[0]) | ((run + t[1]) << 16), (run + t[2]) | ((run + t[3]) << 16),
-                                                           (run + t[4]) | ((run + t[5]) << 16), (run + t[6]) | ((run + t[7]) << 16));
-    }
-    __syncthreads();
-    // first position of bucket b, and (in n) its elements
-    auto bucket_base = [&](int b, int &n) {
+    // first position of bucket b
+    auto bucket_base = [&](int b) {
         const uint32_t w = cnt[b >> 2];
-        const int sh = 8 * (b & 3);
-        n = (int)((w >> sh) & 0xffu);
-        return (int)__dp4a(w & ((1u << sh) - 1u), 0x01010101u, (uint32_t)wbase[b >> 2]);
+        return (int)((w >> 15) + (((w << 5) >> (5 * (b & 3))) & 31u));
     };
 
     // ---------------------------------------------------------------- scatter to the buckets
@@ -207,8 +212,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) skim_sort_bucket_kern
             const int i = i0 + u;
             if (i < ITEMS && i * THREADS + tid < m) {
                 if (!(g[u] >= 0.0f) || g[u] > 3.0e38f) bad |= 2u;
-                int n;
-                const int pos = bucket_base(bucket(x[i < ITEMS ? i : 0]), n) + (int)((slot[i < ITEMS ? i >> 2 : 0] >> (8 * (i & 3))) & 0xffu);
+                const int pos = bucket_base(bucket(x[i < ITEMS ? i : 0])) + (int)((slot[i < ITEMS ? i >> 2 : 0] >> (8 * (i & 3))) & 0xffu);
                 if (SKIM_IDX(pos, m, a.status)) {
                     keys[pos] = x[i < ITEMS ? i : 0];
                     gs[pos] = g[u];
@@ -224,20 +228,19 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) skim_sort_bucket_kern
     // group into the next has to be sorted.  A row with few distinct values is sorted in full (they are counted below), and so
     // are all rows for the exact kernel.
     int nd = ps.misc[0];                     // more than 16 occupied words: more than 16 distinct values
+    auto bucket_end = [&](int b) { return b + 1 < Bk::N ? bucket_base(b + 1) : m; };
     const bool full = a.full_order || nd <= 16;
     for (int p0 = tid * 8; p0 < m; p0 += THREADS * 8) {
         if (!full) {
             if (p0 == 0) continue;
-            int n;
-            const int lo = bucket_base(bucket(keys[p0]), n);
-            if (lo < p0 && lo >= p0 - 8) sort_bucket(keys, gs, lo, n);          // (an earlier start: an earlier border's thread does it)
+            const int b = bucket(keys[p0]), lo = bucket_base(b);
+            if (lo < p0 && lo >= p0 - 8) sort_bucket(keys, gs, lo, bucket_end(b) - lo);          // (an earlier start: an earlier border's thread does it)
         } else {
             // every bucket that starts in these 8 positions (a bucket's other places hold elements of the bucket all along)
             for (int p = p0; p < min(p0 + 8, m);) {
-                int n;
-                const int lo = bucket_base(bucket(keys[p]), n);
-                if (lo >= p0) sort_bucket(keys, gs, lo, n);
-                p = lo + n;
+                const int b = bucket(keys[p]), lo = bucket_base(b), end = bucket_end(b);
+                if (lo >= p0) sort_bucket(keys, gs, lo, end - lo);
+                p = end;
             }
         }
     }
@@ -271,9 +274,10 @@ struct BucketVariant {
 
 #define SKIM_BV(T, I) {T * I, T, skim_sort_bucket_kernel<T, I>}
 
-// About eight elements a thread for short rows; two blocks of 512 threads per SM up to 11 264 columns, one of 1024 beyond.
+// An SM holds 1024 threads; many small blocks wait for their own barriers only (5600 columns: 256 x 22 takes 0.174 ms where
+// 512 x 16 takes 0.217 ms, 4096: 256 x 16 0.132 ms, 512 x 8 0.147 ms), as far as registers hold the row.
 const BucketVariant kVariantsBucket[] = {
-    SKIM_BV(128, 4), SKIM_BV(128, 8), SKIM_BV(256, 8), SKIM_BV(512, 8), SKIM_BV(512, 16), SKIM_BV(512, 22), SKIM_BV(1024, 16), SKIM_BV(1024, 22),
+    SKIM_BV(128, 4), SKIM_BV(128, 8), SKIM_BV(128, 16), SKIM_BV(256, 12), SKIM_BV(256, 16), SKIM_BV(256, 22), SKIM_BV(512, 16), SKIM_BV(512, 22), SKIM_BV(1024, 16), SKIM_BV(1024, 22),
 };
 
 }  // namespace

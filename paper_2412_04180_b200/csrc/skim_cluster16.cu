@@ -129,7 +129,7 @@ struct SortedItems16 {
 
 // HALF_RECORD: the compact row record, for the Lloyd kernel; else the full one, for the exact kernel.
 template <bool HALF_RECORD, int THREADS, int VEC>
-__global__ void __launch_bounds__(THREADS, (THREADS <= 512 ? 2 : 1)) skim_sort16_kernel(ClusterArgs a)
+__global__ void __launch_bounds__(THREADS, 1024 / THREADS) skim_sort16_kernel(ClusterArgs a)
 {
     using K = KeyOps<uint16_t>;
     constexpr int ITEMS = VEC * 8;
@@ -388,8 +388,10 @@ struct Variant16 {
 
 #define SKIM_V16(T, V) {T * V * 8, T, {skim_sort16_kernel<false, T, V>, skim_sort16_kernel<true, T, V>}}
 
+// An SM holds 1024 threads; small blocks wait for their own barriers only (4096 columns: 256 threads of 16 elements take
+// 0.131 ms for 4096 rows, 512 of 8 took 0.153 ms).
 const Variant16 kVariants16[] = {
-    SKIM_V16(128, 1), SKIM_V16(256, 1), SKIM_V16(512, 1), SKIM_V16(512, 2), SKIM_V16(512, 3), SKIM_V16(1024, 2),
+    SKIM_V16(128, 1), SKIM_V16(128, 2), SKIM_V16(256, 2), SKIM_V16(256, 3), SKIM_V16(512, 2), SKIM_V16(512, 3), SKIM_V16(1024, 2),
     SKIM_V16(1024, 3),
 };
 
