@@ -97,6 +97,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) skim_sort_bucket_kern
     float *red = reinterpret_cast<float *>(ps.segtot);                  // free until the record pass
     uint32_t *wsum = reinterpret_cast<uint32_t *>(ps.segtot) + 32;
 
+    skim_let_next_kernel_start();          // (this kernel is an ordinary launch: the one after it waits)
     const int64_t row = a.row0 + blockIdx.x;
     const uint16_t *Wr = a.W + row * a.ld;
     const float *Gr = a.G + row * a.ld;

@@ -69,6 +69,8 @@ __global__ void __launch_bounds__(THREADS) skim_sort_kernel(ClusterArgs a)
     const int lane = tid & 31;
     const int warp = tid >> 5;
     const int m = a.m;
+    skim_wait_for_previous_kernel();
+    skim_let_next_kernel_start();
     const int listed = min(*a.sort_count, a.chunk_rows);
     for (int at = blockIdx.x; at < listed; at += gridDim.x) {
     const int local = a.sort_list[at];
@@ -277,9 +279,8 @@ int skim_launch_cluster(skim_ctx *ctx, const uint16_t *W, const float *importanc
         if (rc) return rc;
         if (scaled) {
             // the rows the buckets could not spread: usually none
-            v->kernel<<<(unsigned)(n < 2 * ctx->sm_count ? n : 2 * ctx->sm_count), v->threads, smem, ctx->stream>>>(a);
-            SKIM_CUDA_OK(cudaGetLastError());
-            ctx->launches += 1;
+            rc = skim_launch_dependent(ctx, v->kernel, dim3((unsigned)(n < 2 * ctx->sm_count ? n : 2 * ctx->sm_count)), v->threads, smem, a);
+            if (rc) return rc;
         }
         if (tev) SKIM_CUDA_OK(cudaEventRecord(tev[1], ctx->stream));
         rc = exact_scratch ? skim_launch_exact(ctx, a, n, exact_scratch, skim_exact_slots(ctx, rows, cols))

@@ -151,6 +151,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) skim_sort16_kernel(Cl
     uint64_t *mbar = reinterpret_cast<uint64_t *>(smem + L.mbar);
     uint32_t *scratch = reinterpret_cast<uint32_t *>(ps.segtot);   // free until the record pass
 
+    skim_let_next_kernel_start();          // (this kernel is an ordinary launch: the one after it waits)
     const int64_t row = a.row0 + blockIdx.x;
     const uint16_t *Wr = a.W + row * a.ld;
     const float *Gr = a.G + row * a.ld;

@@ -191,3 +191,32 @@ __host__ __device__ static inline int64_t skim_row_stride_words(int64_t cols, in
     int64_t w = (cols * (int64_t)b + 31) / 32;
     return (w + 3) / 4 * 4;
 }
+
+// Programmatic dependent launches: the kernel may start while the one before it on the stream drains, and waits itself
+// before it reads what that one (or any earlier one) wrote and before it writes anything.
+__device__ __forceinline__ void skim_wait_for_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void skim_let_next_kernel_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... Params, typename... Args>
+int skim_launch_dependent_on(cudaStream_t stream, void (*kernel)(Params...), dim3 grid, unsigned threads, size_t smem, Args... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    SKIM_CUDA_OK(cudaLaunchKernelEx(&cfg, kernel, args...));
+    return SKIM_OK;
+}
+template <typename... Params, typename... Args>
+int skim_launch_dependent(skim_ctx *ctx, void (*kernel)(Params...), dim3 grid, unsigned threads, size_t smem, Args... args)
+{
+    const int rc = skim_launch_dependent_on(ctx->stream, kernel, grid, threads, smem, args...);
+    if (rc == SKIM_OK) ctx->launches += 1;
+    return rc;
+}

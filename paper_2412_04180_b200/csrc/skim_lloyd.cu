@@ -404,6 +404,7 @@ __global__ void __launch_bounds__(LLOYD_WARPS * 32, 7) skim_lloyd_kernel(Cluster
     extern __shared__ __align__(16) unsigned char gi_all[];      // [LLOYD_WARPS][sk_entries(m)] index entries (binary32, or binary16 with compact records)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int local = blockIdx.x * LLOYD_WARPS + warp;
+    skim_let_next_kernel_start();
     if (blockIdx.x == 0 && threadIdx.x == 0) *a.sort_count = 0;
     if (local >= rows_in_chunk) return;
     LloydSmem &sm = sm_all[warp];
@@ -452,6 +453,8 @@ int skim_launch_lloyd(skim_ctx *ctx, const ClusterArgs &args, int64_t rows)
     // set on every launch: a host-side call of microseconds, and no state shared between contexts
     void (*kernel)(ClusterArgs, int) = args.rec_half ? skim_lloyd_kernel<true> : skim_lloyd_kernel<false>;
     SKIM_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // an ordinary launch: blocks that move in beside the last sort blocks find those blocks' split of shared memory and L1,
+    // with next to no L1 for the records (4096 x 11008: 0.489 instead of 0.44 ms for the whole path)
     kernel<<<blocks, LLOYD_WARPS * 32, smem, ctx->stream>>>(args, (int)rows);
     SKIM_CUDA_OK(cudaGetLastError());
     ctx->launches += 1;

@@ -23,6 +23,9 @@ __global__ void __launch_bounds__(RT) skim_rank_rows_kernel(const uint8_t *__res
     __shared__ int wsum[RT / 32][SKIM_MAX_NBITS];
     __shared__ int gstart[SKIM_MAX_NBITS + 1];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // wait first: the next kernel reads W before its own wait, so whatever wrote W must be done when it starts
+    skim_wait_for_previous_kernel();
+    skim_let_next_kernel_start();
     const int64_t per = (n + RT - 1) / RT;
     const int64_t r0 = min(n, (int64_t)tid * per), r1 = min(n, r0 + per);
     int cnt[SKIM_MAX_NBITS] = {0, 0, 0, 0};
@@ -254,6 +257,7 @@ __global__ void __launch_bounds__(PACK_MAX_THREADS, 8) skim_pack_kernel(PackArgs
 #pragma unroll
         for (int q = 0; q < 4; ++q) raw[q] = __ldg(reinterpret_cast<const uint4 *>(Wr + tid * 32 + 8 * q));
     }
+    skim_wait_for_previous_kernel();
     const int pos = a.row_pos[row];
     const int b = (int)a.bits[row];
     if (pos < 0) return;
@@ -329,9 +333,9 @@ int skim_launch_quantize(skim_ctx *ctx, const uint16_t *W, int64_t rows, int64_t
                          int32_t *row_order, int64_t *group_info, uint16_t *lut)
 {
     SkimWorkspace ws = skim_carve(ctx->ws, rows, cols);
-    skim_rank_rows_kernel<<<1, RT, 0, ctx->stream>>>(bits, rows, cols, bs.n_bits, bs.b_min, ws.row_pos, row_order,
-                                                     (long long *)group_info, ws.status);
-    SKIM_CUDA_OK(cudaGetLastError());
+    int rc = skim_launch_dependent(ctx, skim_rank_rows_kernel, dim3(1), RT, 0, bits, rows, cols, bs.n_bits, bs.b_min, ws.row_pos, row_order,
+                                   (long long *)group_info, ws.status);
+    if (rc) return rc;
     PackArgs a;
     a.W = W;
     a.rscale = ctx->scaled ? ws.rscale : nullptr;
@@ -347,10 +351,7 @@ int skim_launch_quantize(skim_ctx *ctx, const uint16_t *W, int64_t rows, int64_t
     a.vec_ok = ((reinterpret_cast<uintptr_t>(W) & 15u) == 0 && (ld % 8) == 0) ? 1 : 0;
     a.packed = packed;
     a.lut = lut;
-    skim_pack_kernel<<<(unsigned)rows, pack_threads(cols, bs), 0, ctx->stream>>>(a);
-    SKIM_CUDA_OK(cudaGetLastError());
-    ctx->launches += 2;
-    return SKIM_OK;
+    return skim_launch_dependent(ctx, skim_pack_kernel, dim3((unsigned)rows), pack_threads(cols, bs), 0, a);
 }
 
 // ---------------------------------------------------------------- entry point that allocates nothing

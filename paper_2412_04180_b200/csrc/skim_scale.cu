@@ -16,6 +16,8 @@
 //       d loss / d alpha_j = sum_i  -2 g c (w - alpha_j c) + q g w / alpha_j^2   (c, q of the element's
 //       cluster, from the 256-byte table the first kernel left for the row), accumulated in
 //       registers; the row ranges leave partial gradients that the Adam kernel adds in a fixed order.
+// Every kernel of a step is a programmatic dependent of the one before it: it starts while that one drains and fetches
+// what no kernel of the loop writes (the matrix) before it waits.
 //   skim_scale_adam_kernel  sums the partials and the rows' losses (deterministic), applies the
 //       Adam update to the binary64 master copy of alpha.
 #include "skim_internal.cuh"
@@ -44,11 +46,6 @@ struct ScaleArgs {
     int exp2;
     int rows_per_range;
 };
-
-// Every kernel of an Adam step is launched as a programmatic dependent of the one before it: it may start while that
-// one drains, fetches what no kernel of the loop writes (the matrix), and waits here before it touches anything else.
-__device__ __forceinline__ void wait_for_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void let_next_kernel_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // 1 / a for a positive, normal binary64 a (the scale vector is checked to be that): the hardware's approximate
 // reciprocal (better than 20 bits, error e) and one step of the series 1 + e + e^2, within one unit in the last place.  Four
@@ -420,7 +417,7 @@ __global__ void __launch_bounds__(SUM_T, 1) skim_scale_sums_kernel(ScaleArgs a)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     double *alpha = ssmem;
     double2 *part = reinterpret_cast<double2 *>(ssmem + (MODE == SUMS_INIT ? 0 : (a.cols + 1) / 2 * 2));     // [SUM_W][32]
-    let_next_kernel_start();
+    skim_let_next_kernel_start();
     const int64_t stride = skim_ordered_stride(a.cols) / 2;
     const int mine = (int)((a.rows - blockIdx.x + gridDim.x - 1) / gridDim.x);       // rows of this block (at least one)
     const int whole = mine / SUM_W * SUM_W, rest = mine - whole;
@@ -433,7 +430,7 @@ __global__ void __launch_bounds__(SUM_T, 1) skim_scale_sums_kernel(ScaleArgs a)
             for (int u = 0; u < 2 * AHEAD; ++u) asm volatile("prefetch.global.L2 [%0];" ::"l"(p + u * (UNIT / 2) + lane));
         }
     }
-    wait_for_previous_kernel();
+    skim_wait_for_previous_kernel();
     if (MODE != SUMS_INIT) {
         for (int q = threadIdx.x; q < a.cols / 2; q += SUM_T)
             reinterpret_cast<double2 *>(alpha)[q] = __ldg(reinterpret_cast<const double2 *>(a.alpha) + q);
@@ -550,9 +547,9 @@ __global__ void __launch_bounds__(GT, 2) skim_scale_grad_kernel(ScaleArgs a)
 #pragma unroll
         for (int q = 0; q < RB / 2; ++q) tab[h][q] = table_load(a, rb + 2 * q, last);
     };
-    let_next_kernel_start();
+    skim_let_next_kernel_start();
     fetch_rows(0, r0);
-    wait_for_previous_kernel();
+    skim_wait_for_previous_kernel();
     fetch_tables(0, r0);
     double ah[GC], rr[GC], acc[GC];   // alpha / 2, alpha^-2
 #pragma unroll
@@ -596,8 +593,8 @@ __global__ void __launch_bounds__(256) skim_scale_adam_kernel(const double *__re
                                                                double bc1, double bc2, double eps, double *loss_out)
 {
     __shared__ double red[256];
-    let_next_kernel_start();
-    wait_for_previous_kernel();
+    skim_let_next_kernel_start();
+    skim_wait_for_previous_kernel();
     if (blockIdx.x == gridDim.x - 1) {
         // the last block adds the rows' losses: strided partial sums, then a fixed tree
         double s = 0.0;
@@ -668,8 +665,8 @@ __global__ void __launch_bounds__(GT, 2) skim_scale_lf_grad_kernel(ScaleArgs a, 
     const int64_t r0 = (int64_t)blockIdx.y * a.rows_per_range;
     const int64_t r1 = min(a.rows, r0 + a.rows_per_range), last = r1 - 1;
     const double ys = ldexp(-2.0, -a.exp2);
-    let_next_kernel_start();
-    wait_for_previous_kernel();
+    skim_let_next_kernel_start();
+    skim_wait_for_previous_kernel();
     double rr[GC], acc[GC];
 #pragma unroll
     for (int u = 0; u < GC; ++u) {
@@ -727,25 +724,6 @@ size_t skim_scale_lfull_scratch_bytes(int64_t rows, int64_t cols)
 namespace {
 
 // What both updates do first: alpha's master copies, the label-ordered matrix, the per-call constants (G_k, D_k).
-// Launches `kernel` as a programmatic dependent of the kernel before it on the stream.
-template <typename... Params, typename... Args>
-int launch_dependent(skim_ctx *ctx, void (*kernel)(Params...), dim3 grid, unsigned threads, size_t smem, Args... args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = ctx->stream;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    SKIM_CUDA_OK(cudaLaunchKernelEx(&cfg, kernel, args...));
-    ctx->launches += 1;
-    return SKIM_OK;
-}
-
 struct ScalePlan {
     ScaleArgs a;
     unsigned cb, ab;                 // blocks over the columns; Adam: 32 columns a block
@@ -820,7 +798,7 @@ struct AdamSchedule {
 
 int scale_adam(skim_ctx *ctx, const SkimWorkspace &ws, const ScalePlan &p, const AdamSchedule &s, double *loss_trace)
 {
-    return launch_dependent(ctx, skim_scale_adam_kernel, dim3(p.ab + 1), 256, 0, (const double *)ws.grad_part, (const double *)ws.loss_part, p.ranges,
+    return skim_launch_dependent(ctx, skim_scale_adam_kernel, dim3(p.ab + 1), 256, 0, (const double *)ws.grad_part, (const double *)ws.loss_part, p.ranges,
                             p.a.rows, p.a.cols, ws.alpha64, ws.adam_m, ws.adam_v, s.lr, 0.9, 0.999, 1.0 - s.p1, 1.0 - s.p2,
                             1e-8, loss_trace ? loss_trace + (s.t - 1) : nullptr);
 }
@@ -860,11 +838,11 @@ int skim_launch_scale_update_lfull(skim_ctx *ctx, const uint16_t *W, const float
     AdamSchedule sched(lr0, decay, decay_every);
     for (int t = 0; t < steps; ++t) {
         sched.next();
-        rc = launch_dependent(ctx, skim_scale_sums_kernel<SUMS_CENTROIDS>, dim3(p.sum_blocks), SUM_T, sums_smem_bytes((int)cols, false), p.a);
+        rc = skim_launch_dependent(ctx, skim_scale_sums_kernel<SUMS_CENTROIDS>, dim3(p.sum_blocks), SUM_T, sums_smem_bytes((int)cols, false), p.a);
         if (rc) return rc;
         rc = skim_launch_err_lfull(ctx, p.a.D, rows, cols, cols, H, ldh, exp2, sp, nullptr, 1, Y, cols, ws.loss_part, &cl);
         if (rc) return rc;
-        rc = launch_dependent(ctx, skim_scale_lf_grad_kernel, p.grad_grid, GT, 0, p.a, (const float *)Y);
+        rc = skim_launch_dependent(ctx, skim_scale_lf_grad_kernel, p.grad_grid, GT, 0, p.a, (const float *)Y);
         if (rc) return rc;
         rc = scale_adam(ctx, ws, p, sched, loss_trace);
         if (rc) return rc;
@@ -884,9 +862,9 @@ int skim_launch_scale_update(skim_ctx *ctx, const uint16_t *W, const float *impo
     AdamSchedule sched(lr0, decay, decay_every);
     for (int t = 0; t < steps; ++t) {
         sched.next();
-        rc = launch_dependent(ctx, skim_scale_sums_kernel<SUMS_STEP>, dim3(p.sum_blocks), SUM_T, sums_smem_bytes((int)cols, false), p.a);
+        rc = skim_launch_dependent(ctx, skim_scale_sums_kernel<SUMS_STEP>, dim3(p.sum_blocks), SUM_T, sums_smem_bytes((int)cols, false), p.a);
         if (rc) return rc;
-        rc = launch_dependent(ctx, grad, p.grad_grid, GT, 0, p.a);
+        rc = skim_launch_dependent(ctx, grad, p.grad_grid, GT, 0, p.a);
         if (rc) return rc;
         rc = scale_adam(ctx, ws, p, sched, loss_trace);
         if (rc) return rc;
