@@ -272,10 +272,12 @@ __device__ __forceinline__ void lloyd_warp(const unsigned char *rec, const typen
     double err_j = 0.0;
     int gprev = -1;                                   // group of the previous boundary position
     int gstep = 0;                                    // its last move: boundaries keep drifting the same way
+    // The group of the last iteration stays in registers with its prefix sums: most boundaries are in it again.
+    Group<HALF> grp;
+    int gloaded = -1;
     for (int it = 0;; ++it) {
         const float c_up = __shfl_down_sync(0xffffffffu, c, 1);
         int B = m, grp_i = 0, cntk = 0;
-        Group<HALF> grp;
         if (has_boundary) {
             // exact midpoint of two binary32 centroids, rounded down to binary32: x <= midpoint
             // holds for a binary32 x exactly when x <= tf
@@ -304,8 +306,13 @@ __device__ __forceinline__ void lloyd_warp(const unsigned char *rec, const typen
             if (!SKIM_IDX(grp_i, R.ngrp, a.status)) grp_i = 0;
             gstep = gprev >= 0 ? grp_i - gprev : 0;
             gprev = grp_i;
-            const unsigned char *gr = groups + (size_t)grp_i * Group<HALF>::BYTES;
-            grp.load(gr);
+            if (HALF || grp_i != gloaded) {          // (compact records: loading their two sectors always measured as fast)
+                grp.load(groups + (size_t)grp_i * Group<HALF>::BYTES);
+                const double2 sb = segs[grp_i >> SKIM_SEG_SHIFT];       // sums of the earlier segments (shared memory)
+                grp.p.x += sb.x;
+                grp.p.y += sb.y;
+                gloaded = grp_i;
+            }
             cntk = grp.count_le(tf);
             B = min((grp_i << 3) + cntk, m);
         }
@@ -315,9 +322,8 @@ __device__ __forceinline__ void lloyd_warp(const unsigned char *rec, const typen
         double P0 = 0.0, P1 = 0.0, Pc = 0.0;
         if (normal) {
             if (searches) {
-                const double2 sb = segs[grp_i >> SKIM_SEG_SHIFT];   // sums of the earlier segments (shared memory)
-                P0 = sb.x + grp.p.x;
-                P1 = sb.y + grp.p.y;
+                P0 = grp.p.x;
+                P1 = grp.p.y;
                 if (final && !HALF) {
                     Pc = __ldg(&seg[grp_i >> SKIM_SEG_SHIFT].z) + __ldg(reinterpret_cast<const double *>(groups + (size_t)grp_i * SKIM_GROUP_BYTES + 80));
                     add_group<true>(grp, cntk, tf, P0, P1, Pc);
@@ -369,29 +375,60 @@ __device__ __forceinline__ void lloyd_warp(const unsigned char *rec, const typen
     }
 }
 
-// Optional labels of the final assignment, in column order (test/diagnostic output).
-__device__ __forceinline__ void write_codes(const ClusterArgs &a, int64_t row, const LloydSmem &sm)
+// Labels of the final assignment, in column order, from the boundaries the Lloyd kernel left in the record's header: one
+// block per row (the Lloyd kernel's one warp per row took longer over them than over the iterations: 0.235 ms of 0.372 for
+// 4096 x 11008).  A stream: 2 B in, 1 B out per element and width; four probes of shared memory each.
+constexpr int CODES_T = 256;
+
+__global__ void __launch_bounds__(CODES_T) skim_codes_kernel(ClusterArgs a, int vec)
 {
-    const int m = a.m, lane = threadIdx.x & 31;
+    __shared__ float tfs[32];
+    const int tid = threadIdx.x, m = a.m;
+    const int64_t row = a.row0 + blockIdx.x;
+    skim_wait_for_previous_kernel();
+    skim_let_next_kernel_start();
+    if (tid < 32) tfs[tid] = reinterpret_cast<const float *>(a.scratch + (size_t)blockIdx.x * (size_t)a.rec_stride)[tid];
+    __syncthreads();
     const uint16_t *Wr = a.W + row * a.ld;
-    int only = -1;
-    if (a.row_bits) only = (int)a.row_bits[row] - a.bmin;
-    for (int e = lane; e < m; e += 32) {
-        float x = __half2float(__ushort_as_half(Wr[e]));
-        if (a.rscale) x = __fmul_rn(x, a.rscale[e]);
-        int off = 0;
-        for (int bi = 0; bi < a.nb; ++bi) {
-            const int k = 1 << (a.bmin + bi);
-            if (only < 0 || only == bi) {
-                // number of boundaries below x: the boundaries of a width ascend, so log2(k) probes find it
-                int code = 0;
-                for (int step = k >> 1; step >= 1; step >>= 1)
-                    if (sm.tfs[off + code + step - 1] < x) code += step;
-                if (only < 0) a.codes[((int64_t)bi * a.rows + row) * m + e] = (uint8_t)code;
-                else a.codes[row * (int64_t)m + e] = (uint8_t)code;
+    const int only = a.row_bits ? (int)a.row_bits[row] - a.bmin : -1;
+    // number of boundaries below x: the boundaries of a width ascend, so log2(k) probes find it
+    auto code = [&](float x, int off, int k) {
+        int c = 0;
+        for (int step = k >> 1; step >= 1; step >>= 1)
+            if (tfs[off + c + step - 1] < x) c += step;
+        return (uint32_t)c;
+    };
+    int off = 0;
+    for (int bi = 0; bi < a.nb; ++bi) {
+        const int k = 1 << (a.bmin + bi);
+        if (only < 0 || only == bi) {
+            uint8_t *out = only < 0 ? a.codes + ((int64_t)bi * a.rows + row) * m : a.codes + row * (int64_t)m;
+            if (vec) {
+                for (int e = tid * 4; e < m; e += CODES_T * 4) {
+                    const uint2 w = *reinterpret_cast<const uint2 *>(Wr + e);
+                    float r[4] = {1.0f, 1.0f, 1.0f, 1.0f};
+                    if (a.rscale) {
+                        const float4 v = *reinterpret_cast<const float4 *>(a.rscale + e);
+                        r[0] = v.x; r[1] = v.y; r[2] = v.z; r[3] = v.w;
+                    }
+                    uint32_t v = 0u;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const uint32_t h = u < 2 ? w.x : w.y;
+                        const float x = __half2float(__ushort_as_half((uint16_t)((u & 1) ? (h >> 16) : (h & 0xffffu))));
+                        v |= code(a.rscale ? __fmul_rn(x, r[u]) : x, off, k) << (8 * u);
+                    }
+                    *reinterpret_cast<uint32_t *>(out + e) = v;
+                }
+            } else {
+                for (int e = tid; e < m; e += CODES_T) {
+                    float x = __half2float(__ushort_as_half(Wr[e]));
+                    if (a.rscale) x = __fmul_rn(x, a.rscale[e]);
+                    out[e] = (uint8_t)code(x, off, k);
+                }
             }
-            off += k;
         }
+        off += k;
     }
 }
 
@@ -439,9 +476,8 @@ __global__ void __launch_bounds__(LLOYD_WARPS * 32, 7) skim_lloyd_kernel(Cluster
     }
     __syncwarp();
     lloyd_warp<HALF>(rec, gi, segs, nd, a, row, sm);
-    if (!a.codes) return;
-    __syncwarp();
-    write_codes(a, row, sm);
+    // the header has served its purpose: for the codes kernel the boundaries take its place
+    if (a.codes) reinterpret_cast<float *>(const_cast<unsigned char *>(rec))[lane] = sm.tfs[lane];
 }
 
 }  // namespace
@@ -458,5 +494,9 @@ int skim_launch_lloyd(skim_ctx *ctx, const ClusterArgs &args, int64_t rows)
     kernel<<<blocks, LLOYD_WARPS * 32, smem, ctx->stream>>>(args, (int)rows);
     SKIM_CUDA_OK(cudaGetLastError());
     ctx->launches += 1;
+    if (args.codes) {
+        const int vec = args.m % 4 == 0 && args.ld % 4 == 0 && (reinterpret_cast<uintptr_t>(args.W) & 7u) == 0 && (reinterpret_cast<uintptr_t>(args.codes) & 3u) == 0;
+        return skim_launch_dependent(ctx, skim_codes_kernel, dim3((unsigned)rows), CODES_T, 0, args, vec);
+    }
     return SKIM_OK;
 }

@@ -254,14 +254,18 @@ __device__ __forceinline__ double2 table_load(const ScaleArgs &a, int64_t row, i
     const int lane = threadIdx.x & 31;
     return a.tq[min(row + (lane >> 4), last) * KC + (lane & 15)];
 }
-// Shuffle indices of four labels: byte u holds label u, plus 16 for the second row of the pair (a shuffle takes the
-// low five bits of its index, so `>> 8 u` is all an element needs).
-__device__ __forceinline__ uint32_t table_index(uint32_t l, int second) { return (l & 0x0f0f0f0fu) | (second ? 0x10101010u : 0u); }
-__device__ __forceinline__ double2 table_get(const double2 &t, uint32_t index, int u)
-{
-    const int src = (int)(index >> (8 * u));
-    return make_double2(__shfl_sync(0xffffffffu, t.x, src), __shfl_sync(0xffffffffu, t.y, src));
-}
+// A warp's copy of the tables of a batch of rows in shared memory, c and q apart: 16 entries of 8 bytes lie in 16 different
+// bank pairs, so a lookup of either is two wavefronts (16-byte entries took about nine together, four 32-bit shuffles eight).
+template <int RB>
+struct WarpTables {
+    double c[RB * KC], q[RB * KC];
+    __device__ __forceinline__ void put(int pair, const double2 &t)
+    {
+        const int lane = threadIdx.x & 31;
+        c[pair * 32 + lane] = t.x;
+        q[pair * 32 + lane] = t.y;
+    }
+};
 
 // The two elements a lane has of a unit, added to its accumulators.
 template <int MODE>
@@ -395,11 +399,10 @@ __device__ __forceinline__ void residual_columns(const ScaleArgs &a, int64_t row
             const int j = min(jb + u * 128 + lane * 4, j1 - 4);      // lanes past the end repeat the last columns
             const double2 a0 = *reinterpret_cast<const double2 *>(alpha + j), a1 = *reinterpret_cast<const double2 *>(alpha + j + 2);
             const double al[4] = {a0.x, a0.y, a1.x, a1.y};
-            const uint32_t index = table_index(l[u], 0);
             uint32_t h[4];
 #pragma unroll
             for (int v = 0; v < 4; ++v) {
-                const double d = weight_of(w[u], v) - al[v] * __shfl_sync(0xffffffffu, c, (int)(index >> (8 * v)));
+                const double d = weight_of(w[u], v) - al[v] * __shfl_sync(0xffffffffu, c, (int)((l[u] >> (8 * v)) & (KC - 1)));
                 h[v] = __half_as_ushort(__float2half_rn(__fmul_rn((float)d, scale)));
             }
             *reinterpret_cast<uint2 *>(Dr + j) = make_uint2(h[0] | (h[1] << 16), h[2] | (h[3] << 16));
@@ -475,9 +478,8 @@ __global__ void __launch_bounds__(SUM_T, 1) skim_scale_sums_kernel(ScaleArgs a)
 
 // ---------------------------------------------------------------- the gradient of a step
 //
-// A thread owns four columns and walks a range of rows.  The (c_k, q_k) entry of an element comes by four 32-bit
-// shuffles from the row's table, which sits in the lanes (reading 16-byte entries from shared memory by label costs
-// about nine wavefronts a warp, and a barrier per batch of rows); warps do not wait for one another.  Two blocks are resident
+// A thread owns four columns and walks a range of rows.  The (c_k, q_k) entry of an element comes from the warp's own copy
+// of the rows' tables in shared memory; warps do not wait for one another.  Two blocks are resident
 // per SM and the grid is one wave of them.  HBM traffic: 7 B an element.
 template <bool VEC>
 struct GradCols {
@@ -533,6 +535,8 @@ __device__ __forceinline__ void grad_load(const ScaleArgs &a, int64_t row, const
 template <bool VEC>
 __global__ void __launch_bounds__(GT, 2) skim_scale_grad_kernel(ScaleArgs a)
 {
+    __shared__ WarpTables<4> tables[GT / 32];
+    WarpTables<4> &tw = tables[threadIdx.x >> 5];
     constexpr int RB = VEC ? 4 : 2;   // rows of a batch (four column addresses leave fewer registers); two batches take turns in registers, one of them in flight
     const GradCols<VEC> c(blockIdx.x, a.cols);
     const int64_t r0 = (int64_t)blockIdx.y * a.rows_per_range;
@@ -562,19 +566,22 @@ __global__ void __launch_bounds__(GT, 2) skim_scale_grad_kernel(ScaleArgs a)
     for (int64_t rb = r0; rb < r1; rb += 2 * RB) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
+            __syncwarp();
+#pragma unroll
+            for (int q = 0; q < RB / 2; ++q) tw.put(q, tab[h][q]);
+            __syncwarp();
             fetch_rows(h ^ 1, rb + (h + 1) * RB);
             fetch_tables(h ^ 1, rb + (h + 1) * RB);
 #pragma unroll
             for (int q = 0; q < RB; ++q) {
                 if (rb + h * RB + q < r1) {
                     const float g[GC] = {row[h][q].g.x, row[h][q].g.y, row[h][q].g.z, row[h][q].g.w};
-                    const uint32_t index = table_index(row[h][q].l, q & 1);
 #pragma unroll
                     for (int u = 0; u < GC; ++u) {
                         // g (q w / alpha^2 - 2 c (w - alpha c)) with d = 2 c:  g (w (q / alpha^2 - d) + d (d alpha / 2))
-                        const double2 cq = table_get(tab[h][q >> 1], index, u);
-                        const double d = cq.x + cq.x;
-                        const double t = fma(weight_of(row[h][q].w, u), fma(cq.y, rr[u], -d), d * (d * ah[u]));
+                        const int l = q * KC + (int)((row[h][q].l >> (8 * u)) & (KC - 1));
+                        const double c = tw.c[l], d = c + c;
+                        const double t = fma(weight_of(row[h][q].w, u), fma(tw.q[l], rr[u], -d), d * (d * ah[u]));
                         acc[u] = fma((double)g[u], t, acc[u]);
                     }
                 }
@@ -660,6 +667,8 @@ __global__ void skim_scale_finish_kernel(const double *__restrict__ alpha, int c
 // (cols is a multiple of 8 and the rows are aligned: vector loads always).
 __global__ void __launch_bounds__(GT, 2) skim_scale_lf_grad_kernel(ScaleArgs a, const float *Y)
 {
+    __shared__ WarpTables<2> tables[GT / 32];
+    WarpTables<2> &tw = tables[threadIdx.x >> 5];
     constexpr int RB = 2;
     const GradCols<true> c(blockIdx.x, a.cols);
     const int64_t r0 = (int64_t)blockIdx.y * a.rows_per_range;
@@ -691,18 +700,20 @@ __global__ void __launch_bounds__(GT, 2) skim_scale_lf_grad_kernel(ScaleArgs a, 
     for (int64_t rb = r0; rb < r1; rb += 2 * RB) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
+            __syncwarp();
+            tw.put(0, tab[h]);
+            __syncwarp();
             fetch(h ^ 1, rb + (h + 1) * RB);
 #pragma unroll
             for (int q = 0; q < RB; ++q) {
                 if (rb + h * RB + q < r1) {
                     const float g[GC] = {row[h][q].g.x, row[h][q].g.y, row[h][q].g.z, row[h][q].g.w};
                     const float y[GC] = {yv[h][q].x, yv[h][q].y, yv[h][q].z, yv[h][q].w};
-                    const uint32_t index = table_index(row[h][q].l, q & 1);
 #pragma unroll
                     for (int u = 0; u < GC; ++u) {
-                        const double2 cq = table_get(tab[h], index, u);
-                        acc[u] = fma((double)y[u], cq.x, acc[u]);
-                        acc[u] = fma((cq.y * rr[u]) * (double)g[u], weight_of(row[h][q].w, u), acc[u]);
+                        const int l = q * KC + (int)((row[h][q].l >> (8 * u)) & (KC - 1));
+                        acc[u] = fma((double)y[u], tw.c[l], acc[u]);
+                        acc[u] = fma((tw.q[l] * rr[u]) * (double)g[u], weight_of(row[h][q].w, u), acc[u]);
                     }
                 }
             }
