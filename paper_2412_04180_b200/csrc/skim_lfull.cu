@@ -27,6 +27,7 @@
 #include <vector>
 
 #include "skim_internal.cuh"
+#include "skim_labels.cuh"
 
 namespace {
 
@@ -45,17 +46,74 @@ struct ResidualArgs {
     int cols;
     int nb, bmin, sumk;
     int exp2;
-    int vec;                 // rows of W, D (and of the scale vectors) allow 128-bit accesses
+    int vec;                 // rows of D (and of the scale vector) allow 128-bit accesses
     uint16_t *D;
     unsigned long long *status;
 };
 
+// Eight elements per thread and step, the next step's weights in flight.  The label's centroid is one conflict-free lookup in
+// shared memory; the labels themselves come from packed compares (unscaled), so that a narrow width costs little.  Plain stores:
+// what fits stays in L2 for the contraction.
+template <int B>
+__device__ __forceinline__ void residual_row(const ResidualArgs &a, const uint16_t *Wr, uint16_t *Dr, const skiml::RowBounds &rb, const float *cs, uint4 raw)
+{
+    __half2 th[(1 << B) - 1];
+#pragma unroll
+    for (int j = 0; j < (1 << B) - 1; ++j) th[j] = rb.th[j];
+    const float scale = __int_as_float((127 + a.exp2) << 23);       // 2^exp2, exact
+    for (int e0 = threadIdx.x * 8; e0 < a.cols; e0 += RES_T * 8) {
+        uint4 next = make_uint4(0u, 0u, 0u, 0u);
+        if (e0 + RES_T * 8 < a.cols) next = skiml::load8_weights(Wr, e0 + RES_T * 8, a.cols);
+        float w[8];
+        skiml::values8(raw, nullptr, e0, a.cols, w);
+        uint32_t code;
+        if (a.rscale) {
+            float x[8];
+            skiml::values8(raw, a.rscale, e0, a.cols, x);
+            code = skiml::labels8_float<B>(x, rb.tf);
+        } else {
+            code = skiml::labels8_half<B>(raw, th);
+        }
+        float q[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) q[u] = cs[(code >> (u * B)) & ((1u << B) - 1u)];
+        if (a.s) {
+            if (a.vec) {
+                const float4 s0 = *reinterpret_cast<const float4 *>(a.s + e0), s1 = *reinterpret_cast<const float4 *>(a.s + e0 + 4);
+                const float sv[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
+#pragma unroll
+                for (int u = 0; u < 8; ++u) q[u] = __fmul_rn(q[u], sv[u]);
+            } else {
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    if (e0 + u < a.cols) q[u] = __fmul_rn(q[u], a.s[e0 + u]);
+            }
+        }
+        uint32_t out[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const __half2 h = __floats2half2_rn(__fmul_rn(__fsub_rn(w[2 * u], q[2 * u]), scale), __fmul_rn(__fsub_rn(w[2 * u + 1], q[2 * u + 1]), scale));
+            out[u] = *reinterpret_cast<const uint32_t *>(&h);
+        }
+        if (a.vec) {
+            *reinterpret_cast<uint4 *>(Dr + e0) = make_uint4(out[0], out[1], out[2], out[3]);
+        } else {
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (e0 + u < a.cols) Dr[e0 + u] = (uint16_t)((u & 1) ? (out[u >> 1] >> 16) : (out[u >> 1] & 0xffffu));
+        }
+        raw = next;
+    }
+}
+
 __global__ void __launch_bounds__(RES_T) skim_residual_kernel(ResidualArgs a)
 {
-    __shared__ float tf[16];
+    __shared__ skiml::RowBounds rb;
     __shared__ float cs[16];
     const int tid = threadIdx.x;
     const int64_t row = blockIdx.x;
+    const uint16_t *Wr = a.W + row * a.ld;
+    const uint4 raw = skiml::load8_weights(Wr, tid * 8, a.cols);
     const int b = a.row_bits ? (int)a.row_bits[row] : a.width;
     const int bi = b - a.bmin;
     if (bi < 0 || bi >= a.nb) {
@@ -68,62 +126,15 @@ __global__ void __launch_bounds__(RES_T) skim_residual_kernel(ResidualArgs a)
     if (tid < 16) {
         const float cj = c[min(tid, k - 1)];
         cs[tid] = cj;
-        float t = __int_as_float(0x7f800000);
-        if (tid < k - 1) {
-            t = __double2float_rd(0.5 * ((double)cj + (double)c[tid + 1]));
-            if (t == 0.0f) t = 0.0f;
-        }
-        tf[tid] = t;
+        skiml::fill_bounds(rb, tid, c, cj, k);
     }
     __syncthreads();
-    const uint16_t *Wr = a.W + row * a.ld;
     uint16_t *Dr = a.D + row * a.ldd;
-    const float scale = __int_as_float((127 + a.exp2) << 23);       // 2^exp2, exact
-    if (a.vec) {
-        // eight elements per thread and step: one 128-bit load of W, one 128-bit store of D
-        for (int e0 = tid * 8; e0 < a.cols; e0 += RES_T * 8) {
-            const uint4 wv = __ldcs(reinterpret_cast<const uint4 *>(Wr + e0));
-            const uint32_t ww[4] = {wv.x, wv.y, wv.z, wv.w};
-            float rs[8], sv[8];
-            if (a.rscale) {
-                const float4 r0 = *reinterpret_cast<const float4 *>(a.rscale + e0), r1 = *reinterpret_cast<const float4 *>(a.rscale + e0 + 4);
-                rs[0] = r0.x; rs[1] = r0.y; rs[2] = r0.z; rs[3] = r0.w; rs[4] = r1.x; rs[5] = r1.y; rs[6] = r1.z; rs[7] = r1.w;
-            }
-            if (a.s) {
-                const float4 s0 = *reinterpret_cast<const float4 *>(a.s + e0), s1 = *reinterpret_cast<const float4 *>(a.s + e0 + 4);
-                sv[0] = s0.x; sv[1] = s0.y; sv[2] = s0.z; sv[3] = s0.w; sv[4] = s1.x; sv[5] = s1.y; sv[6] = s1.z; sv[7] = s1.w;
-            }
-            uint32_t out[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const float w = __half2float(__ushort_as_half((uint16_t)((u & 1) ? (ww[u >> 1] >> 16) : (ww[u >> 1] & 0xffffu))));
-                float x = w;
-                if (a.rscale) x = __fmul_rn(w, rs[u]);
-                int code = (x > tf[7]) ? 8 : 0;
-                code += (x > tf[code + 3]) ? 4 : 0;
-                code += (x > tf[code + 1]) ? 2 : 0;
-                code += (x > tf[code]) ? 1 : 0;
-                float q = cs[code];
-                if (a.s) q = __fmul_rn(q, sv[u]);
-                const uint32_t h = __half_as_ushort(__float2half_rn(__fmul_rn(__fsub_rn(w, q), scale)));
-                out[u >> 1] |= h << (16 * (u & 1));
-            }
-            __stcs(reinterpret_cast<uint4 *>(Dr + e0), make_uint4(out[0], out[1], out[2], out[3]));
-        }
-        return;
-    }
-    for (int e = tid; e < a.cols; e += RES_T) {
-        const float w = __half2float(__ushort_as_half(Wr[e]));
-        float x = w;
-        if (a.rscale) x = __fmul_rn(w, a.rscale[e]);
-        int code = (x > tf[7]) ? 8 : 0;
-        code += (x > tf[code + 3]) ? 4 : 0;
-        code += (x > tf[code + 1]) ? 2 : 0;
-        code += (x > tf[code]) ? 1 : 0;
-        float q = cs[code];
-        if (a.s) q = __fmul_rn(q, a.s[e]);
-        const float r = __fsub_rn(w, q);
-        Dr[e] = __half_as_ushort(__float2half_rn(__fmul_rn(r, scale)));
+    switch (b) {
+    case 1: residual_row<1>(a, Wr, Dr, rb, cs, raw); break;
+    case 2: residual_row<2>(a, Wr, Dr, rb, cs, raw); break;
+    case 3: residual_row<3>(a, Wr, Dr, rb, cs, raw); break;
+    default: residual_row<4>(a, Wr, Dr, rb, cs, raw); break;
     }
 }
 
@@ -777,8 +788,7 @@ int skim_launch_residual(skim_ctx *ctx, const uint16_t *W, int64_t rows, int64_t
     a.bmin = bs.b_min;
     a.sumk = bs.sumk;
     a.exp2 = exp2;
-    a.vec = ((reinterpret_cast<uintptr_t>(W) & 15u) == 0 && (reinterpret_cast<uintptr_t>(D) & 15u) == 0 && ld % 8 == 0 &&
-             ldd % 8 == 0 && cols % 8 == 0 && (!s || (reinterpret_cast<uintptr_t>(s) & 15u) == 0)) ? 1 : 0;
+    a.vec = ((reinterpret_cast<uintptr_t>(D) & 15u) == 0 && ldd % 8 == 0 && cols % 8 == 0 && (!s || (reinterpret_cast<uintptr_t>(s) & 15u) == 0)) ? 1 : 0;
     a.D = D;
     a.status = ws.status;
     skim_residual_kernel<<<(unsigned)rows, RES_T, 0, ctx->stream>>>(a);

@@ -6,9 +6,10 @@
 //                          every row, row order, group starts and word offsets.
 //   skim_pack_kernel       one block per row: label = number of midpoints below the element
 //                          (packed fp16 compares, two weights per instruction, when no scale is
-//                          installed; a 4-step search in binary32 otherwise); a thread packs whole
-//                          groups of 32 elements into their b words.
+//                          installed; a b-step search in binary32 otherwise); a thread packs whole
+//                          groups of 32 elements into their b words (8 into their b bytes).
 #include "skim_internal.cuh"
+#include "skim_labels.cuh"
 
 namespace {
 
@@ -118,103 +119,40 @@ struct PackArgs {
     uint16_t *lut;
 };
 
-// Labels of 8 fp16 weights (no scale installed) with packed half-precision compares: a weight is
-// above a boundary exactly when it is above the boundary rounded down to fp16, so two weights are
-// compared per instruction and the label is the running sum of the 0/1 results.  Returns the 8
-// labels as B-bit fields.
-template <int B>
-__device__ __forceinline__ uint32_t labels8_half(const uint4 raw, const __half2 *th)
-{
-    const __half2 *p = reinterpret_cast<const __half2 *>(&raw);
-    const __half2 magic = __floats2half2_rn(1024.0f, 1024.0f);   // 1024 + n has n in its low mantissa bits
-    uint32_t v = 0;
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        __half2 cnt = magic;
-#pragma unroll
-        for (int j = 0; j < (1 << B) - 1; ++j) cnt = __hadd2(cnt, __hgt2(p[u], th[j]));
-        const uint32_t bits = *reinterpret_cast<const uint32_t *>(&cnt);
-        v |= (bits & 0xfu) << ((2 * u) * B);
-        v |= ((bits >> 16) & 0xfu) << ((2 * u + 1) * B);
-    }
-    return v;
-}
-
 // Eight blocks of this size are resident per SM at 64 registers.  A block lives for little more than the two round
 // trips of its parameter loads, so many small resident blocks hide them better than few large ones (measured: 64,
 // 128, 192, 256 and 384 threads give 42.9, 40.0, 43.5, 44.3 and 45.8 us for rank + pack of 4096 x 11008).
 constexpr int PACK_MAX_THREADS = 128;
 
-// Labels of 8 elements starting at e0 on the general path (a scale vector installed, unaligned rows, or the ragged
-// end of a row): the clustered value in binary32, then a 4-step search of the binary32 thresholds.
-template <int B>
-__device__ __forceinline__ uint32_t labels8_general(const PackArgs &a, const uint16_t *Wr, int e0, const float *tf)
-{
-    float x[8];
-    if (a.vec_ok && e0 + 8 <= a.cols) {
-        const uint4 raw = *reinterpret_cast<const uint4 *>(Wr + e0);
-        const __half2 *h2 = reinterpret_cast<const __half2 *>(&raw);
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const float2 f = __half22float2(h2[u]);
-            x[2 * u] = f.x;
-            x[2 * u + 1] = f.y;
-        }
-        if (a.rscale) {
-            const float4 r0 = *reinterpret_cast<const float4 *>(a.rscale + e0);
-            const float4 r1 = *reinterpret_cast<const float4 *>(a.rscale + e0 + 4);
-            x[0] = __fmul_rn(x[0], r0.x); x[1] = __fmul_rn(x[1], r0.y);
-            x[2] = __fmul_rn(x[2], r0.z); x[3] = __fmul_rn(x[3], r0.w);
-            x[4] = __fmul_rn(x[4], r1.x); x[5] = __fmul_rn(x[5], r1.y);
-            x[6] = __fmul_rn(x[6], r1.z); x[7] = __fmul_rn(x[7], r1.w);
-        }
-    } else {
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int e = e0 + u;
-            float xv = -__int_as_float(0x7f800000);    // past the row: label 0 (zero padding)
-            if (e < a.cols) {
-                xv = __half2float(__ushort_as_half(Wr[e]));
-                if (a.rscale) xv = __fmul_rn(xv, a.rscale[e]);
-            }
-            x[u] = xv;
-        }
-    }
-    uint32_t v = 0;
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-        int code = (x[u] > tf[7]) ? 8 : 0;
-        code += (x[u] > tf[code + 3]) ? 4 : 0;
-        code += (x[u] > tf[code + 1]) ? 2 : 0;
-        code += (x[u] > tf[code]) ? 1 : 0;
-        v |= (uint32_t)code << (u * B);
-    }
-    return v;
-}
-
-// One row at width B: a thread packs whole groups of 32 elements into their B words -- four 128-bit loads, the
+// One unscaled, aligned row at width B: a thread packs whole groups of 32 elements into their B words -- four 128-bit loads, the
 // labels of 8 elements at a time, the four 8B-bit fields joined with compile-time shifts -- so that no bits cross
-// threads (an earlier version gave a thread 8 elements and merged four threads' fields with 64-bit shuffles, which
-// cost more instructions than the compares).
+// threads.
 template <int B>
-__device__ __forceinline__ void pack_row(const PackArgs &a, const uint16_t *Wr, const __half2 *th, const float *tf,
-                                         uint32_t *dst, int64_t stride, bool fast, uint4 (&raw)[4])
+__device__ __forceinline__ void pack_row(const PackArgs &a, const uint16_t *Wr, const skiml::RowBounds &rb, uint32_t *dst, int64_t stride, uint4 (&raw)[4])
 {
+    __half2 th[(1 << B) - 1];
+#pragma unroll
+    for (int j = 0; j < (1 << B) - 1; ++j) th[j] = rb.th[j];
     const int ngroups = (int)((stride + B - 1) / B);    // a group: 32 elements -> B words
     // `raw` arrives holding the weights of the thread's first group (requested before the row's parameters were)
     for (int grp = threadIdx.x; grp < ngroups; grp += blockDim.x) {
         const int e0 = grp * 32;
         uint32_t v[4];
-        if (fast && e0 + 32 <= a.cols) {
+        if (e0 + 32 <= a.cols) {
             if (grp != (int)threadIdx.x) {
 #pragma unroll
                 for (int q = 0; q < 4; ++q) raw[q] = __ldg(reinterpret_cast<const uint4 *>(Wr + e0 + 8 * q));
             }
 #pragma unroll
-            for (int q = 0; q < 4; ++q) v[q] = labels8_half<B>(raw[q], th);
+            for (int q = 0; q < 4; ++q) v[q] = skiml::labels8_half<B>(raw[q], th);
         } else {
+            // the row's ragged end, and the zero padding behind it
 #pragma unroll
-            for (int q = 0; q < 4; ++q) v[q] = labels8_general<B>(a, Wr, e0 + 8 * q, tf);
+            for (int q = 0; q < 4; ++q) {
+                const int e = e0 + 8 * q;
+                v[q] = e < a.cols ? skiml::labels8_half<B>(skiml::load8_weights(Wr, e, a.cols), th) : 0u;
+                if (e < a.cols && e + 8 > a.cols) v[q] &= (1u << ((a.cols - e) * B)) - 1u;
+            }
         }
         uint32_t word[4] = {0u, 0u, 0u, 0u};
         if constexpr (B == 4) {
@@ -240,10 +178,52 @@ __device__ __forceinline__ void pack_row(const PackArgs &a, const uint16_t *Wr, 
     }
 }
 
+// The same for rows with a scale vector installed, or not 16-byte aligned: a thread takes eight consecutive elements at a
+// time, whose labels are B whole bytes of the packed row, so that loads and stores are contiguous across a warp.  (With
+// groups of 32 a thread's loads of W and 1 / alpha lay 64 and 128 bytes apart across the lanes: 82 us for 4096 x 11008
+// scaled, 62 us for 2000 x 11007, now 47 and 26.)  Bytes past the row are zero.
+template <int B>
+__device__ __forceinline__ void pack_row_bytes(const PackArgs &a, const uint16_t *Wr, const skiml::RowBounds &rb, uint32_t *dst, int bytes, uint4 raw)
+{
+    __half2 th[(1 << B) - 1];
+#pragma unroll
+    for (int j = 0; j < (1 << B) - 1; ++j) th[j] = rb.th[j];
+    const int T = blockDim.x;
+    uint8_t *out = reinterpret_cast<uint8_t *>(dst);
+    // `raw` arrives holding the weights of the thread's first eight elements
+    for (int g = threadIdx.x; g * B < bytes; g += T) {
+        const int e0 = g * 8;
+        uint4 next = make_uint4(0u, 0u, 0u, 0u);
+        if ((g + T) * B < bytes) next = skiml::load8_weights(Wr, e0 + 8 * T, a.cols);
+        uint32_t v = 0u;
+        if (e0 < a.cols) {
+            if (a.rscale) {
+                float x[8];
+                skiml::values8(raw, a.rscale, e0, a.cols, x);
+                v = skiml::labels8_float<B>(x, rb.tf);
+            } else {
+                v = skiml::labels8_half<B>(raw, th);
+            }
+            if (e0 + 8 > a.cols) v &= (1u << ((a.cols - e0) * B)) - 1u;
+        }
+        if constexpr (B == 4) {
+            *reinterpret_cast<uint32_t *>(out + 4 * g) = v;
+        } else if constexpr (B == 2) {
+            *reinterpret_cast<uint16_t *>(out + 2 * g) = (uint16_t)v;
+        } else if constexpr (B == 1) {
+            out[g] = (uint8_t)v;
+        } else {
+#pragma unroll
+            for (int u = 0; u < 3; ++u)
+                if (3 * g + u < bytes) out[3 * g + u] = (uint8_t)(v >> (8 * u));
+        }
+        raw = next;
+    }
+}
+
 __global__ void __launch_bounds__(PACK_MAX_THREADS, 8) skim_pack_kernel(PackArgs a)
 {
-    __shared__ float tf[16];
-    __shared__ __half2 th_s[16];
+    __shared__ skiml::RowBounds rb;
     const int tid = threadIdx.x;
     const int64_t row = blockIdx.x;
     const uint16_t *Wr = a.W + row * a.ld;
@@ -253,7 +233,9 @@ __global__ void __launch_bounds__(PACK_MAX_THREADS, 8) skim_pack_kernel(PackArgs
     uint4 raw[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) raw[q] = make_uint4(0u, 0u, 0u, 0u);
-    if (fast && tid * 32 + 32 <= a.cols) {
+    if (!fast) {
+        raw[0] = skiml::load8_weights(Wr, tid * 8, a.cols);
+    } else if (tid * 32 + 32 <= a.cols) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) raw[q] = __ldg(reinterpret_cast<const uint4 *>(Wr + tid * 32 + 8 * q));
     }
@@ -269,37 +251,41 @@ __global__ void __launch_bounds__(PACK_MAX_THREADS, 8) skim_pack_kernel(PackArgs
     if (tid < 16) {
         const float cj = c[min(tid, k - 1)];
         if (tid < kmax) a.lut[row * kmax + tid] = __half_as_ushort(__float2half_rn(cj));
-        float t = __int_as_float(0x7f800000);
-        if (tid < k - 1) {
-            t = __double2float_rd(0.5 * ((double)cj + (double)c[tid + 1]));
-            if (t == 0.0f) t = 0.0f;
-        }
-        tf[tid] = t;
-        th_s[tid] = __half2half2(__float2half_rd(t));
+        skiml::fill_bounds(rb, tid, c, cj, k);
     }
     __syncthreads();
-    __half2 th[15];
-#pragma unroll
-    for (int j = 0; j < 15; ++j) th[j] = th_s[j];
     const int64_t stride = skim_row_stride_words(a.cols, b);
     uint32_t *dst = a.packed + a.group_info[a.nb + 1 + bi] + (int64_t)(pos - a.group_info[bi]) * stride;
-    switch (b) {
-    case 1: pack_row<1>(a, Wr, th, tf, dst, stride, fast, raw); break;
-    case 2: pack_row<2>(a, Wr, th, tf, dst, stride, fast, raw); break;
-    case 3: pack_row<3>(a, Wr, th, tf, dst, stride, fast, raw); break;
-    default: pack_row<4>(a, Wr, th, tf, dst, stride, fast, raw); break;
+    const int bytes = (int)stride * 4;
+    if (fast) {
+        switch (b) {
+        case 1: pack_row<1>(a, Wr, rb, dst, stride, raw); break;
+        case 2: pack_row<2>(a, Wr, rb, dst, stride, raw); break;
+        case 3: pack_row<3>(a, Wr, rb, dst, stride, raw); break;
+        default: pack_row<4>(a, Wr, rb, dst, stride, raw); break;
+        }
+    } else {
+        switch (b) {
+        case 1: pack_row_bytes<1>(a, Wr, rb, dst, bytes, raw[0]); break;
+        case 2: pack_row_bytes<2>(a, Wr, rb, dst, bytes, raw[0]); break;
+        case 3: pack_row_bytes<3>(a, Wr, rb, dst, bytes, raw[0]); break;
+        default: pack_row_bytes<4>(a, Wr, rb, dst, bytes, raw[0]); break;
+        }
     }
 }
 
-// Threads of a pack block: one per group of 32 elements of the longest packed row, in whole warps, at most
-// PACK_MAX_THREADS (longer rows take several groups per thread).
-static unsigned pack_threads(int64_t cols, const SkimBits &bs)
+// Threads of a pack block: one per group of 32 elements of the longest packed row (fast rows) or per eight elements, in whole
+// warps, at most PACK_MAX_THREADS (longer rows take several rounds).
+static unsigned pack_threads(int64_t cols, const SkimBits &bs, bool fast)
 {
-    int64_t most = 1;
-    for (int u = 0; u < bs.n_bits; ++u) {
-        const int b = bs.b_min + u;
-        const int64_t g = (skim_row_stride_words(cols, b) + b - 1) / b;
-        if (g > most) most = g;
+    int64_t most = (cols + 7) / 8;
+    if (fast) {
+        most = 1;
+        for (int u = 0; u < bs.n_bits; ++u) {
+            const int b = bs.b_min + u;
+            const int64_t g = (skim_row_stride_words(cols, b) + b - 1) / b;
+            if (g > most) most = g;
+        }
     }
     const int64_t t = (most + 31) / 32 * 32;
     return (unsigned)(t > PACK_MAX_THREADS ? PACK_MAX_THREADS : t);
@@ -351,7 +337,7 @@ int skim_launch_quantize(skim_ctx *ctx, const uint16_t *W, int64_t rows, int64_t
     a.vec_ok = ((reinterpret_cast<uintptr_t>(W) & 15u) == 0 && (ld % 8) == 0) ? 1 : 0;
     a.packed = packed;
     a.lut = lut;
-    return skim_launch_dependent(ctx, skim_pack_kernel, dim3((unsigned)rows), pack_threads(cols, bs), 0, a);
+    return skim_launch_dependent(ctx, skim_pack_kernel, dim3((unsigned)rows), pack_threads(cols, bs, a.vec_ok && !a.rscale), 0, a);
 }
 
 // ---------------------------------------------------------------- entry point that allocates nothing
@@ -430,7 +416,7 @@ extern "C" int skim_quantize_static(void *cuda_stream, const uint16_t *W, int64_
     a.vec_ok = ((reinterpret_cast<uintptr_t>(W) & 15u) == 0 && (ld % 8) == 0) ? 1 : 0;
     a.packed = packed;
     a.lut = lut;
-    skim_pack_kernel<<<(unsigned)rows, pack_threads(cols, bs), 0, stream>>>(a);
+    skim_pack_kernel<<<(unsigned)rows, pack_threads(cols, bs, a.vec_ok && !a.rscale), 0, stream>>>(a);
     SKIM_CUDA_OK(cudaGetLastError());
     return SKIM_OK;
 }
