@@ -4,20 +4,16 @@
 //   skim_dequantize  packed codes + per-row codebooks (+ alpha) -> fp16 matrix in source-row order
 //   skim_matvec      y = Wq x taken straight from the packed codes, never forming Wq
 //
-// One warp owns one packed row.  A step covers 256 consecutive elements: the warp fetches the 8b
-// words that hold them with one coalesced load, every lane cuts its 8 codes out of the bit stream
-// (two shuffles and a funnel shift, since 3-bit codes straddle words), looks the codebook entry up
-// in the warp's 16-word copy of the row's codebook in shared memory (16 consecutive words: no bank
-// conflicts, equal indices are broadcast) and meets the per-column vector (alpha, or alpha * x),
-// also in shared memory, where the block put it once for all of its rows.  Both kernels are bound by HBM
-// traffic: b/8 bytes per element in, and for the dequantiser 2 bytes per element out.
+// Codebook lookups go to the warp's copy of the row's codebook in shared memory, 16 consecutive words: no bank conflicts,
+// one wavefront of the L1 data path per 32 elements (a shuffle takes that path for twice as long).
+// A warp takes 256 columns of a row at a time; the per-column vector (alpha, or z = alpha x) sits in shared memory.  What a
+// warp needs of its first row is on its way while that vector is staged.
+//   dequantiser  bound by HBM: b/8 B in and 2 B out per element
+//   mat-vec      bound by the L1 data path (two wavefronts per 32 elements: a lookup each and the reads of z) and issue (five
+//                instructions per element) and, at the usual sizes, by its start and end
 #include "skim_internal.cuh"
 
 namespace {
-
-constexpr int UT = 1024;            // threads per block: 32 rows share one copy of the column vector
-constexpr int UW = UT / 32;
-constexpr int STEP = 256;           // elements per warp step
 
 struct UnpackArgs {
     const uint32_t *packed;
@@ -35,164 +31,269 @@ struct UnpackArgs {
     float *y;                       // mat-vec: [rows]
 };
 
-// Packed row p: its width index, source row and first word.  False when p is not a placed row.
-__device__ __forceinline__ bool locate_row(const UnpackArgs &a, int64_t p, int &width, int64_t &src_row,
-                                           const uint32_t *&words, int &stride)
+// The groups' first packed rows and word offsets, in registers (uniform loads, all at once).
+struct Groups {
+    int start[SKIM_MAX_NBITS + 1];
+    long long word[SKIM_MAX_NBITS];
+    int placed;                     // packed rows (a width outside the bit set was skipped)
+    __device__ __forceinline__ explicit Groups(const UnpackArgs &a)
+    {
+        placed = 0;
+#pragma unroll
+        for (int u = 0; u <= SKIM_MAX_NBITS; ++u) {
+            start[u] = u <= a.nb ? (int)__ldg(a.group_info + u) : 0;
+            if (u < SKIM_MAX_NBITS) word[u] = u < a.nb ? __ldg(a.group_info + a.nb + 1 + u) : 0;
+            if (u == a.nb) placed = start[u];
+        }
+    }
+};
+
+// The shared address of a codebook as the lookups take it.  The lookups are assembly that the compiler does not see as reads of the
+// array: this call, before and after the array is written, keeps them on their side of the stores.
+__device__ __forceinline__ uint32_t codebook_address(const float *book)
 {
-    if (p >= a.rows) return false;
-    int bi = -1;
-    for (int u = 0; u < a.nb; ++u)
-        if (p >= a.group_info[u] && p < a.group_info[u + 1]) bi = u;
-    if (bi < 0) return false;       // beyond the placed rows (a width outside the bit set was skipped)
-    width = a.bmin + bi;
-    stride = (int)skim_row_stride_words(a.cols, width);
-    words = a.packed + a.group_info[a.nb + 1 + bi] + (p - a.group_info[bi]) * (int64_t)stride;
-    src_row = a.row_order[p];
-    if (!SKIM_IDX(src_row, a.rows, nullptr)) return false;
-    return true;
+    uint32_t r;
+    asm volatile("mov.u32 %0, %1;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(book)) : "memory");
+    return r;
 }
 
-// Where entry j of the per-column vector sits in shared memory: inside each block of 256 entries the
-// first quads of all 32 lanes come first, then the second quads, so that a lane's 8 entries are two
-// 16-byte loads that are contiguous across the warp.
+// Codebook entry of a code, the codebook at shared address `book` (64-byte aligned).  `code4` holds the code in bits 2 .. B + 1
+// among others: one logic operation makes the address.
+template <int B>
+__device__ __forceinline__ float lookup(uint32_t book, uint32_t code4)
+{
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"((code4 & (((1u << B) - 1u) << 2)) | book));
+    return v;
+}
+
+constexpr int UT = 1024;            // threads per block, one block per SM
+constexpr int UW = UT / 32;
+constexpr int STEP = 256;           // columns a warp takes at a time
+
+// The eight codes of the lane's elements (8 B bits at byte `at` B of the row), as loaded: at width 3 they may lie in two words, which
+// are only put together when they are used, so that the load does not have to be waited for before.
+template <int B>
+struct LaneCodes {
+    uint32_t lo, hi;
+    __device__ __forceinline__ void load(const uint8_t *row, int at)
+    {
+        hi = 0u;
+        if (B == 4) lo = __ldg(reinterpret_cast<const uint32_t *>(row) + at);
+        else if (B == 2) lo = __ldg(reinterpret_cast<const uint16_t *>(row) + at);
+        else if (B == 1) lo = __ldg(row + at);
+        else {
+            // the row is padded to 16 bytes, and the second word is only asked for where the bits reach into it
+            const uint32_t *w = reinterpret_cast<const uint32_t *>(row) + (3 * at >> 2);
+            lo = __ldg(w);
+            if ((3 * at & 3) > 1) hi = __ldg(w + 1);
+        }
+    }
+    __device__ __forceinline__ uint32_t get(int at) const { return B == 3 ? __funnelshift_r(lo, hi, 8 * (3 * at & 3)) : lo; }
+};
+
+// How a lane's eight values leave: one aligned 16-byte store; or, for rows that are not 16-byte aligned, through the warp's stretch of
+// shared memory, so that the stores are whole words next to one another; or one by one.
+enum Mode { STORE_VEC, STORE_STAGED, STORE_SINGLE, MATVEC };
+
+template <int MODE>
+__device__ __forceinline__ void store8(uint16_t *dst, int j0, int cols, const uint32_t (&h)[4], uint32_t *stage)
+{
+    if (MODE == STORE_VEC && j0 + 8 <= cols) {
+        *reinterpret_cast<uint4 *>(dst + j0) = make_uint4(h[0], h[1], h[2], h[3]);
+        return;
+    }
+    if (MODE != STORE_STAGED) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (j0 + u < cols) dst[j0 + u] = (uint16_t)((u & 1) ? (h[u >> 1] >> 16) : (h[u >> 1] & 0xffffu));
+        return;
+    }
+    const int lane = threadIdx.x & 31;
+    const uint16_t *s16 = reinterpret_cast<const uint16_t *>(stage);
+    const int base = j0 - lane * 8, n = min(STEP, cols - base);            // the warp's first element, and how many
+    *reinterpret_cast<uint4 *>(stage + lane * 4) = make_uint4(h[0], h[1], h[2], h[3]);
+    __syncwarp();
+    const int odd = (int)((reinterpret_cast<uintptr_t>(dst + base) >> 1) & 1u);        // elements before the first whole word
+    if (odd && lane == 0) dst[base] = s16[0];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int e = odd + 2 * (u * 32 + lane);
+        if (e + 1 < n) *reinterpret_cast<uint32_t *>(dst + base + e) = (uint32_t)s16[e] | ((uint32_t)s16[e + 1] << 16);
+        else if (e < n) dst[base + e] = s16[e];
+    }
+    __syncwarp();
+}
+
+// Where the vector's entry of column j sits: inside a block of 256 columns the first quads of all 32 lanes come first, then the second
+// quads, so that a lane's eight are two 16-byte loads that are contiguous across the warp.
 __device__ __forceinline__ int vec_slot(int j)
 {
     const int in = j & (STEP - 1), lane = in >> 3, u = in & 7;
     return (j & ~(STEP - 1)) + (u >> 2) * 128 + lane * 4 + (u & 3);
 }
 
-constexpr int AHEAD = 4;            // steps whose words are fetched together; two such batches are in flight
-
-// The 8 codes of this lane in a step of B-bit codes, cut out of the step's 8B words (lane l < 8B holds
-// word l in `w`), as one word (code u in bits [u*B, (u+1)*B)).
-template <int B>
-__device__ __forceinline__ uint32_t lane_codes(uint32_t w, int lane)
+// Steps [s0, s1) of one row; MATVEC: returns the lane's sum.
+template <int B, int MODE>
+__device__ __forceinline__ float unpack_row(const UnpackArgs &a, const uint8_t *words, uint16_t *dst, int s0, int s1, const float *vec, uint32_t book,
+                                            uint32_t *stage)
 {
-    const int bit = 8 * B * lane;
-    const uint32_t lo = __shfl_sync(0xffffffffu, w, bit >> 5);
-    const uint32_t hi = __shfl_sync(0xffffffffu, w, (bit >> 5) + 1);
-    const uint32_t v = __funnelshift_r(lo, hi, bit & 31);
-    return B == 4 ? v : (v & ((1u << (8 * B)) - 1u));
-}
-
-template <int B, bool MATVEC>
-__device__ __forceinline__ void unpack_row(const UnpackArgs &a, const float *vec, float *book, const uint32_t *words,
-                                           int stride, int64_t src_row, int lane)
-{
-    // the row's codebook, as binary32, in the warp's 16 words of shared memory
-    if (lane < 16) book[lane] = lane < a.kmax ? __half2float(__ushort_as_half(a.lut[src_row * a.kmax + lane])) : 0.0f;
-    __syncwarp();
-    const int steps = (a.cols + STEP - 1) / STEP;
+    constexpr int AHEAD = 4;                // steps whose codes are in flight
+    const int lane = threadIdx.x & 31, last = (a.cols - 1) / 8;      // the row's last group of eight
+    // two batches take turns: the next one is requested as a whole before the current one is worked on (one step at a time, a
+    // load shares its scoreboard with later ones and is waited for with them)
+    LaneCodes<B> codes[AHEAD], next[AHEAD];
     float acc = 0.0f;
-    // the words of the next AHEAD steps are requested before the current ones are worked on
-    uint32_t wv[AHEAD], wn[AHEAD];
 #pragma unroll
-    for (int q = 0; q < AHEAD; ++q) {
-        const int w0 = q * 8 * B + lane;                       // lanes 0 .. 8B-1 fetch a step's words
-        wv[q] = (lane < 8 * B && w0 < stride) ? __ldg(words + w0) : 0u;
-    }
-    for (int t0 = 0; t0 < steps; t0 += AHEAD) {
+    for (int u = 0; u < AHEAD; ++u) codes[u].load(words, min((s0 + u) * 32 + lane, last));
+    for (int t0 = s0; t0 < s1; t0 += AHEAD) {
 #pragma unroll
-        for (int q = 0; q < AHEAD; ++q) {
-            const int w0 = (t0 + AHEAD + q) * 8 * B + lane;
-            wn[q] = (lane < 8 * B && w0 < stride) ? __ldg(words + w0) : 0u;
-        }
+        for (int u = 0; u < AHEAD; ++u) next[u].load(words, min((t0 + AHEAD + u) * 32 + lane, last));
 #pragma unroll
-        for (int q = 0; q < AHEAD; ++q) {
-            const int t = t0 + q;
-            if (t >= steps) break;
-            const uint32_t codes = lane_codes<B>(wv[q], lane);
-            const int j0 = t * STEP + lane * 8;
-            // the step's 256 vector entries are stored as two runs of quads (see vec_slot): both loads are conflict-free;
-            // a dequantiser without a scaling vector has nothing to multiply by and skips them
-            const bool use_vec = MATVEC || a.s != nullptr;
-            float4 va = make_float4(1.f, 1.f, 1.f, 1.f), vb = va;
-            if (use_vec) {
-                va = *reinterpret_cast<const float4 *>(vec + t * STEP + lane * 4);
-                vb = *reinterpret_cast<const float4 *>(vec + t * STEP + 128 + lane * 4);
-            }
-            const float v[8] = {va.x, va.y, va.z, va.w, vb.x, vb.y, vb.z, vb.w};
-            float r[8];
+        for (int u = 0; u < AHEAD; ++u) {
+            const int t = t0 + u;
+            if (t < s1) {
+                const uint32_t c = codes[u].get(min(t * 32 + lane, last));
+                float r[8];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const float e = book[(codes >> (u * B)) & ((1u << B) - 1u)];
-                if (MATVEC) acc = fmaf(e, v[u], acc);
-                else r[u] = use_vec ? __fmul_rn(e, v[u]) : e;
-            }
-            if (!MATVEC) {
-                uint16_t *dst = a.out + src_row * a.ld + j0;
-                if (a.out_vec && j0 + 8 <= a.cols) {
-                    uint32_t h[4];
+                for (int e = 0; e < 8; ++e) r[e] = lookup<B>(book, e * B >= 2 ? c >> (e * B - 2) : c << (2 - e * B));
+                if (MODE == MATVEC || a.s) {
+                    const float4 va = *reinterpret_cast<const float4 *>(vec + t * STEP + lane * 4), vb = *reinterpret_cast<const float4 *>(vec + t * STEP + 128 + lane * 4);
+                    const float v[8] = {va.x, va.y, va.z, va.w, vb.x, vb.y, vb.z, vb.w};
 #pragma unroll
-                    for (int u = 0; u < 4; ++u)
-                        h[u] = (uint32_t)__half_as_ushort(__float2half_rn(r[2 * u])) |
-                               ((uint32_t)__half_as_ushort(__float2half_rn(r[2 * u + 1])) << 16);
-                    *reinterpret_cast<uint4 *>(dst) = make_uint4(h[0], h[1], h[2], h[3]);
-                } else {
+                    for (int e = 0; e < 8; ++e) {
+                        if (MODE == MATVEC) acc = fmaf(r[e], v[e], acc);
+                        else r[e] = __fmul_rn(r[e], v[e]);
+                    }
+                }
+                if constexpr (MODE == MATVEC) continue;
+                else {
+                uint32_t h[4];
 #pragma unroll
-                    for (int u = 0; u < 8; ++u)
-                        if (j0 + u < a.cols) dst[u] = __half_as_ushort(__float2half_rn(r[u]));
+                for (int e = 0; e < 4; ++e) {
+                    const __half2 v = __floats2half2_rn(r[2 * e], r[2 * e + 1]);
+                    h[e] = *reinterpret_cast<const uint32_t *>(&v);
+                }
+                const int j0 = t * STEP + lane * 8;
+                if (MODE == STORE_STAGED || j0 < a.cols) store8<MODE>(dst, j0, a.cols, h, stage);
                 }
             }
         }
 #pragma unroll
-        for (int q = 0; q < AHEAD; ++q) wv[q] = wn[q];
+        for (int u = 0; u < AHEAD; ++u) codes[u] = next[u];
     }
-    if (MATVEC) {
-#pragma unroll
-        for (int off = 16; off; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-        if (lane == 0) a.y[src_row] = acc;
-    }
+    return acc;
 }
 
-template <bool MATVEC>
-__global__ void __launch_bounds__(UT) skim_unpack_kernel(UnpackArgs a)
+// Packed rows are dealt round-robin to the blocks, so that every SM gets the same number (within one); `parts` warps share a
+// row, each with a stretch of its steps (the mat-vec then adds their sums in order).
+template <int MODE>
+__global__ void __launch_bounds__(UT) skim_unpack_kernel(UnpackArgs a, int steps, int parts)
 {
-    extern __shared__ __align__(16) float vec[];          // [cols rounded up to STEP], zero beyond cols
-    __shared__ float books[UW][16];
-    const int padded = (MATVEC || a.s) ? (a.cols + STEP - 1) / STEP * STEP : 0;
-    for (int j = threadIdx.x; j < padded; j += UT) {
-        float v = 0.0f;
-        if (j < a.cols) {
-            v = a.s ? a.s[j] : 1.0f;
-            if (MATVEC) {
-                const float xj = __half2float(__ushort_as_half(a.x[j]));
-                v = a.s ? __fmul_rn(xj, v) : xj;
+    extern __shared__ __align__(16) float vec[];          // [steps][STEP] (scaled, or the mat-vec), then (STORE_STAGED) [UW][STEP / 2] words
+    __shared__ __align__(128) float books[UW][16];
+    __shared__ float sums[UW];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const bool use_vec = MODE == MATVEC || a.s;
+    uint32_t *stage = reinterpret_cast<uint32_t *>(vec + (use_vec ? steps * STEP : 0)) + (MODE == STORE_STAGED ? warp * (STEP / 2) : 0);
+    const Groups g(a);
+    const int part = warp % parts, hop = UW / parts * (int)gridDim.x;
+    const int s0 = steps * part / parts, s1 = steps * (part + 1) / parts;
+    int p = (int)blockIdx.x + warp / parts * (int)gridDim.x;
+    int src = p < g.placed ? __ldg(a.row_order + p) : 0;
+    if (!SKIM_IDX(src, a.rows, nullptr)) src = 0;
+    uint16_t entry = p < g.placed ? __ldg(a.lut + (int64_t)src * a.kmax + min(lane, a.kmax - 1)) : (uint16_t)0;
+    if (use_vec) {
+        for (int j = tid * 4; j < steps * STEP; j += UT * 4) {
+            float v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                v[u] = 0.0f;
+                if (j + u < a.cols) {
+                    v[u] = a.s ? a.s[j + u] : 1.0f;
+                    if (MODE == MATVEC) {
+                        const float x = __half2float(__ushort_as_half(a.x[j + u]));
+                        v[u] = a.s ? __fmul_rn(x, v[u]) : x;
+                    }
+                }
+            }
+            *reinterpret_cast<float4 *>(vec + vec_slot(j)) = make_float4(v[0], v[1], v[2], v[3]);
+        }
+        __syncthreads();
+    }
+    // every warp goes through the same number of rounds: warps that share a row meet at a barrier
+    for (int first_p = (int)blockIdx.x; first_p < g.placed; first_p += hop, p += hop) {
+        float acc = 0.0f;
+        if (p < g.placed) {
+            __syncwarp();
+            if (lane < 16) books[warp][lane] = __half2float(__ushort_as_half(entry));
+            __syncwarp();
+            const uint32_t book = codebook_address(books[warp]);
+            const int nsrc = p + hop < g.placed ? __ldg(a.row_order + p + hop) : 0;      // the next row's, one row early
+            int u = 0, first = g.start[0];
+            long long word = g.word[0];
+#pragma unroll
+            for (int v = 1; v < SKIM_MAX_NBITS; ++v)
+                if (v < a.nb && p >= g.start[v]) { u = v; first = g.start[v]; word = g.word[v]; }
+            const int width = a.bmin + u;
+            const uint8_t *words = reinterpret_cast<const uint8_t *>(a.packed + word + (int64_t)(p - first) * skim_row_stride_words(a.cols, width));
+            uint16_t *dst = a.out + (int64_t)src * a.ld;
+            switch (width) {
+            case 1: acc = unpack_row<1, MODE>(a, words, dst, s0, s1, vec, book, stage); break;
+            case 2: acc = unpack_row<2, MODE>(a, words, dst, s0, s1, vec, book, stage); break;
+            case 3: acc = unpack_row<3, MODE>(a, words, dst, s0, s1, vec, book, stage); break;
+            default: acc = unpack_row<4, MODE>(a, words, dst, s0, s1, vec, book, stage); break;
+            }
+            codebook_address(books[warp]);
+            if (MODE == MATVEC) {
+#pragma unroll
+                for (int off = 16; off; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+                if (parts == 1 && lane == 0) a.y[src] = acc;
+            }
+            if (MODE == MATVEC && parts > 1) {
+                if (lane == 0) sums[warp] = acc;
+            }
+            if (MODE != MATVEC || parts == 1) {
+                src = SKIM_IDX(nsrc, a.rows, nullptr) ? nsrc : 0;
+                entry = __ldg(a.lut + (int64_t)src * a.kmax + min(lane, a.kmax - 1));
             }
         }
-        vec[vec_slot(j)] = v;
-    }
-    __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // rows are dealt round-robin to the blocks, so that every SM gets the same number (within one)
-    for (int64_t p = blockIdx.x + (int64_t)gridDim.x * warp; p < a.rows; p += (int64_t)gridDim.x * UW) {
-        int width = 0, stride = 0;
-        int64_t src_row = 0;
-        const uint32_t *words = nullptr;
-        if (!locate_row(a, p, width, src_row, words, stride)) continue;
-        __syncwarp();
-        switch (width) {
-        case 1: unpack_row<1, MATVEC>(a, vec, books[warp], words, stride, src_row, lane); break;
-        case 2: unpack_row<2, MATVEC>(a, vec, books[warp], words, stride, src_row, lane); break;
-        case 3: unpack_row<3, MATVEC>(a, vec, books[warp], words, stride, src_row, lane); break;
-        default: unpack_row<4, MATVEC>(a, vec, books[warp], words, stride, src_row, lane); break;
+        if (MODE == MATVEC && parts > 1) {
+            __syncthreads();
+            if (p < g.placed) {
+                if (part == 0 && lane == 0) {
+                    for (int q = 1; q < parts; ++q) acc += sums[warp + q];
+                    a.y[src] = acc;
+                }
+                src = p + hop < g.placed ? __ldg(a.row_order + p + hop) : 0;
+                if (!SKIM_IDX(src, a.rows, nullptr)) src = 0;
+                entry = __ldg(a.lut + (int64_t)src * a.kmax + min(lane, a.kmax - 1));
+            }
+            __syncthreads();
         }
     }
 }
 
-template <bool MATVEC>
-int launch_unpack(skim_ctx *ctx, const UnpackArgs &a)
+// with few rows several warps share one
+int unpack_parts(const skim_ctx *ctx, int64_t rows, int steps)
 {
-    const size_t smem = (size_t)((a.cols + STEP - 1) / STEP * STEP) * sizeof(float);
-    if (smem > (size_t)ctx->max_smem_optin) return SKIM_ERR_SHAPE;
+    int parts = 1;
+    while (parts < UW && parts * 2 <= steps && rows * parts * 2 <= (int64_t)ctx->sm_count * UW) parts *= 2;
+    return parts;
+}
+
+int launch_unpack(skim_ctx *ctx, void (*kernel)(UnpackArgs, int, int), const UnpackArgs &a, int steps, size_t smem)
+{
     // set on every launch: a host-side call of microseconds, and no state shared between contexts
-    SKIM_CUDA_OK(cudaFuncSetAttribute(skim_unpack_kernel<MATVEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    const unsigned blocks = (unsigned)(a.rows < ctx->sm_count ? a.rows : ctx->sm_count);   // one block per SM, rows dealt round-robin
-    skim_unpack_kernel<MATVEC><<<blocks, UT, smem, ctx->stream>>>(a);
+    SKIM_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const unsigned blocks = (unsigned)(a.rows < ctx->sm_count ? a.rows : ctx->sm_count);      // one block per SM
+    kernel<<<blocks, UT, smem, ctx->stream>>>(a, steps, unpack_parts(ctx, a.rows, steps));
     SKIM_CUDA_OK(cudaGetLastError());
     ctx->launches += 1;
     return SKIM_OK;
 }
+
+constexpr size_t UNPACK_STATIC_SMEM = UW * 17 * sizeof(float);
 
 }  // namespace
 
@@ -206,7 +307,13 @@ int skim_launch_dequantize(skim_ctx *ctx, const uint32_t *packed, const int32_t 
     a.s = s; a.x = nullptr; a.rows = rows; a.cols = (int)cols; a.nb = bs.n_bits; a.bmin = bs.b_min; a.kmax = 1 << bs.b_max;
     a.out = out; a.ld = ld_out; a.y = nullptr;
     a.out_vec = ((reinterpret_cast<uintptr_t>(out) & 15u) == 0 && (ld_out % 8) == 0) ? 1 : 0;
-    return launch_unpack<false>(ctx, a);
+    const int steps = (int)((cols + STEP - 1) / STEP);
+    const size_t vec = s ? (size_t)steps * STEP * sizeof(float) : 0, stage = (size_t)UW * STEP * 2;
+    if (vec + UNPACK_STATIC_SMEM > (size_t)ctx->max_smem_optin) return SKIM_ERR_SHAPE;
+    if (a.out_vec) return launch_unpack(ctx, skim_unpack_kernel<STORE_VEC>, a, steps, vec);
+    // very long unaligned rows leave no room for the staging of the stores: single 16-bit stores then
+    if (vec + stage + UNPACK_STATIC_SMEM <= (size_t)ctx->max_smem_optin) return launch_unpack(ctx, skim_unpack_kernel<STORE_STAGED>, a, steps, vec + stage);
+    return launch_unpack(ctx, skim_unpack_kernel<STORE_SINGLE>, a, steps, vec);
 }
 
 int skim_launch_matvec(skim_ctx *ctx, const uint32_t *packed, const int32_t *row_order, const int64_t *group_info,
@@ -218,5 +325,8 @@ int skim_launch_matvec(skim_ctx *ctx, const uint32_t *packed, const int32_t *row
     a.packed = packed; a.row_order = row_order; a.group_info = (const long long *)group_info; a.lut = lut;
     a.s = s; a.x = x; a.rows = rows; a.cols = (int)cols; a.nb = bs.n_bits; a.bmin = bs.b_min; a.kmax = 1 << bs.b_max;
     a.out = nullptr; a.ld = 0; a.out_vec = 0; a.y = y;
-    return launch_unpack<true>(ctx, a);
+    const int steps = (int)((cols + STEP - 1) / STEP);
+    const size_t vec = (size_t)steps * STEP * sizeof(float);
+    if (vec + UNPACK_STATIC_SMEM > (size_t)ctx->max_smem_optin) return SKIM_ERR_SHAPE;
+    return launch_unpack(ctx, skim_unpack_kernel<MATVEC>, a, steps, vec);
 }

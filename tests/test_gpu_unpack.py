@@ -116,3 +116,33 @@ def test_unpack_argument_errors(ctx, oracle, skimlib):
     with pytest.raises(skimlib.SkimError) as e:
         ctx.matvec(q, 100000, [1, 2, 3, 4], torch.zeros(100000, dtype=torch.float16, device="cuda"))
     assert e.value.code == -2
+
+
+@pytest.mark.parametrize("rows,cols,pad", [(3, 2049, 0), (5, 255, 1), (2, 8191, 3), (160, 1025, 0), (7, 4104, 8)])
+def test_rows_shared_by_warps_and_unaligned_outputs(ctx, oracle, rows, cols, pad):
+    """Few rows (several warps share one) and output rows at odd addresses (stores staged in shared memory): bit-exact
+    dequantised values with nothing written beside them, and the mat-vec against the same weights."""
+    w, g = inputs.make_rows(rows, cols, 70 + cols)
+    bits = (np.arange(rows) % 4 + 1).astype(np.uint8)
+    res = oracle.cluster_rows(w, g, [1, 2, 3, 4], 5, want_codes=False)
+    c32 = res["centroids"].astype(np.float32)
+    s = torch.from_numpy(inputs.make_scale(cols, 3)).cuda()
+    ctx.reserve(rows, cols)
+    ctx.apply_scale(None)
+    q = ctx.quantize(torch.from_numpy(w).cuda(), torch.from_numpy(bits).cuda(), torch.from_numpy(c32).cuda(), [1, 2, 3, 4])
+    want = ctx.dequantize(q, cols, [1, 2, 3, 4], s=s, out=torch.empty((rows, (cols + 7) // 8 * 8), dtype=torch.float16, device="cuda"))[:, :cols]
+    lut = q["lut"].view(torch.float16).float()
+    em = oracle.emit(w, bits, c32, [1, 2, 3, 4])
+    buf = torch.full((rows, cols + pad), 7.0, dtype=torch.float16, device="cuda")
+    ctx.dequantize(q, cols, [1, 2, 3, 4], s=s, out=buf)
+    assert ctx.get_status() == 0
+    assert torch.equal(buf[:, :cols].view(torch.int16), want.view(torch.int16)) and bool((buf[:, cols:] == 7.0).all())
+    np.testing.assert_array_equal(q["lut"].cpu().numpy().view(np.uint16), em["lut"])
+    # every value is a codebook entry times alpha, the nearest one allowed by the packer's rule
+    near = (want.float()[:, :, None] - (lut[:, None, :] * s[None, :, None]).half().float()).abs().amin(dim=2)
+    assert float(near.max()) == 0.0
+    x = torch.ones(cols, dtype=torch.float16, device="cuda")
+    y = ctx.matvec(q, cols, [1, 2, 3, 4], x, s=s)
+    ref = torch.stack([(lut[i][(lut[i][None, :] * s[:, None]).half().float().sub(want[i].float()[:, None]).abs().argmin(dim=1)].double() * s.double()).sum() for i in range(rows)])
+    mag = (want.double().abs()).sum(dim=1)
+    assert bool(((y.double() - ref).abs() <= 1e-3 * mag).all())
