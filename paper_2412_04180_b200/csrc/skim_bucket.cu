@@ -2,7 +2,7 @@
 // Section 3.2, diagonal form).  One block per row: every element's bucket is a monotone function of its value, chosen so that a bucket holds about one
 // element of a bell-shaped row; one counting pass orders the row up to the order inside the buckets.
 //
-//   load     values (binary32 products where a scale vector is installed, else the binary16 weights) and the sum of |x|,
+//   load     values (binary32 products where a scale vector is installed, else the binary16 weights as binary32) and the sum of |x|,
 //            which sets the buckets' scale.
 //   count    one shared-memory atomic per element; its return value is the element's slot inside its bucket.
 //   scatter  bucket base + slot: value and importance (read from global memory here) go to their bucket's place.
@@ -10,7 +10,7 @@
 //            kernel compares every element with its boundary, so its order does not matter).
 //   then     one pass over the row (skim_cluster_phases.cuh) writes the row record -- group records with
 //            prefix sums, group index, segment table -- to global memory, from which the Lloyd kernel
-//            (skim_lloyd.cu) iterates with one warp per row.
+//            (skim_lloyd.cu) iterates with one warp per row.  Unscaled rows write the compact record.
 //
 // Buckets: v = 1 + |x| / s with s half a standard deviation (from the mean of |x|).  The bits of v grow with |x|: the
 // first three octaves, v in [1, 8), i.e. |x| up to 3.5 deviations, have N/8 buckets each on either side of zero, the next
@@ -81,7 +81,9 @@ __device__ __forceinline__ void sort_bucket(float *keys, float *gs, int lo, int 
     }
 }
 
-template <int THREADS, int ITEMS>
+// SCALED: values times a.rscale, full records; else compact records (its own instance: the choice at run time cost the scaled rows
+// 8-15 %).
+template <int THREADS, int ITEMS, bool SCALED>
 __global__ void __launch_bounds__(THREADS, 1024 / THREADS) skim_sort_bucket_kernel(ClusterArgs a)
 {
     using Bk = Buckets<THREADS>;
@@ -121,7 +123,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) skim_sort_bucket_kern
         for (int i = 0; i < ITEMS; ++i) {
             if ((h[i] & 0x7c00u) == 0x7c00u) bad |= 1u;
             x[i] = __half2float(__ushort_as_half(h[i]));
-            x[i] = __fmul_rn(x[i], (i * THREADS + tid < m) ? a.rscale[i * THREADS + tid] : 1.0f);
+            if constexpr (SCALED) x[i] = __fmul_rn(x[i], (i * THREADS + tid < m) ? a.rscale[i * THREADS + tid] : 1.0f);
             x[i] += 0.0f;                                               // -0 and +0 are one value
             sum += fabsf(x[i]);
         }
@@ -260,7 +262,8 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) skim_sort_bucket_kern
         __syncthreads();
         nd = ps.misc[0];
     }
-    write_row_record<float, THREADS, false>(a, src, ps, nd, (int)blockIdx.x);
+    if constexpr (SCALED) write_row_record<float, THREADS, false>(a, src, ps, nd, (int)blockIdx.x);
+    else write_row_record_half<float, THREADS>(a, src, ps, nd, (int)blockIdx.x);
     if (nd <= 16) {
         collect_distinct<float, THREADS>(src, m, nd, ps);
         write_distinct_values(a, nd, ps.dvals, (int)blockIdx.x);
@@ -270,15 +273,17 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) skim_sort_bucket_kern
 struct BucketVariant {
     int cap;
     int threads;
-    void (*kernel)(ClusterArgs);
+    void (*scaled)(ClusterArgs);
+    void (*unscaled)(ClusterArgs);      // row lengths that the launcher of skim_cluster.cu gives to skim_cluster16.cu have none
 };
 
-#define SKIM_BV(T, I) {T * I, T, skim_sort_bucket_kernel<T, I>}
+#define SKIM_BV(T, I) {T * I, T, skim_sort_bucket_kernel<T, I, true>, nullptr}
+#define SKIM_BV2(T, I) {T * I, T, skim_sort_bucket_kernel<T, I, true>, skim_sort_bucket_kernel<T, I, false>}
 
 // An SM holds 1024 threads; many small blocks wait for their own barriers only (5600 columns: 256 x 22 takes 0.174 ms where
 // 512 x 16 takes 0.217 ms, 4096: 256 x 16 0.132 ms, 512 x 8 0.147 ms), as far as registers hold the row.
 const BucketVariant kVariantsBucket[] = {
-    SKIM_BV(128, 4), SKIM_BV(128, 8), SKIM_BV(128, 16), SKIM_BV(256, 12), SKIM_BV(256, 16), SKIM_BV(256, 22), SKIM_BV(512, 16), SKIM_BV(512, 22), SKIM_BV(1024, 16), SKIM_BV(1024, 22),
+    SKIM_BV2(128, 4), SKIM_BV2(128, 8), SKIM_BV2(128, 16), SKIM_BV2(256, 12), SKIM_BV2(256, 16), SKIM_BV(256, 22), SKIM_BV(512, 16), SKIM_BV(512, 22), SKIM_BV(1024, 16), SKIM_BV(1024, 22),
 };
 
 }  // namespace
@@ -287,11 +292,13 @@ int skim_launch_sort_bucket(skim_ctx *ctx, const ClusterArgs &args, int64_t rows
 {
     for (const BucketVariant &v : kVariantsBucket) {
         if (v.cap < args.m) continue;
+        void (*kernel)(ClusterArgs) = args.rscale ? v.scaled : v.unscaled;
+        if (!kernel) return SKIM_ERR_SHAPE;
         const BucketLayout L = bucket_layout(args.m, v.threads);
         if (L.total > (size_t)ctx->max_smem_optin) return SKIM_ERR_SHAPE;
         // set on every launch: a host-side call of microseconds, and no state shared between contexts
-        SKIM_CUDA_OK(cudaFuncSetAttribute(v.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total));
-        v.kernel<<<(unsigned)rows, v.threads, L.total, ctx->stream>>>(args);
+        SKIM_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total));
+        kernel<<<(unsigned)rows, v.threads, L.total, ctx->stream>>>(args);
         SKIM_CUDA_OK(cudaGetLastError());
         ctx->launches += 1;
         return SKIM_OK;

@@ -373,7 +373,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) skim_sort16_kernel(Cl
         __syncthreads();
         nd = ps.misc[0];
     }
-    if constexpr (HALF_RECORD) write_row_record_half<THREADS>(a, src, ps, nd, (int)blockIdx.x);
+    if constexpr (HALF_RECORD) write_row_record_half<uint16_t, THREADS>(a, src, ps, nd, (int)blockIdx.x);
     else write_row_record<uint16_t, THREADS, false>(a, src, ps, nd, (int)blockIdx.x);
     if (nd <= 16) {
         collect_distinct<uint16_t, THREADS>(src, m, nd, ps);
@@ -388,11 +388,12 @@ struct Variant16 {
 };
 
 #define SKIM_V16(T, V) {T * V * 8, T, {skim_sort16_kernel<false, T, V>, skim_sort16_kernel<true, T, V>}}
+#define SKIM_V16F(T, V) {T * V * 8, T, {skim_sort16_kernel<false, T, V>, nullptr}}      // short rows with compact records: skim_bucket.cu
 
 // An SM holds 1024 threads; small blocks wait for their own barriers only (4096 columns: 256 threads of 16 elements take
 // 0.131 ms for 4096 rows, 512 of 8 took 0.153 ms).
 const Variant16 kVariants16[] = {
-    SKIM_V16(128, 1), SKIM_V16(128, 2), SKIM_V16(256, 2), SKIM_V16(256, 3), SKIM_V16(512, 2), SKIM_V16(512, 3), SKIM_V16(1024, 2),
+    SKIM_V16F(128, 1), SKIM_V16F(128, 2), SKIM_V16(256, 2), SKIM_V16(256, 3), SKIM_V16(512, 2), SKIM_V16(512, 3), SKIM_V16(1024, 2),
     SKIM_V16(1024, 3),
 };
 
@@ -405,6 +406,7 @@ int skim_launch_sort16(skim_ctx *ctx, const ClusterArgs &args, int64_t rows)
         const Layout16 L = layout16(args.m, v.threads);
         if (L.total > (size_t)ctx->max_smem_optin) continue;
         void (*kernel)(ClusterArgs) = v.kernel[args.rec_half ? 1 : 0];
+        if (!kernel) return SKIM_ERR_SHAPE;
         // set on every launch: a host-side call of microseconds, and no state shared between contexts
         SKIM_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total));
         kernel<<<(unsigned)rows, v.threads, L.total, ctx->stream>>>(args);

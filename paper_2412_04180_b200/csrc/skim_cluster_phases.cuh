@@ -94,6 +94,7 @@ struct ClusterArgs {
     long long rec_stride;     // bytes between row records
     int64_t row0;             // first row of the current chunk
     int rec_half;             // compact records (no scale installed: every value is a binary16 number)
+    int unordered;            // compact records: elements inside a group are in no order (bucket kernel)
     int full_order;           // the reader wants order inside the groups too (exact kernel)
     int chunk_rows;           // rows of the current chunk
     int *sort_list;           // rows (indexes inside the chunk) the bucket kernel left to the radix kernel, and how many; the
@@ -367,11 +368,11 @@ __device__ __forceinline__ void st_sector(void *p, unsigned long long a, unsigne
     asm volatile("st.global.v4.b64 [%0], {%1, %2, %3, %4};" ::"l"(p), "l"(a), "l"(b), "l"(c), "l"(d) : "memory");
 }
 
-// The compact row record (see SKIM_GROUP_BYTES_HALF) from a row sorted by 16-bit keys; the counterpart of
+// The compact row record (see SKIM_GROUP_BYTES_HALF) of an unscaled row; the counterpart of
 // write_row_record for unscaled rows.  One pass, one group per lane; only the sums of g and g*x are
 // scanned, the g*x^2 terms are added up per warp and meet in the row total.  nd: the distinct-value count
 // (any number above 16 stands for "more than 16").  Call with all threads.
-template <int THREADS, typename Src>
+template <typename KeyT, int THREADS, typename Src>
 __device__ __forceinline__ void write_row_record_half(const ClusterArgs &a, const Src &src, PhaseSmem &ps, int nd, int local_row)
 {
     constexpr int NW = THREADS / 32;
@@ -389,21 +390,24 @@ __device__ __forceinline__ void write_row_record_half(const ClusterArgs &a, cons
         float first = 0.0f;
         if (q < R.ngrp) {
             const int e = q << 3;
-            uint16_t ks[8];
+            KeyT ks[8];
             float gs[8];
             const unsigned gbits = src.group(e, m, ks, gs);
             uint32_t hb[8];
             double xd[8];
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
-                const uint16_t k = ks[u];
-                const uint16_t h = (e + u < m) ? ((k & 0x8000u) ? (uint16_t)(k & 0x7fffu) : (uint16_t)~k) : (uint16_t)SKIM_PAD_HALF;
+                uint16_t h;
+                if constexpr (sizeof(KeyT) == 2) h = (ks[u] & 0x8000u) ? (uint16_t)(ks[u] & 0x7fffu) : (uint16_t)~ks[u];
+                else h = __half_as_ushort(__float2half_rn(KeyOps<KeyT>::to_float(ks[u])));         // exact: no scale installed
+                if (e + u >= m) h = (uint16_t)SKIM_PAD_HALF;
                 hb[u] = h;
                 xd[u] = (double)__half2float(__ushort_as_half(h));
             }
             xq0 = (unsigned long long)(hb[0] | (hb[1] << 16)) | ((unsigned long long)(hb[2] | (hb[3] << 16)) << 32);
             xq1 = (unsigned long long)(hb[4] | (hb[5] << 16)) | ((unsigned long long)(hb[6] | (hb[7] << 16)) << 32);
-            first = (float)xd[0];
+            // the smallest value: inside a group a row of the bucket kernel is in no order
+            first = sizeof(KeyT) == 2 ? (float)xd[0] : (float)fmin(fmin(fmin(xd[0], xd[1]), fmin(xd[2], xd[3])), fmin(fmin(xd[4], xd[5]), fmin(xd[6], xd[7])));
             st_sector(rec + R.groups + (size_t)q * SKIM_GROUP_BYTES_HALF + 32, gs);
             double t0[8], t1[8], t2[8];
 #pragma unroll
@@ -485,7 +489,7 @@ __device__ __forceinline__ void write_distinct_values(const ClusterArgs &a, int 
 
 }  // namespace skimk
 
-// Bucket sort kernel (skim_bucket.cu), a scale vector installed: writes the row records of a chunk, or puts rows on args.sort_list.
+// Bucket sort kernel (skim_bucket.cu): writes the row records of a chunk, or puts rows on args.sort_list.
 int skim_launch_sort_bucket(skim_ctx *ctx, const skimk::ClusterArgs &args, int64_t rows);
 // fp16-key sort kernel (skim_cluster16.cu): writes the row records of a chunk; no scale vector installed.
 int skim_launch_sort16(skim_ctx *ctx, const skimk::ClusterArgs &args, int64_t rows);

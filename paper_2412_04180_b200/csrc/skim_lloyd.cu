@@ -41,12 +41,26 @@ __device__ __forceinline__ void ld_sector(const unsigned char *p, float4 &a, flo
                  : "l"(p));
 }
 
+// The n-th smallest of eight values (n from 0).
+__device__ __forceinline__ float nth_of_8(const float (&x)[8], int n)
+{
+    float v = x[0];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        int rank = 0;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) rank += (w < u ? x[w] <= x[u] : x[w] < x[u]) ? 1 : 0;
+        if (rank == n) v = x[u];
+    }
+    return v;
+}
+
 // One group record in registers.  HALF = false: the full record (three sectors: binary32 values | importances |
 // sums incl. g*x^2); HALF = true: the compact record of unscaled rows (two sectors: binary16 values
 // and the sums of g and g*x | importances).
-template <bool HALF> struct Group;
+template <bool HALF, bool UNORDERED> struct Group;
 
-template <> struct Group<false> {
+template <bool UNORDERED> struct Group<false, UNORDERED> {
     static constexpr int BYTES = SKIM_GROUP_BYTES;
     float4 xa, xb, ga, gb;
     double2 p;   // prefix sums of g and g*x at the group's first element
@@ -73,24 +87,17 @@ template <> struct Group<false> {
         float4 a, b;
         ld_sector(groups + (size_t)(idx >> 3) * BYTES, a, b);
         const float x[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-        float v = x[0];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            int rank = 0;
-#pragma unroll
-            for (int w = 0; w < 8; ++w) rank += (w < u ? x[w] <= x[u] : x[w] < x[u]) ? 1 : 0;
-            if (rank == (idx & 7)) v = x[u];
-        }
-        return v;
+        return nth_of_8(x, idx & 7);
     }
-    __device__ __forceinline__ void in_prefix(int, float t, bool (&in)[8]) const
+    // importances of the values <= t, zero for the others
+    __device__ __forceinline__ void masked(int, float t, float (&g)[8]) const
     {
-        in[0] = xa.x <= t; in[1] = xa.y <= t; in[2] = xa.z <= t; in[3] = xa.w <= t;
-        in[4] = xb.x <= t; in[5] = xb.y <= t; in[6] = xb.z <= t; in[7] = xb.w <= t;
+        g[0] = xa.x <= t ? ga.x : 0.0f; g[1] = xa.y <= t ? ga.y : 0.0f; g[2] = xa.z <= t ? ga.z : 0.0f; g[3] = xa.w <= t ? ga.w : 0.0f;
+        g[4] = xb.x <= t ? gb.x : 0.0f; g[5] = xb.y <= t ? gb.y : 0.0f; g[6] = xb.z <= t ? gb.z : 0.0f; g[7] = xb.w <= t ? gb.w : 0.0f;
     }
 };
 
-template <> struct Group<true> {
+template <bool UNORDERED> struct Group<true, UNORDERED> {
     static constexpr int BYTES = SKIM_GROUP_BYTES_HALF;
     uint32_t xh[4];      // 8 binary16 values
     float4 ga, gb;
@@ -122,15 +129,32 @@ template <> struct Group<true> {
             x[2 * u + 1] = (double)f.y;
         }
     }
-    // values ascend
-    __device__ __forceinline__ void in_prefix(int n, float, bool (&in)[8]) const
+    // importances of the n values <= t, zero for the others.  UNORDERED: by comparison; else the values ascend.
+    __device__ __forceinline__ void masked(int n, float t, float (&g)[8]) const
     {
+        g[0] = ga.x; g[1] = ga.y; g[2] = ga.z; g[3] = ga.w;
+        g[4] = gb.x; g[5] = gb.y; g[6] = gb.z; g[7] = gb.w;
+        if constexpr (UNORDERED) {
+            const __half2 th = __half2half2(__float2half_rd(t));
 #pragma unroll
-        for (int u = 0; u < 8; ++u) in[u] = u < n;
+            for (int u = 0; u < 4; ++u) {
+                const uint32_t k = __hle2_mask(*reinterpret_cast<const __half2 *>(&xh[u]), th);
+                g[2 * u] = __uint_as_float(__float_as_uint(g[2 * u]) & __byte_perm(k, 0u, 0x1010));
+                g[2 * u + 1] = __uint_as_float(__float_as_uint(g[2 * u + 1]) & __byte_perm(k, 0u, 0x3232));
+            }
+        } else {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) g[u] = u < n ? g[u] : 0.0f;
+        }
     }
     static __device__ __forceinline__ float value_at(const unsigned char *groups, int idx)
     {
-        return __half2float(__ushort_as_half(__ldg(reinterpret_cast<const unsigned short *>(groups + (size_t)(idx >> 3) * BYTES) + (idx & 7))));
+        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(groups + (size_t)(idx >> 3) * BYTES));
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+        float x[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) x[u] = __half2float(__ushort_as_half((uint16_t)((u & 1) ? (w[u >> 1] >> 16) : (w[u >> 1] & 0xffffu))));
+        return nth_of_8(x, idx & 7);
     }
 };
 
@@ -140,14 +164,13 @@ template <bool WANT_C, typename G>
 __device__ __forceinline__ void add_group(const G &grp, int n, float t, double &s0, double &s1, double &s2)
 {
     double xs[8];
-    bool in[8];
+    float gs[8];
     grp.values(xs);
-    grp.in_prefix(n, t, in);
-    const float gs[8] = {grp.ga.x, grp.ga.y, grp.ga.z, grp.ga.w, grp.gb.x, grp.gb.y, grp.gb.z, grp.gb.w};
+    grp.masked(n, t, gs);
     double t0[8], t1[8], t2[8];
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-        const double g = (double)(in[u] ? gs[u] : 0.0f), x = xs[u];   // padding values are finite, so 0 * x = 0
+        const double g = (double)gs[u], x = xs[u];   // padding values are finite, so 0 * x = 0
         t0[u] = g;
         t1[u] = g * x;
         if (WANT_C) t2[u] = t1[u] * x;
@@ -238,7 +261,7 @@ __device__ __forceinline__ double quotient(double s1, double s0)
 // window); loads that one group record, which gives the exact boundary position (values), the
 // prefix sums at the group start and the few elements in between.
 // On return sm.tfs[L] holds the boundary (largest binary32 value still assigned to centroid L).
-template <bool HALF>
+template <bool HALF, bool UNORDERED>
 __device__ __forceinline__ void lloyd_warp(const unsigned char *rec, const typename Window<HALF>::Entry *gi, const double2 *segs,
                                            int nd, const ClusterArgs &a, int64_t row, LloydSmem &sm)
 {
@@ -264,7 +287,7 @@ __device__ __forceinline__ void lloyd_warp(const unsigned char *rec, const typen
     if (degenerate) c = sm.dvals[min(j, nd - 1)];
     if (normal) {
         const int idx = (int)(((long long)(2 * j + 1) * m) / (2 * k));
-        if (SKIM_IDX(idx, m, a.status)) c = Group<HALF>::value_at(groups, idx);
+        if (SKIM_IDX(idx, m, a.status)) c = Group<HALF, UNORDERED>::value_at(groups, idx);
     }
 
     int Bprev = -1;
@@ -273,7 +296,7 @@ __device__ __forceinline__ void lloyd_warp(const unsigned char *rec, const typen
     int gprev = -1;                                   // group of the previous boundary position
     int gstep = 0;                                    // its last move: boundaries keep drifting the same way
     // The group of the last iteration stays in registers with its prefix sums: most boundaries are in it again.
-    Group<HALF> grp;
+    Group<HALF, UNORDERED> grp;
     int gloaded = -1;
     for (int it = 0;; ++it) {
         const float c_up = __shfl_down_sync(0xffffffffu, c, 1);
@@ -307,7 +330,7 @@ __device__ __forceinline__ void lloyd_warp(const unsigned char *rec, const typen
             gstep = gprev >= 0 ? grp_i - gprev : 0;
             gprev = grp_i;
             if (HALF || grp_i != gloaded) {          // (compact records: loading their two sectors always measured as fast)
-                grp.load(groups + (size_t)grp_i * Group<HALF>::BYTES);
+                grp.load(groups + (size_t)grp_i * Group<HALF, UNORDERED>::BYTES);
                 const double2 sb = segs[grp_i >> SKIM_SEG_SHIFT];       // sums of the earlier segments (shared memory)
                 grp.p.x += sb.x;
                 grp.p.y += sb.y;
@@ -434,7 +457,7 @@ __global__ void __launch_bounds__(CODES_T) skim_codes_kernel(ClusterArgs a, int 
 
 // Seven blocks of four rows per SM: an eighth would hold the kernel to 64 registers, which measured slower on every
 // shape (the full-record form spills there).
-template <bool HALF>
+template <bool HALF, bool UNORDERED>
 __global__ void __launch_bounds__(LLOYD_WARPS * 32, 7) skim_lloyd_kernel(ClusterArgs a, int rows_in_chunk)
 {
     __shared__ LloydSmem sm_all[LLOYD_WARPS];
@@ -475,7 +498,7 @@ __global__ void __launch_bounds__(LLOYD_WARPS * 32, 7) skim_lloyd_kernel(Cluster
         }
     }
     __syncwarp();
-    lloyd_warp<HALF>(rec, gi, segs, nd, a, row, sm);
+    lloyd_warp<HALF, UNORDERED>(rec, gi, segs, nd, a, row, sm);
     // the header has served its purpose: for the codes kernel the boundaries take its place
     if (a.codes) reinterpret_cast<float *>(const_cast<unsigned char *>(rec))[lane] = sm.tfs[lane];
 }
@@ -487,7 +510,7 @@ int skim_launch_lloyd(skim_ctx *ctx, const ClusterArgs &args, int64_t rows)
     const unsigned blocks = (unsigned)((rows + LLOYD_WARPS - 1) / LLOYD_WARPS);
     const size_t smem = (size_t)LLOYD_WARPS * lloyd_warp_bytes(args.m, args.rec_half != 0);
     // set on every launch: a host-side call of microseconds, and no state shared between contexts
-    void (*kernel)(ClusterArgs, int) = args.rec_half ? skim_lloyd_kernel<true> : skim_lloyd_kernel<false>;
+    void (*kernel)(ClusterArgs, int) = !args.rec_half ? skim_lloyd_kernel<false, true> : args.unordered ? skim_lloyd_kernel<true, true> : skim_lloyd_kernel<true, false>;
     SKIM_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     // an ordinary launch: blocks that move in beside the last sort blocks find those blocks' split of shared memory and L1,
     // with next to no L1 for the records (4096 x 11008: 0.489 instead of 0.44 ms for the whole path)

@@ -125,6 +125,21 @@ def test_llama_row_lengths_on_a_row_subset(ctx, oracle, cols, seed, sigma):
     assert exact > 0.98
 
 
+@pytest.mark.parametrize("cols", [129, 512, 513, 1025, 2048, 2049, 3072, 3584, 3585, 4097, 5632, 5633, 8193, 11265, 16385, 22528])
+@pytest.mark.parametrize("scaled", [False, True])
+def test_rows_spread_and_clumped_in_one_matrix(ctx, oracle, cols, scaled):
+    """Row lengths at the edges of the sort kernels' sizes; every other row is one that buckets of equal spacing cannot spread."""
+    w, g = inputs.make_rows(6, cols, 9000 + cols)
+    w[1] = np.random.default_rng(cols).choice(np.float16([-0.5, 0.125, 0.25, 1.0]), cols)      # four values
+    w[3] = (1.0 + np.arange(cols) % 64 / 1024).astype(np.float16)                             # a clump away from zero ...
+    w[3, :3] = -0.02
+    w[5, 1::2] = w[5, 0]                                                                      # half of a row equal
+    s = inputs.make_scale(cols, 23) if scaled else None
+    ora = oracle.cluster_rows(w, g, BITS, 8, s=s)
+    cent, err, codes = _gpu_cluster(ctx, w, g, BITS, 8, s=s)
+    check_cluster(ora, cent, err, codes, _values(w, s), BITS, label=f"cols={cols} scaled={scaled}")
+
+
 def test_scaled_long_rows(ctx, oracle):
     cols = 22016
     w, g = inputs.make_rows(8192, cols, 5001, 0, 12, importance_sigma=2.0)
