@@ -92,7 +92,7 @@ int skim_destroy(skim_ctx *ctx)
     if (ctx && ctx->copy_ready) {
         DeviceGuard guard(ctx->device);
         cudaStreamDestroy(ctx->copy_stream);
-        for (int k = 0; k < SKIM_HOST_CHUNKS; ++k) cudaEventDestroy(ctx->copy_done[k]);
+        for (int k = 0; k < SKIM_HOST_EVENTS; ++k) cudaEventDestroy(ctx->copy_done[k]);
         cudaEventDestroy(ctx->main_idle);
     }
     if (ctx && ctx->timing_ready) {
@@ -481,6 +481,8 @@ int skim_scale_update_lfull(skim_ctx *ctx, const uint16_t *W, const float *impor
 // ---------------------------------------------------------------- host-buffer path
 
 namespace {
+constexpr int64_t HOST_CHUNK_ELEMENTS = 1 << 20;      // the host-buffer entry point cuts its last chunks down to this
+
 struct Staging {
     uint16_t *W;
     float *G;
@@ -543,7 +545,7 @@ int skim_quantize_matrix_host(skim_ctx *ctx, const uint16_t *W_host, const float
     cudaStream_t st = ctx->stream;
     if (!ctx->copy_ready) {
         SKIM_CUDA_OK(cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking));
-        for (int k = 0; k < SKIM_HOST_CHUNKS; ++k)
+        for (int k = 0; k < SKIM_HOST_EVENTS; ++k)
             SKIM_CUDA_OK(cudaEventCreateWithFlags(&ctx->copy_done[k], cudaEventDisableTiming));
         SKIM_CUDA_OK(cudaEventCreateWithFlags(&ctx->main_idle, cudaEventDisableTiming));
         ctx->copy_ready = true;
@@ -551,12 +553,16 @@ int skim_quantize_matrix_host(skim_ctx *ctx, const uint16_t *W_host, const float
     // the staging area may still be read by earlier work on the main stream
     SKIM_CUDA_OK(cudaEventRecord(ctx->main_idle, st));
     SKIM_CUDA_OK(cudaStreamWaitEvent(ctx->copy_stream, ctx->main_idle, 0));
-    // rows travel in chunks: chunk k is clustered while chunk k+1 is still on the bus
+    // Rows travel in chunks: chunk k is clustered while chunk k+1 is still on the bus.  The bus is the bound (4096 x 11008: 4.92 of
+    // 5.4 ms); what follows the last byte is the clustering of the last chunk, so the last chunks halve -- down to
+    // HOST_CHUNK_ELEMENTS: a smaller chunk arrives faster (1 M elements: 0.11 ms) than the chunk before it is clustered.
     const int64_t per = (rows + SKIM_HOST_CHUNKS - 1) / SKIM_HOST_CHUNKS;
     const int64_t chunk = per < 256 ? (rows < 256 ? rows : 256) : per;
     int k = 0;
-    for (int64_t r0 = 0; r0 < rows; r0 += chunk, ++k) {
-        const int64_t n = rows - r0 < chunk ? rows - r0 : chunk;
+    int64_t n;
+    for (int64_t r0 = 0; r0 < rows; r0 += n, ++k) {
+        n = rows - r0 < chunk ? rows - r0 : chunk;
+        if (n == rows - r0 && k < SKIM_HOST_EVENTS - 2 && n / 2 * cols >= HOST_CHUNK_ELEMENTS) n -= n / 2;
         SKIM_CUDA_OK(cudaMemcpyAsync(s.W + r0 * cols, W_host + r0 * cols, (size_t)n * cols * 2, cudaMemcpyHostToDevice,
                                      ctx->copy_stream));
         SKIM_CUDA_OK(cudaMemcpyAsync(s.G + r0 * cols, importance_host + r0 * cols, (size_t)n * cols * 4,
@@ -569,14 +575,15 @@ int skim_quantize_matrix_host(skim_ctx *ctx, const uint16_t *W_host, const float
     }
     rc = skim_allocate_bits(ctx, s.err, rows, bit_set, n_bits, budget, s.bits, nullptr);
     if (rc) return rc;
+    // errors and widths travel back beside the packer
+    SKIM_CUDA_OK(cudaEventRecord(ctx->main_idle, st));
+    SKIM_CUDA_OK(cudaStreamWaitEvent(ctx->copy_stream, ctx->main_idle, 0));
     rc = skim_quantize(ctx, s.W, rows, cols, cols, s.bits, s.centroids, bit_set, n_bits, s.packed, s.row_order,
                        s.group_info, s.lut);
     if (rc) return rc;
-    if (err_host) SKIM_CUDA_OK(cudaMemcpyAsync(err_host, s.err, (size_t)rows * n_bits * 4, cudaMemcpyDeviceToHost, st));
-    if (bits_host) SKIM_CUDA_OK(cudaMemcpyAsync(bits_host, s.bits, (size_t)rows, cudaMemcpyDeviceToHost, st));
-    if (row_order_host) SKIM_CUDA_OK(cudaMemcpyAsync(row_order_host, s.row_order, (size_t)rows * 4, cudaMemcpyDeviceToHost, st));
-    if (lut_host)
-        SKIM_CUDA_OK(cudaMemcpyAsync(lut_host, s.lut, (size_t)rows * (size_t)(1 << bs.b_max) * 2, cudaMemcpyDeviceToHost, st));
+    if (err_host)
+        SKIM_CUDA_OK(cudaMemcpyAsync(err_host, s.err, (size_t)rows * n_bits * 4, cudaMemcpyDeviceToHost, ctx->copy_stream));
+    if (bits_host) SKIM_CUDA_OK(cudaMemcpyAsync(bits_host, s.bits, (size_t)rows, cudaMemcpyDeviceToHost, ctx->copy_stream));
     int64_t info[2 * (SKIM_MAX_NBITS + 1)];
     SKIM_CUDA_OK(cudaMemcpyAsync(info, s.group_info, (size_t)(2 * (n_bits + 1)) * 8, cudaMemcpyDeviceToHost, st));
     SKIM_CUDA_OK(cudaStreamSynchronize(st));
@@ -586,8 +593,12 @@ int skim_quantize_matrix_host(skim_ctx *ctx, const uint16_t *W_host, const float
         // only the words the allocation really uses travel back
         const size_t words = (size_t)info[2 * n_bits + 1];
         SKIM_CUDA_OK(cudaMemcpyAsync(packed_host, s.packed, words * 4, cudaMemcpyDeviceToHost, st));
-        SKIM_CUDA_OK(cudaStreamSynchronize(st));
     }
+    if (row_order_host) SKIM_CUDA_OK(cudaMemcpyAsync(row_order_host, s.row_order, (size_t)rows * 4, cudaMemcpyDeviceToHost, st));
+    if (lut_host)
+        SKIM_CUDA_OK(cudaMemcpyAsync(lut_host, s.lut, (size_t)rows * (size_t)(1 << bs.b_max) * 2, cudaMemcpyDeviceToHost, st));
+    SKIM_CUDA_OK(cudaStreamSynchronize(st));
+    SKIM_CUDA_OK(cudaStreamSynchronize(ctx->copy_stream));
     return SKIM_OK;
 }
 

@@ -8,7 +8,8 @@
 #include "skim.h"
 
 #define SKIM_MAX_NBITS SKIM_MAX_BIT
-#define SKIM_HOST_CHUNKS 8   // row chunks of the host-buffer entry point
+#define SKIM_HOST_CHUNKS 8   // row chunks of the host-buffer entry point, and how many with the last one cut further
+#define SKIM_HOST_EVENTS 14
 #define SKIM_MAX_SUMK 30  // 2 + 4 + 8 + 16: one warp lane per centroid
 #define SKIM_TIMING_SLOTS 256   // clustering chunks whose kernel times skim_kernel_timing can hold
 
@@ -25,7 +26,7 @@ struct skim_ctx {
     // host-buffer entry point: a second stream for the host-to-device copies, so that the copy
     // of one row chunk runs under the clustering of the previous one (created on first use)
     cudaStream_t copy_stream;
-    cudaEvent_t copy_done[SKIM_HOST_CHUNKS];
+    cudaEvent_t copy_done[SKIM_HOST_EVENTS];
     cudaEvent_t main_idle;
     bool copy_ready;
     // optional kernel timing: events before the sort kernel, between the two kernels and after

@@ -158,6 +158,26 @@ def test_host_buffer_entry_point(ctx, oracle, skimlib):
     assert e.value.code == -5
 
 
+@pytest.mark.parametrize("rows,cols", [(255, 8192), (256, 8192), (257, 16001), (520, 9000), (2100, 5000)])
+def test_host_buffer_chunks_cut_at_the_end(ctx, skimlib, rows, cols):
+    """Matrices around the sizes at which the last row chunks are halved: the device-buffer path's results, bit for bit."""
+    w, g = inputs.make_rows(rows, cols, 43)
+    cent, err, bits, total, out = _pipeline(ctx, w, g, 3, 2.5)
+    staging = torch.empty(skimlib.Skim.host_staging_bytes(rows, cols, BITS), dtype=torch.uint8, device="cuda")
+    _, mx = skimlib.Skim.packed_layout(rows, cols, BITS)
+    h = dict(err=torch.zeros((rows, 4)), bits=torch.zeros(rows, dtype=torch.uint8), packed=torch.zeros(mx // 4, dtype=torch.int32),
+             row_order=torch.zeros(rows, dtype=torch.int32), group_info=torch.zeros(10, dtype=torch.int64),
+             lut=torch.zeros((rows, 16), dtype=torch.int16))
+    h = {k: v.pin_memory() for k, v in h.items()}
+    ctx.quantize_matrix_host(torch.from_numpy(w).pin_memory(), torch.from_numpy(g).pin_memory(), BITS, 3, 2.5, staging, h)
+    words = int(out["group_info"][-1])
+    np.testing.assert_array_equal(h["err"].numpy(), err)
+    np.testing.assert_array_equal(h["bits"].numpy(), bits)
+    np.testing.assert_array_equal(h["packed"].numpy()[:words], out["packed"][:words])
+    for k in ("group_info", "row_order", "lut"):
+        np.testing.assert_array_equal(h[k].numpy(), out[k])
+
+
 def test_full_matrix_every_row(ctx, oracle):
     """Every row of the benchmark's 4096 x 11008 matrix (the launch configuration the benchmark times):
     centroids and errors of all four widths against the oracle, row by row.  A row whose
