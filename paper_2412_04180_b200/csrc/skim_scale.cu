@@ -45,6 +45,7 @@ struct ScaleArgs {
     uint16_t *D;            // L-full loss: [rows][cols] binary16 residual * 2^exp2
     int exp2;
     int rows_per_range;
+    int grad_warps;         // warps of a gradient block side by side over the columns; its other warps take other rows
 };
 
 // 1 / a for a positive, normal binary64 a (the scale vector is checked to be that): the hardware's approximate
@@ -227,6 +228,61 @@ __global__ void __launch_bounds__(OT) skim_scale_order_kernel(ScaleArgs a)
     for (int q = tid; q < total / 2; q += OT) dst[q] = src[q];
 }
 
+// Short rows: padding to whole units and the reductions at every cluster's end would cost more than the elements do (22016 x 128:
+// 8 clusters of 16 elements padded to 64 each).  Such rows are written without padding, by one warp each, in column order inside a
+// cluster; ord_end counts elements.  Whole step, before and after: 22016 x 128 85 -> 49 us, 9000 x 300 43 -> 28.5 us; at 4096 x 1500 36.6 -> 43.6 us,
+// since the longest cluster decides.  Up to 1024 columns it pays where every warp of the sums kernel has a row of its own (4096 x 700 28.4 ->
+// 26.1 us, ordering 9000 x 1000 170 -> 100 us; 1000 x 1001 16.9 -> 19.0 us).
+constexpr int SHORT_COLS = 512, SHORT_COLS_MANY_ROWS = 1024;
+constexpr int OST = 256;
+
+__global__ void __launch_bounds__(OST) skim_scale_order_short_kernel(ScaleArgs a)
+{
+    __shared__ int count_all[OST / 32][2 * KC];
+    const int lane = threadIdx.x & 31;
+    int *count = count_all[threadIdx.x >> 5];                  // entry KC: columns past the end
+    const int64_t row = (int64_t)blockIdx.x * (OST / 32) + (threadIdx.x >> 5);
+    if (row >= a.rows) return;                                 // (whole warps; no block-wide barrier follows)
+    const uint16_t *Wr = a.W + row * a.ld;
+    const float *Gr = a.G + row * a.ld;
+    const uint8_t *Lr = a.labels + row * (int64_t)a.cols;
+    uint2 *dst = a.ord + row * skim_ordered_stride(a.cols);
+    count[lane] = 0;
+    __syncwarp();
+    for (int j0 = 0; j0 < a.cols; j0 += 32) {
+        const int l = j0 + lane < a.cols ? (int)(Lr[j0 + lane] & (KC - 1)) : KC;
+        const uint32_t same = __match_any_sync(0xffffffffu, l);
+        if ((same & ((1u << lane) - 1u)) == 0u) count[l] += __popc(same);
+        __syncwarp();
+    }
+    const int n = count[lane & (KC - 1)];
+    int inc = n;
+#pragma unroll
+    for (int off = 1; off < KC; off <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, inc, off, KC);
+        if ((lane & (KC - 1)) >= off) inc += t;
+    }
+    __syncwarp();
+    if (lane < KC) {
+        a.ord_end[row * KC + lane] = (uint16_t)inc;
+        count[lane] = inc - n;
+    }
+    __syncwarp();
+    for (int j0 = 0; j0 < a.cols; j0 += 32) {
+        const int j = j0 + lane;
+        const bool in = j < a.cols;
+        const int l = in ? (int)(Lr[j] & (KC - 1)) : KC;
+        const uint32_t w = in ? (uint32_t)Wr[j] : 0u;
+        const float g = in ? Gr[j] : 0.0f;
+        const uint32_t same = __match_any_sync(0xffffffffu, l), below = same & ((1u << lane) - 1u);
+        const int pos = count[l] + __popc(below);
+        __syncwarp();
+        if (below == 0u) count[l] += __popc(same);
+        if (in && SKIM_IDX(pos, a.cols, nullptr)) dst[pos] = make_uint2(__float_as_uint(g), (w << 16) | (uint32_t)j);
+        __syncwarp();
+    }
+}
+
 // ---------------------------------------------------------------- the sums of a step
 
 constexpr int SUM_T = 768;                 // threads per block of the sums kernel, one block per SM (80 registers)
@@ -341,6 +397,40 @@ __device__ __forceinline__ void sum_units(const uint4 *src, int end, int t0, int
     }
 }
 
+// The same sums of a short row, all of it: the lanes are dealt to the clusters in equal groups (a power of two of clusters, so
+// 2 to 32 lanes each), a lane takes every so-manieth element of its cluster.
+template <int MODE>
+__device__ __forceinline__ void sum_short(const uint2 *src, int end, const double *alpha, double &vx, double &vb)
+{
+    constexpr int AT_ONCE = 4;
+    const int lane = threadIdx.x & 31;
+    const int before = __shfl_up_sync(0xffffffffu, end, 1, KC);
+    const uint32_t full = __ballot_sync(0xffffffffu, end > ((lane & (KC - 1)) ? before : 0)) & 0xffffu;
+    const int lg = full > 1u ? 32 - __clz(31 - __clz(full)) : 0;       // clusters up to the last one with members: at most 2^lg
+    const int sh = 5 - lg, per = 1 << sh, k = lane >> sh;
+    const int stop = __shfl_sync(0xffffffffu, end, k);
+    const int start = __shfl_sync(0xffffffffu, end, max(k - 1, 0));
+    double acc[3] = {0.0, 0.0, 0.0};
+    for (int i = (k ? start : 0) + (lane & (per - 1)); i < stop; i += AT_ONCE * per) {
+        uint2 v[AT_ONCE];
+#pragma unroll
+        for (int u = 0; u < AT_ONCE; ++u) v[u] = i + u * per < stop ? src[i + u * per] : make_uint2(0u, 0u);
+#pragma unroll
+        for (int u = 0; u < AT_ONCE; ++u) add_element<MODE>(v[u].x, v[u].y, alpha, acc);
+    }
+    __syncwarp();
+    for (int off = per >> 1; off; off >>= 1) {
+        acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], off);
+        if (MODE != SUMS_CENTROIDS) acc[1] += __shfl_xor_sync(0xffffffffu, acc[1], off);
+        if (MODE == SUMS_STEP) acc[2] += __shfl_xor_sync(0xffffffffu, acc[2], off);
+    }
+    const int from = (lane & (KC - 1)) << sh;                          // beyond the last lane: an empty cluster
+    const double s0 = __shfl_sync(0xffffffffu, acc[0], from & 31), s1 = __shfl_sync(0xffffffffu, acc[1], from & 31);
+    const double s2 = __shfl_sync(0xffffffffu, acc[2], from & 31);
+    vx = from < 32 ? (lane < KC ? s0 : s1) : 0.0;
+    vb = from < 32 ? s2 : 0.0;
+}
+
 // What the sums of a row are turned into (lanes as sum_units leaves them).
 //   SUMS_INIT       the per-call constants (G_k, D_k)
 //   SUMS_STEP       (c_k, q_k) and the row's loss
@@ -413,7 +503,7 @@ __device__ __forceinline__ void residual_columns(const ScaleArgs &a, int64_t row
 // One block per SM, rows dealt round-robin to the blocks.  A warp takes whole rows while there are rows for all of the
 // block's warps; the rows that are left are shared by the warps in equal stretches, whose sums meet in shared memory in a
 // fixed order.  Bound by HBM: 8 B an element.
-template <int MODE>
+template <int MODE, bool SHORT>
 __global__ void __launch_bounds__(SUM_T, 1) skim_scale_sums_kernel(ScaleArgs a)
 {
     extern __shared__ __align__(16) double ssmem[];
@@ -424,7 +514,7 @@ __global__ void __launch_bounds__(SUM_T, 1) skim_scale_sums_kernel(ScaleArgs a)
     const int64_t stride = skim_ordered_stride(a.cols) / 2;
     const int mine = (int)((a.rows - blockIdx.x + gridDim.x - 1) / gridDim.x);       // rows of this block (at least one)
     const int whole = mine / SUM_W * SUM_W, rest = mine - whole;
-    if (MODE != SUMS_INIT) {
+    if (MODE != SUMS_INIT && !SHORT) {
         // the start of this warp's first row, while the previous kernel ends
         const int r = whole ? warp : warp / (SUM_W / rest);
         if (r < mine) {
@@ -441,38 +531,50 @@ __global__ void __launch_bounds__(SUM_T, 1) skim_scale_sums_kernel(ScaleArgs a)
         __syncthreads();
     }
     double vx, vb;
-    for (int r = warp; r < whole; r += SUM_W) {
-        const int64_t row = blockIdx.x + (int64_t)gridDim.x * r;
-        const int end = a.ord_end[row * KC + (lane & 15)];
-        sum_units<MODE>(reinterpret_cast<const uint4 *>(a.ord) + row * stride, end, 0, __shfl_sync(0xffffffffu, end, KC - 1), alpha, vx, vb);
-        const double c = finish_row<MODE>(a, row, vx, vb);
-        if (MODE == SUMS_CENTROIDS) residual_columns(a, row, 0, a.cols, alpha, c);
-    }
-    if (rest == 0) return;
-    const int per_row = SUM_W / rest, idx = warp / per_row, sub = warp - idx * per_row;
-    const int64_t row = blockIdx.x + (int64_t)gridDim.x * (whole + idx);
-    if (idx < rest) {
-        const int end = a.ord_end[row * KC + (lane & 15)];
-        const int total = __shfl_sync(0xffffffffu, end, KC - 1);
-        const int t0 = total * sub / per_row, t1 = total * (sub + 1) / per_row;
-        sum_units<MODE>(reinterpret_cast<const uint4 *>(a.ord) + row * stride, end, t0, t1, alpha, vx, vb);
-        part[threadIdx.x] = make_double2(vx, vb);
-    }
-    __syncthreads();
-    if (idx < rest && sub == 0) {
-        for (int q = 1; q < per_row; ++q) {
-            const double2 o = part[threadIdx.x + 32 * q];
-            vx += o.x;
-            vb += o.y;
+    if constexpr (SHORT) {
+        int end = warp < mine ? (int)a.ord_end[(blockIdx.x + (int64_t)gridDim.x * warp) * KC + (lane & 15)] : 0;
+        for (int r = warp; r < mine; r += SUM_W) {
+            const int64_t row = blockIdx.x + (int64_t)gridDim.x * r, next = row + (int64_t)gridDim.x * SUM_W;
+            const int ahead = r + SUM_W < mine ? (int)a.ord_end[next * KC + (lane & 15)] : 0;
+            sum_short<MODE>(a.ord + row * stride * 2, end, alpha, vx, vb);
+            const double c = finish_row<MODE>(a, row, vx, vb);
+            if (MODE == SUMS_CENTROIDS) residual_columns(a, row, 0, a.cols, alpha, c);
+            end = ahead;
         }
-        const double c = finish_row<MODE>(a, row, vx, vb);
-        if (MODE == SUMS_CENTROIDS) part[threadIdx.x].x = c;
-    }
-    if (MODE == SUMS_CENTROIDS) {
-        // the row's columns are shared by the same warps (in fours: cols is a multiple of 8 on this path)
+    } else {
+        for (int r = warp; r < whole; r += SUM_W) {
+            const int64_t row = blockIdx.x + (int64_t)gridDim.x * r;
+            const int end = a.ord_end[row * KC + (lane & 15)];
+            sum_units<MODE>(reinterpret_cast<const uint4 *>(a.ord) + row * stride, end, 0, __shfl_sync(0xffffffffu, end, KC - 1), alpha, vx, vb);
+            const double c = finish_row<MODE>(a, row, vx, vb);
+            if (MODE == SUMS_CENTROIDS) residual_columns(a, row, 0, a.cols, alpha, c);
+        }
+        if (rest == 0) return;
+        const int per_row = SUM_W / rest, idx = warp / per_row, sub = warp - idx * per_row;
+        const int64_t row = blockIdx.x + (int64_t)gridDim.x * (whole + idx);
+        if (idx < rest) {
+            const int end = a.ord_end[row * KC + (lane & 15)];
+            const int total = __shfl_sync(0xffffffffu, end, KC - 1);
+            const int t0 = total * sub / per_row, t1 = total * (sub + 1) / per_row;
+            sum_units<MODE>(reinterpret_cast<const uint4 *>(a.ord) + row * stride, end, t0, t1, alpha, vx, vb);
+            part[threadIdx.x] = make_double2(vx, vb);
+        }
         __syncthreads();
-        const int quads = a.cols / 4, q0 = quads * sub / per_row, q1 = quads * (sub + 1) / per_row;
-        if (idx < rest && q0 < q1) residual_columns(a, row, q0 * 4, q1 * 4, alpha, part[idx * per_row * 32 + lane].x);
+        if (idx < rest && sub == 0) {
+            for (int q = 1; q < per_row; ++q) {
+                const double2 o = part[threadIdx.x + 32 * q];
+                vx += o.x;
+                vb += o.y;
+            }
+            const double c = finish_row<MODE>(a, row, vx, vb);
+            if (MODE == SUMS_CENTROIDS) part[threadIdx.x].x = c;
+        }
+        if (MODE == SUMS_CENTROIDS) {
+            // the row's columns are shared by the same warps (in fours: cols is a multiple of 8 on this path)
+            __syncthreads();
+            const int quads = a.cols / 4, q0 = quads * sub / per_row, q1 = quads * (sub + 1) / per_row;
+            if (idx < rest && q0 < q1) residual_columns(a, row, q0 * 4, q1 * 4, alpha, part[idx * per_row * 32 + lane].x);
+        }
     }
 }
 
@@ -487,16 +589,17 @@ struct GradCols {
     bool in[VEC ? 1 : GC];
     // VEC: four consecutive columns (cols % 4 == 0: all inside or all outside).  Otherwise four columns a block width
     // apart, so that scalar loads are contiguous across a warp.
-    __device__ __forceinline__ GradCols(int tile, int cols)
+    // thread t of the `width` threads that share a tile
+    __device__ __forceinline__ GradCols(int tile, int cols, int t, int width)
     {
         if constexpr (VEC) {
-            const int c = (tile * GT + threadIdx.x) * GC;
+            const int c = (tile * width + t) * GC;
             in[0] = c < cols;
             j[0] = min(c, cols - GC);
         } else {
 #pragma unroll
             for (int u = 0; u < GC; ++u) {
-                const int c = (tile * GC + u) * GT + threadIdx.x;
+                const int c = (tile * GC + u) * width + t;
                 in[u] = c < cols;
                 j[u] = min(c, cols - 1);
             }
@@ -532,15 +635,19 @@ __device__ __forceinline__ void grad_load(const ScaleArgs &a, int64_t row, const
     }
 }
 
-template <bool VEC>
+// NARROW: the block's warps share the rows as well (its own instance: the wide form has no register to spare)
+template <bool VEC, bool NARROW>
 __global__ void __launch_bounds__(GT, 2) skim_scale_grad_kernel(ScaleArgs a)
 {
     __shared__ WarpTables<4> tables[GT / 32];
     WarpTables<4> &tw = tables[threadIdx.x >> 5];
     constexpr int RB = VEC ? 4 : 2;   // rows of a batch (four column addresses leave fewer registers); two batches take turns in registers, one of them in flight
-    const GradCols<VEC> c(blockIdx.x, a.cols);
-    const int64_t r0 = (int64_t)blockIdx.y * a.rows_per_range;
-    const int64_t r1 = min(a.rows, r0 + a.rows_per_range), last = r1 - 1;
+    const int side = NARROW ? a.grad_warps : GT / 32, subs = (GT / 32) / side, sub = NARROW ? (int)(threadIdx.x >> 5) / side : 0;
+    const GradCols<VEC> c(blockIdx.x, a.cols, (int)threadIdx.x - sub * side * 32, side * 32);
+    const int64_t b0 = (int64_t)blockIdx.y * a.rows_per_range, b1 = min(a.rows, b0 + a.rows_per_range), last = b1 - 1;
+    // this warp's share of the block's rows (none for the warps left over)
+    const int64_t share = NARROW ? (b1 - b0 + subs - 1) / subs : 0, r0 = NARROW ? min(b1, b0 + sub * share) : b0;
+    const int64_t r1 = NARROW ? (sub < subs ? min(b1, r0 + share) : r0) : b1;
     GradRow row[2][RB];
     double2 tab[2][RB / 2];
     auto fetch_rows = [&](int h, int64_t rb) {
@@ -588,6 +695,17 @@ __global__ void __launch_bounds__(GT, 2) skim_scale_grad_kernel(ScaleArgs a)
             }
         }
     }
+    if constexpr (NARROW) {
+        // the shares' sums, in the order of the rows
+        __shared__ double red[GC][GT];
+#pragma unroll
+        for (int u = 0; u < GC; ++u) red[u][threadIdx.x] = acc[u];
+        __syncthreads();
+        if (sub != 0) return;
+        for (int q = 1; q < subs; ++q)
+#pragma unroll
+            for (int u = 0; u < GC; ++u) acc[u] += red[u][threadIdx.x + q * side * 32];
+    }
 #pragma unroll
     for (int u = 0; u < GC; ++u)
         if (c.inside(u)) a.grad_part[(int64_t)blockIdx.y * a.cols + c.col(u)] = acc[u];
@@ -605,6 +723,7 @@ __global__ void __launch_bounds__(256) skim_scale_adam_kernel(const double *__re
     if (blockIdx.x == gridDim.x - 1) {
         // the last block adds the rows' losses: strided partial sums, then a fixed tree
         double s = 0.0;
+#pragma unroll 8
         for (int64_t i = threadIdx.x; i < rows; i += 256) s += loss_row[i];
         red[threadIdx.x] = s;
         __syncthreads();
@@ -670,7 +789,7 @@ __global__ void __launch_bounds__(GT, 2) skim_scale_lf_grad_kernel(ScaleArgs a, 
     __shared__ WarpTables<2> tables[GT / 32];
     WarpTables<2> &tw = tables[threadIdx.x >> 5];
     constexpr int RB = 2;
-    const GradCols<true> c(blockIdx.x, a.cols);
+    const GradCols<true> c(blockIdx.x, a.cols, (int)threadIdx.x, GT);
     const int64_t r0 = (int64_t)blockIdx.y * a.rows_per_range;
     const int64_t r1 = min(a.rows, r0 + a.rows_per_range), last = r1 - 1;
     const double ys = ldexp(-2.0, -a.exp2);
@@ -736,6 +855,7 @@ namespace {
 
 // What both updates do first: alpha's master copies, the label-ordered matrix, the per-call constants (G_k, D_k).
 struct ScalePlan {
+    void (*step)(ScaleArgs), (*centroids)(ScaleArgs);      // the sums kernel by row length
     ScaleArgs a;
     unsigned cb, ab;                 // blocks over the columns; Adam: 32 columns a block
     dim3 grad_grid;
@@ -772,6 +892,9 @@ int scale_begin(skim_ctx *ctx, const SkimWorkspace &ws, const uint16_t *W, const
     if (ranges > SKIM_SCALE_MAX_CTAS) ranges = SKIM_SCALE_MAX_CTAS;
     if (ranges > rows) ranges = (int)rows;
     if (ranges < 1) ranges = 1;
+    // warps side by side over the columns: narrow matrices would leave most of a block idle (22016 x 128: 7 warps of 8;
+    // a step 49 -> 30 us)
+    a.grad_warps = tiles > 1 || cols > GT / 2 * GC ? GT / 32 : (int)((cols + 32 * GC - 1) / (32 * GC));
     a.rows_per_range = (int)((rows + ranges - 1) / ranges);
     p->ranges = (int)((rows + a.rows_per_range - 1) / a.rows_per_range);
     p->grad_grid = dim3((unsigned)tiles, (unsigned)p->ranges);
@@ -779,15 +902,20 @@ int scale_begin(skim_ctx *ctx, const SkimWorkspace &ws, const uint16_t *W, const
     p->sum_blocks = (unsigned)(rows < ctx->sm_count ? rows : ctx->sm_count);
     // set on every launch: host-side calls of microseconds, and no state shared between contexts
     const int sm_order = (int)order_smem_bytes((int)cols), sm_init = (int)sums_smem_bytes((int)cols, true), sm_sums = (int)sums_smem_bytes((int)cols, false);
+    const bool is_short = cols <= SHORT_COLS || (cols <= SHORT_COLS_MANY_ROWS && rows >= (int64_t)SUM_W * ctx->sm_count);
+    void (*init)(ScaleArgs) = is_short ? skim_scale_sums_kernel<SUMS_INIT, true> : skim_scale_sums_kernel<SUMS_INIT, false>;
+    p->step = is_short ? skim_scale_sums_kernel<SUMS_STEP, true> : skim_scale_sums_kernel<SUMS_STEP, false>;
+    p->centroids = is_short ? skim_scale_sums_kernel<SUMS_CENTROIDS, true> : skim_scale_sums_kernel<SUMS_CENTROIDS, false>;
     SKIM_CUDA_OK(cudaFuncSetAttribute(skim_scale_order_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sm_order));
-    SKIM_CUDA_OK(cudaFuncSetAttribute(skim_scale_sums_kernel<SUMS_INIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm_init));
-    SKIM_CUDA_OK(cudaFuncSetAttribute(skim_scale_sums_kernel<SUMS_STEP>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm_sums));
-    SKIM_CUDA_OK(cudaFuncSetAttribute(skim_scale_sums_kernel<SUMS_CENTROIDS>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm_sums));
+    SKIM_CUDA_OK(cudaFuncSetAttribute(init, cudaFuncAttributeMaxDynamicSharedMemorySize, sm_init));
+    SKIM_CUDA_OK(cudaFuncSetAttribute(p->step, cudaFuncAttributeMaxDynamicSharedMemorySize, sm_sums));
+    SKIM_CUDA_OK(cudaFuncSetAttribute(p->centroids, cudaFuncAttributeMaxDynamicSharedMemorySize, sm_sums));
     skim_scale_init_kernel<<<p->cb, 256, 0, ctx->stream>>>(alpha, (int)cols, ws.alpha64, ws.adam_m, ws.adam_v, ws.status);
     SKIM_CUDA_OK(cudaGetLastError());
-    skim_scale_order_kernel<<<(unsigned)rows, OT, sm_order, ctx->stream>>>(a);
+    if (is_short) skim_scale_order_short_kernel<<<(unsigned)((rows + OST / 32 - 1) / (OST / 32)), OST, 0, ctx->stream>>>(a);
+    else skim_scale_order_kernel<<<(unsigned)rows, OT, sm_order, ctx->stream>>>(a);
     SKIM_CUDA_OK(cudaGetLastError());
-    skim_scale_sums_kernel<SUMS_INIT><<<p->sum_blocks, SUM_T, sm_init, ctx->stream>>>(a);
+    init<<<p->sum_blocks, SUM_T, sm_init, ctx->stream>>>(a);
     SKIM_CUDA_OK(cudaGetLastError());
     ctx->launches += 3;
     return SKIM_OK;
@@ -849,7 +977,7 @@ int skim_launch_scale_update_lfull(skim_ctx *ctx, const uint16_t *W, const float
     AdamSchedule sched(lr0, decay, decay_every);
     for (int t = 0; t < steps; ++t) {
         sched.next();
-        rc = skim_launch_dependent(ctx, skim_scale_sums_kernel<SUMS_CENTROIDS>, dim3(p.sum_blocks), SUM_T, sums_smem_bytes((int)cols, false), p.a);
+        rc = skim_launch_dependent(ctx, p.centroids, dim3(p.sum_blocks), SUM_T, sums_smem_bytes((int)cols, false), p.a);
         if (rc) return rc;
         rc = skim_launch_err_lfull(ctx, p.a.D, rows, cols, cols, H, ldh, exp2, sp, nullptr, 1, Y, cols, ws.loss_part, &cl);
         if (rc) return rc;
@@ -869,11 +997,13 @@ int skim_launch_scale_update(skim_ctx *ctx, const uint16_t *W, const float *impo
     ScalePlan p;
     int rc = scale_begin(ctx, ws, W, importance, rows, cols, ld, labels, alpha, &p);
     if (rc) return rc;
-    auto grad = p.a.vec ? skim_scale_grad_kernel<true> : skim_scale_grad_kernel<false>;
+    const bool narrow = p.a.grad_warps < GT / 32;
+    auto grad = p.a.vec ? (narrow ? skim_scale_grad_kernel<true, true> : skim_scale_grad_kernel<true, false>)
+                        : (narrow ? skim_scale_grad_kernel<false, true> : skim_scale_grad_kernel<false, false>);
     AdamSchedule sched(lr0, decay, decay_every);
     for (int t = 0; t < steps; ++t) {
         sched.next();
-        rc = skim_launch_dependent(ctx, skim_scale_sums_kernel<SUMS_STEP>, dim3(p.sum_blocks), SUM_T, sums_smem_bytes((int)cols, false), p.a);
+        rc = skim_launch_dependent(ctx, p.step, dim3(p.sum_blocks), SUM_T, sums_smem_bytes((int)cols, false), p.a);
         if (rc) return rc;
         rc = skim_launch_dependent(ctx, grad, p.grad_grid, GT, 0, p.a);
         if (rc) return rc;

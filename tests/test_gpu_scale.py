@@ -57,6 +57,13 @@ def test_scale_update_label_layouts(ctx, oracle, rows, cols, kind):
     np.testing.assert_allclose(alpha.cpu().numpy().astype(np.float64), want, rtol=1e-6, atol=0)
 
 
+@pytest.mark.parametrize("rows,cols,kind", [(40, 128, "mixed"), (17, 129, "mixed"), (300, 389, "rare"), (50, 512, "one"), (50, 513, "column"),
+                                            (3553, 516, "mixed"), (3600, 1024, "mixed"), (3600, 1025, "rare")])
+def test_scale_update_narrow_matrices(ctx, oracle, rows, cols, kind):
+    """Row lengths and row counts around the rules for short rows, and blocks of the gradient kernel that hold several row shares."""
+    test_scale_update_label_layouts(ctx, oracle, rows, cols, kind)
+
+
 def test_scale_update_wide_rows(ctx, oracle):
     rows, cols = 6, 22016
     w, g = inputs.make_rows(8192, cols, 5001, 0, rows, importance_sigma=2.0)
