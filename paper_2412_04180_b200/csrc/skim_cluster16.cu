@@ -1,5 +1,6 @@
 // fp16-key row-sorting kernel, the first half of the row clustering (SKIM Algorithm 3, error pre-recording loop; objective of
-// Section 3.2, diagonal form) where no scale vector is installed.
+// Section 3.2, diagonal form) where no scale vector is installed: rows too long for skim_bucket.cu to be faster, and all
+// rows of the exact clustering.
 //
 // With no scale the clustered value IS the fp16 weight, so a 16-bit order-preserving key is exact
 // and the sort moves one 32-bit word per element: (key << 16) | column.

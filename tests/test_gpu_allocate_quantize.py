@@ -50,6 +50,22 @@ def test_allocation_heavy_ties_and_special_tables(ctx, oracle):
             np.testing.assert_array_equal(got, want, err_msg=f"table {t} total {total}")
 
 
+@pytest.mark.parametrize("rows", [170, 171, 172, 4096, 4097, 22016])
+@pytest.mark.parametrize("kind", ["equal", "two", "clump", "octaves"])
+def test_allocation_of_clumped_keys(ctx, oracle, rows, kind):
+    """Numbers of keys around what is ranked directly and what stays in registers; gains that one split of their range leaves together."""
+    rng = np.random.default_rng(rows)
+    gain = {"equal": lambda: np.full((rows, 3), 0.25), "two": lambda: rng.choice([0.25, np.nextafter(np.float32(0.25), np.float32(1))], (rows, 3)),
+            "clump": lambda: np.where(rng.random((rows, 3)) < 0.01, 1e20, 1.0 + rng.integers(0, 50, (rows, 3)) * 2.0**-20),
+            "octaves": lambda: 2.0 ** rng.integers(-100, 100, (rows, 3))}[kind]()
+    err = np.concatenate([np.cumsum(gain[:, ::-1], axis=1)[:, ::-1], np.zeros((rows, 1))], axis=1).astype(np.float32)
+    for budget in (1.0 + 1.0 / rows, 2.25, 2.5, 4.0 - 1.0 / rows):
+        want, total = oracle.allocate_bits(err, 1, budget)
+        got, gtotal = _alloc(ctx, err, BITS, budget)
+        assert gtotal == total
+        np.testing.assert_array_equal(got, want, err_msg=f"budget={budget}")
+
+
 @pytest.mark.parametrize("rows", [1, 33, 1000, 4096, 9000])
 def test_floor_started_allocation_matches_oracle(ctx, oracle, rows):
     """skim_allocate_bits_floor: every row starts at floor(budget); bit-exact against the oracle's loop."""
@@ -180,6 +196,15 @@ def test_packed_codes_unaligned_leading_dimension(ctx, oracle):
     w, g = inputs.make_rows(rows, cols, 12)
     cent32 = oracle.cluster_rows(w, g, [2, 3], 6, want_codes=False)["centroids"].astype(np.float32)
     _emit_both(ctx, oracle, w, (np.arange(rows) % 2 + 2).astype(np.uint8), cent32, [2, 3])
+
+
+@pytest.mark.parametrize("cols", [1, 7, 9, 31, 33, 1000, 1023, 1032, 2049, 4099])
+def test_packed_codes_with_scale_at_ragged_lengths(ctx, oracle, cols):
+    rows = 13
+    w, g = inputs.make_rows(rows, cols, 500 + cols)
+    s = inputs.make_scale(cols, 9)
+    cent32 = oracle.cluster_rows(w, g, BITS, 4, s=s, want_codes=False)["centroids"].astype(np.float32)
+    _emit_both(ctx, oracle, w, (np.arange(rows) % 4 + 1).astype(np.uint8), cent32, BITS, s=s)
 
 
 def test_elements_exactly_at_midpoints(ctx, oracle):

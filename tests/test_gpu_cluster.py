@@ -140,6 +140,25 @@ def test_rows_spread_and_clumped_in_one_matrix(ctx, oracle, cols, scaled):
     check_cluster(ora, cent, err, codes, _values(w, s), BITS, label=f"cols={cols} scaled={scaled}")
 
 
+@pytest.mark.parametrize("cols", [512, 1001, 3584, 4096, 4097])
+@pytest.mark.parametrize("scaled", [False, True])
+def test_matrices_at_odd_addresses(ctx, oracle, cols, scaled):
+    """Matrices that begin one element into an allocation: no row is aligned for vector loads."""
+    w, g = inputs.make_rows(5, cols, 9500 + cols)
+    s = inputs.make_scale(cols, 29) if scaled else None
+    ora = oracle.cluster_rows(w, g, BITS, 8, s=s)
+    W = torch.empty(w.size + 1, dtype=torch.float16, device="cuda")[1:].view(w.shape)
+    G = torch.empty(g.size + 1, dtype=torch.float32, device="cuda")[1:].view(g.shape)
+    W.copy_(torch.from_numpy(w))
+    G.copy_(torch.from_numpy(g))
+    ctx.reserve(*w.shape)
+    ctx.apply_scale(torch.from_numpy(s).cuda() if scaled else None)
+    cent, codes, err = ctx.cluster_rows(W, G, BITS, 8, want_codes=True)
+    assert ctx.get_status() == 0
+    ctx.apply_scale(None)
+    check_cluster(ora, cent.cpu().numpy(), err.cpu().numpy(), codes.cpu().numpy(), _values(w, s), BITS, label=f"cols={cols} scaled={scaled}")
+
+
 def test_scaled_long_rows(ctx, oracle):
     cols = 22016
     w, g = inputs.make_rows(8192, cols, 5001, 0, 12, importance_sigma=2.0)
