@@ -274,6 +274,8 @@ __global__ void __launch_bounds__(UT) skim_unpack_kernel(UnpackArgs a, int steps
     }
 }
 
+constexpr size_t UNPACK_STATIC_SMEM = UW * 17 * sizeof(float);
+
 // with few rows several warps share one
 int unpack_parts(const skim_ctx *ctx, int64_t rows, int steps)
 {
@@ -284,16 +286,16 @@ int unpack_parts(const skim_ctx *ctx, int64_t rows, int steps)
 
 int launch_unpack(skim_ctx *ctx, void (*kernel)(UnpackArgs, int, int), const UnpackArgs &a, int steps, size_t smem)
 {
-    // set on every launch: a host-side call of microseconds, and no state shared between contexts
-    SKIM_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // Set on every launch that needs it, to the same value: no state shared between contexts.  The calls on small matrices are bound
+    // by the host, and this one is a twelfth of their time, so it is left out within the 48 KB that need no permission.
+    if (smem + UNPACK_STATIC_SMEM > 48 * 1024)
+        SKIM_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->max_smem_optin - (int)UNPACK_STATIC_SMEM));
     const unsigned blocks = (unsigned)(a.rows < ctx->sm_count ? a.rows : ctx->sm_count);      // one block per SM
     kernel<<<blocks, UT, smem, ctx->stream>>>(a, steps, unpack_parts(ctx, a.rows, steps));
     SKIM_CUDA_OK(cudaGetLastError());
     ctx->launches += 1;
     return SKIM_OK;
 }
-
-constexpr size_t UNPACK_STATIC_SMEM = UW * 17 * sizeof(float);
 
 }  // namespace
 
