@@ -25,15 +25,16 @@ namespace {
 
 struct DeviceGuard {
     int prev;
-    bool ok;
-    explicit DeviceGuard(int dev) : prev(-1), ok(false)
+    bool ok, changed;
+    explicit DeviceGuard(int dev) : prev(-1), ok(false), changed(false)
     {
         if (cudaGetDevice(&prev) != cudaSuccess) return;
-        ok = (prev == dev) || (cudaSetDevice(dev) == cudaSuccess);
+        changed = prev != dev;
+        ok = !changed || (cudaSetDevice(dev) == cudaSuccess);
     }
     ~DeviceGuard()
     {
-        if (ok && prev >= 0) cudaSetDevice(prev);
+        if (changed) cudaSetDevice(prev);
     }
 };
 

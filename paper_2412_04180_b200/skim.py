@@ -7,6 +7,7 @@ loudly when the library has not been built, and every call needs CUDA tensors.
 from __future__ import annotations
 
 import ctypes as C
+import functools
 import os
 
 import torch
@@ -46,6 +47,11 @@ def lib():
         _lib.skim_strerror.argtypes = [C.c_int]
         _lib.skim_launch_count.restype = C.c_int64
         _lib.skim_launch_count.argtypes = [C.c_void_p]
+        # the calls that a decoded token makes are bound by the host: declared types let plain integers through, which
+        # costs a third of wrapping every argument
+        vp, i64 = C.c_void_p, C.c_int64
+        _lib.skim_dequantize.argtypes = [vp] * 6 + [i64, i64, vp, C.c_int, vp, i64]
+        _lib.skim_matvec.argtypes = [vp] * 7 + [i64, i64, vp, C.c_int, vp]
     return _lib
 
 
@@ -56,8 +62,13 @@ def _ptr(t):
 
 
 def _bits(bit_set):
-    arr = (C.c_int * len(bit_set))(*[int(b) for b in bit_set])
-    return arr, len(bit_set), sum(1 << int(b) for b in bit_set)
+    return _bits_of(tuple(int(b) for b in bit_set))
+
+
+@functools.lru_cache(maxsize=64)
+def _bits_of(widths):
+    """The C array of the widths (the library only reads it), their number and the number of centroids."""
+    return (C.c_int * len(widths))(*widths), len(widths), sum(1 << b for b in widths)
 
 
 def _chk(rc, where):
@@ -266,9 +277,9 @@ class Skim:
             _dev(s, torch.float32, "s")
         if out is None:
             out = torch.empty((rows, cols), dtype=torch.float16, device=q["packed"].device)
-        _chk(lib().skim_dequantize(self._h, _ptr(q["packed"]), _ptr(q["row_order"]), _ptr(q["group_info"]),
-                                   _ptr(q["lut"]), _ptr(s), C.c_int64(rows), C.c_int64(cols), arr, C.c_int(nb),
-                                   _ptr(out), C.c_int64(out.stride(0))), "skim_dequantize")
+        _chk(lib().skim_dequantize(self._h, q["packed"].data_ptr(), q["row_order"].data_ptr(), q["group_info"].data_ptr(),
+                                   q["lut"].data_ptr(), None if s is None else s.data_ptr(), rows, cols, arr, nb,
+                                   out.data_ptr(), out.stride(0)), "skim_dequantize")
         return out
 
     def matvec(self, q, cols, bit_set, x, s=None, out=None):
@@ -280,9 +291,9 @@ class Skim:
             _dev(s, torch.float32, "s")
         if out is None:
             out = torch.empty((rows,), dtype=torch.float32, device=x.device)
-        _chk(lib().skim_matvec(self._h, _ptr(q["packed"]), _ptr(q["row_order"]), _ptr(q["group_info"]), _ptr(q["lut"]),
-                               _ptr(s), _ptr(x), C.c_int64(rows), C.c_int64(cols), arr, C.c_int(nb), _ptr(out)),
-             "skim_matvec")
+        _chk(lib().skim_matvec(self._h, q["packed"].data_ptr(), q["row_order"].data_ptr(), q["group_info"].data_ptr(),
+                               q["lut"].data_ptr(), None if s is None else s.data_ptr(), x.data_ptr(), rows, cols, arr, nb,
+                               out.data_ptr()), "skim_matvec")
         return out
 
     def scale_update(self, W, importance, labels, alpha, steps=120, lr0=0.01, decay=0.5, decay_every=40,
