@@ -150,7 +150,9 @@ int skim_cluster_rows_exact(skim_ctx *ctx, const uint16_t *W, const float *impor
  * Algorithm 1.  All rows start at b_min; the row with the largest error reduction
  * err[i][b_i] - err[i][b_i+1] (differences taken in binary64; lowest row index on ties) gains a
  * bit until the total is T = floor(rows * budget + 1e-6).  Reductions may be negative.
- *   err         [rows][n_bits] binary32 (column u is width bit_set[u])
+ *   err         [rows][n_bits] binary32 (column u is width bit_set[u]).  An entry may be infinite, e.g. to rule a
+ *               width out; a row with a reduction that is not a number (two infinities side by side, NaN) gets
+ *               some width of bit_set, the total still being T.
  *   bits        out [rows] uint8
  *   total_bits  host out, may be NULL: T (computed on the host, no synchronisation)
  */

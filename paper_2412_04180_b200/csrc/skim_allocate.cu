@@ -10,11 +10,13 @@
 // resolved by row-major rank.  One block: the work is latency, and the fewer passes the better -- an 8-bit radix select,
 // whose first digits are the same for all keys, took eight (4096 rows: 20.5 us; 22 016 rows: 108 us).
 #include "skim_internal.cuh"
+#include "skim_key_range.h"
 
 namespace {
 
 constexpr int AT = 1024;  // threads of the single block
-constexpr int BINS = 2048;
+constexpr int BINS = 1 << SkimKeyRange::PART_BITS;
+static_assert(BINS == 2 * AT, "a thread has two bins");
 constexpr int LIST_CAP = 512;    // live keys that are ranked directly
 
 __device__ __forceinline__ unsigned long long ordered_bits(double v)
@@ -59,7 +61,7 @@ __global__ void __launch_bounds__(AT) skim_allocate_kernel(const float *__restri
     constexpr int STEPS_MAX = SKIM_MAX_NBITS - 1;
     constexpr int NC = CACHE_ROWS > 0 ? CACHE_ROWS : 1;
     __shared__ unsigned int hist[BINS];
-    __shared__ unsigned long long s_lo, s_hi;    // the live keys lie in [s_lo, s_hi]
+    __shared__ SkimKeyRange s_range;             // of the live keys
     __shared__ long long s_need;                 // the wanted key is the s_need-th largest of them
     __shared__ unsigned int s_live;
     __shared__ long long wsum[AT / 32];
@@ -140,17 +142,16 @@ __global__ void __launch_bounds__(AT) skim_allocate_kernel(const float *__restri
             lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, off));
             hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, off));
         }
-        if (lane == 0) { s_lo = lo; s_hi = hi; s_need = K; s_live = (unsigned)min((long long)n * steps, 0xffffffffll); s_count = 0u; }
+        if (lane == 0) { s_range.lo = lo; s_range.hi = hi; s_need = K; s_live = (unsigned)min((long long)n * steps, 0xffffffffll); s_count = 0u; }
     }
     __syncthreads();
 
     // ---- narrow the range down to the part that holds the K-th largest key
-    while (s_live > (unsigned)LIST_CAP && s_lo < s_hi) {
-        const unsigned long long base = s_lo, span = s_hi - s_lo;
-        const int bits_used = 64 - __clzll((long long)span), shift = bits_used > 11 ? bits_used - 11 : 0;
+    while (s_live > (unsigned)LIST_CAP && s_range.lo < s_range.hi) {
+        const SkimKeyRange range = s_range;
+        const int shift = range.shift();
         each_key([&](unsigned long long key) {
-            const unsigned long long d = key - base;            // keys below the range wrap round to large numbers
-            if (d <= span) atomicAdd(&hist[(unsigned)(d >> shift)], 1u);
+            if (range.holds(key)) atomicAdd(&hist[range.part_of(key, shift)], 1u);
         });
         __syncthreads();
         // suffix counts: thread t has bins 2t and 2t + 1
@@ -171,27 +172,25 @@ __global__ void __launch_bounds__(AT) skim_allocate_kernel(const float *__restri
         __syncthreads();
         if (above < need && need <= above + c1 + c0) {
             const bool upper = need <= above + c1;
-            const unsigned long long first = base + ((unsigned long long)(2 * tid + (upper ? 1 : 0)) << shift);
             s_need = upper ? need - above : need - above - c1;
             s_live = upper ? c1 : c0;
-            s_lo = first;
-            s_hi = min(base + span, first + ((1ull << shift) - 1ull));
+            s_range = range.part(2u * tid + (upper ? 1u : 0u), shift);
         }
         __syncthreads();
     }
-    if (s_lo == s_hi) {
+    if (s_range.lo == s_range.hi) {
         // one value is left: all live keys equal it
-        if (tid == 0) { s_thr = s_lo; s_take = s_need; }
+        if (tid == 0) { s_thr = s_range.lo; s_take = s_need; }
     } else {
-        const unsigned long long base = s_lo, span = s_hi - s_lo;
+        const SkimKeyRange range = s_range;
         each_key([&](unsigned long long key) {
-            if (key - base <= span) {
+            if (range.holds(key)) {
                 const unsigned at = atomicAdd(&s_count, 1u);
-                if (SKIM_IDX(at, LIST_CAP, nullptr)) list[at] = key;
+                if (at < (unsigned)LIST_CAP) list[at] = key;      // (there are s_live <= LIST_CAP of them)
             }
         });
         __syncthreads();
-        const unsigned cnt = s_count;
+        const unsigned cnt = min(s_count, (unsigned)LIST_CAP);
         if ((unsigned)tid < cnt) {
             const unsigned long long key = list[tid];
             unsigned greater = 0u, equal = 0u;

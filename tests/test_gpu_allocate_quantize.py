@@ -66,6 +66,32 @@ def test_allocation_of_clumped_keys(ctx, oracle, rows, kind):
         np.testing.assert_array_equal(got, want, err_msg=f"budget={budget}")
 
 
+@pytest.mark.parametrize("rows", [3, 170, 2000, 4097])
+def test_allocation_of_infinite_entries(ctx, oracle, rows):
+    """Widths ruled out by an infinite error, beside a negative gain: the keys span nearly all of 64 bits.  (The selection's
+    arithmetic over the same tables is checked on the host in test_key_range_cpu.py.)"""
+    rng = np.random.default_rng(rows)
+    err = np.sort(rng.random((rows, 4)), axis=1)[:, ::-1].astype(np.float32)
+    tables = []
+    for share_first, share_last in ((1.0, 0.0), (0.4, 0.0), (0.4, 0.3)):
+        e = err.copy()
+        e[rng.random(rows) < share_first, 0] = np.inf
+        e[rng.random(rows) < share_last, 3] = np.inf
+        e[rows // 2] = [0.5, 0.501, 0.4, 0.3]
+        tables.append(e)
+    nan = tables[0].copy()
+    nan[::3, 1] = np.inf                                              # inf - inf is not a number
+    nan[1::7, 2] = np.nan
+    for budget in (1.0 + 1.0 / rows, 1.5, 2.25, 3.0, 4.0 - 1.0 / rows):
+        for t, e in enumerate(tables):
+            want, total = oracle.allocate_bits(e, 1, budget)
+            got, gtotal = _alloc(ctx, e, BITS, budget)
+            assert gtotal == total
+            np.testing.assert_array_equal(got, want, err_msg=f"table {t} budget={budget}")
+        got, gtotal = _alloc(ctx, nan, BITS, budget)                  # no order to compare: the total and the widths' range
+        assert int(got.sum()) == gtotal and got.min() >= 1 and got.max() <= 4
+
+
 @pytest.mark.parametrize("rows", [1, 33, 1000, 4096, 9000])
 def test_floor_started_allocation_matches_oracle(ctx, oracle, rows):
     """skim_allocate_bits_floor: every row starts at floor(budget); bit-exact against the oracle's loop."""
