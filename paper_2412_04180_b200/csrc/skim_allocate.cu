@@ -303,7 +303,11 @@ __global__ void __launch_bounds__(AT) skim_allocate_optimal_kernel(const float *
         if (cost) *cost = prev[K];
         long long s = K;
         for (int64_t i = n - 1; i >= 0; --i) {
-            const int u = choice[(size_t)i * (size_t)(K + 1) + (size_t)s];
+            // s <= (i + 1)(nb - 1) here, so its choice has been written.  Where every way to s costs infinitely much no choice was
+            // better than 0: the rows before take at most i (nb - 1), so that s stays a state that they have
+            const long long least = s - i * (nb - 1);
+            long long u = choice[(size_t)i * (size_t)(K + 1) + (size_t)s];
+            if (u < least) u = least;
             bits[i] = (uint8_t)(bmin + u);
             s -= u;
         }

@@ -143,6 +143,28 @@ def test_optimal_allocation_matches_oracle(ctx, oracle, rows):
     np.testing.assert_array_equal(got.cpu().numpy(), want)
 
 
+@pytest.mark.parametrize("rows", [1, 2, 300])
+def test_optimal_allocation_of_infinite_entries(ctx, oracle, rows):
+    """Infinite errors: with a finite way to the total the oracle's result; without one (a row that is infinite at every width)
+    some widths of the set with the right total.  The backward walk restated on the host: test_optimal_walk in test_key_range_cpu.py."""
+    rng = np.random.default_rng(rows)
+    err = np.sort(rng.random((rows, 4)), axis=1)[:, ::-1].astype(np.float32)
+    err[rng.random(rows) < 0.3, 3] = np.inf
+    none = err.copy()
+    none[rows // 2] = np.inf
+    none[0] = np.nan
+    for budget in (1.0, 1.5, 2.25, 3.0):
+        want, total, cost = oracle.allocate_optimal(err, 1, budget)
+        got, gtotal, gcost = ctx.allocate_optimal(torch.from_numpy(err).cuda(), BITS, budget)
+        assert gtotal == total and gcost == cost
+        np.testing.assert_array_equal(got.cpu().numpy(), want)
+    for table in (none, np.full((rows, 4), np.inf, np.float32)):
+        for budget in (1.0, 1.5, 2.25, 3.0, 4.0):
+            got, gtotal, _ = ctx.allocate_optimal(torch.from_numpy(table).cuda(), BITS, budget)
+            got = got.cpu().numpy()
+            assert int(got.sum()) == gtotal and got.min() >= 1 and got.max() <= 4
+
+
 @pytest.mark.parametrize("bit_set", [[2, 3], [1, 2, 3], [3, 4], [4]])
 def test_allocation_other_bit_sets(ctx, oracle, bit_set):
     err = inputs.make_error_table(777, len(bit_set), 9, monotone=False, ties=True)

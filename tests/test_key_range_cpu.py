@@ -96,6 +96,24 @@ def test_selection_stays_inside_its_list(select, name):
     _check(select, keys)
 
 
+@pytest.mark.parametrize("nb", [2, 3, 4])
+def test_optimal_walk(nb):
+    """The dynamic programme's backward walk where choices carry no information (every way infinitely dear: all choices 0, or any
+    other value a state can have): the state stays one that the rows before can have, and the walk ends at 0."""
+    rng = np.random.default_rng(nb)
+    for rows in (1, 2, 5, 40):
+        for K in range(0, rows * (nb - 1) + 1, max(1, rows // 5)):
+            for any_choice in (False, True):
+                s = K
+                for i in range(rows - 1, -1, -1):
+                    assert 0 <= s <= min(K, (i + 1) * (nb - 1))          # the states whose choice the kernel writes
+                    u = int(rng.integers(0, min(s, nb - 1) + 1)) if any_choice else 0
+                    u = max(u, s - i * (nb - 1))
+                    assert 0 <= u <= nb - 1
+                    s -= u
+                assert s == 0
+
+
 @pytest.mark.parametrize("lo,hi", [(0, 2**64 - 1), (2**63 + 12345, 2**64 - 1), (2**64 - 4096, 2**64 - 1), (0, 4095), (7, 2**53 + 9)])
 def test_selection_over_extreme_ranges(select, lo, hi):
     rng = np.random.default_rng(lo % 1000 + 1)
