@@ -311,7 +311,9 @@ int skim_scale_update(skim_ctx *ctx, const uint16_t *W, const float *importance,
  *
  * skim_err_lfull:  err[i * err_stride] = ( sum_j sum_k D_ij H_jk D_ik ) / 4^exp2
  *   H          [cols][ldh] binary16 (device), the Gram matrix X X^T of the layer's inputs; only its symmetric
- *              part matters.  16-byte aligned, ldh % 8 == 0.  cols % 8 == 0.
+ *              part matters.  16-byte aligned, ldh % 8 == 0.  cols % 8 == 0.  Where H equals its transpose bit for bit
+ *              (copy one triangle over the other if it was computed in full) a large call does half of the
+ *              products: 4096 x 11008 0.38 instead of 0.71 ms.
  *   scratch    device, 256-byte aligned, at least skim_err_lfull_bytes(rows, cols) bytes
  *   err        out binary32; err_stride elements between rows (n_bits to fill one column of the error table)
  * The products are exact in binary32 and are accumulated in binary32 by the tensor cores (cols terms per output

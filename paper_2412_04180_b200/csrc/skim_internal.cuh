@@ -41,7 +41,7 @@ struct skim_ctx {
 // Workspace layout (all offsets 256-byte aligned), carved per call for the call's (rows, cols).
 // The status word and the reciprocal scale sit at fixed offsets, so they persist across calls.
 struct SkimWorkspace {
-    unsigned long long *status;  // word 0: status bits; words 1, 2: Lloyd iterations run and rows counted (skim_lloyd_iterations); word 4: length of sort_list
+    unsigned long long *status;  // word 0: status bits; words 1, 2: Lloyd iterations run and rows counted (skim_lloyd_iterations); word 4: length of sort_list; word 5: skim_lfull_leave_flag
     float *rscale;               // [cols]     reciprocal of the installed scale vector
     int32_t *row_pos;            // [rows]     packed-row index of every source row
     double *alpha64;             // [cols]     scale-update master copy of alpha
@@ -76,6 +76,9 @@ __host__ __device__ static inline int64_t skim_ordered_stride(int64_t cols)
 {
     return (cols + SKIM_ORDER_UNIT - 1) / SKIM_ORDER_UNIT * SKIM_ORDER_UNIT + 16 * SKIM_ORDER_UNIT;
 }
+
+// The half contraction's leave flag (skim_lfull.cu), in the status words at the start of the workspace: zero between calls.
+static inline unsigned *skim_lfull_leave_flag(void *ws) { return (unsigned *)((unsigned long long *)ws + 5); }
 
 static inline size_t skim_align256(size_t v) { return (v + 255) & ~(size_t)255; }
 

@@ -148,6 +148,7 @@ constexpr int UMMA_K = 16;
 constexpr int A_BYTES = CM * BK * 2, BOX_BYTES = CB * BK * 2, STAGE_BYTES = A_BYTES + 2 * BOX_BYTES;     // per CTA
 constexpr int EPI_WARPS = 8;                    // two for every quarter of the accumulator's rows, each with half of the columns
 constexpr int GEMM_THREADS = (2 + EPI_WARPS) * 32;
+constexpr int LEAVE_POLL = 8;                   // the producer of the half contraction looks at the leave flag every so many K blocks
 constexpr int CHECK_WARPS = 4;                  // further warps of the half contraction: they compare H with its transpose
 constexpr int SPLIT_MAX = 8;                    // ranges of K a tile of the last round is cut into, at most
 constexpr int HALF_MIN_ROWS = 768, HALF_MIN_NT = 4;
@@ -172,10 +173,14 @@ struct GemmSync {
     uint64_t empty[STAGES];
     uint64_t tmem_full[2];
     uint64_t tmem_empty[2];
+    uint64_t drained;            // half contraction: the MMAs issued are done (both CTAs)
     uint32_t tmem_base;
-    int abort;
-    int asym;
+    int abort;                   // a wait ran out
+    int asym;                    // half contraction: this CTA's warps have found (or been told) that H is not symmetric
+    int leave;                   // half contraction: both CTAs stop where they are
+    int issued[2];               // half contraction: K blocks that the CTAs' producers have issued
 };
+static_assert(sizeof(GemmSync) <= 256, "the barriers' part of gemm_smem");
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -218,12 +223,14 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity)
                  : "memory");
     return ok != 0;
 }
-// Bounded wait.  False when the block is aborting (this wait ran out, or another role's did).
-__device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, volatile int *abort_flag)
+// Bounded wait.  False when the block is aborting (this wait ran out, or another role's did) or, unless it is to go on all
+// the same, leaving.
+__device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, GemmSync &sync, bool leaving_too = false)
 {
+    volatile int *abort_flag = &sync.abort, *leave_flag = &sync.leave;
     const long long t0 = clock64();
     while (!mbar_try_wait(bar, parity)) {
-        if (*abort_flag) return false;
+        if (*abort_flag || (*leave_flag && !leaving_too)) return false;
         if (clock64() - t0 > WAIT_LIMIT_CYCLES) {
             *abort_flag = 1;
             return false;
@@ -231,6 +238,18 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, volati
     }
     return true;
 }
+__device__ __forceinline__ void store_cluster(uint32_t addr, int v)
+{
+    asm volatile("st.relaxed.cluster.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+// A flag in global memory that other blocks of the launch may set.
+__device__ __forceinline__ unsigned flag_load(const unsigned *p)
+{
+    unsigned v;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void flag_set(unsigned *p) { asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(1u) : "memory"); }
 
 // Into this CTA's shared memory; the bytes are counted by the mbarrier at `bar` (an address in either CTA of the pair).
 __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, uint32_t bar, int x, int y)
@@ -308,8 +327,9 @@ struct GemmArgs {
     float *Y;                // optional [rows][ldy]: the product D H itself (the scaling-vector update needs it)
     int64_t ldy;
     SkimLfullClusters cl;    // with Y, optional: sums of Y alpha by cluster
-    int *asym;               // [asym_n] per block of the half contraction: H is not symmetric in the part it compared
+    int *asym;               // [asym_n] per block of the half contraction: H is not symmetric in the part it compared, or the block left
     int asym_n;
+    unsigned *leave;         // half contraction: some block has found H not symmetric (zero between calls)
     int piece_kb;            // half contraction: a tile's list of K blocks is cut into pieces of about this length
     unsigned long long *status;
 };
@@ -389,15 +409,17 @@ __device__ __forceinline__ int unit_index(int t, int nunits)
 
 // Compares H with its transpose, one warp per pair of blocks H[32 I .. +32][64 J .. +64] and H[64 J ..][32 I ..] at or
 // above the diagonal.  A lane compares an 8 x 8 sub-block against its mirror image in registers; whole sectors on either side.
-// The ragged end (fewer than 8 rows or columns cannot occur: cols is a multiple of 8).  Returns nonzero on a difference.
-__device__ __forceinline__ uint32_t compare_transpose(const uint16_t *H, int64_t ldh, int cols, int first, int step)
+// The ragged end (fewer than 8 rows or columns cannot occur: cols is a multiple of 8).  True, and *leave set, at the first
+// difference; true as well as soon as some other warp of the launch has set it.
+__device__ __forceinline__ bool compare_transpose(const uint16_t *H, int64_t ldh, int cols, int first, int step, unsigned *leave)
 {
     const int lane = threadIdx.x & 31;
     const int ni = (cols + 31) / 32, nj = (cols + 63) / 64;
-    uint32_t diff = 0u;
     for (long long t = first; t < (long long)ni * nj; t += step) {
         const int I = (int)(t % ni), J = (int)(t / ni);
         if (64 * J + 64 <= 32 * I) continue;                  // below the diagonal: the mirror pair is compared
+        const unsigned left = flag_load(leave);
+        uint32_t diff = 0u;
         const int r0 = 32 * I + (lane >> 3) * 8, c0 = 64 * J + (lane & 7) * 8;
         if (r0 < cols && c0 < cols) {
             uint4 x[8], y[8];
@@ -418,8 +440,12 @@ __device__ __forceinline__ uint32_t compare_transpose(const uint16_t *H, int64_t
                 }
             }
         }
+        if (__any_sync(0xffffffffu, (diff | left) != 0u)) {
+            if (lane == 0) flag_set(leave);
+            return true;
+        }
     }
-    return diff;
+    return false;
 }
 
 // Adds y_j alpha_j of 32 consecutive columns to the row's sums by cluster (slot k of this thread at slot[k * CM]).  The
@@ -464,8 +490,10 @@ __device__ __forceinline__ bool epilogue_barrier_or(bool v)
 }
 __device__ __forceinline__ void epilogue_barrier() { asm volatile("bar.sync 1, %0;" ::"n"(EPI_WARPS * 32) : "memory"); }
 
-// HALF: the half contraction for a symmetric H, launched first; it leaves in a.asym whether H was.  Otherwise the full
-// contraction; with a.asym given it is the fallback of a half launch and leaves at once unless H was not symmetric.
+// HALF: the half contraction for a symmetric H, launched first; a.asym then says whether H was.  At the first difference that
+// the checking warps find all pairs stop where they are (within a few K blocks), so that an H that is symmetric up to rounding
+// only costs little more than the full contraction.  !HALF: the full contraction; with a.asym given it is the fallback of a
+// half launch and returns at once unless H was not symmetric.
 template <bool HALF>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS + (HALF ? CHECK_WARPS * 32 : 0), 1)
 skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, GemmArgs a, const uint16_t *H, int64_t ldh)
@@ -476,7 +504,6 @@ skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
     GemmSync &sy = *reinterpret_cast<GemmSync *>(tiles + (size_t)NST * STAGE_BYTES);
     float *dot_s = reinterpret_cast<float *>(tiles + (size_t)NST * STAGE_BYTES + 256);                           // [CM]
     EpilogueSmem &ep = *reinterpret_cast<EpilogueSmem *>(tiles + (size_t)NST * STAGE_BYTES + 256 + CM * sizeof(float));   // not for HALF
-    volatile int *abort_flag = &sy.abort;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nkb = (a.cols + BK - 1) / BK;
     const int ntiles = a.mt * a.nt;
@@ -488,6 +515,7 @@ skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
     } else if (a.asym) {
         int any = 0;
         for (int i = threadIdx.x; i < a.asym_n; i += GEMM_THREADS) any |= a.asym[i];
+        if (blockIdx.x == 0 && threadIdx.x == 0) *a.leave = 0u;
         if (!__syncthreads_or(any)) return;
     }
 
@@ -496,8 +524,10 @@ skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
         // full and tmem_empty are used in the first CTA only; the other two in both
         for (int s = 0; s < NST; ++s) { mbar_init(&sy.full[s], 1); mbar_init(&sy.empty[s], 1); }
         for (int s = 0; s < 2; ++s) { mbar_init(&sy.tmem_full[s], 1); mbar_init(&sy.tmem_empty[s], 2 * EPI_WARPS); }
+        mbar_init(&sy.drained, 1);
         sy.abort = 0;
         sy.asym = 0;
+        sy.leave = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
@@ -510,12 +540,22 @@ skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
     tc_fence_after();
     const uint32_t tmem_base = sy.tmem_base;
 
+    // one K block of operands: this CTA's half of either
+    auto load_block = [&](int stage, int k, int m0, int b0, int boxes) {
+        unsigned char *sa = tiles + (size_t)stage * STAGE_BYTES;
+        if (rank == 0) mbar_expect_tx(&sy.full[stage], 2 * (A_BYTES + boxes * BOX_BYTES));
+        const uint32_t bar = cluster_addr(&sy.full[stage], 0);
+        tma_load_2d(sa, &map_a, bar, k, m0);
+        for (int b = 0; b < boxes; ++b) tma_load_2d(sa + A_BYTES + b * BOX_BYTES, &map_b, bar, k, b0 + b * CB);
+    };
     if (warp == 0) {
-        // ------------------------------------------------------------ TMA producer (one lane): this CTA's half of either operand
+        // ------------------------------------------------------------ TMA producer (one lane)
         if (lane == 0) {
             int stage = 0;
             uint32_t phase = 0;
             bool ok = true;
+            int issued = 0;
+            unsigned left = 0u;                               // the leave flag as it was LEAVE_POLL blocks ago: its load is never waited for
             for (int t = 0; t * ((int)gridDim.x / 2) < nunits && ok; ++t) {
                 const int u = unit_index<HALF>(t, nunits);
                 if (u < 0) continue;
@@ -524,15 +564,23 @@ skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
                 const int boxes = w.n / (2 * CB), b0 = n0 + w.n_off + (int)rank * (w.n / 2);
                 for (int l = w.kb0; l < w.kb1; ++l) {
                     const int kb = HALF ? n0 / BK + l : l;
-                    if (!(ok = mbar_wait(&sy.empty[stage], phase ^ 1u, abort_flag))) break;
-                    unsigned char *sa = tiles + (size_t)stage * STAGE_BYTES;
-                    if (rank == 0) mbar_expect_tx(&sy.full[stage], 2 * (A_BYTES + boxes * BOX_BYTES));
-                    const uint32_t bar = cluster_addr(&sy.full[stage], 0);
-                    tma_load_2d(sa, &map_a, bar, kb * BK, m0);
-                    for (int b = 0; b < boxes; ++b) tma_load_2d(sa + A_BYTES + b * BOX_BYTES, &map_b, bar, kb * BK, b0 + b * CB);
+                    if (HALF && issued % LEAVE_POLL == 0) {
+                        if (left) {
+                            *(volatile int *)&sy.leave = 1;
+                            store_cluster(cluster_addr(&sy.leave, rank ^ 1u), 1);
+                            ok = false;
+                            break;
+                        }
+                        left = flag_load(a.leave);
+                    }
+                    if (!(ok = mbar_wait(&sy.empty[stage], phase ^ 1u, sy))) break;
+                    load_block(stage, kb * BK, m0, b0, boxes);
+                    ++issued;
                     if (++stage == NST) { stage = 0; phase ^= 1u; }
                 }
             }
+            if (HALF)
+                for (uint32_t r = 0; r < 2; ++r) store_cluster(cluster_addr(&sy.issued[rank], r), issued);
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer (one lane of the first CTA)
@@ -546,11 +594,11 @@ skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
                 if (u < 0) continue;
                 const GemmUnit w = HALF ? half_unit(a, half, u, nkb) : unit_of(a, u, nkb);
                 const int as = it & 1;
-                if (!(ok = mbar_wait(&sy.tmem_empty[as], (((uint32_t)it >> 1) & 1u) ^ 1u, abort_flag))) break;
+                if (!(ok = mbar_wait(&sy.tmem_empty[as], (((uint32_t)it >> 1) & 1u) ^ 1u, sy))) break;
                 tc_fence_after();
                 const uint32_t tmem_d = tmem_base + (uint32_t)(as * BN), idesc = umma_idesc(w.n);
                 for (int kb = w.kb0; kb < w.kb1; ++kb) {          // HALF: list positions
-                    if (!(ok = mbar_wait(&sy.full[stage], phase, abort_flag))) break;
+                    if (!(ok = mbar_wait(&sy.full[stage], phase, sy))) break;
                     tc_fence_after();
                     const uint32_t sa = smem_u32(tiles + (size_t)stage * STAGE_BYTES), sb = sa + A_BYTES;
 #pragma unroll
@@ -563,11 +611,12 @@ skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
                 if (ok) umma_commit(&sy.tmem_full[as]);      // the accumulator is complete once all MMAs are
                 ++it;
             }
+            if (HALF) umma_commit(&sy.drained);
         }
     } else if (HALF && warp >= GEMM_THREADS / 32) {
         // ------------------------------------------------------------ H against its transpose, under the contraction
-        const uint32_t diff = compare_transpose(H, ldh, a.cols, (int)blockIdx.x * CHECK_WARPS + warp - GEMM_THREADS / 32, (int)gridDim.x * CHECK_WARPS);
-        if (diff) sy.asym = 1;
+        if (compare_transpose(H, ldh, a.cols, (int)blockIdx.x * CHECK_WARPS + warp - GEMM_THREADS / 32, (int)gridDim.x * CHECK_WARPS, a.leave))
+            sy.asym = 1;
     } else {
         // ------------------------------------------------------------ epilogue: one row per thread, half of the tile's columns
         const int q = warp & 3;                               // the tensor-memory lane quarter this warp may read
@@ -606,7 +655,7 @@ skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
             };
             fetch(c0, dv, lv);
             epilogue_barrier();                               // alpha is in place
-            ok = mbar_wait(&sy.tmem_full[as], ((uint32_t)it >> 1) & 1u, abort_flag);
+            ok = mbar_wait(&sy.tmem_full[as], ((uint32_t)it >> 1) & 1u, sy);
             ok = __all_sync(0xffffffffu, ok);
             float acc = 0.0f;
             if (ok) {
@@ -668,7 +717,25 @@ skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
     // ---------------------------------------------------------------- teardown (every path comes here)
     tc_fence_before();
     __syncthreads();
-    if (HALF && threadIdx.x == 0) a.asym[blockIdx.x] = sy.asym;
+    if (HALF) {
+        // A pair that leaves has copies and MMAs in flight, and one of its producers may be ahead of the other, whose bytes
+        // the pair's mbarriers then still expect.  Both issue as many blocks as the one ahead has (of anything; their stages
+        // are free for both: one commit frees a stage in both CTAs), and wait until all of it has landed and the MMAs are done.
+        cluster_sync();                // the counts and the leave flag are in place
+        if (threadIdx.x == 0) {
+            a.asym[blockIdx.x] = sy.asym | sy.leave;
+            bool ok = !sy.abort;
+            const int most = max(sy.issued[0], sy.issued[1]);
+            for (int b = sy.issued[rank]; b < most && ok; ++b) {
+                ok = mbar_wait(&sy.empty[b % NST], (((uint32_t)(b / NST)) & 1u) ^ 1u, sy, true);
+                if (ok) load_block(b % NST, 0, 0, 0, BN / (2 * CB));
+            }
+            if (rank == 0)
+                for (int b = max(0, most - NST); b < most && ok; ++b) ok = mbar_wait(&sy.full[b % NST], ((uint32_t)(b / NST)) & 1u, sy, true);
+            if (ok) mbar_wait(&sy.drained, 0u, sy, true);
+        }
+        __syncthreads();
+    }
     if (sy.abort) {
         // a wait ran out: give the bulk copies that may still be in flight time to land before the block's
         // shared memory is released (about a millisecond), and report
@@ -861,6 +928,7 @@ int skim_launch_err_lfull(skim_ctx *ctx, const uint16_t *D, int64_t rows, int64_
     // contraction is no slower.
     a.asym = nullptr;
     a.asym_n = 0;
+    a.leave = skim_lfull_leave_flag(ctx->ws);
     a.piece_kb = nkb;
     if (!Y && rows >= HALF_MIN_ROWS && a.nt >= HALF_MIN_NT && ctx->sm_count * sizeof(int) <= HALF_FLAG_BYTES) {
         // pieces of about the full contraction's length (the accumulator's rounding errors grow with it), or half of that

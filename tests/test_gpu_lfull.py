@@ -181,3 +181,63 @@ def test_lfull_half_contraction_of_a_symmetric_matrix(ctx, oracle, rows, cols, s
         H[cols - 1, 0] += np.float16(3.0)
     sel = np.unique(np.concatenate([[0, 127, 128, rows - 1], rng.choice(rows, 20)]))
     _check_err(ctx, oracle, D, H, 8, rows=sel, label=f"{rows}x{cols} {symmetric}")
+
+
+@pytest.mark.parametrize("rows,cols", [(770, 4432), (2100, 4104), (4100, 2056), (16000, 1032)])
+def test_lfull_leaves_the_half_contraction(ctx, oracle, rows, cols):
+    """H that differs from its transpose everywhere by a rounding, or in one entry that is compared early, late or in between: the
+    pairs of CTAs stop at different places, and the full contraction's result is the same bit for bit on every run.  Calls
+    with a symmetric H in between take the half contraction again."""
+    ctx.reserve(rows, cols)
+    rng = np.random.default_rng(rows + cols)
+    D = (rng.standard_normal((rows, cols)) * 2).astype(np.float16)
+    H = inputs.make_gram(cols, 90 + cols)
+    rounding = H.copy()
+    at = rng.random(H.shape) < 0.05
+    rounding[at] = (rounding[at].astype(np.float32) * np.float32(1 + 2.0**-10)).astype(np.float16)
+    variants = [rounding]
+    for i, j in ((1, 0), (cols // 2, cols // 2 + 1), (3, cols - 1), (cols - 1, cols - 9)):
+        h = H.copy()
+        h[i, j] += np.float16(0.5)
+        variants.append(h)
+    Dg, Hg = torch.from_numpy(D).cuda(), torch.from_numpy(H).cuda()
+    sel = np.unique(np.concatenate([[0, 127, 128, rows - 1], rng.choice(rows, 8)]))
+    _check_err(ctx, oracle, D, H, 8, rows=sel, label=f"{rows}x{cols} symmetric")
+    sym = ctx.err_lfull(Dg, Hg, exp2=8)
+    for v, h in enumerate(variants):
+        first = _check_err(ctx, oracle, D, h, 8, rows=sel, label=f"{rows}x{cols} variant {v}").astype(np.float32)
+        hg = torch.from_numpy(h).cuda()
+        for _ in range(6):
+            np.testing.assert_array_equal(ctx.err_lfull(Dg, hg, exp2=8).cpu().numpy(), first)
+            assert torch.equal(ctx.err_lfull(Dg, Hg, exp2=8), sym)
+    assert ctx.get_status() == 0
+
+
+def test_lfull_costs_little_more_for_an_unsymmetric_matrix(ctx):
+    """The half contraction takes about half of the full one's time; a call that has to run the full one after all must not also
+    run the half one to its end (which made it 2.9 times the time of the symmetric call)."""
+    rows, cols = 4096, 8192
+    ctx.reserve(rows, cols)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(5)
+    D = torch.randn((rows, cols), generator=gen, device="cuda").half()
+    X = torch.randn((cols, 64), generator=gen, device="cuda")
+    H = (X @ X.T / 64).half()
+    H = torch.triu(H) + torch.triu(H, 1).T
+    other = H.clone()
+    other[1::3] = (other[1::3].float() * (1 + 2.0**-10)).half()
+
+    def median_ms(h):
+        times = []
+        for _ in range(7):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            ctx.err_lfull(D, h)
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b))
+        return sorted(times)[3]
+
+    median_ms(H)
+    assert median_ms(other) < 2.3 * median_ms(H)
+    assert ctx.get_status() == 0
