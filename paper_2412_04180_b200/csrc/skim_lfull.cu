@@ -152,6 +152,7 @@ constexpr int LEAVE_POLL = 8;                   // the producer of the half cont
 constexpr int CHECK_WARPS = 4;                  // further warps of the half contraction: they compare H with its transpose
 constexpr int SPLIT_MAX = 8;                    // ranges of K a tile of the last round is cut into, at most
 constexpr int HALF_MIN_ROWS = 768, HALF_MIN_NT = 4;
+constexpr double HALF_MIN_PRODUCTS = 1.5e10;    // rows * cols^2
 constexpr size_t HALF_FLAG_BYTES = 4096;         // symmetry flags of up to 1024 blocks
 constexpr int TMEM_COLS = 512;                  // two accumulator stages of BN binary32 columns
 constexpr long long WAIT_LIMIT_CYCLES = 400000000ll;   // about 0.2 s; a whole launch takes milliseconds
@@ -924,13 +925,15 @@ int skim_launch_err_lfull(skim_ctx *ctx, const uint16_t *D, int64_t rows, int64_
     }
     // Half the contraction where H turns out symmetric, as a Gram matrix is.  The comparison of H with its transpose
     // reads all of H (2 B per entry) under a contraction of rows MACs per entry: at the measured rates the two take equally long
-    // near 700 rows; below that, or with so few column tiles that the diagonal blocks are most of the work, the full
-    // contraction is no slower.
+    // near 700 rows (512 x 11008 145 us in full, 158 halved; 768 x 11008 204 and 161).  The further launch, the longer start and
+    // the pair's teardown cost 6 us, so the products saved must take longer: us per call in full and halved, 1536 x 1536 17.6 and 23.0,
+    // 4096 x 1536 25.6 and 29.1, 1024 x 3072 27.1 and 29.2, 3072 x 2048 29.2 and 31.3, 4096 x 2048 37.3 and 35.2, 2048 x 3072
+    // 39.1 and 37.4, 8192 x 1536 44.5 and 39.4, 1024 x 4096 53.8 and 42.5.
     a.asym = nullptr;
     a.asym_n = 0;
     a.leave = skim_lfull_leave_flag(ctx->ws);
     a.piece_kb = nkb;
-    if (!Y && rows >= HALF_MIN_ROWS && a.nt >= HALF_MIN_NT && ctx->sm_count * sizeof(int) <= HALF_FLAG_BYTES) {
+    if (!Y && rows >= HALF_MIN_ROWS && a.nt >= HALF_MIN_NT && (double)rows * (double)cols * (double)cols >= HALF_MIN_PRODUCTS && ctx->sm_count * sizeof(int) <= HALF_FLAG_BYTES) {
         // pieces of about the full contraction's length (the accumulator's rounding errors grow with it), or half of that
         // where it balances the blocks clearly better
         double best = 0.0;
