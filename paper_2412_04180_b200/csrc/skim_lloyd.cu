@@ -382,7 +382,14 @@ __device__ __forceinline__ void lloyd_warp(const unsigned char *rec, const typen
         // a cluster without weight keeps its centroid.  S0 is a difference of rounded prefix sums: over a
         // run of zero importances that crosses a group or segment border it is rounding noise of either
         // sign, not 0, so "has weight" means: above 2^-40 of the prefix it was taken from
-        if (normal && S0 > P0 * 0x1p-40) c = (float)quotient(S1, S0);
+        // Likewise S1 over a run of zeros (a pruned row): its terms are 0 and the prefixes equal but for their rounding, about 2^-49
+        // of them.  The mean is 0 then, not that noise: zeros lie on the midpoint of a centroid 0 and its copies (the start
+        // values repeat), which decides where they all go.  (The centroid moves by 2^-46 P1 / S0 at most, elsewhere too.)
+        const bool zero_mean = fabs(S1) <= fabs(P1) * 0x1p-46;
+        if (normal && S0 > P0 * 0x1p-40) {
+            c = (float)quotient(S1, S0);
+            if (zero_mean) c = 0.0f;
+        }
     }
     sm.errs[lane] = err_j;
     sm.tfs[lane] = has_boundary ? tf : INF;

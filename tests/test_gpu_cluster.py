@@ -321,3 +321,48 @@ def test_early_exit_switch_and_iteration_count(ctx):
     assert 0 < it_on <= it_off
     ctx.cluster_rows(W, G, BITS, iters)
     assert ctx.lloyd_iterations() == (0, 0)      # nothing is counted while timing is off
+
+
+@pytest.mark.parametrize("cols", [33, 128, 513, 2049, 3073, 3584, 3585, 5632, 11008, 22528])
+@pytest.mark.parametrize("scaled", [False, True])
+def test_rows_with_zeros(ctx, oracle, cols, scaled):
+    """Pruned rows: few zeros, as many as a bucket takes and one more, half, nearly all, all; zeros of either sign; zeros beside
+    values of one sign only and beside a clump that no bucket spreads."""
+    w, g = inputs.make_rows(14, cols, 9700 + cols)
+    rng = np.random.default_rng(cols)
+    w[w == 0] = np.float16(0.001)
+    for r, zeros in enumerate([1, 15, 16, 31, 32, 48, cols // 2, cols - cols // 10, cols - 1, cols]):
+        w[r, rng.permutation(cols)[:min(zeros, cols)]] = np.float16(0.0 if r % 2 else -0.0)
+    w[6, ::3] = np.where(w[6, ::3] == 0, np.float16(0.0), w[6, ::3])
+    w[10] = np.abs(w[10])
+    w[11] = -np.abs(w[11])
+    w[10:12, ::2] = 0
+    w[12] = 1.0 + np.arange(cols) % 64 / 1024
+    w[12, ::2] = 0
+    w[13, ::4] = 0
+    g[13, ::8] = 0                                                    # some zeros without weight
+    s = inputs.make_scale(cols, 31) if scaled else None
+    ora = oracle.cluster_rows(w, g, BITS, 8, s=s)
+    cent, err, codes = _gpu_cluster(ctx, w, g, BITS, 8, s=s)
+    check_cluster(ora, cent, err, codes, _values(w, s), BITS, label=f"cols={cols} scaled={scaled}")
+    again = _gpu_cluster(ctx, w, g, BITS, 8, s=s)
+    for a, b in zip((cent, err, codes), again):
+        np.testing.assert_allclose(a, b, rtol=1e-6)
+
+
+def test_exact_clustering_of_rows_with_zeros(ctx, oracle):
+    """All buckets in order (the exact kernel reads whole rows in order), with the zeros between them."""
+    w, g = inputs.make_rows(5, 600, 9800)
+    s = inputs.make_scale(600, 37)
+    for r, step in enumerate((2, 3, 5)):
+        w[r, ::step] = 0
+    w[3] = np.abs(w[3])
+    w[3, ::2] = 0
+    ctx.reserve(*w.shape)
+    for scale in (None, s):
+        ctx.apply_scale(torch.from_numpy(scale).cuda() if scale is not None else None)
+        cent, err = ctx.cluster_rows_exact(torch.from_numpy(w).cuda(), torch.from_numpy(g).cuda(), BITS)
+        want = oracle.cluster_rows_exact(w, g, BITS, s=scale)
+        np.testing.assert_allclose(err.cpu().numpy(), want["err"], rtol=1e-6, atol=1e-12)
+    ctx.apply_scale(None)
+    assert ctx.get_status() == 0
