@@ -14,8 +14,10 @@
 //
 // Buckets: v = 1 + |x| / s with s half a standard deviation (from the mean of |x|).  The bits of v grow with |x|: the
 // first three octaves, v in [1, 8), i.e. |x| up to 3.5 deviations, have N/8 buckets each on either side of zero, the next
-// eight share N/8 (N = 32 per thread).  A row whose values this cannot spread (a bucket with BUCKET_LIMIT elements, or 32
-// in three neighbouring ones: few distinct values, a clump) is put on a list and sorted by the radix kernel of skim_cluster.cu.
+// eight share N/8 (N = 32 per thread).  A row whose values this cannot spread (a bucket with BUCKET_LIMIT elements, or 32 in
+// three neighbouring ones: few distinct values, a clump) is put on a list, for the fp16-key kernel of skim_cluster16.cu or, where
+// scaled, the radix kernel of skim_cluster.cu.  Such a matrix takes 1.1 to 1.4 times what those kernels alone would (sort of 4096
+// rows of a few nearby values, us: 2000 columns 169, 3000 columns 256, 11008 scaled 1281; a bell-shaped row 63, 93, 349).
 //
 // Zeros (a pruned matrix) are one value and need no bucket: a row that cannot be spread and has zeros is read again and spread with
 // its zeros between the negative and the positive buckets in column order, by ballots, the scale taken from the other elements.
@@ -100,6 +102,7 @@ __device__ __forceinline__ int bucket_base(const uint32_t *cnt, int b)
 
 struct Spread {
     bool done;          // false: the row cannot be spread
+    bool zeros_only;    // ... but perhaps if its zeros are kept apart
     unsigned bad;
     float inv_s;        // of the buckets
 };
@@ -120,7 +123,7 @@ __device__ __forceinline__ Spread spread_row(const uint16_t *Wr, const float *Gr
     float *red = reinterpret_cast<float *>(ps.segtot);                  // free until the record pass
     uint32_t *wsum = reinterpret_cast<uint32_t *>(ps.segtot) + 32;
     uint32_t *wzeros = bucket_zeros(ps);
-    Spread r{false, 0u, 0.0f};
+    Spread r{false, true, 0u, 0.0f};
 
     // ------------------------------------------------------------ load
     float x[ITEMS];
@@ -157,8 +160,8 @@ __device__ __forceinline__ Spread spread_row(const uint16_t *Wr, const float *Gr
         if (zeros < ZEROS_APART) return r;
         others -= (int)zeros;
     } else {
-        // a row with many zeros is not tried without: one of 32 elements looked at tells
-        if (__syncthreads_count(tid < m && x[0] == 0.0f ? 1 : 0) > THREADS / 32) return r;
+        // a row with many zeros is not tried without: one of 32 elements looked at, and at least ZEROS_APART of them
+        if (__syncthreads_count(tid < m && x[0] == 0.0f ? 1 : 0) >= max(THREADS / 32, (int)ZEROS_APART)) return r;
     }
     sum = 0.0f;
     for (int w = 0; w < NW; ++w) sum += red[w];
@@ -183,6 +186,7 @@ __device__ __forceinline__ Spread spread_row(const uint16_t *Wr, const float *Gr
     __syncthreads();
 
     // ------------------------------------------------------------ counters -> bases
+    bool crowded = false;
     {
         uint4 v[2];
         uint32_t s = 0u, occupied = 0u;
@@ -211,14 +215,18 @@ __device__ __forceinline__ Spread spread_row(const uint16_t *Wr, const float *Gr
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
             const uint32_t c0 = w[u] & 0xffu, c1 = c0 + ((w[u] >> 8) & 0xffu), c2 = c1 + ((w[u] >> 16) & 0xffu), c3 = c2 + (w[u] >> 24);
-            over |= c2 > 31u;
+            crowded |= c2 > 31u;
             w[u] = (run << 15) | c0 | (c1 << 5) | (c2 << 10);
             run += c3;
         }
 #pragma unroll
         for (int u = 0; u < 2; ++u) reinterpret_cast<uint4 *>(cnt)[2 * tid + u] = v[u];
     }
-    if (__syncthreads_or(over ? 1 : 0)) return r;
+    if (__syncthreads_or(over || crowded ? 1 : 0)) {
+        // (zeros fall into the first bucket of thread THREADS / 2)
+        r.zeros_only = !__syncthreads_or(crowded && tid != THREADS / 2 ? 1 : 0);
+        return r;
+    }
 
     // ------------------------------------------------------------ scatter to the buckets
     constexpr int GB = 8;                                           // importances in flight
@@ -292,7 +300,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) skim_sort_bucket_kern
     }
     Spread sp = spread_row<THREADS, ITEMS, SCALED, false>(Wr, Gr, a.rscale, m, a.status);
     bool apart = false;                    // the zeros lie between the negative and the positive buckets
-    if (!sp.done) {
+    if (!sp.done && sp.zeros_only) {
         __syncthreads();
         if (tid == 0) ps.misc[0] = 0;
         sp = spread_row_zeros_apart<THREADS, ITEMS, SCALED>(Wr, Gr, a.rscale, m, a.status);
@@ -300,7 +308,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) skim_sort_bucket_kern
     }
     if (sp.bad) atomicOr(a.status, (unsigned long long)sp.bad);
     if (!sp.done) {
-        // not a row for buckets: the radix kernel takes it
+        // not a row for buckets: the kernel after this one takes it
         if (tid == 0) {
             const int at = atomicAdd(a.sort_count, 1);
             if (SKIM_IDX(at, a.chunk_rows, a.status)) a.sort_list[at] = (int)blockIdx.x;

@@ -7,9 +7,9 @@
 // on one warp while two rows filled an SM's shared memory; from global memory (the hot lines stay in
 // L1) every SM keeps 28 rows in flight.
 //
-// Long unscaled rows are sorted by skim_cluster16.cu, the others by skim_bucket.cu.  This file: the radix
-// sort kernel for the rows the bucket kernel cannot spread (few distinct values, clumps), and the host-side
-// launcher of the whole clustering.
+// Long unscaled rows are sorted by skim_cluster16.cu, the others by skim_bucket.cu.  Rows that the bucket kernel cannot spread (few
+// distinct values, clumps) go on a list: unscaled ones to skim_cluster16.cu, scaled ones to the radix sort kernel of this
+// file.  With it the host-side launcher of the whole clustering.
 //
 // One thread block owns one row at a time.
 //   1. load   the row's (value, importance) pairs into registers; the value is turned into an
@@ -32,20 +32,19 @@ constexpr int BUCKET_UNSCALED_COLS = 3584;
 constexpr int RADIX_BITS = 8;
 constexpr int RADIX = 1 << RADIX_BITS;
 
-template <typename KeyT> struct Passes;
-template <> struct Passes<uint32_t> { static constexpr int N = 4; };
+constexpr int PASSES = 32 / RADIX_BITS;
 
 // Shared-memory layout, computed identically on host and device.
 struct SmemLayout {
     size_t keys, gs, uni, dbase, phase, total;
 };
 
-__host__ __device__ inline SmemLayout smem_layout(int cap, int key_bytes, int nwarps)
+__host__ __device__ inline SmemLayout smem_layout(int cap, int nwarps)
 {
     SmemLayout L;
     size_t off = 0;
     auto take = [&](size_t b) { size_t o = off; off += (b + 15) & ~(size_t)15; return o; };
-    L.keys = take((size_t)cap * key_bytes);
+    L.keys = take((size_t)cap * 4);
     L.gs = take((size_t)cap * 4);
     L.uni = take((size_t)nwarps * RADIX * 4);
     L.dbase = take(RADIX * 4);
@@ -55,16 +54,15 @@ __host__ __device__ inline SmemLayout smem_layout(int cap, int key_bytes, int nw
 }
 
 // Takes the rows of a.sort_list (blocks leave at once when it is empty, the usual case).
-template <typename KeyT, int THREADS, int ITEMS>
+template <int THREADS, int ITEMS>
 __global__ void __launch_bounds__(THREADS) skim_sort_kernel(ClusterArgs a)
 {
-    using K = KeyOps<KeyT>;
-    constexpr int PASSES = Passes<KeyT>::N;
+    using K = KeyOps<uint32_t>;
     constexpr int NW = THREADS / 32;
     constexpr int CAP = THREADS * ITEMS;
     extern __shared__ __align__(16) unsigned char smem[];
-    const SmemLayout L = smem_layout(CAP, (int)sizeof(KeyT), NW);
-    KeyT *skeys = reinterpret_cast<KeyT *>(smem + L.keys);
+    const SmemLayout L = smem_layout(CAP, NW);
+    uint32_t *skeys = reinterpret_cast<uint32_t *>(smem + L.keys);
     float *sg = reinterpret_cast<float *>(smem + L.gs);
     uint32_t *cnt = reinterpret_cast<uint32_t *>(smem + L.uni);
     uint32_t *dbase = reinterpret_cast<uint32_t *>(smem + L.dbase);
@@ -84,7 +82,7 @@ __global__ void __launch_bounds__(THREADS) skim_sort_kernel(ClusterArgs a)
     const float *Gr = a.G + row * a.ld;
 
     // ---------------------------------------------------------------- 1. load
-    KeyT key[ITEMS];
+    uint32_t key[ITEMS];
     float val[ITEMS];
     unsigned bad = 0;
 #pragma unroll
@@ -96,7 +94,7 @@ __global__ void __launch_bounds__(THREADS) skim_sort_kernel(ClusterArgs a)
             if ((h & 0x7c00u) == 0x7c00u) bad |= 1u;
             if (!(g >= 0.0f) || g > 3.0e38f) bad |= 2u;
             float x = __half2float(__ushort_as_half(h));
-            if (a.rscale) x = __fmul_rn(x, a.rscale[e]);
+            x = __fmul_rn(x, a.rscale[e]);
             if (x == 0.0f) x = 0.0f;
             key[i] = K::from_float(x);
             val[i] = g;
@@ -185,21 +183,10 @@ __global__ void __launch_bounds__(THREADS) skim_sort_kernel(ClusterArgs a)
     // ---------------------------------------------------------------- 3. row record for the Lloyd kernel
     if (tid == 0) { ps.misc[0] = 0; ps.misc[1] = 0; }
     __syncthreads();
-    const SortedArrays<KeyT> src{skeys, sg};
-    int nd;
-    if (a.rec_half) {
-        int distinct = 0;
-        for (int p = tid; p < m; p += THREADS) distinct += (p == 0 || skeys[p] != skeys[p - 1]) ? 1 : 0;
-        distinct = __reduce_add_sync(0xffffffffu, distinct);
-        if (lane == 0 && distinct) atomicAdd(&ps.misc[0], distinct);
-        __syncthreads();
-        nd = ps.misc[0];
-        write_row_record_half<KeyT, THREADS>(a, src, ps, nd, local);
-    } else {
-        nd = write_row_record<KeyT, THREADS, true>(a, src, ps, 0, local);
-    }
+    const SortedArrays<uint32_t> src{skeys, sg};
+    const int nd = write_row_record<uint32_t, THREADS, true>(a, src, ps, 0, local);
     if (nd <= 16) {
-        collect_distinct<KeyT, THREADS>(src, m, nd, ps);
+        collect_distinct<uint32_t, THREADS>(src, m, nd, ps);
         write_distinct_values(a, nd, ps.dvals, local);
     }
     __syncthreads();
@@ -209,21 +196,22 @@ __global__ void __launch_bounds__(THREADS) skim_sort_kernel(ClusterArgs a)
 struct Variant {
     int cap;
     int threads;
-    int key_bytes;
     void (*kernel)(ClusterArgs);
 };
 
-#define SKIM_VARIANT(T, I) {T * I, T, 4, skim_sort_kernel<uint32_t, T, I>}
+#define SKIM_VARIANT(T, I) {T * I, T, skim_sort_kernel<T, I>}
 
-const Variant kVariants32[] = {SKIM_VARIANT(512, 8), SKIM_VARIANT(512, 22), SKIM_VARIANT(512, 44)};
-constexpr int kNumVariants = 3;
+// A row pays for the whole size: with 512 x 8, 22 and 44 only, 4096 refused rows of 5600 columns took 1167 us, with 512 x 16 890.
+const Variant kVariants32[] = {SKIM_VARIANT(256, 2), SKIM_VARIANT(256, 8), SKIM_VARIANT(512, 8), SKIM_VARIANT(512, 16), SKIM_VARIANT(512, 22),
+                               SKIM_VARIANT(512, 32), SKIM_VARIANT(512, 44)};
+constexpr int kNumVariants = sizeof(kVariants32) / sizeof(kVariants32[0]);
 
 // Picks the smallest variant that holds `cols` and fits shared memory.
 const Variant *pick_variant(const Variant *table, int64_t cols, int max_smem, size_t *smem)
 {
     for (int v = 0; v < kNumVariants; ++v) {
         if (table[v].cap < cols) continue;
-        const SmemLayout L = smem_layout(table[v].cap, table[v].key_bytes, table[v].threads / 32);
+        const SmemLayout L = smem_layout(table[v].cap, table[v].threads / 32);
         if (L.total <= (size_t)max_smem) { *smem = L.total; return &table[v]; }
     }
     return nullptr;
@@ -280,7 +268,7 @@ int skim_launch_cluster(skim_ctx *ctx, const uint16_t *W, const float *importanc
     const Variant *v = nullptr;
     const bool bucket = scaled || (a.rec_half && cols <= BUCKET_UNSCALED_COLS);
     a.unordered = bucket ? 1 : 0;
-    if (bucket) {
+    if (scaled) {
         v = pick_variant(kVariants32, cols, ctx->max_smem_optin, &smem);
         if (!v) return SKIM_ERR_SHAPE;
         SKIM_CUDA_OK(cudaFuncSetAttribute(v->kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -297,7 +285,8 @@ int skim_launch_cluster(skim_ctx *ctx, const uint16_t *W, const float *importanc
         if (rc) return rc;
         if (bucket) {
             // the rows the buckets could not spread: usually none
-            rc = skim_launch_dependent(ctx, v->kernel, dim3((unsigned)(n < 2 * ctx->sm_count ? n : 2 * ctx->sm_count)), v->threads, smem, a);
+            if (scaled) rc = skim_launch_dependent(ctx, v->kernel, dim3(skim_list_blocks(ctx, v->threads, n)), v->threads, smem, a);
+            else rc = skim_launch_sort16(ctx, a, n, true);
             if (rc) return rc;
         }
         if (tev) SKIM_CUDA_OK(cudaEventRecord(tev[1], ctx->stream));

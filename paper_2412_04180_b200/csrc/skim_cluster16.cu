@@ -128,9 +128,10 @@ struct SortedItems16 {
     __device__ __forceinline__ uint16_t key_at(int p) const { return (uint16_t)(items[p] >> 16); }
 };
 
-// HALF_RECORD: the compact row record, for the Lloyd kernel; else the full one, for the exact kernel.
-template <bool HALF_RECORD, int THREADS, int VEC>
-__global__ void __launch_bounds__(THREADS, 1024 / THREADS) skim_sort16_kernel(ClusterArgs a)
+// One row, by the whole block; local: its index inside the chunk.  FIRST: sets the mbarrier up; parity: of its phase.  False: the
+// importance row never arrived (flagged; the row's record is marked invalid).
+template <bool HALF_RECORD, int THREADS, int VEC, bool FIRST>
+__device__ __forceinline__ bool sort16_row(const ClusterArgs &a, int local, uint32_t parity)
 {
     using K = KeyOps<uint16_t>;
     constexpr int ITEMS = VEC * 8;
@@ -152,8 +153,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) skim_sort16_kernel(Cl
     uint64_t *mbar = reinterpret_cast<uint64_t *>(smem + L.mbar);
     uint32_t *scratch = reinterpret_cast<uint32_t *>(ps.segtot);   // free until the record pass
 
-    skim_let_next_kernel_start();          // (this kernel is an ordinary launch: the one after it waits)
-    const int64_t row = a.row0 + blockIdx.x;
+    const int64_t row = a.row0 + local;
     const uint16_t *Wr = a.W + row * a.ld;
     const float *Gr = a.G + row * a.ld;
     // the importance row lands at the place in its 16-byte block that it has in global memory
@@ -163,7 +163,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) skim_sort16_kernel(Cl
 
     // ---------------------------------------------------------------- set-up
     if (tid == 0) {
-        mbar_init(mbar, 1);
+        if (FIRST) mbar_init(mbar, 1);
         ps.misc[0] = 0;
         ps.misc[1] = 0;
     }
@@ -347,16 +347,16 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) skim_sort16_kernel(Cl
     // ---------------------------------------------------------------- the importance row must have landed
     // (the vote below is also the barrier that ends pass 1)
     {
-        const bool landed = mbar_wait_bounded(mbar, 0);
+        const bool landed = mbar_wait_bounded(mbar, parity);
         if (!__syncthreads_and(landed ? 1 : 0)) {
             // the copy never arrived: flag it, give it one more bounded chance to drain, leave
             // and mark the row record invalid, so that the Lloyd kernel skips the row
             if (tid == 0) {
                 atomicOr(a.status, (unsigned long long)SKIM_STATUS_TIMEOUT);
-                *reinterpret_cast<int *>(a.scratch + (size_t)blockIdx.x * (size_t)a.rec_stride) = -1;
+                *reinterpret_cast<int *>(a.scratch + (size_t)local * (size_t)a.rec_stride) = -1;
             }
-            mbar_wait_bounded(mbar, 0);
-            return;
+            mbar_wait_bounded(mbar, parity);
+            return false;
         }
     }
     // ---------------------------------------------------------------- row record
@@ -374,11 +374,40 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) skim_sort16_kernel(Cl
         __syncthreads();
         nd = ps.misc[0];
     }
-    if constexpr (HALF_RECORD) write_row_record_half<uint16_t, THREADS>(a, src, ps, nd, (int)blockIdx.x);
-    else write_row_record<uint16_t, THREADS, false>(a, src, ps, nd, (int)blockIdx.x);
+    if constexpr (HALF_RECORD) write_row_record_half<uint16_t, THREADS>(a, src, ps, nd, local);
+    else write_row_record<uint16_t, THREADS, false>(a, src, ps, nd, local);
     if (nd <= 16) {
         collect_distinct<uint16_t, THREADS>(src, m, nd, ps);
-        write_distinct_values(a, nd, ps.dvals, (int)blockIdx.x);
+        write_distinct_values(a, nd, ps.dvals, local);
+    }
+    return true;
+}
+
+// HALF_RECORD: the compact row record, for the Lloyd kernel; else the full one, for the exact kernel.
+template <bool HALF_RECORD, int THREADS, int VEC>
+__global__ void __launch_bounds__(THREADS, 1024 / THREADS) skim_sort16_kernel(ClusterArgs a)
+{
+    skim_let_next_kernel_start();          // (this kernel is an ordinary launch: the one after it waits)
+    sort16_row<HALF_RECORD, THREADS, VEC, true>(a, (int)blockIdx.x, 0u);
+}
+
+// The rows that the bucket kernel has put on a.sort_list (usually none).
+template <int THREADS, int VEC>
+__global__ void __launch_bounds__(THREADS, 1024 / THREADS) skim_sort16_list_kernel(ClusterArgs a)
+{
+    skim_wait_for_previous_kernel();
+    skim_let_next_kernel_start();
+    const int listed = min(*a.sort_count, a.chunk_rows);
+    if ((int)blockIdx.x >= listed) return;
+    extern __shared__ __align__(16) unsigned char smem[];
+    if (threadIdx.x == 0) mbar_init(reinterpret_cast<uint64_t *>(smem + layout16(a.m, THREADS).mbar), 1);      // (a barrier follows)
+    bool ok = true;
+    uint32_t parity = 0u;
+    for (int at = blockIdx.x; at < listed; at += gridDim.x, parity ^= 1u) {
+        const int local = a.sort_list[at];
+        if (ok) ok = sort16_row<true, THREADS, VEC, false>(a, local, parity);
+        else if (threadIdx.x == 0) *reinterpret_cast<int *>(a.scratch + (size_t)local * (size_t)a.rec_stride) = -1;      // a copy may still be in flight
+        __syncthreads();
     }
 }
 
@@ -390,6 +419,7 @@ struct Variant16 {
 
 #define SKIM_V16(T, V) {T * V * 8, T, {skim_sort16_kernel<false, T, V>, skim_sort16_kernel<true, T, V>}}
 #define SKIM_V16F(T, V) {T * V * 8, T, {skim_sort16_kernel<false, T, V>, nullptr}}      // short rows with compact records: skim_bucket.cu
+#define SKIM_V16L(T, V) {T * V * 8, T, {nullptr, skim_sort16_list_kernel<T, V>}}
 
 // An SM holds 1024 threads; small blocks wait for their own barriers only (4096 columns: 256 threads of 16 elements take
 // 0.131 ms for 4096 rows, 512 of 8 took 0.153 ms).
@@ -397,23 +427,31 @@ const Variant16 kVariants16[] = {
     SKIM_V16F(128, 1), SKIM_V16F(128, 2), SKIM_V16(256, 2), SKIM_V16(256, 3), SKIM_V16(512, 2), SKIM_V16(512, 3), SKIM_V16(1024, 2),
     SKIM_V16(1024, 3),
 };
+// The rows that the bucket kernel refuses.  No smaller blocks: short rows are mostly the work on the 4096 counters, and the launch,
+// which usually finds the list empty, has fewer blocks (1184 of 128 threads cost 0.7 us, 592 of 256 nothing measurable).
+const Variant16 kListVariants16[] = {SKIM_V16L(256, 1), SKIM_V16L(512, 1)};
+
+template <int N>
+const Variant16 *pick16(const Variant16 (&table)[N], const skim_ctx *ctx, int m)
+{
+    for (const Variant16 &v : table)
+        if (v.cap >= m && layout16(m, v.threads).total <= (size_t)ctx->max_smem_optin) return &v;
+    return nullptr;
+}
 
 }  // namespace
 
-int skim_launch_sort16(skim_ctx *ctx, const ClusterArgs &args, int64_t rows)
+int skim_launch_sort16(skim_ctx *ctx, const ClusterArgs &args, int64_t rows, bool listed)
 {
-    for (const Variant16 &v : kVariants16) {
-        if (v.cap < args.m) continue;
-        const Layout16 L = layout16(args.m, v.threads);
-        if (L.total > (size_t)ctx->max_smem_optin) continue;
-        void (*kernel)(ClusterArgs) = v.kernel[args.rec_half ? 1 : 0];
-        if (!kernel) return SKIM_ERR_SHAPE;
-        // set on every launch: a host-side call of microseconds, and no state shared between contexts
-        SKIM_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total));
-        kernel<<<(unsigned)rows, v.threads, L.total, ctx->stream>>>(args);
-        SKIM_CUDA_OK(cudaGetLastError());
-        ctx->launches += 1;
-        return SKIM_OK;
-    }
-    return SKIM_ERR_SHAPE;
+    const Variant16 *v = listed ? pick16(kListVariants16, ctx, args.m) : pick16(kVariants16, ctx, args.m);
+    void (*kernel)(ClusterArgs) = v ? v->kernel[args.rec_half ? 1 : 0] : nullptr;
+    if (!kernel) return SKIM_ERR_SHAPE;
+    const size_t smem = layout16(args.m, v->threads).total;
+    // set on every launch: a host-side call of microseconds, and no state shared between contexts
+    SKIM_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (listed) return skim_launch_dependent(ctx, kernel, dim3(skim_list_blocks(ctx, v->threads, rows)), v->threads, smem, args);
+    kernel<<<(unsigned)rows, v->threads, smem, ctx->stream>>>(args);
+    SKIM_CUDA_OK(cudaGetLastError());
+    ctx->launches += 1;
+    return SKIM_OK;
 }

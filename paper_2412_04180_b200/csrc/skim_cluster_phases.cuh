@@ -489,10 +489,17 @@ __device__ __forceinline__ void write_distinct_values(const ClusterArgs &a, int 
 
 }  // namespace skimk
 
+// Blocks of the kernels that take the rows on args.sort_list: as many as an SM holds.
+static inline unsigned skim_list_blocks(const skim_ctx *ctx, int threads, int64_t rows)
+{
+    const int64_t blocks = (int64_t)ctx->sm_count * (1024 / threads);
+    return (unsigned)(rows < blocks ? rows : blocks);
+}
 // Bucket sort kernel (skim_bucket.cu): writes the row records of a chunk, or puts rows on args.sort_list.
 int skim_launch_sort_bucket(skim_ctx *ctx, const skimk::ClusterArgs &args, int64_t rows);
-// fp16-key sort kernel (skim_cluster16.cu): writes the row records of a chunk; no scale vector installed.
-int skim_launch_sort16(skim_ctx *ctx, const skimk::ClusterArgs &args, int64_t rows);
+// fp16-key sort kernel (skim_cluster16.cu): writes the row records of a chunk, or of the rows on args.sort_list; no scale vector
+// installed.
+int skim_launch_sort16(skim_ctx *ctx, const skimk::ClusterArgs &args, int64_t rows, bool listed = false);
 // Exact clustering kernel (skim_exact.cu): one block per row record; `scratch` holds `slots` slots of
 // skim_exact_slot_bytes(cols) bytes.
 int skim_launch_exact(skim_ctx *ctx, const skimk::ClusterArgs &args, int64_t rows, void *scratch, int slots);

@@ -396,3 +396,38 @@ def test_pruned_matrices_cost_little_more(ctx, rows, cols, scaled):
     assert _cluster_us(ctx, pruned, G) < 1.6 * _cluster_us(ctx, W, G)
     ctx.apply_scale(None)
     assert ctx.get_status() == 0
+
+
+@pytest.mark.parametrize("rows,cols", [(3000, 65), (1300, 1025), (700, 3001), (330, 5000)])
+@pytest.mark.parametrize("scaled", [False, True])
+def test_matrices_of_refused_rows(ctx, oracle, rows, cols, scaled):
+    """More rows that no bucket spreads than blocks of the kernel that takes them: a block goes through several."""
+    w, g = inputs.make_rows(rows, cols, 9900 + cols)
+    w[:] = (1.0 + 0.25 * w.astype(np.float32)).astype(np.float16)       # few values, a clump away from zero
+    w[:, 0] = -0.02
+    w[rows // 2] *= np.float16(0.5)
+    s = None
+    if scaled:
+        s = np.ones(cols, np.float32)
+        s[::7] = 2.0
+    ora = oracle.cluster_rows(w, g, BITS, 5, s=s, want_codes=False)
+    cent, err, _ = _gpu_cluster(ctx, w, g, BITS, 5, s=s, codes=False)
+    check_cluster(ora, cent, err, None, _values(w, s), BITS, label=f"{rows}x{cols} scaled={scaled}")
+
+
+@pytest.mark.parametrize("rows,cols,scaled,most", [(20000, 128, False, 3.5), (4096, 700, False, 3.0), (4096, 3000, False, 2.6), (4096, 3000, True, 4.2)])
+def test_refused_matrices_go_to_a_sort_of_their_size(ctx, rows, cols, scaled, most):
+    """All rows a clump of nearby values, against the same matrix around zero.  A radix sort of 4096 elements, whatever the rows' length,
+    took 5 to 8 times as long."""
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(cols)
+    W = torch.randn((rows, cols), generator=gen, device="cuda") * 0.02
+    G = torch.randn((rows, cols), generator=gen, device="cuda").exp()
+    clump = (1.0 + 0.01 * W).half()
+    W = W.half()
+    ctx.reserve(rows, cols)
+    ctx.apply_scale(torch.ones(cols, device="cuda") if scaled else None)
+    _cluster_us(ctx, W, G)
+    assert _cluster_us(ctx, clump, G) < most * _cluster_us(ctx, W, G)
+    ctx.apply_scale(None)
+    assert ctx.get_status() == 0
