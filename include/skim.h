@@ -41,6 +41,10 @@
  *     all inside [1, SKIM_MAX_BIT].  Width b has 2^b centroids.  "sumk" below is the sum of
  *     2^b over bit_set; a row's centroid record is the concatenation of its width blocks in
  *     bit_set order, each block ascending.
+ *   - Sums have a fixed order: the same inputs give the same bits on every run, with one exception.  Without a scale
+ *     vector the clustering adds the elements of equal weight in no fixed order, so an error (and a centroid, where
+ *     importances beside one another differ by more than 2^15) may differ by a rounding of the binary64 sums,
+ *     which the rounding to binary32 nearly always hides.
  *   - The value that is clustered is x = float(W_ij) when no scale is installed, else the
  *     binary32 product float(W_ij) * r_j with r_j = 1.0f / s_j.
  */

@@ -73,13 +73,16 @@ __host__ __device__ inline BucketLayout bucket_layout(int m, int threads)
     return L;
 }
 
-// Insertion sort of n elements by one thread.
+// Insertion sort of n elements by one thread.  BOTH: equal values by importance.
+template <bool BOTH>
 __device__ __forceinline__ void sort_bucket(float *keys, float *gs, int lo, int n)
 {
     for (int i = lo + 1; i < lo + n; ++i) {
         const float k = keys[i], g = gs[i];
         int j = i;
-        for (float y; j > lo && (y = keys[j - 1]) > k; --j) {
+        for (; j > lo; --j) {
+            const float y = keys[j - 1];
+            if (BOTH ? (y < k || (y == k && gs[j - 1] <= g)) : !(y > k)) break;
             keys[j] = y;
             gs[j] = gs[j - 1];
         }
@@ -321,7 +324,9 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) skim_sort_bucket_kern
     // ---------------------------------------------------------------- order where it matters
     // The Lloyd kernel asks for groups of 8 in order, not for order inside a group: only a bucket that reaches from one
     // group into the next has to be sorted.  A row with few distinct values is sorted in full (they are counted below), and so
-    // are all rows for the exact kernel.
+    // are all rows for the exact kernel.  Scaled rows come out the same on every run (the record pass orders their groups).  An
+    // unscaled value has 11 bits, so a group's sums of g and g x are exact unless its importances spread over 2^15, whatever
+    // their order; the row total of g x^2 may differ in its last bit between runs, as it does from the fp16-key kernel.
     int nd = ps.misc[0];                     // more than 16 occupied words: more than 16 distinct values
     auto bucket_end = [&](int b) { return b + 1 < Bk::N ? bucket_base(cnt, b + 1) - (apart && b + 1 == Bk::HALF ? (int)bucket_zeros(ps)[NW] : 0) : m; };
     const bool full = a.full_order || nd <= 16;
@@ -329,14 +334,14 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) skim_sort_bucket_kern
         if (!full) {
             if (p0 == 0) continue;
             const int b = bucket(keys[p0]), lo = bucket_base(cnt, b);
-            if (lo < p0 && lo >= p0 - 8) sort_bucket(keys, gs, lo, bucket_end(b) - lo);          // (an earlier start: an earlier border's thread does it)
+            if (lo < p0 && lo >= p0 - 8) sort_bucket<SCALED>(keys, gs, lo, bucket_end(b) - lo);          // (an earlier start: an earlier border's thread does it)
         } else {
             // every bucket that starts in these 8 positions (a bucket's other places hold elements of the bucket all along)
             for (int p = p0; p < min(p0 + 8, m);) {
                 const float key = keys[p];
                 const int b = bucket(key), lo = bucket_base(cnt, b), end = bucket_end(b);
                 const bool zero = apart && key == 0.0f;              // (its bucket begins behind the zeros)
-                if (lo >= p0 && !zero) sort_bucket(keys, gs, lo, end - lo);
+                if (lo >= p0 && !zero) sort_bucket<SCALED>(keys, gs, lo, end - lo);
                 p = zero ? lo : end;
             }
         }

@@ -6,6 +6,8 @@
 // and skim_exact.cu.
 #pragma once
 
+#include <type_traits>
+
 #include "skim_internal.cuh"
 
 namespace skimk {
@@ -109,7 +111,7 @@ struct ClusterArgs {
 //   seg     one 32-byte entry per segment of 32 groups (256 elements): the binary64 sums of g,
 //           g*x and g*x^2 over all earlier segments; entry nseg holds the row totals
 //   groups  one 96-byte record per group of 8 elements (no value of a group above one of the next; inside a
-//           group the radix kernels leave order, the bucket kernel need not), three whole 32-byte sectors: the 8
+//           group the radix kernels leave order, and scaled rows of the bucket kernel are put in order), three whole 32-byte sectors: the 8
 //           values | the 8 importances | the binary64 sums of g, g*x and g*x^2 from the start of
 //           the group's segment to the group's first element (and 8 bytes of padding).  With the
 //           segment entry that is everything a boundary needs in one Lloyd iteration.  The last
@@ -222,6 +224,36 @@ __device__ __forceinline__ void collect_distinct(const Src &src, int m, int nd, 
     __syncthreads();
 }
 
+// Eight (value, importance) pairs in ascending order, by Batcher's odd-even merging network: 19 exchanges in registers.  BOTH: equal
+// values by importance.
+template <bool BOTH>
+__device__ __forceinline__ void merge8(float *k, float *g)
+{
+    auto exchange = [&](int i, int j) {
+        const float ki = k[i], kj = k[j], gi = g[i], gj = g[j];
+        const bool swap = ki > kj || (BOTH && ki == kj && gi > gj);
+        k[i] = fminf(ki, kj);
+        k[j] = fmaxf(ki, kj);
+        g[i] = swap ? gj : gi;
+        g[j] = swap ? gi : gj;
+    };
+    exchange(0, 1); exchange(2, 3); exchange(4, 5); exchange(6, 7);
+    exchange(0, 2); exchange(1, 3); exchange(4, 6); exchange(5, 7);
+    exchange(1, 2); exchange(5, 6);
+    exchange(0, 4); exchange(1, 5); exchange(2, 6); exchange(3, 7);
+    exchange(2, 4); exchange(3, 5);
+    exchange(1, 2); exchange(3, 4); exchange(5, 6);
+}
+// (Equal values are rare, or the row has few of them: the second pass, for them, is skipped.  All in one pass took 2-3 % more of the kernel.)
+__device__ __forceinline__ void order8(float *k, float *g)
+{
+    merge8<false>(k, g);
+    bool tie = false;
+#pragma unroll
+    for (int u = 0; u < 7; ++u) tie |= k[u] == k[u + 1] && g[u] > g[u + 1];
+    if (tie) merge8<true>(k, g);
+}
+
 // Writes the row record from the sorted row (a source, see above; padded to whole groups: largest
 // key / zero importance).  One pass: a lane takes 2^(SKIM_SEG_SHIFT - 5) adjacent groups of 8 elements (one, as measured best), decodes them,
 // stores their values and importances, sums g, g*x, g*x^2 in binary64 (pairwise); one warp scan over
@@ -257,6 +289,18 @@ __device__ __forceinline__ int write_row_record(const ClusterArgs &a, const Src 
                 KeyT ks[8];
                 float gs[8], x[8];
                 const unsigned gbits = src.group(e, m, ks, gs);
+                if constexpr (std::is_same<KeyT, float>::value) {
+                    // The bucket kernel leaves the elements of a bucket in the order in which its counting atomics came in, another one on
+                    // every run.  The product of two binary32 numbers fills a binary64 one, so the sums below (and the Lloyd
+                    // kernel's) depend on the order in their last bit: a group is put in order here.  It costs 4-12 % of the
+                    // kernel (4096 x 11008 349 -> 373 us, 4096 x 4096 121 -> 135); ordering the buckets in shared memory took 57 %.
+                    if (!a.full_order) {
+#pragma unroll
+                        for (int u = 0; u < 8; ++u)
+                            if (e + u >= m) ks[u] = SKIM_PAD_VALUE;
+                        order8(ks, gs);
+                    }
+                }
                 KeyT prev = (COUNT && e > 0) ? src.key_at(e - 1) : (KeyT)0;
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
@@ -270,8 +314,7 @@ __device__ __forceinline__ int write_row_record(const ClusterArgs &a, const Src 
                 unsigned char *gr = rec + R.groups + (size_t)q * SKIM_GROUP_BYTES;
                 st_sector(gr, x);
                 st_sector(gr + 32, gs);
-                // the smallest value: inside a group a row of the bucket kernel is in no order
-                first[h] = fminf(fminf(fminf(x[0], x[1]), fminf(x[2], x[3])), fminf(fminf(x[4], x[5]), fminf(x[6], x[7])));
+                first[h] = x[0];
                 double t0[8], t1[8], t2[8];
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {

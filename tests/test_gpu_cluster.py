@@ -431,3 +431,29 @@ def test_refused_matrices_go_to_a_sort_of_their_size(ctx, rows, cols, scaled, mo
     assert _cluster_us(ctx, clump, G) < most * _cluster_us(ctx, W, G)
     ctx.apply_scale(None)
     assert ctx.get_status() == 0
+
+
+@pytest.mark.parametrize("rows,cols", [(700, 129), (300, 1500), (300, 3000), (300, 4096), (200, 5000), (200, 11008), (100, 16500), (100, 22528)])
+def test_scaled_rows_are_the_same_on_every_run(ctx, rows, cols):
+    """The workspace holds the row records (sorted groups and their binary64 prefix sums): every byte of it is the same whatever order the
+    counting atomics came in.  Rows with zeros kept apart and with equal values among them; none that the buckets refuse (their
+    list has an order of its own)."""
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(cols)
+    W = (torch.randn((rows, cols), generator=gen, device="cuda") * 0.02).half()
+    W[::5] = torch.where(W[::5].abs() < 0.01, torch.zeros_like(W[::5]), W[::5])
+    G = (1.5 * torch.randn((rows, cols), generator=gen, device="cuda")).exp()
+    s = torch.exp(0.25 * torch.randn((cols,), generator=gen, device="cuda"))
+    s[: cols // 2] = 1.0                                                # products of equal weights are equal there
+    ctx.set_workspace(torch.zeros(ctx.workspace_bytes(rows, cols), dtype=torch.uint8, device="cuda"))
+    ctx.apply_scale(s)
+    first = None
+    for _ in range(8):
+        cent, _, err = ctx.cluster_rows(W, G, BITS, 6)
+        out = (ctx._ws.clone(), cent.clone(), err.clone())
+        if first is None:
+            first = out
+        for a, b in zip(first, out):
+            assert torch.equal(a.view(torch.uint8) if a.dtype != torch.uint8 else a, b.view(torch.uint8) if b.dtype != torch.uint8 else b)
+    ctx.apply_scale(None)
+    assert ctx.get_status() == 0
