@@ -429,7 +429,7 @@ const Variant16 kVariants16[] = {
 };
 // The rows that the bucket kernel refuses.  No smaller blocks: short rows are mostly the work on the 4096 counters, and the launch,
 // which usually finds the list empty, has fewer blocks (1184 of 128 threads cost 0.7 us, 592 of 256 nothing measurable).
-const Variant16 kListVariants16[] = {SKIM_V16L(256, 1), SKIM_V16L(512, 1)};
+const Variant16 kVariantsList16[] = {SKIM_V16L(256, 1), SKIM_V16L(512, 1)};
 
 template <int N>
 const Variant16 *pick16(const Variant16 (&table)[N], const skim_ctx *ctx, int m)
@@ -443,7 +443,7 @@ const Variant16 *pick16(const Variant16 (&table)[N], const skim_ctx *ctx, int m)
 
 int skim_launch_sort16(skim_ctx *ctx, const ClusterArgs &args, int64_t rows, bool listed)
 {
-    const Variant16 *v = listed ? pick16(kListVariants16, ctx, args.m) : pick16(kVariants16, ctx, args.m);
+    const Variant16 *v = listed ? pick16(kVariantsList16, ctx, args.m) : pick16(kVariants16, ctx, args.m);
     void (*kernel)(ClusterArgs) = v ? v->kernel[args.rec_half ? 1 : 0] : nullptr;
     if (!kernel) return SKIM_ERR_SHAPE;
     const size_t smem = layout16(args.m, v->threads).total;
