@@ -94,8 +94,12 @@ int skim_max_cols(const skim_ctx *ctx, int64_t *out);
  * The workspace must be 256-byte aligned and stays owned by the caller.  It also stores the
  * installed scale vector, so it must outlive every call that follows skim_apply_scale.  Most of
  * it is the clustering's scratch: about 13 bytes per element for min(rows, 8192) rows (the sorted
- * rows with their prefix sums, which the sort kernel hands to the Lloyd kernel); the scale update
- * adds 8 bytes x 296 x cols of partial gradients and 520 bytes per row.
+ * rows with their prefix sums, which the sort kernel hands to the Lloyd kernel).  The scale updates
+ * put their label-ordered copy of the matrix in the same place, 8 bytes per element of ALL rows (of more than 512
+ * columns: and up to 1087 elements of padding per row), which is more above 8192 rows (22016 x 8192:
+ * 1.66 GB instead of 0.92) and in narrow matrices; they also need 8 bytes x 296 x cols of partial gradients and 556 bytes per
+ * row.  The other calls ask for what they use only: a program that never calls a scale update may hand over
+ * skim_workspace_bytes(min(rows, 8192), cols) plus 640 bytes for each further row plus 4096.
  * skim_set_workspace UNINSTALLS a scale vector that is installed (its reciprocal lives in the old
  * workspace): call skim_apply_scale again afterwards.  The caller must not release the old workspace
  * before the work already enqueued on the context's stream has finished. */

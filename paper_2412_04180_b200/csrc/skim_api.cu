@@ -47,11 +47,11 @@ int check_matrix(const skim_ctx *ctx, int64_t rows, int64_t cols, int64_t ld)
     return SKIM_OK;
 }
 
-int check_workspace(const skim_ctx *ctx, int64_t rows, int64_t cols)
+int check_workspace(const skim_ctx *ctx, int64_t rows, int64_t cols, bool scale_update = false)
 {
     if (!ctx->ws) return SKIM_ERR_WORKSPACE;
     const SkimWorkspace need = skim_carve(nullptr, rows, cols);
-    return need.bytes <= ctx->ws_bytes ? SKIM_OK : SKIM_ERR_WORKSPACE;
+    return (scale_update ? need.bytes : need.bytes_no_update) <= ctx->ws_bytes ? SKIM_OK : SKIM_ERR_WORKSPACE;
 }
 
 }  // namespace
@@ -397,7 +397,7 @@ int skim_scale_update(skim_ctx *ctx, const uint16_t *W, const float *importance,
     int rc = check_matrix(ctx, rows, cols, ld);
     if (rc) return rc;
     if (rows < 1 || steps < 0 || decay_every < 1 || !(lr0 > 0.0f) || !(decay > 0.0f)) return SKIM_ERR_SHAPE;
-    rc = check_workspace(ctx, rows, cols);
+    rc = check_workspace(ctx, rows, cols, true);
     if (rc) return rc;
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return SKIM_ERR_CUDA;
@@ -469,7 +469,7 @@ int skim_scale_update_lfull(skim_ctx *ctx, const uint16_t *W, const float *impor
     if ((reinterpret_cast<uintptr_t>(W) & 15u) || (reinterpret_cast<uintptr_t>(importance) & 15u) ||
         (reinterpret_cast<uintptr_t>(labels) & 15u) || (reinterpret_cast<uintptr_t>(H) & 15u))
         return SKIM_ERR_ALIGN;
-    rc = check_workspace(ctx, rows, cols);
+    rc = check_workspace(ctx, rows, cols, true);
     if (rc) return rc;
     if ((reinterpret_cast<uintptr_t>(scratch) & 255u) != 0 || scratch_bytes < skim_scale_lfull_scratch_bytes(rows, cols))
         return SKIM_ERR_WORKSPACE;

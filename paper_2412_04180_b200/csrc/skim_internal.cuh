@@ -54,7 +54,8 @@ struct SkimWorkspace {
     uint16_t *scale_ord_end;     // [rows][16]  scale update: steps of the clusters in the label-ordered rows
     int *sort_list;              // [min(rows, SKIM_CLUSTER_CHUNK_ROWS)] rows the bucket sort kernel leaves to the radix kernel
     unsigned char *cluster_scratch;  // [min(rows, SKIM_CLUSTER_CHUNK_ROWS)] row records of the clustering; during a scale update the label-ordered matrix
-    size_t bytes;
+    size_t bytes;                // enough for every call
+    size_t bytes_no_update;      // enough for every call but the scale updates (the records, not the label-ordered matrix)
 };
 
 #define SKIM_SCALE_MAX_CTAS 296
@@ -68,12 +69,15 @@ __host__ __device__ static inline size_t skim_cluster_record_bytes(int64_t cols)
     return (13 * m8 + 1024 + 127) & ~(size_t)127;
 }
 
-// The label-ordered matrix of the scale update (skim_scale.cu): elements (8 bytes each) of a row, at most, with 16
-// clusters padded to whole units of 64; and the bytes behind the last row that its readers may fetch.
+// The label-ordered matrix of the scale update (skim_scale.cu): elements (8 bytes each) of a row, at most -- rows of up to
+// SKIM_ORDER_SHORT_COLS have no padding (an even number of elements), the others have 16 clusters padded to whole units of
+// 64 -- and the bytes behind the last row that its readers may fetch.
 #define SKIM_ORDER_UNIT 64
+#define SKIM_ORDER_SHORT_COLS 512
 #define SKIM_ORDER_SLACK 8192
 __host__ __device__ static inline int64_t skim_ordered_stride(int64_t cols)
 {
+    if (cols <= SKIM_ORDER_SHORT_COLS) return (cols + 1) / 2 * 2;
     return (cols + SKIM_ORDER_UNIT - 1) / SKIM_ORDER_UNIT * SKIM_ORDER_UNIT + 16 * SKIM_ORDER_UNIT;
 }
 
@@ -102,6 +106,7 @@ static inline SkimWorkspace skim_carve(void *base, int64_t rows, int64_t cols)
     w.sort_list = (int *)take((size_t)(rows < SKIM_CLUSTER_CHUNK_ROWS ? rows : SKIM_CLUSTER_CHUNK_ROWS) * 4);
     const size_t records = (size_t)(rows < SKIM_CLUSTER_CHUNK_ROWS ? rows : SKIM_CLUSTER_CHUNK_ROWS) * skim_cluster_record_bytes(cols);
     const size_t ordered = (size_t)rows * (size_t)skim_ordered_stride(cols) * 8 + SKIM_ORDER_SLACK;
+    w.bytes_no_update = off + skim_align256(records);
     w.cluster_scratch = (unsigned char *)take(records > ordered ? records : ordered);
     w.bytes = off;
     return w;

@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(OT) skim_scale_order_kernel(ScaleArgs a)
 // cluster; ord_end counts elements.  Whole step, before and after: 22016 x 128 85 -> 49 us, 9000 x 300 43 -> 28.5 us; at 4096 x 1500 36.6 -> 43.6 us,
 // since the longest cluster decides.  Up to 1024 columns it pays where every warp of the sums kernel has a row of its own (4096 x 700 28.4 ->
 // 26.1 us, ordering 9000 x 1000 170 -> 100 us; 1000 x 1001 16.9 -> 19.0 us).
-constexpr int SHORT_COLS = 512, SHORT_COLS_MANY_ROWS = 1024;
+constexpr int SHORT_COLS = SKIM_ORDER_SHORT_COLS, SHORT_COLS_MANY_ROWS = 1024;
 constexpr int OST = 256;
 
 __global__ void __launch_bounds__(OST) skim_scale_order_short_kernel(ScaleArgs a)

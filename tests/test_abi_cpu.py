@@ -41,6 +41,20 @@ def test_packed_layout(lib, oracle):
     assert strides == [oracle.row_stride_words(100, 2), oracle.row_stride_words(100, 3)]
 
 
+def test_workspace_sizes(lib):
+    """Short rows are label-ordered without padding; the matrix of the scale update is the only part that grows with all rows."""
+    from paper_2412_04180_b200.skim import Skim
+    record = lambda cols: 13 * (cols + 7) + 1152                      # bytes of a row record, at most
+    for rows, cols in [(1, 1), (22016, 128), (22016, 511), (22016, 512), (9000, 300), (100000, 64)]:
+        ordered = 8 * rows * (cols + 1) + 8192
+        fixed = 296 * 8 * max(cols, 1) + 28 * cols + 556 * rows + 8 * 296 + 4 * 8192 + 16 * 256
+        assert Skim.workspace_bytes(rows, cols) <= fixed + max(ordered, min(rows, 8192) * record(cols)), (rows, cols)
+    for rows, cols in [(4096, 11008), (22016, 8192), (8192, 22016), (256, 513)]:
+        ordered = 8 * rows * (cols + 63 + 1024) + 8192
+        fixed = 296 * 8 * cols + 28 * cols + 556 * rows + 8 * 296 + 4 * 8192 + 16 * 256
+        assert Skim.workspace_bytes(rows, cols) <= fixed + max(ordered, min(rows, 8192) * record(cols)), (rows, cols)
+
+
 def test_argument_errors_without_a_device(lib):
     from paper_2412_04180_b200.skim import Skim, SkimError
     with pytest.raises(SkimError) as e:

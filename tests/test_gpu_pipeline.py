@@ -313,3 +313,38 @@ def test_config5_schedule_on_a_row_subset(ctx, oracle, mat):
                                     label=f"config5/{mat}", trace_rtol=1e-5, alpha_rtol=1e-4, alpha_atol=1e-4)
     assert len(losses) == 5
 
+
+
+@pytest.mark.parametrize("rows,cols", [(9000, 40), (8200, 700), (300, 200)])
+def test_workspace_without_scale_update(ctx, rows, cols):
+    """Every call but the scale updates runs in the smaller workspace that the header states, with the same results; a scale update
+    there is refused on the host."""
+    from paper_2412_04180_b200.skim import SkimError
+    w, g = inputs.make_rows(rows, cols, 77)
+    W, G = torch.from_numpy(w).cuda(), torch.from_numpy(g).cuda()
+    alpha = torch.from_numpy(inputs.make_scale(cols, 5)).cuda()
+
+    def run():
+        ctx.apply_scale(alpha)
+        cent, _, err = ctx.cluster_rows(W, G, BITS, 5)
+        bits, _ = ctx.allocate_bits(err, BITS, 2.25)
+        q = ctx.quantize(W, bits, cent, BITS)
+        cent2, labels, _ = ctx.cluster_rows_at(W, G, bits, BITS, 5)
+        n = int(q["group_info"][-1].item())
+        return [cent, err, bits, q["packed"][:n], q["lut"], labels]
+
+    full = ctx.workspace_bytes(rows, cols)
+    less = ctx.workspace_bytes(min(rows, 8192), cols) + 640 * max(rows - 8192, 0) + 4096
+    ctx.set_workspace(torch.empty(full, dtype=torch.uint8, device="cuda"))
+    want = run()
+    ctx.set_workspace(torch.empty(less // 256 * 256, dtype=torch.uint8, device="cuda"))
+    for a, b in zip(run(), want):
+        assert torch.equal(a, b)
+    if less < full:
+        with pytest.raises(SkimError) as e:
+            ctx.scale_update(W, G, want[-1], alpha.clone(), steps=1)
+        assert e.value.code == -5
+    ctx.set_workspace(torch.empty(full, dtype=torch.uint8, device="cuda"))
+    ctx.scale_update(W, G, want[-1], alpha.clone(), steps=1)
+    ctx.apply_scale(None)
+    assert ctx.get_status() == 0
