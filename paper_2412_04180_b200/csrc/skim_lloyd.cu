@@ -241,11 +241,12 @@ template <> struct Window<true> {
 
 // s1 / s0 for s0 > 0: binary32 reciprocal seed and two binary64 Newton corrections (relative
 // error about 2^-60, i.e. the correctly rounded quotient up to the last bit or so); operands far
-// outside the binary32 range take the plain division.
-__device__ __forceinline__ double quotient(double s1, double s0)
+// outside the binary32 range take the plain division.  zero: the quotient is 0 instead (one branch for both rare cases; a
+// selection at the end took 2 % of the kernel).
+__device__ __forceinline__ double quotient(double s1, double s0, bool zero)
 {
     const float s0f = (float)s0;
-    if (!(s0f > 1e-30f && s0f < 1e30f) || !(fabs(s1) < 1e30)) return s1 / s0;
+    if (!(s0f > 1e-30f && s0f < 1e30f) || !(fabs(s1) < 1e30) || zero) return zero ? 0.0 : s1 / s0;
     const float rf = __frcp_rn(s0f);
     const double rd = (double)rf;
     double q = (double)((float)s1 * rf);
@@ -385,11 +386,7 @@ __device__ __forceinline__ void lloyd_warp(const unsigned char *rec, const typen
         // Likewise S1 over a run of zeros (a pruned row): its terms are 0 and the prefixes equal but for their rounding, about 2^-49
         // of them.  The mean is 0 then, not that noise: zeros lie on the midpoint of a centroid 0 and its copies (the start
         // values repeat), which decides where they all go.  (The centroid moves by 2^-46 P1 / S0 at most, elsewhere too.)
-        const bool zero_mean = fabs(S1) <= fabs(P1) * 0x1p-46;
-        if (normal && S0 > P0 * 0x1p-40) {
-            c = (float)quotient(S1, S0);
-            if (zero_mean) c = 0.0f;
-        }
+        if (normal && S0 > P0 * 0x1p-40) c = (float)quotient(S1, S0, fabs(S1) <= fabs(P1) * 0x1p-46);
     }
     sm.errs[lane] = err_j;
     sm.tfs[lane] = has_boundary ? tf : INF;
