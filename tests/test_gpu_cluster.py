@@ -170,9 +170,8 @@ def test_scaled_long_rows(ctx, oracle):
 
 @pytest.mark.parametrize("cols", [8192, 11008, 16384])
 def test_scaled_rows_at_llama_lengths(ctx, oracle, cols):
-    """Scaled rows go through the 32-bit-key sort kernel; these three lengths take its three largest
-    variants below the 22 016-column one (8192 is the row length of the 22016 x 8192 matrix that
-    the scaling alternation runs on)."""
+    """Scaled rows go through the bucket sort kernel; these lengths take three of its larger sizes (8192 is the row length of the
+    22016 x 8192 matrix that the scaling alternation runs on)."""
     w, g = inputs.make_rows(24, cols, 8100 + cols, importance_sigma=2.0)
     s = inputs.make_scale(cols, 29)
     ora = oracle.cluster_rows(w, g, BITS, 50, s=s)

@@ -99,9 +99,9 @@ def test_lfull_special_matrices(ctx, oracle):
 
 @pytest.mark.parametrize("cols", [968, 1160, 2560])
 def test_lfull_error_full_and_split_rounds(ctx, oracle, cols):
-    """4096 rows are 32 row tiles.  On a 148-SM part 968 columns give 128 tiles (one round, nothing cut), 1160
-    columns 160 tiles (one full round, the 12 tiles left cut into 8 ranges of K each), 2560 columns 320 tiles (two
-    full rounds, 24 tiles cut into 6 ranges): rows from full tiles and from cut tiles are compared with the oracle."""
+    """4096 rows are 16 row tiles of 256, a tile for one of the 74 pairs of SMs.  968 columns give 64 tiles (one round, nothing cut), 1160
+    columns 80 (one full round, the 6 tiles left cut along K), 2560 columns 160 (two full rounds, 12 tiles cut; as a
+    symmetric matrix it takes the half contraction): rows from full tiles and from cut tiles are compared with the oracle."""
     rows = 4096
     ctx.reserve(rows, cols)
     rng = np.random.default_rng(cols)
@@ -169,10 +169,11 @@ def test_lfull_argument_errors(ctx, skimlib):
 
 
 @pytest.mark.parametrize("rows,cols,symmetric", [(768, 776, True), (1000, 1096, True), (770, 2056, True), (4100, 1024, True), (897, 4104, True),
-                                                 (1000, 1096, False), (770, 2056, False), (767, 1096, True)])
+                                                 (1000, 1096, False), (770, 2056, False), (767, 1096, True),
+                                                 (768, 4424, True), (767, 4432, True), (770, 4432, False), (3700, 2016, True), (3570, 2048, True), (15000, 1000, True), (14900, 1000, True)])
 def test_lfull_half_contraction_of_a_symmetric_matrix(ctx, oracle, rows, cols, symmetric):
-    """Enough rows and columns for the half contraction: symmetric H, and one that differs from its transpose in a
-    single corner entry (the full contraction must take over)."""
+    """Symmetric H, and one that differs from its transpose in a single corner entry (the full contraction must take over), on either
+    side of the rule for the half contraction: 768 rows, four column tiles, rows * cols^2 = 1.5e10 (the smaller calls run in full)."""
     ctx.reserve(rows, cols)
     rng = np.random.default_rng(rows + cols)
     D = (rng.standard_normal((rows, cols)) * 2).astype(np.float16)
