@@ -17,7 +17,7 @@
 // operands brought in by TMA (cp.async.bulk.tensor, 128-byte swizzle) through a 6-stage shared-memory ring.  A CTA
 // fetches its 128 rows of D and half of the tile's rows of H (32 KB per K block of 64; a tile of its own of 128 x 256
 // took 48 KB for the same MMA time, more than the L2 delivers to an SM meanwhile).  Warp 0 issues the TMA loads, warp 1
-// allocates tensor memory and, in the first CTA, issues the MMAs of both, warps 2-5 read the accumulators back
+// allocates tensor memory and, in the first CTA, issues the MMAs of both, eight warps read the accumulators back
 // (tcgen05.ld) and do the dot product with the matching D tile.  No TMA multicast: every CTA fetches its own operands.
 // Every wait on an mbarrier is bounded: after WAIT_LIMIT_CYCLES the waiting role raises the block's abort flag,
 // sets SKIM_STATUS_TIMEOUT, and all roles leave their loops; tensor memory is freed on every path.
@@ -152,7 +152,8 @@ constexpr int LEAVE_POLL = 8;                   // the producer of the half cont
 constexpr int CHECK_WARPS = 4;                  // further warps of the half contraction: they compare H with its transpose
 constexpr int SPLIT_MAX = 8;                    // ranges of K a tile of the last round is cut into, at most
 constexpr int HALF_MIN_ROWS = 768, HALF_MIN_NT = 4;
-constexpr double HALF_MIN_PRODUCTS = 1.5e10;    // rows * cols^2
+constexpr double HALF_MIN_SAVING = 14.0;         // K blocks of a pair (6 us) that the half contraction must save
+constexpr double EPILOGUE_KB = 10.0;             // K blocks' worth of MMA time of an epilogue (256 columns read back and multiplied)
 constexpr size_t HALF_FLAG_BYTES = 4096;         // symmetry flags of up to 1024 blocks
 constexpr int TMEM_COLS = 512;                  // two accumulator stages of BN binary32 columns
 constexpr long long WAIT_LIMIT_CYCLES = 400000000ll;   // about 0.2 s; a whole launch takes milliseconds
@@ -224,14 +225,14 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity)
                  : "memory");
     return ok != 0;
 }
-// Bounded wait.  False when the block is aborting (this wait ran out, or another role's did) or, unless it is to go on all
-// the same, leaving.
-__device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, GemmSync &sync, bool leaving_too = false)
+// Bounded wait.  False when the block is aborting (this wait ran out, or another role's did) or, with LEAVES, leaving.
+template <bool LEAVES>
+__device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, GemmSync &sync)
 {
     volatile int *abort_flag = &sync.abort, *leave_flag = &sync.leave;
     const long long t0 = clock64();
     while (!mbar_try_wait(bar, parity)) {
-        if (*abort_flag || (*leave_flag && !leaving_too)) return false;
+        if (*abort_flag || (LEAVES && *leave_flag)) return false;
         if (clock64() - t0 > WAIT_LIMIT_CYCLES) {
             *abort_flag = 1;
             return false;
@@ -574,7 +575,7 @@ skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
                         }
                         left = flag_load(a.leave);
                     }
-                    if (!(ok = mbar_wait(&sy.empty[stage], phase ^ 1u, sy))) break;
+                    if (!(ok = mbar_wait<HALF>(&sy.empty[stage], phase ^ 1u, sy))) break;
                     load_block(stage, kb * BK, m0, b0, boxes);
                     ++issued;
                     if (++stage == NST) { stage = 0; phase ^= 1u; }
@@ -595,11 +596,11 @@ skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
                 if (u < 0) continue;
                 const GemmUnit w = HALF ? half_unit(a, half, u, nkb) : unit_of(a, u, nkb);
                 const int as = it & 1;
-                if (!(ok = mbar_wait(&sy.tmem_empty[as], (((uint32_t)it >> 1) & 1u) ^ 1u, sy))) break;
+                if (!(ok = mbar_wait<HALF>(&sy.tmem_empty[as], (((uint32_t)it >> 1) & 1u) ^ 1u, sy))) break;
                 tc_fence_after();
                 const uint32_t tmem_d = tmem_base + (uint32_t)(as * BN), idesc = umma_idesc(w.n);
                 for (int kb = w.kb0; kb < w.kb1; ++kb) {          // HALF: list positions
-                    if (!(ok = mbar_wait(&sy.full[stage], phase, sy))) break;
+                    if (!(ok = mbar_wait<HALF>(&sy.full[stage], phase, sy))) break;
                     tc_fence_after();
                     const uint32_t sa = smem_u32(tiles + (size_t)stage * STAGE_BYTES), sb = sa + A_BYTES;
 #pragma unroll
@@ -656,7 +657,7 @@ skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
             };
             fetch(c0, dv, lv);
             epilogue_barrier();                               // alpha is in place
-            ok = mbar_wait(&sy.tmem_full[as], ((uint32_t)it >> 1) & 1u, sy);
+            ok = mbar_wait<HALF>(&sy.tmem_full[as], ((uint32_t)it >> 1) & 1u, sy);
             ok = __all_sync(0xffffffffu, ok);
             float acc = 0.0f;
             if (ok) {
@@ -728,12 +729,12 @@ skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
             bool ok = !sy.abort;
             const int most = max(sy.issued[0], sy.issued[1]);
             for (int b = sy.issued[rank]; b < most && ok; ++b) {
-                ok = mbar_wait(&sy.empty[b % NST], (((uint32_t)(b / NST)) & 1u) ^ 1u, sy, true);
+                ok = mbar_wait<false>(&sy.empty[b % NST], (((uint32_t)(b / NST)) & 1u) ^ 1u, sy);
                 if (ok) load_block(b % NST, 0, 0, 0, BN / (2 * CB));
             }
             if (rank == 0)
-                for (int b = max(0, most - NST); b < most && ok; ++b) ok = mbar_wait(&sy.full[b % NST], ((uint32_t)(b / NST)) & 1u, sy, true);
-            if (ok) mbar_wait(&sy.drained, 0u, sy, true);
+                for (int b = max(0, most - NST); b < most && ok; ++b) ok = mbar_wait<false>(&sy.full[b % NST], ((uint32_t)(b / NST)) & 1u, sy);
+            if (ok) mbar_wait<false>(&sy.drained, 0u, sy);
         }
         __syncthreads();
     }
@@ -800,7 +801,6 @@ skim_lfull_reduce_kernel(GemmArgs a, int exp2, float *__restrict__ err, int64_t 
 // piece also costs its epilogue, which hides under the next piece's MMAs unless that one is shorter.
 double half_makespan(int mt, int nt, int nkb, int piece_kb, int pairs)
 {
-    constexpr double EPILOGUE = 10.0;          // K blocks' worth of MMA time (256 columns read back and multiplied)
     std::vector<double> load(pairs, 0.0);
     int u = 0;
     for (int nb = 0; nb < nt; ++nb) {
@@ -808,12 +808,12 @@ double half_makespan(int mt, int nt, int nkb, int piece_kb, int pairs)
         const double len = (double)half_len(nb, nkb) / p;
         for (int r = 0; r < p * mt; ++r, ++u) {
             const int t = u / pairs, b = u % pairs;
-            load[(t & 1) ? pairs - 1 - b : b] += len > EPILOGUE ? len : EPILOGUE;
+            load[(t & 1) ? pairs - 1 - b : b] += len > EPILOGUE_KB ? len : EPILOGUE_KB;
         }
     }
     double most = 0.0;
     for (double v : load) most = v > most ? v : most;
-    return most + EPILOGUE;
+    return most + EPILOGUE_KB;
 }
 
 int encode_map(CUtensorMap *map, const uint16_t *base, int64_t rows, int64_t cols, int64_t ld, int box_rows)
@@ -926,14 +926,15 @@ int skim_launch_err_lfull(skim_ctx *ctx, const uint16_t *D, int64_t rows, int64_
     // Half the contraction where H turns out symmetric, as a Gram matrix is.  The comparison of H with its transpose
     // reads all of H (2 B per entry) under a contraction of rows MACs per entry: at the measured rates the two take equally long
     // near 700 rows (512 x 11008 145 us in full, 158 halved; 768 x 11008 204 and 161).  The further launch, the longer start and
-    // the pair's teardown cost 6 us, so the products saved must take longer: us per call in full and halved, 1536 x 1536 17.6 and 23.0,
-    // 4096 x 1536 25.6 and 29.1, 1024 x 3072 27.1 and 29.2, 3072 x 2048 29.2 and 31.3, 4096 x 2048 37.3 and 35.2, 2048 x 3072
-    // 39.1 and 37.4, 8192 x 1536 44.5 and 39.4, 1024 x 4096 53.8 and 42.5.
+    // the pair's teardown cost 6 us, so the busiest pair must save more than that.  us per call in full and halved where the rule
+    // says full: 1536 x 1536 16.6 and 22.7, 1298 x 3072 31.6 and 37.0, 8192 x 1280 32.0 and 37.0, 768 x 6144 51.8 and 55.6; and
+    // where it says halved: 1298 x 3216 39.1 and 35.0, 4096 x 1792 39.1 and 30.9, 6000 x 1280 40.7 and 28.8, 1024 x 4096 47.3 and 41.1.
     a.asym = nullptr;
     a.asym_n = 0;
     a.leave = skim_lfull_leave_flag(ctx->ws);
     a.piece_kb = nkb;
-    if (!Y && rows >= HALF_MIN_ROWS && a.nt >= HALF_MIN_NT && (double)rows * (double)cols * (double)cols >= HALF_MIN_PRODUCTS && ctx->sm_count * sizeof(int) <= HALF_FLAG_BYTES) {
+    bool halved = !Y && rows >= HALF_MIN_ROWS && a.nt >= HALF_MIN_NT && ctx->sm_count * sizeof(int) <= HALF_FLAG_BYTES;
+    if (halved) {
         // pieces of about the full contraction's length (the accumulator's rounding errors grow with it), or half of that
         // where it balances the blocks clearly better
         double best = 0.0;
@@ -943,6 +944,13 @@ int skim_launch_err_lfull(skim_ctx *ctx, const uint16_t *D, int64_t rows, int64_
             const double v = half_makespan(a.mt, a.nt, nkb, piece, pairs);
             if (c == c0 || v < best * 0.95) { best = v; a.piece_kb = piece; }
         }
+        // the full contraction's rounds of whole tiles, then of cut ones (a piece takes an epilogue's time at least)
+        const int cut = (tiles - a.full_tiles) * a.split;
+        auto round_kb = [](double kb) { return kb > EPILOGUE_KB ? kb : EPILOGUE_KB; };
+        const double full = (a.full_tiles + pairs - 1) / pairs * round_kb(nkb) + (cut + pairs - 1) / pairs * round_kb((double)nkb / a.split) + EPILOGUE_KB;
+        halved = full - best >= HALF_MIN_SAVING;
+    }
+    if (halved) {
         a.asym = (int *)((char *)scratch + skim_lfull_scratch_bytes(rows, cols) - HALF_FLAG_BYTES);
         a.asym_n = 2 * pairs;
         SKIM_CUDA_OK(cudaFuncSetAttribute(skim_lfull_gemm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem(true)));

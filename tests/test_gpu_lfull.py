@@ -170,10 +170,10 @@ def test_lfull_argument_errors(ctx, skimlib):
 
 @pytest.mark.parametrize("rows,cols,symmetric", [(768, 776, True), (1000, 1096, True), (770, 2056, True), (4100, 1024, True), (897, 4104, True),
                                                  (1000, 1096, False), (770, 2056, False), (767, 1096, True),
-                                                 (768, 4424, True), (767, 4432, True), (770, 4432, False), (3700, 2016, True), (3570, 2048, True), (15000, 1000, True), (14900, 1000, True)])
+                                                 (768, 4424, True), (767, 4432, True), (770, 4432, False), (3700, 2016, True), (1298, 3072, True), (1298, 3216, True), (15000, 1000, True), (2048, 2560, True), (2049, 2560, False)])
 def test_lfull_half_contraction_of_a_symmetric_matrix(ctx, oracle, rows, cols, symmetric):
     """Symmetric H, and one that differs from its transpose in a single corner entry (the full contraction must take over), on either
-    side of the rule for the half contraction: 768 rows, four column tiles, rows * cols^2 = 1.5e10 (the smaller calls run in full)."""
+    side of the rule for the half contraction: 768 rows, four column tiles, what the busiest pair of SMs saves (the smaller calls run in full)."""
     ctx.reserve(rows, cols)
     rng = np.random.default_rng(rows + cols)
     D = (rng.standard_normal((rows, cols)) * 2).astype(np.float16)
@@ -184,7 +184,7 @@ def test_lfull_half_contraction_of_a_symmetric_matrix(ctx, oracle, rows, cols, s
     _check_err(ctx, oracle, D, H, 8, rows=sel, label=f"{rows}x{cols} {symmetric}")
 
 
-@pytest.mark.parametrize("rows,cols", [(770, 4432), (2100, 4104), (4100, 2056), (16000, 1032)])
+@pytest.mark.parametrize("rows,cols", [(768, 4424), (1026, 4104), (2100, 4104), (4100, 2056), (16000, 1032), (1298, 3216)])
 def test_lfull_leaves_the_half_contraction(ctx, oracle, rows, cols):
     """H that differs from its transpose everywhere by a rounding, or in one entry that is compared early, late or in between: the
     pairs of CTAs stop at different places, and the full contraction's result is the same bit for bit on every run.  Calls
