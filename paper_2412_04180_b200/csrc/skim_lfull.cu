@@ -613,7 +613,7 @@ skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
                 if (ok) umma_commit(&sy.tmem_full[as]);      // the accumulator is complete once all MMAs are
                 ++it;
             }
-            if (HALF) umma_commit(&sy.drained);
+            if (HALF && !ok) umma_commit(&sy.drained);       // leaving
         }
     } else if (HALF && warp >= GEMM_THREADS / 32) {
         // ------------------------------------------------------------ H against its transpose, under the contraction
@@ -726,7 +726,8 @@ skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
         cluster_sync();                // the counts and the leave flag are in place
         if (threadIdx.x == 0) {
             a.asym[blockIdx.x] = sy.asym | sy.leave;
-            bool ok = !sy.abort;
+            // (a producer that has issued its last block never raises the flag, so a pair that leaves has not finished)
+            bool ok = sy.leave && !sy.abort;
             const int most = max(sy.issued[0], sy.issued[1]);
             for (int b = sy.issued[rank]; b < most && ok; ++b) {
                 ok = mbar_wait<false>(&sy.empty[b % NST], (((uint32_t)(b / NST)) & 1u) ^ 1u, sy);
