@@ -7,7 +7,8 @@
 //   count    one shared-memory atomic per element; its return value is the element's slot inside its bucket.
 //   scatter  bucket base + slot: value and importance (read from global memory here) go to their bucket's place.
 //   order    the buckets that reach from one group of 8 into the next are sorted (groups ascend; inside a group the Lloyd
-//            kernel compares every element with its boundary, so its order does not matter).
+//            kernel compares every element with its boundary, so its order does not matter; in scaled rows the record pass
+//            puts the group in order, for sums that are the same on every run).
 //   then     one pass over the row (skim_cluster_phases.cuh) writes the row record -- group records with
 //            prefix sums, group index, segment table -- to global memory, from which the Lloyd kernel
 //            (skim_lloyd.cu) iterates with one warp per row.  Unscaled rows write the compact record.
@@ -17,13 +18,13 @@
 // eight share N/8 (N = 32 per thread).  A row whose values this cannot spread (a bucket with BUCKET_LIMIT elements, or 32 in
 // three neighbouring ones: few distinct values, a clump) is put on a list, for the fp16-key kernel of skim_cluster16.cu or, where
 // scaled, the radix kernel of skim_cluster.cu.  Such a matrix takes 1.1 to 1.4 times what those kernels alone would (sort of 4096
-// rows of a few nearby values, us: 2000 columns 169, 3000 columns 256, 11008 scaled 1281; a bell-shaped row 63, 93, 349).
+// rows of a few nearby values, us: 2000 columns 169, 3000 columns 256, 11008 scaled 1281; of bell-shaped rows 64, 93, 374).
 //
 // Zeros (a pruned matrix) are one value and need no bucket: a row that cannot be spread and has zeros is read again and spread with
 // its zeros between the negative and the positive buckets in column order, by ballots, the scale taken from the other elements.
 // (One pass that always looks for zeros cost rows without any 4-15 %: every register is taken.)  Sort of a matrix with half of its
-// weights zero, us, before (all its rows went to the radix kernel) and now: 4096 x 11008 scaled 1313 -> 405, 4096 x 3000 403 -> 111,
-// 20000 x 128 1444 -> 118; the same matrices unpruned 354, 93 and 98.
+// weights zero, us, before (all its rows went to the radix kernel) and now: 4096 x 11008 scaled 1313 -> 447, 4096 x 3000 403 -> 110,
+// 20000 x 128 1444 -> 118; the same matrices unpruned 374, 93 and 98.
 //
 // Why not a radix sort: rows of 32-bit keys took four passes, each with ballots or random shared-memory traffic of all
 // elements (1.17 ms for 4096 x 11008); 16-bit keys two (0.284 ms).  What bounds this kernel is the same resource,
