@@ -279,8 +279,8 @@ int skim_dequantize(skim_ctx *ctx, const uint32_t *packed, const int32_t *row_or
 /*
  * y = Wq x straight from the packed form, Wq as defined for skim_dequantize but never rounded to
  * binary16 or stored: y_i = sum_j float(lut[i][code_ij]) * z_j with z_j = float(x_j) * s_j in
- * binary32 (z = x when s == NULL).  The sum is accumulated in binary32 (per lane in element
- * order, then a 5-level tree), so |y_i - exact| <= (cols/32 + 8) * 2^-24 * sum_j |term_ij|.
+ * binary32 (z = x when s == NULL).  The sum is accumulated in binary32 (per lane in four
+ * interleaved sums in element order, then a tree), so |y_i - exact| <= (cols/32 + 8) * 2^-24 * sum_j |term_ij|.
  *   x  [cols] binary16 bit patterns (device);  y  out [rows] binary32, source-row order (device)
  */
 int skim_matvec(skim_ctx *ctx, const uint32_t *packed, const int32_t *row_order, const int64_t *group_info,

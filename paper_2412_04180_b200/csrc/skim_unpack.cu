@@ -4,13 +4,16 @@
 //   skim_dequantize  packed codes + per-row codebooks (+ alpha) -> fp16 matrix in source-row order
 //   skim_matvec      y = Wq x taken straight from the packed codes, never forming Wq
 //
-// Codebook lookups go to the warp's copy of the row's codebook in shared memory, 16 consecutive words: no bank conflicts,
-// one wavefront of the L1 data path per 32 elements (a shuffle takes that path for twice as long).
-// A warp takes 256 columns of a row at a time; the per-column vector (alpha, or z = alpha x) sits in shared memory.  What a
-// warp needs of its first row is on its way while that vector is staged.
-//   dequantiser  bound by its writes: b/8 B in and 2 B out per element (4096 x 11008 24.4 us, a plain fill of the output 24.3)
-//   mat-vec      bound by the L1 data path (2.7 wavefronts per 32 elements: a lookup each, the reads of z and the packed words; busy
-//                13.2 of 17.3 us at 4096 x 11008), then by issue and, at the usual sizes, by its start and end
+// The codebook of a warp's row sits in registers, as planes of its entries' low and high bytes: a byte permutation takes four codes at
+// once out of eight entries, so that a lookup costs two permutations per four elements (four at width 4) and no memory access.  (A load
+// from the warp's copy in shared memory, as before, is a wavefront of the L1 data path per 32 elements, and its address two more
+// operations per element.)  A warp takes 256 columns of a row at a time, eight a lane; the per-column vector (alpha, or z = alpha x) sits
+// in shared memory.  What a warp needs of its first row is on its way while that vector is staged.
+//   mat-vec      bound by the integer pipe (16 lanes a clock and scheduler: about 3 operations per element there), then by its start and
+//                end.  4096 x 11008 at 3.0 bits 18.7 -> 13.9 us, 22016 x 8192 55.6 -> 44.2 us
+//   dequantiser  bound by its writes: b/8 B in and 2 B out per element (4096 x 11008 26.8 -> 26.5 us scaled, 25.0 -> 23.7 unscaled; 4096 x
+//                4096 13.6 -> 11.6).  Lanes that own 32 columns and walk rows, the codes brought by bulk copies: 24.7 unscaled, and 22.6 for
+//                the mat-vec (too few warps for the chain of a row).  Requesting whole rows into L2 first: slower by 5 % at 22016 x 8192
 #include "skim_internal.cuh"
 
 namespace {
@@ -48,48 +51,119 @@ struct Groups {
     }
 };
 
-// The shared address of a codebook as the lookups take it.  The lookups are assembly that the compiler does not see as reads of the
-// array: this call, before and after the array is written, keeps them on their side of the stores.
-__device__ __forceinline__ uint32_t codebook_address(const float *book)
+// Eight codes of B bits (the low 8 B bits of x; above them anything) as the eight nibbles of a word.
+template <int B>
+__device__ __forceinline__ uint32_t nibbles(uint32_t x)
 {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %1;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(book)) : "memory");
-    return r;
+    if constexpr (B == 4) {
+        return x;
+    } else if constexpr (B == 3) {
+        // halves of 12 bits, bytes of 6, nibbles of 3; what comes along above each is cleared at the end
+        const uint32_t y = (x & 0x00000fffu) | ((x << 4) & 0xfffff000u);
+        const uint32_t z = (y & 0x00ff00ffu) | ((y << 2) & 0xff00ff00u);
+        return ((z & 0x0f0f0f0fu) | ((z << 1) & 0xf0f0f0f0u)) & 0x77777777u;
+    } else if constexpr (B == 2) {
+        const uint32_t y = __byte_perm(x, 0u, 0x4140);
+        const uint32_t z = (y | (y << 4)) & 0x0f0f0f0fu;
+        return (z | (z << 2)) & 0x33333333u;
+    } else {
+        const uint32_t y = (x | (x << 12)) & 0x000f000fu;
+        const uint32_t z = (y | (y << 6)) & 0x03030303u;
+        return (z | (z << 3)) & 0x11111111u;
+    }
 }
 
-// Codebook entry of a code, the codebook at shared address `book` (64-byte aligned).  `code4` holds the code in bits 2 .. B + 1
-// among others: one logic operation makes the address.
+// A codebook in registers, as byte planes: lo[i], hi[i] hold the low and high bytes of entries 4 i .. 4 i + 3.
 template <int B>
-__device__ __forceinline__ float lookup(uint32_t book, uint32_t code4)
+struct Book {
+    static constexpr int N = B == 4 ? 4 : B == 3 ? 2 : 1;
+    uint32_t lo[N], hi[N];
+    // entries: binary16, 8-byte aligned
+    __device__ __forceinline__ explicit Book(const uint16_t *entries)
+    {
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            const uint2 e = reinterpret_cast<const uint2 *>(entries)[i];
+            lo[i] = __byte_perm(e.x, e.y, 0x6420);
+            hi[i] = __byte_perm(e.x, e.y, 0x7531);
+        }
+    }
+    // The entries of eight codes, two a word.
+    __device__ __forceinline__ void look_up(uint32_t n, uint32_t (&h)[4]) const
+    {
+        // a permutation takes four selectors of 4 bits, whose top bit must be clear
+        const uint32_t s = B == 4 ? n & 0x77777777u : n;
+        const uint32_t top = B == 4 ? (n >> 3) & 0x11111111u : 0u;
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const uint32_t su = u ? s >> 16 : s;
+            uint32_t l, g;
+            if constexpr (B == 4) {
+                const uint32_t upper = __byte_perm(0x0000ff00u, 0u, u ? top >> 16 : top);       // the bytes of codes 8 .. 15
+                l = (__byte_perm(lo[0], lo[1], su) & ~upper) | (__byte_perm(lo[2], lo[3], su) & upper);
+                g = (__byte_perm(hi[0], hi[1], su) & ~upper) | (__byte_perm(hi[2], hi[3], su) & upper);
+            } else {
+                l = __byte_perm(lo[0], lo[N - 1], su);
+                g = __byte_perm(hi[0], hi[N - 1], su);
+            }
+            h[2 * u] = __byte_perm(l, g, 0x5140);
+            h[2 * u + 1] = __byte_perm(l, g, 0x7362);
+        }
+    }
+};
+
+// Two binary32 operations in one instruction; the same results as two.
+__device__ __forceinline__ unsigned long long pack2(float a, float b)
 {
-    float v;
-    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"((code4 & (((1u << B) - 1u) << 2)) | book));
-    return v;
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack2(unsigned long long v, float &a, float &b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c)
+{
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b)
+{
+    unsigned long long r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
 }
 
 constexpr int UT = 1024;            // threads per block, one block per SM
 constexpr int UW = UT / 32;
 constexpr int STEP = 256;           // columns a warp takes at a time
 
-// The eight codes of the lane's elements (8 B bits at byte `at` B of the row), as loaded: at width 3 they may lie in two words, which
-// are only put together when they are used, so that the load does not have to be waited for before.
+// The lane's codes of a row, from step t on: those of a step are 8 B bits at byte (32 t + lane) B, asked for with `ask` and put together with `get` when
+// they are used, so that the load does not have to be waited for before.
 template <int B>
 struct LaneCodes {
-    uint32_t lo, hi;
-    __device__ __forceinline__ void load(const uint8_t *row, int at)
+    const unsigned char *at, *at2;  // for B = 3 the word that holds its first byte, and the next one if the bits reach into it
+    int shift;                      // B = 3: the first byte's bit in its word
+    __device__ __forceinline__ LaneCodes(const uint32_t *row, int lane, int t)
     {
-        hi = 0u;
-        if (B == 4) lo = __ldg(reinterpret_cast<const uint32_t *>(row) + at);
-        else if (B == 2) lo = __ldg(reinterpret_cast<const uint16_t *>(row) + at);
-        else if (B == 1) lo = __ldg(row + at);
-        else {
-            // the row is padded to 16 bytes, and the second word is only asked for where the bits reach into it
-            const uint32_t *w = reinterpret_cast<const uint32_t *>(row) + (3 * at >> 2);
-            lo = __ldg(w);
-            if ((3 * at & 3) > 1) hi = __ldg(w + 1);
-        }
+        shift = 8 * (3 * lane & 3);
+        at = reinterpret_cast<const unsigned char *>(row) + t * (32 * B) + (B == 3 ? 3 * lane & ~3 : B * lane);
+        at2 = at + (shift > 8 ? 4 : 0);
     }
-    __device__ __forceinline__ uint32_t get(int at) const { return B == 3 ? __funnelshift_r(lo, hi, 8 * (3 * at & 3)) : lo; }
+    // of the t-th step from here
+    __device__ __forceinline__ uint2 ask(int t) const
+    {
+        const int o = t * (32 * B);
+        if (B == 4) return make_uint2(__ldg(reinterpret_cast<const uint32_t *>(at + o)), 0u);
+        if (B == 2) return make_uint2(__ldg(reinterpret_cast<const uint16_t *>(at + o)), 0u);
+        if (B == 1) return make_uint2(__ldg(at + o), 0u);
+        return make_uint2(__ldg(reinterpret_cast<const uint32_t *>(at + o)), __ldg(reinterpret_cast<const uint32_t *>(at2 + o)));
+    }
+    __device__ __forceinline__ void advance(int t)
+    {
+        at += t * (32 * B);
+        at2 += t * (32 * B);
+    }
+    __device__ __forceinline__ uint32_t get(const uint2 &v) const { return B == 3 ? __funnelshift_r(v.x, v.y, shift) : v.x; }
 };
 
 // How a lane's eight values leave: one aligned 16-byte store; or, for rows that are not 16-byte aligned, through the warp's stretch of
@@ -135,54 +209,80 @@ __device__ __forceinline__ int vec_slot(int j)
 
 // Steps [s0, s1) of one row; MATVEC: returns the lane's sum.
 template <int B, int MODE>
-__device__ __forceinline__ float unpack_row(const UnpackArgs &a, const uint8_t *words, uint16_t *dst, int s0, int s1, const float *vec, uint32_t book,
+__device__ __forceinline__ float unpack_row(const UnpackArgs &a, const uint32_t *words, uint16_t *dst, int s0, int s1, const float *vec, const uint16_t *entries,
                                             uint32_t *stage)
 {
     constexpr int AHEAD = 4;                // steps whose codes are in flight
-    const int lane = threadIdx.x & 31, last = (a.cols - 1) / 8;      // the row's last group of eight
-    // two batches take turns: the next one is requested as a whole before the current one is worked on (one step at a time, a
-    // load shares its scoreboard with later ones and is waited for with them)
-    LaneCodes<B> codes[AHEAD], next[AHEAD];
-    float acc = 0.0f;
+    const int lane = threadIdx.x & 31;
+    const Book<B> book(entries);
+    LaneCodes<B> codes(words, lane, s0);
+    const float *v4 = vec + s0 * STEP + lane * 4;
+    int j0 = s0 * STEP + lane * 8;
+    unsigned long long acc[2] = {0ull, 0ull};
+    auto step = [&](int u0, const uint2 &raw, bool whole) {
+        uint32_t h[4];
+        book.look_up(nibbles<B>(codes.get(raw)), h);
+        if (MODE == MATVEC || a.s) {
+            const ulonglong2 va = *reinterpret_cast<const ulonglong2 *>(v4 + u0 * STEP), vb = *reinterpret_cast<const ulonglong2 *>(v4 + u0 * STEP + 128);
+            const unsigned long long v[4] = {va.x, va.y, vb.x, vb.y};
 #pragma unroll
-    for (int u = 0; u < AHEAD; ++u) codes[u].load(words, min((s0 + u) * 32 + lane, last));
-    for (int t0 = s0; t0 < s1; t0 += AHEAD) {
-#pragma unroll
-        for (int u = 0; u < AHEAD; ++u) next[u].load(words, min((t0 + AHEAD + u) * 32 + lane, last));
-#pragma unroll
-        for (int u = 0; u < AHEAD; ++u) {
-            const int t = t0 + u;
-            if (t < s1) {
-                const uint32_t c = codes[u].get(min(t * 32 + lane, last));
-                float r[8];
-#pragma unroll
-                for (int e = 0; e < 8; ++e) r[e] = lookup<B>(book, e * B >= 2 ? c >> (e * B - 2) : c << (2 - e * B));
-                if (MODE == MATVEC || a.s) {
-                    const float4 va = *reinterpret_cast<const float4 *>(vec + t * STEP + lane * 4), vb = *reinterpret_cast<const float4 *>(vec + t * STEP + 128 + lane * 4);
-                    const float v[8] = {va.x, va.y, va.z, va.w, vb.x, vb.y, vb.z, vb.w};
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) {
-                        if (MODE == MATVEC) acc = fmaf(r[e], v[e], acc);
-                        else r[e] = __fmul_rn(r[e], v[e]);
-                    }
-                }
-                if constexpr (MODE == MATVEC) continue;
-                else {
-                uint32_t h[4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const __half2 v = __floats2half2_rn(r[2 * e], r[2 * e + 1]);
-                    h[e] = *reinterpret_cast<const uint32_t *>(&v);
-                }
-                const int j0 = t * STEP + lane * 8;
-                if (MODE == STORE_STAGED || j0 < a.cols) store8<MODE>(dst, j0, a.cols, h, stage);
+            for (int u = 0; u < 4; ++u) {
+                const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&h[u]));
+                if constexpr (MODE == MATVEC) {
+                    acc[u & 1] = fma2(pack2(f.x, f.y), v[u], acc[u & 1]);
+                } else {
+                    float p, q;
+                    unpack2(mul2(pack2(f.x, f.y), v[u]), p, q);
+                    const __half2 r = __floats2half2_rn(p, q);
+                    h[u] = *reinterpret_cast<const uint32_t *>(&r);
                 }
             }
         }
+        if constexpr (MODE != MATVEC) {
+            const int j = j0 + u0 * STEP;
+            if (MODE == STORE_VEC && whole)
+                *reinterpret_cast<uint4 *>(dst + j) = make_uint4(h[0], h[1], h[2], h[3]);
+            else
+                store8<MODE>(dst, j, a.cols, h, stage);
+        }
+    };
+    // By AHEAD steps: two batches take turns, the next one requested as a whole before the current one is worked on (one step at a
+    // time, a load shares its scoreboard with later ones and is waited for with them).  The last batch holds what is left, and the row's
+    // ragged end: lanes past it have nothing (STORE_STAGED: they help with the stores).
+    const int batches = max(min(s1, a.cols / STEP) - s0, 0) / AHEAD, left = s1 - s0 - batches * AHEAD;
+    uint2 now[AHEAD], next[AHEAD];
+    auto ask_left = [&](int j, uint2 (&to)[AHEAD]) {
 #pragma unroll
-        for (int u = 0; u < AHEAD; ++u) codes[u] = next[u];
+        for (int u = 0; u < AHEAD; ++u) to[u] = u < left && j + u * STEP < a.cols ? codes.ask(u) : make_uint2(0u, 0u);
+    };
+    if (batches) {
+#pragma unroll
+        for (int u = 0; u < AHEAD; ++u) now[u] = codes.ask(u);
+    } else {
+        ask_left(j0, now);
     }
-    return acc;
+    for (int b = 1; b <= batches; ++b) {
+        codes.advance(AHEAD);
+        if (b < batches) {
+#pragma unroll
+            for (int u = 0; u < AHEAD; ++u) next[u] = codes.ask(u);
+        } else {
+            ask_left(j0 + AHEAD * STEP, next);
+        }
+#pragma unroll
+        for (int u = 0; u < AHEAD; ++u) step(u, now[u], true);
+        v4 += AHEAD * STEP;
+        j0 += AHEAD * STEP;
+#pragma unroll
+        for (int u = 0; u < AHEAD; ++u) now[u] = next[u];
+    }
+#pragma unroll
+    for (int u = 0; u < AHEAD; ++u)
+        if (u < left && (MODE == STORE_STAGED || j0 + u * STEP < a.cols)) step(u, now[u], j0 + u * STEP - lane * 8 + STEP <= a.cols);
+    float p, q, r, v;
+    unpack2(acc[0], p, q);
+    unpack2(acc[1], r, v);
+    return (p + q) + (r + v);
 }
 
 // Packed rows are dealt round-robin to the blocks, so that every SM gets the same number (within one); `parts` warps share a
@@ -191,11 +291,13 @@ template <int MODE>
 __global__ void __launch_bounds__(UT) skim_unpack_kernel(UnpackArgs a, int steps, int parts)
 {
     extern __shared__ __align__(16) float vec[];          // [steps][STEP] (scaled, or the mat-vec), then (STORE_STAGED) [UW][STEP / 2] words
-    __shared__ __align__(128) float books[UW][16];
+    __shared__ __align__(16) uint16_t books[UW][16];
     __shared__ float sums[UW];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const bool use_vec = MODE == MATVEC || a.s;
     uint32_t *stage = reinterpret_cast<uint32_t *>(vec + (use_vec ? steps * STEP : 0)) + (MODE == STORE_STAGED ? warp * (STEP / 2) : 0);
+    skim_let_next_kernel_start();
+    skim_wait_for_previous_kernel();
     const Groups g(a);
     const int part = warp % parts, hop = UW / parts * (int)gridDim.x;
     const int s0 = steps * part / parts, s1 = steps * (part + 1) / parts;
@@ -226,9 +328,9 @@ __global__ void __launch_bounds__(UT) skim_unpack_kernel(UnpackArgs a, int steps
         float acc = 0.0f;
         if (p < g.placed) {
             __syncwarp();
-            if (lane < 16) books[warp][lane] = __half2float(__ushort_as_half(entry));
+            if (lane < 16) books[warp][lane] = entry;
             __syncwarp();
-            const uint32_t book = codebook_address(books[warp]);
+            const uint16_t *book = books[warp];
             const int nsrc = p + hop < g.placed ? __ldg(a.row_order + p + hop) : 0;      // the next row's, one row early
             int u = 0, first = g.start[0];
             long long word = g.word[0];
@@ -236,7 +338,7 @@ __global__ void __launch_bounds__(UT) skim_unpack_kernel(UnpackArgs a, int steps
             for (int v = 1; v < SKIM_MAX_NBITS; ++v)
                 if (v < a.nb && p >= g.start[v]) { u = v; first = g.start[v]; word = g.word[v]; }
             const int width = a.bmin + u;
-            const uint8_t *words = reinterpret_cast<const uint8_t *>(a.packed + word + (int64_t)(p - first) * skim_row_stride_words(a.cols, width));
+            const uint32_t *words = a.packed + word + (int64_t)(p - first) * skim_row_stride_words(a.cols, width);
             uint16_t *dst = a.out + (int64_t)src * a.ld;
             switch (width) {
             case 1: acc = unpack_row<1, MODE>(a, words, dst, s0, s1, vec, book, stage); break;
@@ -244,7 +346,6 @@ __global__ void __launch_bounds__(UT) skim_unpack_kernel(UnpackArgs a, int steps
             case 3: acc = unpack_row<3, MODE>(a, words, dst, s0, s1, vec, book, stage); break;
             default: acc = unpack_row<4, MODE>(a, words, dst, s0, s1, vec, book, stage); break;
             }
-            codebook_address(books[warp]);
             if (MODE == MATVEC) {
 #pragma unroll
                 for (int off = 16; off; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
@@ -291,10 +392,7 @@ int launch_unpack(skim_ctx *ctx, void (*kernel)(UnpackArgs, int, int), const Unp
     if (smem + UNPACK_STATIC_SMEM > 48 * 1024)
         SKIM_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->max_smem_optin - (int)UNPACK_STATIC_SMEM));
     const unsigned blocks = (unsigned)(a.rows < ctx->sm_count ? a.rows : ctx->sm_count);      // one block per SM
-    kernel<<<blocks, UT, smem, ctx->stream>>>(a, steps, unpack_parts(ctx, a.rows, steps));
-    SKIM_CUDA_OK(cudaGetLastError());
-    ctx->launches += 1;
-    return SKIM_OK;
+    return skim_launch_dependent(ctx, kernel, dim3(blocks), UT, smem, a, steps, unpack_parts(ctx, a.rows, steps));
 }
 
 }  // namespace

@@ -65,6 +65,17 @@ def test_unpack_matches_oracle_on_ragged_widths(ctx, oracle, cols, scaled):
     _check(ctx, oracle, em, s, cols, [1, 2, 3, 4], cols)
 
 
+@pytest.mark.parametrize("cols", [1016, 1023, 1024, 1025, 1281, 2040, 2048, 2056, 3328])
+@pytest.mark.parametrize("width", [1, 2, 3, 4])
+def test_unpack_around_whole_batches(ctx, oracle, cols, width):
+    """Rows that end just before, at and behind four steps of 256 columns (codes are requested by four steps), every code of every width,
+    codebook entries of either sign and subnormal ones."""
+    em, s = _synthetic_emit(oracle, 9, cols, [1, 2, 3, 4], 900 + cols, width % 2 == 0, widths=[width] * 9)
+    em["lut"][::3, : 1 << width] = np.arange(1 << width, dtype=np.uint16) * 0x0801 + 3          # subnormal and small values, all bytes in use
+    em["lut"][1::3, 0] = 0x8001
+    _check(ctx, oracle, em, s, cols, [1, 2, 3, 4], cols + width)
+
+
 @pytest.mark.parametrize("bit_set", [[1], [2, 3], [3], [3, 4], [4], [1, 2, 3]])
 def test_unpack_other_bit_sets_and_unaligned_output(ctx, oracle, bit_set):
     em, s = _synthetic_emit(oracle, 65, 777, bit_set, 31 + len(bit_set), True)
