@@ -19,6 +19,11 @@
 //            thousand times another (the minimiser jumps where an outlier enters the prefix), and a thousand nodes
 //            can share one split point (it stays put while the elements behind it weigh nothing).  Nodes that end inside a
 //            thread's stretch are written at once; the rest meet in a segmented minimum over the lanes, then over the warps.
+//            Not every position is needed: only F_K(m), K the largest width, is asked of the last layer, so layer K - 1 is needed at the split
+//            points of that alone, and so on down.  The minimisers of a layer lie at or above the ones of the layer before it,
+//            t_{j-1}(i) <= t_j(i) (the cost is Monge), so when layer j - 1 is known, layer j needs no position below
+//            L_j = t_{j-1}(t_{j-1}(... (m))), K - j times, and no split point below t_{j-1}(L_j).  With 16 clusters that leaves about 60 %
+//            of all candidates: 256 x 4096 928 -> 703 us.
 //   result   for every width the split points are walked back from the row's end; centroid = weighted mean of
 //            its interval (an interval without weight: mean of its first and last value), error = F_k(m).
 // All widths share the layers: F_2, F_4, F_8, F_16 are read off on the way.
@@ -196,18 +201,22 @@ __global__ void __launch_bounds__(XT, 1024 / XT) skim_exact_kernel(ClusterArgs a
         __syncthreads();
 
         // ------------------------------------------------------------ layers 2 .. kmax
-        const int layers = min(min(kmax, nd - 1), m);         // widths with k >= nd take the distinct values instead
+        // up to the largest width with k < nd (the others take the distinct values instead)
+        int layers = kmax;
+        while (layers >= nd) layers >>= 1;
+        // Positions below lowest = L_j are not needed in layer j, and split points below tmin not tried (see the top of the file); L_1 = 1.
+        int lowest = layers > 2 ? 2 : m, tmin = 1;
         for (int j = 2; j <= layers; ++j) {
-            const int n = m - j + 1;                           // positions p = 1 .. n  <->  i = j + p - 1
+            const int n = m - lowest + 1;                      // positions p = 1 .. n  <->  i = lowest + p - 1
             int L = 1;
             while ((1 << L) - 1 < n) ++L;
-            if (tid == 0) optarr[0] = (uint16_t)(j - 1);
+            if (tid == 0) optarr[0] = (uint16_t)tmin;
             __syncthreads();
             for (int lev = 0; lev < L; ++lev) {
                 const int sh_h = L - 1 - lev, h = 1 << sh_h;
                 const int nvalid = (n / h + 1) >> 1;                 // nodes (2q + 1) h <= n of this level
                 // a node's position, and the range of split points its two finished neighbours leave it
-                auto node_i = [&](int q) { return j + ((2 * q + 1) << sh_h) - 1; };
+                auto node_i = [&](int q) { return lowest + ((2 * q + 1) << sh_h) - 1; };
                 auto node_tlo = [&](int q) { return (int)optarr[(2 * q) << sh_h]; };
                 auto node_thi = [&](int q) {
                     const int thi = node_i(q) - 1, right = (2 * q + 2) << sh_h;
@@ -215,7 +224,7 @@ __global__ void __launch_bounds__(XT, 1024 / XT) skim_exact_kernel(ClusterArgs a
                 };
                 // the list of candidates: node q has P(q) = tlo(q) - tlo(0) + q before its own tlo(q) .. thi(q) (where the limit
                 // t < i cuts a range short of its right neighbour's minimiser, the missing split points are skipped)
-                const int tmin = (int)optarr[0], total = node_thi(nvalid - 1) - tmin + nvalid;
+                const int total = node_thi(nvalid - 1) - tmin + nvalid;
                 const int chunk = ((total + XT - 1) / XT) | 1;       // odd: neighbouring lanes' reads fall into different banks
                 const int xa = min(tid * chunk, total), xb = min(xa + chunk, total);
                 Cand head{__longlong_as_double(0x7ff0000000000000ll), -1, 0}, cur{head.v, X_NONE, 0};
@@ -307,13 +316,13 @@ __global__ void __launch_bounds__(XT, 1024 / XT) skim_exact_kernel(ClusterArgs a
             // go by from the top, each read in full before it is written.
             uint16_t *Tj = T + (size_t)j * (m + 1);
             constexpr int PER = 4;
-            for (int base = j + (n - 1) / (PER * XT) * (PER * XT); base >= j; base -= PER * XT) {
+            for (int base = lowest + (n - 1) / (PER * XT) * (PER * XT); base >= lowest; base -= PER * XT) {
                 double an[PER];
 #pragma unroll
                 for (int u = 0; u < PER; ++u) {
                     const int i = base + tid + u * XT;
                     if (i <= m) {
-                        const int t = optarr[i - j + 1];
+                        const int t = optarr[i - lowest + 1];
                         Tj[i] = (uint16_t)t;
                         double t0, t1, av, i0, i1, ia;
                         Q.load(t, t0, t1, av);
@@ -329,6 +338,12 @@ __global__ void __launch_bounds__(XT, 1024 / XT) skim_exact_kernel(ClusterArgs a
                     if (i <= m) Q.set_a(i, an[u]);
                 }
             }
+            // the next layer's limits, from this one's minimisers
+            int x = m;
+            for (int u = layers - j - 1; u > 0; --u) x = max((int)optarr[x - lowest + 1], lowest);
+            x = max(x, lowest + 1);
+            if (j < layers) tmin = max((int)optarr[x - lowest + 1], lowest);
+            lowest = x;
             __syncthreads();
         }
 

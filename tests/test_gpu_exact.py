@@ -101,3 +101,24 @@ def test_exact_block_sizes(ctx, oracle, rows, cols):
     ora = oracle.cluster_rows_exact(w[-n:], g[-n:], BITS)
     np.testing.assert_allclose(err.cpu().numpy()[-n:], ora["err"], rtol=1e-6)
     assert bool((torch.diff(cent[:, 14:], dim=1) >= 0).all())
+
+
+@pytest.mark.parametrize("bit_set", [[1, 2, 3, 4], [1, 2, 3], [4], [1]])
+def test_exact_rows_whose_weight_lies_at_one_end(ctx, oracle, bit_set):
+    """Layers leave out positions that the chain of split points cannot reach: rows where that is nearly all of them, or nearly none."""
+    cols = 300
+    rng = np.random.default_rng(77)
+    w = np.sort(rng.standard_normal((12, cols)), axis=1).astype(np.float16)
+    g = np.exp(rng.standard_normal((12, cols))).astype(np.float32)
+    g[0, :250] *= 1e-6                                     # at the upper end
+    g[1, 50:] *= 1e-6                                      # at the lower end
+    g[2, 150:] = 0.0
+    g[3, :150] = 0.0
+    g[4, 40:260] = 0.0
+    w[5] = (np.exp(w[5].astype(np.float64) * 2)).astype(np.float16)
+    w[6, -1] = 4000.0                                      # an outlier at either end
+    w[7, 0] = -4000.0
+    for i, d in ((8, 17), (9, 18), (10, 24), (11, 33)):    # hardly more distinct values than clusters
+        w[i] = (rng.integers(0, d, cols) * 0.25 - 2).astype(np.float16)
+        w[i, :d] = (np.arange(d) * 0.25 - 2).astype(np.float16)
+    _check(ctx, oracle, w, g, bit_set, label="one end")
