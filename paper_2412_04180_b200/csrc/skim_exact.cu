@@ -65,14 +65,22 @@ __device__ __forceinline__ Cand shfl_up(const Cand &c, int off)
     r.t = __shfl_up_sync(0xffffffffu, c.t, off);
     return r;
 }
-// Every lane's candidate becomes the best of its node's candidates in this and the lower lanes (nodes ascend).
+// Every lane's candidate becomes the best of its node's candidates in this and the lower lanes (nodes ascend, so the doubling stops
+// as soon as no node reaches that far).
 __device__ __forceinline__ void segmented_min(Cand &c)
 {
     const int lane = threadIdx.x & 31;
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
-        const Cand o = shfl_up(c, off);
-        if (lane >= off && o.q == c.q && better(o, c)) c = o;
+        const int q = __shfl_up_sync(0xffffffffu, c.q, off);
+        const bool same = lane >= off && q == c.q;
+        if (!__any_sync(0xffffffffu, same)) break;
+        const double v = __shfl_up_sync(0xffffffffu, c.v, off);
+        const int t = __shfl_up_sync(0xffffffffu, c.t, off);
+        if (same && (v < c.v || (v == c.v && t < c.t))) {
+            c.v = v;
+            c.t = t;
+        }
     }
 }
 
@@ -214,7 +222,7 @@ __global__ void __launch_bounds__(XT, 1024 / XT) skim_exact_kernel(ClusterArgs a
             __syncthreads();
             for (int lev = 0; lev < L; ++lev) {
                 const int sh_h = L - 1 - lev, h = 1 << sh_h;
-                const int nvalid = (n / h + 1) >> 1;                 // nodes (2q + 1) h <= n of this level
+                const int nvalid = ((n >> sh_h) + 1) >> 1;                 // nodes (2q + 1) h <= n of this level
                 // a node's position, and the range of split points its two finished neighbours leave it
                 auto node_i = [&](int q) { return lowest + ((2 * q + 1) << sh_h) - 1; };
                 auto node_tlo = [&](int q) { return (int)optarr[(2 * q) << sh_h]; };
@@ -235,38 +243,43 @@ __global__ void __launch_bounds__(XT, 1024 / XT) skim_exact_kernel(ClusterArgs a
                         const int mid = (lo + hi + 1) >> 1;
                         if (node_tlo(mid) - tmin + mid <= xa) lo = mid; else hi = mid - 1;
                     }
-                    int q = lo, i = node_i(q), t = xa - q + tmin;
-                    first = q;
+                    int i = node_i(lo), t = xa - lo + tmin, o = (2 * lo + 1) << sh_h;       // o: the node's place in the tree
+                    first = lo;
                     // `end`: the last split point that is counted as the node's (a split point past its limit i - 1 is replaced by that)
-                    int end = (q + 1 < nvalid) ? node_tlo(q + 1) : node_thi(q);
-                    double i0, i1, ia;
-                    Q.load(i, i0, i1, ia);
-                    double best = __longlong_as_double(0x7ff0000000000000ll);
-                    int bt = min(t, i - 1);
-                    for (int x = xa;;) {
+                    int end = (lo + 1 < nvalid) ? node_tlo(lo + 1) : node_thi(lo);
+                    double i0, i1;
+                    Q.load_i(i, i0, i1);
+                    const double none = __longlong_as_double(0x7ff0000000000000ll);
+                    double best = none, head_v = none;
+                    int bt = min(t, i - 1), head_t = -1;
+                    // a node that ends inside the stretch is written at once; where it began in an earlier one (the first), its
+                    // minimiser is written again below
+                    for (int left = xb - xa; left > 0; --left) {
                         const int te = min(t, i - 1);
                         double t0, t1, av;
                         Q.load(te, t0, t1, av);
                         const double s0 = i0 - t0, s1 = i1 - t1;
                         const double v = s0 > 0.0 ? av - square_over(s1, s0) : av;
-                        if (v < best) { best = v; bt = te; }
-                        if (++x == xb) break;
-                        const bool fin = t == end;
-                        ++t;
-                        if (fin) {
-                            // node q ends inside the stretch: its minimiser is known, unless it began in an earlier one
-                            if (q == first) head = Cand{best, q, bt}; else optarr[(2 * q + 1) << sh_h] = (uint16_t)bt;
-                            ++q;
-                            t = end;
+                        const bool less = v < best;
+                        best = less ? v : best;
+                        bt = less ? te : bt;
+                        if (t == end && left > 1) {
+                            optarr[o] = (uint16_t)bt;
+                            head_v = head_t < 0 ? best : head_v;
+                            head_t = head_t < 0 ? bt : head_t;
+                            o += 2 << sh_h;
                             i += 2 << sh_h;
-                            const int right = (2 * q + 2) << sh_h;
+                            best = none;
+                            bt = min(end, i - 1);
+                            const int right = o + h;
                             end = right <= n ? (int)optarr[right] : i - 1;
                             Q.load_i(i, i0, i1);
-                            best = __longlong_as_double(0x7ff0000000000000ll);
-                            bt = min(t, i - 1);
+                        } else {
+                            ++t;
                         }
                     }
-                    cur = Cand{best, q, bt};
+                    if (head_t >= 0) head = Cand{head_v, first, head_t};
+                    cur = Cand{best, o >> (sh_h + 1), bt};
                 }
                 // ---- over the lanes
                 segmented_min(cur);
