@@ -8,7 +8,9 @@
 // evaluations.  One block owns a row and reads the row record the sort kernels leave (sorted values and
 // importances by groups of 8 with their binary64 prefix sums).
 //
-//   prefix   the record's two-level prefix sums become flat arrays P0, P1, P2 (sums of g, g x, g x^2) and
+//   prefix   the record's two-level prefix sums become flat arrays P0, P1, P2 (sums of g, g x, g x^2) with a position per distinct
+//            value -- no optimum splits equal values, and a row of 11 008 binary16 weights has some 6600 values (512 x 11008
+//            3972 -> 2632 us, 256 x 4096 with 3280 values a row 648 -> 597) -- and
 //            A = F_{j-1} - P2: the cost of a candidate is A(t) - S1^2 / S0 up to a term of i alone, so a candidate needs
 //            (P0, P1, A)(t), 24 bytes.  They sit in shared memory where the row fits, else in global memory.
 //   layer    positions are visited like the in-order nodes of a perfect binary tree, level by level: a node's
@@ -23,7 +25,7 @@
 //            points of that alone, and so on down.  The minimisers of a layer lie at or above the ones of the layer before it,
 //            t_{j-1}(i) <= t_j(i) (the cost is Monge), so when layer j - 1 is known, layer j needs no position below
 //            L_j = t_{j-1}(t_{j-1}(... (m))), K - j times, and no split point below t_{j-1}(L_j).  With 16 clusters that leaves about 60 %
-//            of all candidates: 256 x 4096 928 -> 703 us.
+//            of all candidates: 256 x 4096 952 -> 726 us a call.
 //   result   for every width the split points are walked back from the row's end; centroid = weighted mean of
 //            its interval (an interval without weight: mean of its first and last value), error = F_k(m).
 // All widths share the layers: F_2, F_4, F_8, F_16 are read off on the way.
@@ -153,15 +155,15 @@ __global__ void __launch_bounds__(XT, 1024 / XT) skim_exact_kernel(ClusterArgs a
     extern __shared__ __align__(16) unsigned char xsmem[];
     constexpr int NW = XT / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int m = a.m;
-    const RowRecord R = row_record(m);
-    const ExactSlot S = exact_slot(m);
+    const int cols = a.m;
+    const RowRecord R = row_record(cols);
+    const ExactSlot S = exact_slot(cols);
     unsigned char *slot = scratch + (size_t)blockIdx.x * slot_bytes;
     uint16_t *T = reinterpret_cast<uint16_t *>(slot + S.t);
     uint16_t *optarr = reinterpret_cast<uint16_t *>(xsmem);           // minimisers of the current layer by node position
-    ExactShared &sh = *reinterpret_cast<ExactShared *>(xsmem + exact_optarr_bytes(m));
+    ExactShared &sh = *reinterpret_cast<ExactShared *>(xsmem + exact_optarr_bytes(cols));
     Sums<PLACE> Q;
-    Q.init(xsmem + exact_optarr_bytes(m) + ((sizeof(ExactShared) + 15) & ~(size_t)15), slot + S.q, m);
+    Q.init(xsmem + exact_optarr_bytes(cols) + ((sizeof(ExactShared) + 15) & ~(size_t)15), slot + S.q, cols);
     const int kmax = 1 << (a.bmin + a.nb - 1);
     if (blockIdx.x == 0 && tid == 0) *a.sort_count = 0;
 
@@ -175,25 +177,68 @@ __global__ void __launch_bounds__(XT, 1024 / XT) skim_exact_kernel(ClusterArgs a
         const unsigned char *groups = rec + R.groups;
         const double4 *seg = reinterpret_cast<const double4 *>(rec + R.seg);
 
-        // ------------------------------------------------------------ flat prefix sums
-        for (int q = tid; q < R.ngrp; q += XT) {
-            const unsigned char *gr = groups + (size_t)q * SKIM_GROUP_BYTES;
-            const float4 xa = *reinterpret_cast<const float4 *>(gr), xb = *reinterpret_cast<const float4 *>(gr + 16);
-            const float4 ga = *reinterpret_cast<const float4 *>(gr + 32), gb = *reinterpret_cast<const float4 *>(gr + 48);
-            const double4 gp = *reinterpret_cast<const double4 *>(gr + 64);
-            const double4 sb = seg[q >> SKIM_SEG_SHIFT];
-            double p0 = sb.x + gp.x, p1 = sb.y + gp.y, p2 = sb.z + gp.z;
-            const float xs[8] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y, xb.z, xb.w};
-            const float gs[8] = {ga.x, ga.y, ga.z, ga.w, gb.x, gb.y, gb.z, gb.w};
+        // ------------------------------------------------------------ flat prefix sums, a position per distinct value
+        float *xv = reinterpret_cast<float *>(T);                   // the values: rows 0 and 1 of T hold no minimisers
+        int m;                                                       // distinct values
+        {
+            const float *gi = reinterpret_cast<const float *>(rec + R.gi);
+            const int per = (R.ngrp + XT - 1) / XT, q0 = min(tid * per, R.ngrp), q1 = min(q0 + per, R.ngrp);
+            // bit u: element u of group q is the last one of its value
+            auto last_of_value = [&](int q, const float (&xs)[8]) {
+                const float next = q + 1 < R.ngrp ? gi[q + 1] : SKIM_PAD_VALUE;
+                uint32_t r = 0u;
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                Q.set(q * 8 + u, p0, p1, p2);
-                const double g = (double)gs[u], x = (double)xs[u];      // padding: g = 0
-                p0 += g;
-                p1 += g * x;
-                p2 += g * x * x;
+                for (int u = 0; u < 8; ++u)
+                    if (q * 8 + u < cols && (q * 8 + u == cols - 1 || xs[u] != (u < 7 ? xs[u < 7 ? u + 1 : 7] : next))) r |= 1u << u;
+                return r;
+            };
+            auto load_values = [&](int q, float (&xs)[8]) {
+                const float4 xa = *reinterpret_cast<const float4 *>(groups + (size_t)q * SKIM_GROUP_BYTES), xb = *reinterpret_cast<const float4 *>(groups + (size_t)q * SKIM_GROUP_BYTES + 16);
+                xs[0] = xa.x; xs[1] = xa.y; xs[2] = xa.z; xs[3] = xa.w; xs[4] = xb.x; xs[5] = xb.y; xs[6] = xb.z; xs[7] = xb.w;
+            };
+            int own = 0;
+            for (int q = q0; q < q1; ++q) {
+                float xs[8];
+                load_values(q, xs);
+                own += __popc(last_of_value(q, xs));
             }
-            if (q == R.ngrp - 1) Q.set(q * 8 + 8, p0, p1, p2);
+            int inc = own;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const int t = __shfl_up_sync(0xffffffffu, inc, off);
+                if (lane >= off) inc += t;
+            }
+            if (lane == 31) sh.first[warp] = inc;
+            __syncthreads();
+            int at = inc - own;
+            m = 0;
+            for (int w = 0; w < NW; ++w) {
+                if (w < warp) at += sh.first[w];
+                m += sh.first[w];
+            }
+            for (int q = q0; q < q1; ++q) {
+                float xs[8];
+                load_values(q, xs);
+                const unsigned char *gr = groups + (size_t)q * SKIM_GROUP_BYTES;
+                const float4 ga = *reinterpret_cast<const float4 *>(gr + 32), gb = *reinterpret_cast<const float4 *>(gr + 48);
+                const double4 gp = *reinterpret_cast<const double4 *>(gr + 64);
+                const double4 sb = seg[q >> SKIM_SEG_SHIFT];
+                double p0 = sb.x + gp.x, p1 = sb.y + gp.y, p2 = sb.z + gp.z;
+                const float gs[8] = {ga.x, ga.y, ga.z, ga.w, gb.x, gb.y, gb.z, gb.w};
+                const uint32_t ends = last_of_value(q, xs);
+                if (q == 0) Q.set(0, p0, p1, p2);
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const double g = (double)gs[u], x = (double)xs[u];      // padding: g = 0
+                    p0 += g;
+                    p1 += g * x;
+                    p2 += g * x * x;
+                    if (ends >> u & 1u) {
+                        xv[at] = xs[u];
+                        Q.set(++at, p0, p1, p2);
+                    }
+                }
+            }
         }
         __syncthreads();
 
@@ -327,7 +372,7 @@ __global__ void __launch_bounds__(XT, 1024 / XT) skim_exact_kernel(ClusterArgs a
             }
             // F_j - P2 becomes the previous layer.  A position needs the old values of lower ones only: stretches of positions
             // go by from the top, each read in full before it is written.
-            uint16_t *Tj = T + (size_t)j * (m + 1);
+            uint16_t *Tj = T + (size_t)j * (cols + 1);
             constexpr int PER = 4;
             for (int base = lowest + (n - 1) / (PER * XT) * (PER * XT); base >= lowest; base -= PER * XT) {
                 double an[PER];
@@ -376,7 +421,7 @@ __global__ void __launch_bounds__(XT, 1024 / XT) skim_exact_kernel(ClusterArgs a
                 double total = 0.0, i0, i1, ia;
                 Q.load(m, i0, i1, ia);
                 for (int jj = k; jj >= 1; --jj) {
-                    const int t = (jj == 1) ? 0 : (int)T[(size_t)jj * (m + 1) + i];
+                    const int t = (jj == 1) ? 0 : (int)T[(size_t)jj * (cols + 1) + i];
                     double t0, t1, ta;
                     Q.load(t, t0, t1, ta);
                     const double s0 = i0 - t0, s1 = i1 - t1;
@@ -385,9 +430,7 @@ __global__ void __launch_bounds__(XT, 1024 / XT) skim_exact_kernel(ClusterArgs a
                         c = (float)(s1 / s0);
                         total += (Q.get_p2(i) - Q.get_p2(t)) - s1 * s1 / s0;
                     } else {
-                        const float xf = *(reinterpret_cast<const float *>(groups + (size_t)(t >> 3) * SKIM_GROUP_BYTES) + (t & 7));
-                        const float xl = *(reinterpret_cast<const float *>(groups + (size_t)((i - 1) >> 3) * SKIM_GROUP_BYTES) + ((i - 1) & 7));
-                        c = (float)(0.5 * ((double)xf + (double)xl));
+                        c = (float)(0.5 * ((double)xv[t] + (double)xv[i - 1]));
                     }
                     cout[jj - 1] = c;
                     i = t;
