@@ -319,6 +319,21 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t *v)
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+// Whole 32-byte sectors in one access: a lane of the epilogue has a row of its own, so that narrower ones take the L1 data path once per
+// lane each (and a store of half a sector the L2 twice).
+__device__ __forceinline__ void ld_sector(const void *p, uint4 &a, uint4 &b)
+{
+    asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
+                 : "l"(p));
+}
+__device__ __forceinline__ void st_sector(void *p, const uint32_t *v)
+{
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]),
+                 "r"(v[6]), "r"(v[7])
+                 : "memory");
+}
+
 struct GemmArgs {
     const uint16_t *D;       // [rows][ldd] binary16 (also operand A, through its tensor map)
     int64_t ldd;
@@ -331,6 +346,7 @@ struct GemmArgs {
     SkimLfullClusters cl;    // with Y, optional: sums of Y alpha by cluster
     int *asym;               // [asym_n] per block of the half contraction: H is not symmetric in the part it compared, or the block left
     int asym_n;
+    int sectors;             // rows of D (and labels) start at whole sectors, and cols is a multiple of 32
     unsigned *leave;         // half contraction: some block has found H not symmetric (zero between calls)
     int piece_kb;            // half contraction: a tile's list of K blocks is cut into pieces of about this length
     unsigned long long *status;
@@ -647,6 +663,21 @@ skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
             uint4 dv[4], dn[4];
             uint2 lv[4], ln[4];
             auto fetch = [&](int c, uint4 (&d)[4], uint2 (&l)[4]) {
+                if (a.sectors) {
+                    const int col = n0 + c;
+                    const bool in = c < c0 + w.n / 2 && col < a.cols;                 // cols is a multiple of 32
+#pragma unroll
+                    for (int v = 0; v < 4; v += 2) {
+                        d[v] = d[v + 1] = make_uint4(0u, 0u, 0u, 0u);
+                        if (in) ld_sector(drow + col + v * 8, d[v], d[v + 1]);
+                    }
+                    if (by_cluster) {
+                        uint4 x = make_uint4(0u, 0u, 0u, 0u), y = x;
+                        if (in) ld_sector(a.cl.labels + lrow * a.cols + col, x, y);
+                        l[0] = make_uint2(x.x, x.y); l[1] = make_uint2(x.z, x.w); l[2] = make_uint2(y.x, y.y); l[3] = make_uint2(y.z, y.w);
+                    }
+                    return;
+                }
 #pragma unroll
                 for (int v = 0; v < 4; ++v) {
                     const int col = n0 + c + v * 8;
@@ -671,9 +702,8 @@ skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
                     if (!HALF && a.Y && row < a.rows) {
                         float *yrow = a.Y + (int64_t)row * a.ldy + col;
 #pragma unroll
-                        for (int g = 0; g < 8; ++g)
-                            if (col + g * 4 + 4 <= a.cols)
-                                *reinterpret_cast<uint4 *>(yrow + g * 4) = make_uint4(v[g * 4], v[g * 4 + 1], v[g * 4 + 2], v[g * 4 + 3]);
+                        for (int g = 0; g < 4; ++g)
+                            if (col + g * 8 + 8 <= a.cols) st_sector(yrow + g * 8, v + g * 8);
                     }
                     // columns past the matrix have a zero accumulator and a zero alpha
                     if (by_cluster) add_by_cluster(slot, v, lv, ep.alpha + c);
@@ -898,6 +928,7 @@ int skim_launch_err_lfull(skim_ctx *ctx, const uint16_t *D, int64_t rows, int64_
     a.Y = Y;
     a.ldy = ldy;
     a.cl = clusters ? *clusters : SkimLfullClusters{};
+    a.sectors = cols % 32 == 0 && ((reinterpret_cast<uintptr_t>(D) | (uintptr_t)ldd * 2) & 31u) == 0 && (!clusters || (reinterpret_cast<uintptr_t>(clusters->labels) & 31u) == 0);
     const size_t smem = gemm_smem(false);
     a.status = (unsigned long long *)ctx->ws;
     SKIM_CUDA_OK(cudaFuncSetAttribute(skim_lfull_gemm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
