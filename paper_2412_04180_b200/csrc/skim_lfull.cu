@@ -112,6 +112,8 @@ __global__ void __launch_bounds__(RES_T) skim_residual_kernel(ResidualArgs a)
     __shared__ float cs[16];
     const int tid = threadIdx.x;
     const int64_t row = blockIdx.x;
+    skim_wait_for_previous_kernel();
+    skim_let_next_kernel_start();
     const uint16_t *Wr = a.W + row * a.ld;
     const uint4 raw = skiml::load8_weights(Wr, tid * 8, a.cols);
     const int b = a.row_bits ? (int)a.row_bits[row] : a.width;
@@ -527,6 +529,8 @@ skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
     const int ntiles = a.mt * a.nt;
     int nunits = a.full_tiles + (ntiles - a.full_tiles) * a.split;
     HalfList half = {0, 0, HALF ? half_pieces(0, nkb, a.piece_kb) : 1};
+    if (!a.Y) skim_let_next_kernel_start();
+    if (!HALF && a.asym) skim_wait_for_previous_kernel();
     if (HALF) {
         nunits = 0;
         for (int nb = 0; nb < a.nt; ++nb) nunits += a.mt * half_pieces(nb, nkb, a.piece_kb);
@@ -556,6 +560,7 @@ skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
     __syncthreads();
     cluster_sync();
     tc_fence_after();
+    if (HALF || !a.asym) skim_wait_for_previous_kernel();      // nothing is read or written before it
     const uint32_t tmem_base = sy.tmem_base;
 
     // one K block of operands: this CTA's half of either
@@ -790,6 +795,8 @@ constexpr int RED_WARPS = 8;
 __global__ void __launch_bounds__(RED_WARPS * 32)
 skim_lfull_reduce_kernel(GemmArgs a, int exp2, float *__restrict__ err, int64_t err_stride, double *__restrict__ err64)
 {
+    skim_wait_for_previous_kernel();
+    if (!a.Y) skim_let_next_kernel_start();
     bool half = false;
     if (a.asym) {
         int any = 0;
@@ -890,10 +897,7 @@ int skim_launch_residual(skim_ctx *ctx, const uint16_t *W, int64_t rows, int64_t
     a.vec = ((reinterpret_cast<uintptr_t>(D) & 15u) == 0 && ldd % 8 == 0 && cols % 8 == 0 && (!s || (reinterpret_cast<uintptr_t>(s) & 15u) == 0)) ? 1 : 0;
     a.D = D;
     a.status = ws.status;
-    skim_residual_kernel<<<(unsigned)rows, RES_T, 0, ctx->stream>>>(a);
-    SKIM_CUDA_OK(cudaGetLastError());
-    ctx->launches += 1;
-    return SKIM_OK;
+    return skim_launch_dependent(ctx, skim_residual_kernel, dim3((unsigned)rows), RES_T, 0, a);
 }
 
 size_t skim_lfull_cluster_bytes(int64_t rows, int64_t cols)
@@ -986,16 +990,23 @@ int skim_launch_err_lfull(skim_ctx *ctx, const uint16_t *D, int64_t rows, int64_
         a.asym = (int *)((char *)scratch + skim_lfull_scratch_bytes(rows, cols) - HALF_FLAG_BYTES);
         a.asym_n = 2 * pairs;
         SKIM_CUDA_OK(cudaFuncSetAttribute(skim_lfull_gemm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem(true)));
-        skim_lfull_gemm_kernel<true><<<(unsigned)(2 * pairs), GEMM_THREADS + CHECK_WARPS * 32, gemm_smem(true), ctx->stream>>>(map_a, map_b, a, H, ldh);
-        SKIM_CUDA_OK(cudaGetLastError());
-        ctx->launches += 1;
+        rc = skim_launch_dependent(ctx, skim_lfull_gemm_kernel<true>, dim3((unsigned)(2 * pairs)), GEMM_THREADS + CHECK_WARPS * 32, gemm_smem(true), map_a, map_b, a, H, ldh);
+        if (rc) return rc;
     }
     const int units = a.full_tiles + (tiles - a.full_tiles) * a.split;
     const unsigned blocks = (unsigned)(2 * (units < pairs ? units : pairs));    // persistent: one CTA per SM
-    skim_lfull_gemm_kernel<false><<<blocks, GEMM_THREADS, smem, ctx->stream>>>(map_a, map_b, a, H, ldh);
-    SKIM_CUDA_OK(cudaGetLastError());
-    skim_lfull_reduce_kernel<<<(unsigned)((rows + RED_WARPS - 1) / RED_WARPS), RED_WARPS * 32, 0, ctx->stream>>>(a, exp2, err, err_stride, err64);
-    SKIM_CUDA_OK(cudaGetLastError());
-    ctx->launches += 2;
-    return SKIM_OK;
+    const dim3 red((unsigned)((rows + RED_WARPS - 1) / RED_WARPS));
+    if (Y) {
+        // In the scaling-vector update the dependents' blocks, moving in under the contraction and its reduction, cost more than the
+        // launches they save (a step of 4096 x 4096: 257 us so, 249 with ordinary launches).
+        skim_lfull_gemm_kernel<false><<<blocks, GEMM_THREADS, smem, ctx->stream>>>(map_a, map_b, a, H, ldh);
+        SKIM_CUDA_OK(cudaGetLastError());
+        skim_lfull_reduce_kernel<<<red, RED_WARPS * 32, 0, ctx->stream>>>(a, exp2, err, err_stride, err64);
+        SKIM_CUDA_OK(cudaGetLastError());
+        ctx->launches += 2;
+        return SKIM_OK;
+    }
+    rc = skim_launch_dependent(ctx, skim_lfull_gemm_kernel<false>, dim3(blocks), GEMM_THREADS, smem, map_a, map_b, a, H, ldh);
+    if (rc) return rc;
+    return skim_launch_dependent(ctx, skim_lfull_reduce_kernel, red, RED_WARPS * 32, 0, a, exp2, err, err_stride, err64);
 }
