@@ -16,6 +16,8 @@ namespace {
 using namespace skimk;
 
 constexpr int LLOYD_WARPS = 4;   // rows per block
+constexpr int LLOYD_BLOCKS = 7;  // per SM
+constexpr size_t LLOYD_BESIDE = 3072;   // static shared memory of a block, and what the system takes
 constexpr int WIN = 16;          // group-index entries held in registers
 
 // dynamic shared memory of one warp: the group index (binary32, or binary16 with compact records), then 16 bytes
@@ -26,6 +28,9 @@ __host__ __device__ inline size_t lloyd_warp_bytes(int m, bool half_index)
     const size_t idx = ((size_t)sk_entries(m) * (half_index ? 2 : 4) + 15) & ~(size_t)15;
     return idx + (size_t)(nseg + 1) * 16;
 }
+
+// a copy of a row's compact group records
+__host__ __device__ inline size_t lloyd_near_bytes(int m) { return (size_t)((m + 7) >> 3) * SKIM_GROUP_BYTES_HALF; }
 
 struct LloydSmem {
     double errs[32];
@@ -109,6 +114,14 @@ template <bool UNORDERED> struct Group<true, UNORDERED> {
         xh[0] = (uint32_t)q0; xh[1] = (uint32_t)(q0 >> 32); xh[2] = (uint32_t)q1; xh[3] = (uint32_t)(q1 >> 32);
         p = make_double2(__longlong_as_double((long long)q2), __longlong_as_double((long long)q3));
         ld_sector(gr + 32, ga, gb);
+    }
+    __device__ __forceinline__ void load_shared(const unsigned char *gr)
+    {
+        const uint4 v = *reinterpret_cast<const uint4 *>(gr);
+        xh[0] = v.x; xh[1] = v.y; xh[2] = v.z; xh[3] = v.w;
+        p = *reinterpret_cast<const double2 *>(gr + 16);
+        ga = *reinterpret_cast<const float4 *>(gr + 32);
+        gb = *reinterpret_cast<const float4 *>(gr + 48);
     }
     // a binary16 value is <= t exactly when it is <= t rounded down to binary16: four packed compares
     __device__ __forceinline__ int count_le(float t) const
@@ -262,8 +275,9 @@ __device__ __forceinline__ double quotient(double s1, double s0, bool zero)
 // window); loads that one group record, which gives the exact boundary position (values), the
 // prefix sums at the group start and the few elements in between.
 // On return sm.tfs[L] holds the boundary (largest binary32 value still assigned to centroid L).
-template <bool HALF, bool UNORDERED>
-__device__ __forceinline__ void lloyd_warp(const unsigned char *rec, const typename Window<HALF>::Entry *gi, const double2 *segs,
+// LOCAL: `near`, a copy of the group records in shared memory, is read instead of the record.
+template <bool HALF, bool UNORDERED, bool LOCAL>
+__device__ __forceinline__ void lloyd_warp(const unsigned char *rec, const unsigned char *near, const typename Window<HALF>::Entry *gi, const double2 *segs,
                                            int nd, const ClusterArgs &a, int64_t row, LloydSmem &sm)
 {
     const int lane = threadIdx.x & 31;
@@ -331,7 +345,8 @@ __device__ __forceinline__ void lloyd_warp(const unsigned char *rec, const typen
             gstep = gprev >= 0 ? grp_i - gprev : 0;
             gprev = grp_i;
             if (HALF || grp_i != gloaded) {          // (compact records: loading their two sectors always measured as fast)
-                grp.load(groups + (size_t)grp_i * Group<HALF, UNORDERED>::BYTES);
+                if constexpr (LOCAL) grp.load_shared(near + (size_t)grp_i * Group<HALF, UNORDERED>::BYTES);
+                else grp.load(groups + (size_t)grp_i * Group<HALF, UNORDERED>::BYTES);
                 const double2 sb = segs[grp_i >> SKIM_SEG_SHIFT];       // sums of the earlier segments (shared memory)
                 grp.p.x += sb.x;
                 grp.p.y += sb.y;
@@ -461,8 +476,8 @@ __global__ void __launch_bounds__(CODES_T) skim_codes_kernel(ClusterArgs a, int 
 
 // Seven blocks of four rows per SM: an eighth would hold the kernel to 64 registers, which measured slower on every
 // shape (the full-record form spills there).
-template <bool HALF, bool UNORDERED>
-__global__ void __launch_bounds__(LLOYD_WARPS * 32, 7) skim_lloyd_kernel(ClusterArgs a, int rows_in_chunk)
+template <bool HALF, bool UNORDERED, bool LOCAL>
+__global__ void __launch_bounds__(LLOYD_WARPS * 32, LLOYD_BLOCKS) skim_lloyd_kernel(ClusterArgs a, int rows_in_chunk)
 {
     __shared__ LloydSmem sm_all[LLOYD_WARPS];
     extern __shared__ __align__(16) unsigned char gi_all[];      // [LLOYD_WARPS][sk_entries(m)] index entries (binary32, or binary16 with compact records)
@@ -481,7 +496,13 @@ __global__ void __launch_bounds__(LLOYD_WARPS * 32, 7) skim_lloyd_kernel(Cluster
     // the row's group index, copied once
     const int nsk = sk_entries(a.m);
     typedef typename Window<HALF>::Entry Entry;
-    const size_t per_warp = lloyd_warp_bytes(a.m, HALF);
+    const size_t per_warp = lloyd_warp_bytes(a.m, HALF) + (LOCAL ? lloyd_near_bytes(a.m) : 0);
+    unsigned char *near = gi_all + (size_t)warp * per_warp + lloyd_warp_bytes(a.m, HALF);
+    if constexpr (LOCAL) {
+        const RowRecord R = row_record(a.m, true);
+        for (int i = lane; i < R.ngrp * (SKIM_GROUP_BYTES_HALF / 16); i += 32)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(near + 16 * i)), "l"(rec + R.groups + 16 * i) : "memory");
+    }
     Entry *gi = reinterpret_cast<Entry *>(gi_all + (size_t)warp * per_warp);
     double2 *segs = reinterpret_cast<double2 *>(gi_all + (size_t)warp * per_warp + (((size_t)nsk * sizeof(Entry) + 15) & ~(size_t)15));
     {
@@ -501,8 +522,9 @@ __global__ void __launch_bounds__(LLOYD_WARPS * 32, 7) skim_lloyd_kernel(Cluster
             }
         }
     }
+    if constexpr (LOCAL) asm volatile("cp.async.wait_all;" ::: "memory");
     __syncwarp();
-    lloyd_warp<HALF, UNORDERED>(rec, gi, segs, nd, a, row, sm);
+    lloyd_warp<HALF, UNORDERED, LOCAL>(rec, near, gi, segs, nd, a, row, sm);
     // the header has served its purpose: for the codes kernel the boundaries take its place
     if (a.codes) reinterpret_cast<float *>(const_cast<unsigned char *>(rec))[lane] = sm.tfs[lane];
 }
@@ -512,9 +534,18 @@ __global__ void __launch_bounds__(LLOYD_WARPS * 32, 7) skim_lloyd_kernel(Cluster
 int skim_launch_lloyd(skim_ctx *ctx, const ClusterArgs &args, int64_t rows)
 {
     const unsigned blocks = (unsigned)((rows + LLOYD_WARPS - 1) / LLOYD_WARPS);
-    const size_t smem = (size_t)LLOYD_WARPS * lloyd_warp_bytes(args.m, args.rec_half != 0);
+    size_t smem = (size_t)LLOYD_WARPS * lloyd_warp_bytes(args.m, args.rec_half != 0);
+    // Few rows: the compact records fit into shared memory with the launch still one wave, and an iteration then waits for no load from
+    // L2.  Lloyd kernel, us, without and with: 1000 x 3001 55.7 and 49.8, 500 x 4096 55.8 and 47.6, 1000 x 1000 38.4 and 37.2; where
+    // a second wave would follow (8192 x 300, 14 us a wave) it costs 2 %.  (Full records are half as long again: not tried.)
+    const size_t near = smem + (size_t)LLOYD_WARPS * lloyd_near_bytes(args.m);
+    const int64_t beside = (int64_t)((size_t)ctx->max_smem_optin / (near + LLOYD_BESIDE));       // blocks of an SM
+    const bool local = args.rec_half && (int64_t)blocks <= ctx->sm_count * (beside < LLOYD_BLOCKS ? beside : LLOYD_BLOCKS);
+    if (local) smem = near;
     // set on every launch: a host-side call of microseconds, and no state shared between contexts
-    void (*kernel)(ClusterArgs, int) = !args.rec_half ? skim_lloyd_kernel<false, true> : args.unordered ? skim_lloyd_kernel<true, true> : skim_lloyd_kernel<true, false>;
+    void (*kernel)(ClusterArgs, int) = !args.rec_half ? skim_lloyd_kernel<false, true, false>
+                                     : local ? (args.unordered ? skim_lloyd_kernel<true, true, true> : skim_lloyd_kernel<true, false, true>)
+                                             : (args.unordered ? skim_lloyd_kernel<true, true, false> : skim_lloyd_kernel<true, false, false>);
     SKIM_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     // an ordinary launch: blocks that move in beside the last sort blocks find those blocks' split of shared memory and L1,
     // with next to no L1 for the records (4096 x 11008: 0.489 instead of 0.44 ms for the whole path)
