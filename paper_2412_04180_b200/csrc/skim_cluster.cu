@@ -25,10 +25,10 @@ namespace {
 using namespace skimk;
 
 // Unscaled rows up to this length go to the bucket kernel too.  The fp16-key kernel clears and scans its counters twice whatever
-// the row length: sorting took 70 us there and 33 us in buckets at 4096 x 700, 182 and 115 at 8192 x 2000, 124 and 107 at
-// 4096 x 3500; at 4096 columns both take 129, and the rows are in order inside the groups, which saves the Lloyd kernel its comparisons
-// (up to 6 %).
-constexpr int BUCKET_UNSCALED_COLS = 3584;
+// the row length, and places every element twice: us for 4096 rows there and in buckets, 700 columns 70 and 33, 4096 129.6 and 107.2, 5600 161.4
+// and 154.1, 8192 238.8 and 222.1.  Behind it the buckets' counters leave fewer blocks on an SM: 11 008 columns 289.4 and 308.1, 2000 rows of 22 016
+// 334 and 365 (of 16 000 263 and 255).
+constexpr int BUCKET_UNSCALED_COLS = 8192;
 constexpr int RADIX_BITS = 8;
 constexpr int RADIX = 1 << RADIX_BITS;
 

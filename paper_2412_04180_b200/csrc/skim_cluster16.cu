@@ -421,15 +421,14 @@ struct Variant16 {
 #define SKIM_V16F(T, V) {T * V * 8, T, {skim_sort16_kernel<false, T, V>, nullptr}}      // short rows with compact records: skim_bucket.cu
 #define SKIM_V16L(T, V) {T * V * 8, T, {nullptr, skim_sort16_list_kernel<T, V>}}
 
-// An SM holds 1024 threads; small blocks wait for their own barriers only (4096 columns: 256 threads of 16 elements take
-// 0.131 ms for 4096 rows, 512 of 8 took 0.153 ms).
+// An SM holds 1024 threads; small blocks wait for their own barriers only.
 const Variant16 kVariants16[] = {
-    SKIM_V16F(128, 1), SKIM_V16F(128, 2), SKIM_V16(256, 2), SKIM_V16(256, 3), SKIM_V16(512, 2), SKIM_V16(512, 3), SKIM_V16(1024, 2),
+    SKIM_V16F(128, 1), SKIM_V16F(128, 2), SKIM_V16F(256, 2), SKIM_V16F(256, 3), SKIM_V16F(512, 2), SKIM_V16(512, 3), SKIM_V16(1024, 2),
     SKIM_V16(1024, 3),
 };
 // The rows that the bucket kernel refuses.  No smaller blocks: short rows are mostly the work on the 4096 counters, and the launch,
 // which usually finds the list empty, has fewer blocks (1184 of 128 threads cost 0.7 us, 592 of 256 nothing measurable).
-const Variant16 kVariantsList16[] = {SKIM_V16L(256, 1), SKIM_V16L(512, 1)};
+const Variant16 kVariantsList16[] = {SKIM_V16L(256, 1), SKIM_V16L(512, 1), SKIM_V16L(256, 3), SKIM_V16L(512, 2)};
 
 template <int N>
 const Variant16 *pick16(const Variant16 (&table)[N], const skim_ctx *ctx, int m)

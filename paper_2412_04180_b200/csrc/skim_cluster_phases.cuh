@@ -433,24 +433,42 @@ __device__ __forceinline__ void write_row_record_half(const ClusterArgs &a, cons
         float first = 0.0f;
         if (q < R.ngrp) {
             const int e = q << 3;
-            KeyT ks[8];
             float gs[8];
-            const unsigned gbits = src.group(e, m, ks, gs);
-            uint32_t hb[8];
             double xd[8];
+            unsigned gbits;
+            if constexpr (std::is_same<KeyT, uint4>::value) {
+                // eight binary16 values as they lie, padded
+                uint4 k;
+                gbits = src.group(e, m, k, gs);
+                xq0 = (unsigned long long)k.x | ((unsigned long long)k.y << 32);
+                xq1 = (unsigned long long)k.z | ((unsigned long long)k.w << 32);
+                const __half2 v[4] = {*reinterpret_cast<const __half2 *>(&k.x), *reinterpret_cast<const __half2 *>(&k.y), *reinterpret_cast<const __half2 *>(&k.z),
+                                      *reinterpret_cast<const __half2 *>(&k.w)};
+                const __half2 least = __hmin2(__hmin2(v[0], v[1]), __hmin2(v[2], v[3]));
+                first = __half2float(__hmin(__low2half(least), __high2half(least)));
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                uint16_t h;
-                if constexpr (sizeof(KeyT) == 2) h = (ks[u] & 0x8000u) ? (uint16_t)(ks[u] & 0x7fffu) : (uint16_t)~ks[u];
-                else h = __half_as_ushort(__float2half_rn(KeyOps<KeyT>::to_float(ks[u])));         // exact: no scale installed
-                if (e + u >= m) h = (uint16_t)SKIM_PAD_HALF;
-                hb[u] = h;
-                xd[u] = (double)__half2float(__ushort_as_half(h));
+                for (int u = 0; u < 4; ++u) {
+                    const float2 f = __half22float2(v[u]);
+                    xd[2 * u] = (double)f.x;
+                    xd[2 * u + 1] = (double)f.y;
+                }
+            } else {
+                // order-preserving images of binary16 patterns, ascending
+                static_assert(std::is_same<KeyT, uint16_t>::value, "keys of the fp16-key kernel");
+                KeyT ks[8];
+                gbits = src.group(e, m, ks, gs);
+                uint32_t hb[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    uint16_t h = (ks[u] & 0x8000u) ? (uint16_t)(ks[u] & 0x7fffu) : (uint16_t)~ks[u];
+                    if (e + u >= m) h = (uint16_t)SKIM_PAD_HALF;
+                    hb[u] = h;
+                    xd[u] = (double)__half2float(__ushort_as_half(h));
+                }
+                xq0 = (unsigned long long)(hb[0] | (hb[1] << 16)) | ((unsigned long long)(hb[2] | (hb[3] << 16)) << 32);
+                xq1 = (unsigned long long)(hb[4] | (hb[5] << 16)) | ((unsigned long long)(hb[6] | (hb[7] << 16)) << 32);
+                first = (float)xd[0];
             }
-            xq0 = (unsigned long long)(hb[0] | (hb[1] << 16)) | ((unsigned long long)(hb[2] | (hb[3] << 16)) << 32);
-            xq1 = (unsigned long long)(hb[4] | (hb[5] << 16)) | ((unsigned long long)(hb[6] | (hb[7] << 16)) << 32);
-            // the smallest value: inside a group a row of the bucket kernel is in no order
-            first = sizeof(KeyT) == 2 ? (float)xd[0] : (float)fmin(fmin(fmin(xd[0], xd[1]), fmin(xd[2], xd[3])), fmin(fmin(xd[4], xd[5]), fmin(xd[6], xd[7])));
             st_sector(rec + R.groups + (size_t)q * SKIM_GROUP_BYTES_HALF + 32, gs);
             double t0[8], t1[8], t2[8];
 #pragma unroll

@@ -125,7 +125,7 @@ def test_llama_row_lengths_on_a_row_subset(ctx, oracle, cols, seed, sigma):
     assert exact > 0.98
 
 
-@pytest.mark.parametrize("cols", [129, 512, 513, 1025, 2048, 2049, 3072, 3584, 3585, 4097, 5632, 5633, 8193, 11265, 16385, 22528])
+@pytest.mark.parametrize("cols", [129, 512, 513, 1025, 2048, 2049, 3072, 3584, 3585, 4096, 4097, 5632, 5633, 8192, 8193, 11265, 16385, 22528])
 @pytest.mark.parametrize("scaled", [False, True])
 def test_rows_spread_and_clumped_in_one_matrix(ctx, oracle, cols, scaled):
     """Row lengths at the edges of the sort kernels' sizes; every other row is one that buckets of equal spacing cannot spread."""
@@ -397,7 +397,7 @@ def test_pruned_matrices_cost_little_more(ctx, rows, cols, scaled):
     assert ctx.get_status() == 0
 
 
-@pytest.mark.parametrize("rows,cols", [(3000, 65), (1300, 1025), (700, 3001), (330, 5000)])
+@pytest.mark.parametrize("rows,cols", [(3000, 65), (1300, 1025), (700, 3001), (330, 5000), (310, 8000)])
 @pytest.mark.parametrize("scaled", [False, True])
 def test_matrices_of_refused_rows(ctx, oracle, rows, cols, scaled):
     """More rows that no bucket spreads than blocks of the kernel that takes them: a block goes through several."""
