@@ -290,7 +290,8 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) skim_sort_bucket_kern
     uint32_t *cnt = reinterpret_cast<uint32_t *>(smem + L.uni);         // four counters a word
     PhaseSmem &ps = *reinterpret_cast<PhaseSmem *>(smem + L.phase);
 
-    skim_let_next_kernel_start();          // (this kernel is an ordinary launch: the one after it waits)
+    skim_let_next_kernel_start();
+    skim_wait_for_previous_kernel();
     const int64_t row = a.row0 + blockIdx.x;
     const uint16_t *Wr = a.W + row * a.ld;
     const float *Gr = a.G + row * a.ld;
@@ -637,7 +638,8 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) skim_sort_bucket16_ke
     const uint16_t *base = reinterpret_cast<const uint16_t *>(smem + L.base);
     PhaseSmem &ps = *reinterpret_cast<PhaseSmem *>(smem + L.phase);
 
-    skim_let_next_kernel_start();          // (this kernel is an ordinary launch: the one after it waits)
+    skim_let_next_kernel_start();
+    skim_wait_for_previous_kernel();
     const int64_t row = a.row0 + blockIdx.x;
     const uint16_t *Wr = a.W + row * a.ld;
     const float *Gr = a.G + row * a.ld;
@@ -739,10 +741,7 @@ int skim_launch_sort_bucket(skim_ctx *ctx, const ClusterArgs &args, int64_t rows
         if (smem > (size_t)ctx->max_smem_optin) return SKIM_ERR_SHAPE;
         // set on every launch: a host-side call of microseconds, and no state shared between contexts
         SKIM_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        kernel<<<(unsigned)rows, v.threads, smem, ctx->stream>>>(args);
-        SKIM_CUDA_OK(cudaGetLastError());
-        ctx->launches += 1;
-        return SKIM_OK;
+        return skim_launch_dependent(ctx, kernel, dim3((unsigned)rows), v.threads, smem, args);
     }
     return SKIM_ERR_SHAPE;
 }

@@ -387,7 +387,8 @@ __device__ __forceinline__ bool sort16_row(const ClusterArgs &a, int local, uint
 template <bool HALF_RECORD, int THREADS, int VEC>
 __global__ void __launch_bounds__(THREADS, 1024 / THREADS) skim_sort16_kernel(ClusterArgs a)
 {
-    skim_let_next_kernel_start();          // (this kernel is an ordinary launch: the one after it waits)
+    skim_let_next_kernel_start();
+    skim_wait_for_previous_kernel();
     sort16_row<HALF_RECORD, THREADS, VEC, true>(a, (int)blockIdx.x, 0u);
 }
 
@@ -449,8 +450,5 @@ int skim_launch_sort16(skim_ctx *ctx, const ClusterArgs &args, int64_t rows, boo
     // set on every launch: a host-side call of microseconds, and no state shared between contexts
     SKIM_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     if (listed) return skim_launch_dependent(ctx, kernel, dim3(skim_list_blocks(ctx, v->threads, rows)), v->threads, smem, args);
-    kernel<<<(unsigned)rows, v->threads, smem, ctx->stream>>>(args);
-    SKIM_CUDA_OK(cudaGetLastError());
-    ctx->launches += 1;
-    return SKIM_OK;
+    return skim_launch_dependent(ctx, kernel, dim3((unsigned)rows), v->threads, smem, args);
 }

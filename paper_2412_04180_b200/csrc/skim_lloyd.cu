@@ -17,6 +17,7 @@ using namespace skimk;
 
 constexpr int LLOYD_WARPS = 4;   // rows per block
 constexpr int LLOYD_BLOCKS = 7;  // per SM
+constexpr int LLOYD_LOCAL_COLS = 1024;
 constexpr size_t LLOYD_BESIDE = 3072;   // static shared memory of a block, and what the system takes
 constexpr int WIN = 16;          // group-index entries held in registers
 
@@ -484,6 +485,7 @@ __global__ void __launch_bounds__(LLOYD_WARPS * 32, LLOYD_BLOCKS) skim_lloyd_ker
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int local = blockIdx.x * LLOYD_WARPS + warp;
     skim_let_next_kernel_start();
+    skim_wait_for_previous_kernel();
     if (blockIdx.x == 0 && threadIdx.x == 0) *a.sort_count = 0;
     if (local >= rows_in_chunk) return;
     LloydSmem &sm = sm_all[warp];
@@ -537,21 +539,27 @@ int skim_launch_lloyd(skim_ctx *ctx, const ClusterArgs &args, int64_t rows)
     size_t smem = (size_t)LLOYD_WARPS * lloyd_warp_bytes(args.m, args.rec_half != 0);
     // Few rows: the compact records fit into shared memory with the launch still one wave, and an iteration then waits for no load from
     // L2.  Lloyd kernel, us, without and with: 1000 x 3001 55.7 and 49.8, 500 x 4096 55.8 and 47.6, 1000 x 1000 38.4 and 37.2; where
-    // a second wave would follow (8192 x 300, 14 us a wave) it costs 2 %.  (Full records are half as long again: not tried.)
+    // a second wave would follow (8192 x 300, 14 us a wave) it costs 2 %, and short rows (2000 x 700 38.5 and 38.9) are in L1 anyway.  (Full
+    // records are half as long again: not tried.)
     const size_t near = smem + (size_t)LLOYD_WARPS * lloyd_near_bytes(args.m);
     const int64_t beside = (int64_t)((size_t)ctx->max_smem_optin / (near + LLOYD_BESIDE));       // blocks of an SM
-    const bool local = args.rec_half && (int64_t)blocks <= ctx->sm_count * (beside < LLOYD_BLOCKS ? beside : LLOYD_BLOCKS);
+    const bool local = args.rec_half && args.m >= LLOYD_LOCAL_COLS && (int64_t)blocks <= ctx->sm_count * (beside < LLOYD_BLOCKS ? beside : LLOYD_BLOCKS);
     if (local) smem = near;
     // set on every launch: a host-side call of microseconds, and no state shared between contexts
     void (*kernel)(ClusterArgs, int) = !args.rec_half ? skim_lloyd_kernel<false, true, false>
                                      : local ? (args.unordered ? skim_lloyd_kernel<true, true, true> : skim_lloyd_kernel<true, false, true>)
                                              : (args.unordered ? skim_lloyd_kernel<true, true, false> : skim_lloyd_kernel<true, false, false>);
     SKIM_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    // an ordinary launch: blocks that move in beside the last sort blocks find those blocks' split of shared memory and L1,
-    // with next to no L1 for the records (4096 x 11008: 0.489 instead of 0.44 ms for the whole path)
-    kernel<<<blocks, LLOYD_WARPS * 32, smem, ctx->stream>>>(args, (int)rows);
-    SKIM_CUDA_OK(cudaGetLastError());
-    ctx->launches += 1;
+    // Few rows: a programmatic dependent (with the sort kernel one too, a pipeline of 256 x 512 47.1 -> 43.0 us, 1000 x 3001 90.9 -> 86.7).  Otherwise an ordinary launch: blocks that move in beside the last sort blocks find those
+    // blocks' split of shared memory and L1, with next to no L1 for the records (4096 x 11008: 0.489 instead of 0.44 ms for the whole path).
+    if ((int64_t)blocks <= ctx->sm_count * 2) {
+        const int rc = skim_launch_dependent(ctx, kernel, dim3(blocks), LLOYD_WARPS * 32, smem, args, (int)rows);
+        if (rc) return rc;
+    } else {
+        kernel<<<blocks, LLOYD_WARPS * 32, smem, ctx->stream>>>(args, (int)rows);
+        SKIM_CUDA_OK(cudaGetLastError());
+        ctx->launches += 1;
+    }
     if (args.codes) {
         const int vec = args.m % 4 == 0 && args.ld % 4 == 0 && (reinterpret_cast<uintptr_t>(args.W) & 7u) == 0 && (reinterpret_cast<uintptr_t>(args.codes) & 3u) == 0;
         return skim_launch_dependent(ctx, skim_codes_kernel, dim3((unsigned)rows), CODES_T, 0, args, vec);
