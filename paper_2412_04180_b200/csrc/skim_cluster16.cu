@@ -105,6 +105,11 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity
     return false;
 }
 
+// Where item p of the row lies in `buf`: every second eight pieces of 16 bytes have their pairs swapped, so that neither the record pass (32
+// bytes a lane) nor pass 1 (a stretch of a multiple of 32 bytes a thread) meets a bank twice.  us: 4096 x 11008 289.6 -> 287.4, 2000 x
+// 22016 334.5 -> 328.3.
+__device__ __forceinline__ int item_place(int p) { return p ^ (p >> 3 & 4); }
+
 // The sorted row of this kernel: packed items (key << 16 | column) in sorted order, and the raw
 // importance row, which the record pass reads through the column index.
 struct SortedItems16 {
@@ -113,7 +118,8 @@ struct SortedItems16 {
     unsigned long long *status;
     __device__ __forceinline__ unsigned group(int e, int m, uint16_t *ks, float *gs) const
     {
-        const uint4 a = *reinterpret_cast<const uint4 *>(items + e), b = *reinterpret_cast<const uint4 *>(items + e + 4);
+        const int at = item_place(e);
+        const uint4 a = *reinterpret_cast<const uint4 *>(items + at), b = *reinterpret_cast<const uint4 *>(items + (at ^ 4));
         const uint32_t it[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
         unsigned bits = 0u;
 #pragma unroll
@@ -125,7 +131,7 @@ struct SortedItems16 {
         }
         return bits;      // not validated here
     }
-    __device__ __forceinline__ uint16_t key_at(int p) const { return (uint16_t)(items[p] >> 16); }
+    __device__ __forceinline__ uint16_t key_at(int p) const { return (uint16_t)(items[item_place(p)] >> 16); }
 };
 
 // One row, by the whole block; local: its index inside the chunk.  FIRST: sets the mbarrier up; parity: of its phase.  False: the
@@ -169,7 +175,7 @@ __device__ __forceinline__ bool sort16_row(const ClusterArgs &a, int local, uint
     }
     for (int d = tid; d < D0; d += THREADS) C0[d] = 0u;
     for (int d = tid; d < D1 * THREADS / 2; d += THREADS) cnt1w[d] = 0u;
-    if (tid < mpad - m) buf[m + tid] = PAD_ITEM;
+    if (tid < mpad - m) buf[item_place(m + tid)] = PAD_ITEM;
     __syncthreads();
 
     // ---------------------------------------------------------------- load, keys, pass-0 histogram
@@ -247,7 +253,7 @@ __device__ __forceinline__ bool sort16_row(const ClusterArgs &a, int local, uint
             const uint32_t key = item[i] >> 16;
             const uint32_t pos = C0[key & (D0 - 1)] + (item[i] & 0xffffu);      // bin base + slot
             const uint32_t col = (uint32_t)(((i >> 3) * THREADS + tid) * 8 + (i & 7));
-            if (SKIM_IDX(pos, m, a.status)) buf[pos] = (key << 16) | col;
+            if (SKIM_IDX(pos, m, a.status)) buf[item_place((int)pos)] = (key << 16) | col;
             // one more item of digit key >> 12 in the stretch of pass-1 owner pos / ITEMS
             const uint32_t owner = pos / ITEMS;
             if (SKIM_IDX(owner, THREADS, a.status))
@@ -315,7 +321,7 @@ __device__ __forceinline__ bool sort16_row(const ClusterArgs &a, int local, uint
     for (int i = 0; i < ITEMS; i += 4) {
         const int p = tid * ITEMS + i;
         uint4 v = make_uint4(NO_ITEM, NO_ITEM, NO_ITEM, NO_ITEM);
-        if (p < m) v = *reinterpret_cast<const uint4 *>(buf + p);     // past m: padding items, or the NO_ITEM of a later word
+        if (p < m) v = *reinterpret_cast<const uint4 *>(buf + item_place(p));     // past m: padding items, or the NO_ITEM of a later word
         item[i] = v.x; item[i + 1] = v.y; item[i + 2] = v.z; item[i + 3] = v.w;
     }
     __syncthreads();
@@ -340,7 +346,7 @@ __device__ __forceinline__ bool sort16_row(const ClusterArgs &a, int local, uint
             uint16_t *c = cnt1 + (item[i] >> (16 + D0_BITS)) * THREADS + tid;
             const uint32_t pos = *c;
             *c = (uint16_t)(pos + 1u);
-            if (SKIM_IDX(pos, m, a.status)) buf[pos] = item[i];
+            if (SKIM_IDX(pos, m, a.status)) buf[item_place((int)pos)] = item[i];
         }
     }
 
