@@ -397,6 +397,21 @@ def test_pruned_matrices_cost_little_more(ctx, rows, cols, scaled):
     assert ctx.get_status() == 0
 
 
+@pytest.mark.parametrize("rows,cols,most", [(592, 22016, 0.61), (148, 22016, 0.28)])
+def test_fewer_long_rows_take_less_time(ctx, rows, cols, most):
+    """Unscaled rows beyond the buckets, against 1192 rows (measured 0.55 and 0.25; with Lloyd blocks that moved in beside the sort's and
+    waited through it 0.67 and 0.31)."""
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(cols)
+    W = (torch.randn((1192, cols), generator=gen, device="cuda") * 0.02).half()
+    G = torch.randn((1192, cols), generator=gen, device="cuda").exp()
+    ctx.reserve(*W.shape)
+    ctx.apply_scale(None)
+    _cluster_us(ctx, W, G)
+    assert _cluster_us(ctx, W[:rows], G[:rows]) < most * _cluster_us(ctx, W, G)
+    assert ctx.get_status() == 0
+
+
 @pytest.mark.parametrize("rows,cols", [(3000, 65), (1300, 1025), (700, 3001), (330, 5000), (310, 8000)])
 @pytest.mark.parametrize("scaled", [False, True])
 def test_matrices_of_refused_rows(ctx, oracle, rows, cols, scaled):
