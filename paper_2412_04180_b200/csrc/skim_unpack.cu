@@ -15,6 +15,7 @@
 //                4096 13.6 -> 11.6).  Lanes that own 32 columns and walk rows, the codes brought by bulk copies: 24.7 unscaled, and 22.6 for
 //                the mat-vec (too few warps for the chain of a row).  Requesting whole rows into L2 first: slower by 5 % at 22016 x 8192
 #include "skim_internal.cuh"
+#include "skim_lane_words.h"
 
 namespace {
 
@@ -142,28 +143,29 @@ constexpr int STEP = 256;           // columns a warp takes at a time
 template <int B>
 struct LaneCodes {
     const unsigned char *at, *at2;  // for B = 3 the word that holds its first byte, and the next one if the bits reach into it
-    int shift;                      // B = 3: the first byte's bit in its word
-    __device__ __forceinline__ LaneCodes(const uint32_t *row, int lane, int t)
+    SkimLaneWords3 words;           // B = 3
+    __device__ __forceinline__ LaneCodes(const uint32_t *row, int lane, int t) : words(lane)
     {
-        shift = 8 * (3 * lane & 3);
-        at = reinterpret_cast<const unsigned char *>(row) + t * (32 * B) + (B == 3 ? 3 * lane & ~3 : B * lane);
-        at2 = at + (shift > 8 ? 4 : 0);
+        at = reinterpret_cast<const unsigned char *>(row) + t * (32 * B) + (B == 3 ? 4 * words.first : B * lane);
+        at2 = at + (words.reaches_next(8) ? 4 : 0);
     }
-    // of the t-th step from here
-    __device__ __forceinline__ uint2 ask(int t) const
+    // of the t-th step from here, of which the row has `columns` columns from the lane's first one on (8: or more)
+    __device__ __forceinline__ uint2 ask(int t, int columns = 8) const
     {
         const int o = t * (32 * B);
         if (B == 4) return make_uint2(__ldg(reinterpret_cast<const uint32_t *>(at + o)), 0u);
         if (B == 2) return make_uint2(__ldg(reinterpret_cast<const uint16_t *>(at + o)), 0u);
         if (B == 1) return make_uint2(__ldg(at + o), 0u);
-        return make_uint2(__ldg(reinterpret_cast<const uint32_t *>(at + o)), __ldg(reinterpret_cast<const uint32_t *>(at2 + o)));
+        // (whole: read without a branch; else 0, the code of the columns past the row's end)
+        const bool second = columns >= 8 || words.reaches_next(columns);
+        return make_uint2(__ldg(reinterpret_cast<const uint32_t *>(at + o)), second ? __ldg(reinterpret_cast<const uint32_t *>(at2 + o)) : 0u);
     }
     __device__ __forceinline__ void advance(int t)
     {
         at += t * (32 * B);
         at2 += t * (32 * B);
     }
-    __device__ __forceinline__ uint32_t get(const uint2 &v) const { return B == 3 ? __funnelshift_r(v.x, v.y, shift) : v.x; }
+    __device__ __forceinline__ uint32_t get(const uint2 &v) const { return B == 3 ? __funnelshift_r(v.x, v.y, words.shift) : v.x; }
 };
 
 // How a lane's eight values leave: one aligned 16-byte store; or, for rows that are not 16-byte aligned, through the warp's stretch of
@@ -253,7 +255,7 @@ __device__ __forceinline__ float unpack_row(const UnpackArgs &a, const uint32_t 
     uint2 now[AHEAD], next[AHEAD];
     auto ask_left = [&](int j, uint2 (&to)[AHEAD]) {
 #pragma unroll
-        for (int u = 0; u < AHEAD; ++u) to[u] = u < left && j + u * STEP < a.cols ? codes.ask(u) : make_uint2(0u, 0u);
+        for (int u = 0; u < AHEAD; ++u) to[u] = u < left && j + u * STEP < a.cols ? codes.ask(u, a.cols - j - u * STEP) : make_uint2(0u, 0u);
     };
     if (batches) {
 #pragma unroll

@@ -65,6 +65,22 @@ def test_unpack_matches_oracle_on_ragged_widths(ctx, oracle, cols, scaled):
     _check(ctx, oracle, em, s, cols, [1, 2, 3, 4], cols)
 
 
+@pytest.mark.parametrize("cols", [41, 42, 81, 83, 85, 169, 1065, 1109])
+@pytest.mark.parametrize("scaled", [False, True])
+def test_unpack_rows_of_three_bits_that_fill_their_words(ctx, oracle, cols, scaled):
+    """The last codes end in the last of the row's 16-byte padded words; the codes of a whole group of eight would reach past it, for the last row out of
+    the buffer (csrc/skim_lane_words.h).  Then every code 1, and entries from 2 on infinite: none of them is taken for the columns past the end."""
+    em, s = _synthetic_emit(oracle, 5, cols, [3], 500 + cols, scaled)
+    assert em["packed"].size == 5 * ((cols * 3 + 127) // 128 * 4)
+    _check(ctx, oracle, em, s, cols, [3], cols)
+    q = _to_gpu(em)
+    q["lut"][:, 2:] = 0x7C00
+    row = np.packbits(np.pad(np.tile(np.array([1, 0, 0], np.uint8), cols), (0, -3 * cols % 128)), bitorder="little").view("<i4")
+    q["packed"][:] = torch.from_numpy(np.tile(row, 5)).cuda()
+    y = ctx.matvec(q, cols, [3], torch.ones(cols, dtype=torch.float16, device="cuda"))
+    assert bool(torch.isfinite(y).all())
+
+
 @pytest.mark.parametrize("cols", [1016, 1023, 1024, 1025, 1281, 2040, 2048, 2056, 3328])
 @pytest.mark.parametrize("width", [1, 2, 3, 4])
 def test_unpack_around_whole_batches(ctx, oracle, cols, width):
