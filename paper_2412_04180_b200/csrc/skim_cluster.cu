@@ -53,7 +53,9 @@ __host__ __device__ inline SmemLayout smem_layout(int cap, int nwarps)
     return L;
 }
 
-// Takes the rows of a.sort_list (blocks leave at once when it is empty, the usual case).
+// Takes the rows of a.sort_list (blocks leave at once when it is empty, the usual case).  The kernel after this one may start as the blocks leave, no
+// earlier: the Lloyd blocks of few rows, moving in beside blocks that sort, waited there with their split of shared memory and L1 (clustering of rows
+// that are all listed, us, let in at once and now: 1000 x 11008 scaled 384 and 353, 300 x 8192 scaled 114 and 111, 500 x 1500 unscaled 39 and 35).
 template <int THREADS, int ITEMS>
 __global__ void __launch_bounds__(THREADS) skim_sort_kernel(ClusterArgs a)
 {
@@ -73,7 +75,6 @@ __global__ void __launch_bounds__(THREADS) skim_sort_kernel(ClusterArgs a)
     const int warp = tid >> 5;
     const int m = a.m;
     skim_wait_for_previous_kernel();
-    skim_let_next_kernel_start();
     const int listed = min(*a.sort_count, a.chunk_rows);
     for (int at = blockIdx.x; at < listed; at += gridDim.x) {
     const int local = a.sort_list[at];

@@ -398,12 +398,11 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) skim_sort16_kernel(Cl
     sort16_row<HALF_RECORD, THREADS, VEC, true>(a, (int)blockIdx.x, 0u);
 }
 
-// The rows that the bucket kernel has put on a.sort_list (usually none).
+// The rows that the bucket kernel has put on a.sort_list (usually none).  The next kernel may start as the blocks leave (see skim_cluster.cu).
 template <int THREADS, int VEC>
 __global__ void __launch_bounds__(THREADS, 1024 / THREADS) skim_sort16_list_kernel(ClusterArgs a)
 {
     skim_wait_for_previous_kernel();
-    skim_let_next_kernel_start();
     const int listed = min(*a.sort_count, a.chunk_rows);
     if ((int)blockIdx.x >= listed) return;
     extern __shared__ __align__(16) unsigned char smem[];
