@@ -16,9 +16,9 @@
 // Buckets: v = 1 + |x| / s with s half a standard deviation (from the mean of |x|).  The bits of v grow with |x|: the
 // first three octaves, v in [1, 8), i.e. |x| up to 3.5 deviations, have N/8 buckets each on either side of zero, the next
 // eight share N/8 (N = 32 per thread).  A row whose values this cannot spread (a bucket with BUCKET_LIMIT elements, or 32 in
-// three neighbouring ones: few distinct values, a clump) is put on a list, for the fp16-key kernel of skim_cluster16.cu or, where
-// scaled, the radix kernel of skim_cluster.cu.  Such a matrix takes 1.1 to 1.4 times what those kernels alone would (sort of 4096
-// rows of a few nearby values, us: 11008 scaled 1281; of bell-shaped rows 374).
+// three neighbouring ones; unscaled rows: see there) is sorted by 16-bit keys (skim_sort16.cuh), by the block itself or through a list by the kernel
+// of skim_cluster16.cu, or, where scaled, goes through the list to the radix kernel of skim_cluster.cu (sort of 4096 x 11008 scaled, us: a few nearby
+// values 1281, bell-shaped rows 374).
 //
 // Zeros (a pruned matrix) are one value and need no bucket: a row that cannot be spread and has zeros is read again and spread with
 // its zeros between the negative and the positive buckets in column order, by ballots, the scale taken from the other elements.
@@ -29,7 +29,9 @@
 // Why not a radix sort: rows of 32-bit keys took four passes, each with ballots or random shared-memory traffic of all
 // elements (1.17 ms for 4096 x 11008); 16-bit keys two (0.284 ms).  What bounds this kernel is the same resource,
 // shared-memory wavefronts of random accesses, but there is one counting atomic and one scatter per element.
-#include "skim_cluster_phases.cuh"
+#include "skim_sort16.cuh"
+
+#include <algorithm>
 
 namespace {
 
@@ -400,6 +402,23 @@ __host__ __device__ inline Bucket16Layout bucket16_layout(int m, int threads)
     return L;
 }
 
+// A row is refused for a bucket with more than BUCKET16_SLOTS elements, or for crowded words (three neighbouring buckets with 32 elements): more than
+// two of a thread's eight, or any in more than CROWDED threads.  A bucket across the border of two groups is put in order by one thread, in time that
+// grows with its square.  A row with a narrow centre and long tails has a few crowded words (sort and Lloyd, 4096 x 5000: 263 us refused and 220 spread);
+// spreading values about 0.3 with a deviation of 0.02, whose words are crowded throughout, took 328 us for 4096 x 4096 where refusing them takes 190.
+// A row of few values or a clump is told by the first EARLY elements of every thread: one of their buckets holds EARLY_SLOTS already.  Otherwise all its
+// elements queue for a few counters (us for 4096 rows of a clump, 4096 columns 314 -> 243, 8192 578 -> 449).
+//
+// The block sorts a refused row itself where it has 256 threads or more: that takes no more shared memory than the buckets (44 KB each at 4096
+// columns), the failed attempt's waits are covered by the SM's other blocks, and no other kernel has to look for such rows (2.8 us).
+// Smaller blocks would lose an eighth of their number by it; their rows go on a list.
+// us for 4096 rows of a clump (in brackets: values about 0.3), by the fp16-key kernel alone, by buckets and a list, and now: 3700 columns 229 308 231 (173 219
+// 187), 4096 243 331 242 (178 224 190), 5000 273 459 291 (190 247 235), 8192 444 590 449 (310 372 341).  Bell-shaped rows: 160 132 128, 163 139 135, 187 177 172,
+// 280 262 254.
+constexpr uint32_t BUCKET16_SLOTS = 32, EARLY_SLOTS = 12;
+__host__ __device__ constexpr bool sorts_refused_rows(int threads) { return threads >= 256; }
+template <int THREADS> constexpr int CROWDED = sorts_refused_rows(THREADS) ? THREADS / 64 : 0;
+
 __device__ __forceinline__ float key_value(uint16_t h) { return __half2float(__ushort_as_half(h)); }
 
 // Where the first position of bucket b lies in `base`: a thread writes 64 bytes, four pieces whose order is another one every second
@@ -491,6 +510,8 @@ __device__ __forceinline__ Spread spread_row16(const uint16_t *Wr, const float *
     // ------------------------------------------------------------ count: slots inside the buckets
     uint32_t slot[(ITEMS + 3) / 4];
     uint32_t most = 0u;
+    constexpr int EARLY = sorts_refused_rows(THREADS) ? 2 : 0;
+    bool clumped = false;               // a value or a clump of them takes a bucket after EARLY of the thread's elements
 #pragma unroll
     for (int i = 0; i < ITEMS; ++i) {
         if ((i & 3) == 0) slot[i >> 2] = 0u;
@@ -501,13 +522,25 @@ __device__ __forceinline__ Spread spread_row16(const uint16_t *Wr, const float *
             const uint32_t s = __funnelshift_r(atomicAdd(cnt + (b >> 2), __funnelshift_l(1u, 1u, 8u * b)), 0u, 8u * b & 31u) & 0xffu;
             most = max(most, s);
             slot[i >> 2] |= s << (8 * (i & 3));
+            clumped |= i < EARLY && s >= EARLY_SLOTS && item[i] != 0u;
             item[i] |= (uint32_t)base_place((int)b) << 16;
         }
+        // (no barrier for it: a warp that sees one leaves the others to count on)
+        if (i == EARLY - 1 && __any_sync(0xffffffffu, clumped)) {
+            clumped = true;
+            break;
+        }
     }
+    if (clumped) ps.misc[2] = 1;
+    if (most >= BUCKET16_SLOTS) ps.misc[3] = 1;
     __syncthreads();
+    if (ps.misc[2]) {
+        r.zeros_only = false;
+        return r;
+    }
 
     // ------------------------------------------------------------ counters -> first positions
-    bool crowded = false;
+    int crowded = 0;
     {
         uint4 v[2];
         uint32_t s = 0u, occupied = 0u;
@@ -537,7 +570,7 @@ __device__ __forceinline__ Spread spread_row16(const uint16_t *Wr, const float *
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
             const uint32_t before = w[u] * 0x01010100u;             // bytes: elements of the word's buckets before each one
-            crowded |= before >> 24 > 31u;
+            crowded += before >> 24 > 31u ? 1 : 0;
             const uint32_t both = run * 0x10001u;
             out[2 * u] = both + __byte_perm(before, 0u, 0x4140);
             out[2 * u + 1] = both + __byte_perm(before, 0u, 0x4342);
@@ -547,6 +580,7 @@ __device__ __forceinline__ Spread spread_row16(const uint16_t *Wr, const float *
         for (int u = 0; u < 4; ++u) reinterpret_cast<uint4 *>(base)[4 * tid + (u ^ (tid >> 1 & 3))] = make_uint4(out[4 * u], out[4 * u + 1], out[4 * u + 2], out[4 * u + 3]);
         if (tid < SPARE) base[Bk::N + tid] = (uint16_t)m;            // the last bucket's end; elements past the row are not placed
     }
+    if (CROWDED<THREADS> && crowded > 2) ps.misc[3] = 1;
     // importances, a batch ahead of the one that is placed
     constexpr int GB = 8;
     float g[2][GB];
@@ -555,7 +589,7 @@ __device__ __forceinline__ Spread spread_row16(const uint16_t *Wr, const float *
         for (int u = 0; u < GB; ++u) to[u] = (i0 + u < ITEMS && (i0 + u) * THREADS + tid < m) ? Gr[(i0 + u) * THREADS + tid] : 0.0f;
     };
     fetch(0, g[0]);
-    if (__syncthreads_or(most >= (uint32_t)BUCKET_LIMIT || crowded ? 1 : 0)) {
+    if (__syncthreads_count(crowded ? 1 : 0) > CROWDED<THREADS> || ps.misc[3]) {
         // (zeros fall into the first bucket of thread THREADS / 2)
         r.zeros_only = !__syncthreads_or(crowded && tid != THREADS / 2 ? 1 : 0);
         return r;
@@ -624,8 +658,12 @@ struct SortedHalves {
     __device__ __forceinline__ float key_at(int p) const { return key_value(keys[p]); }
 };
 
+// (its own function, as above)
 template <int THREADS, int ITEMS>
-__global__ void __launch_bounds__(THREADS, 1024 / THREADS) skim_sort_bucket16_kernel(ClusterArgs a)
+__device__ __noinline__ void sort_refused_row(const ClusterArgs &a) { sort16_row<true, THREADS, (ITEMS + 7) / 8, true>(a, (int)blockIdx.x, 0u); }
+
+template <int THREADS, int ITEMS>
+__global__ void __launch_bounds__(THREADS, 1024 / THREADS) skim_sort_bucket16_kernel(const __grid_constant__ ClusterArgs a)
 {
     using Bk = Buckets<THREADS>;
     constexpr int NW = THREADS / 32;
@@ -638,7 +676,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) skim_sort_bucket16_ke
     const uint16_t *base = reinterpret_cast<const uint16_t *>(smem + L.base);
     PhaseSmem &ps = *reinterpret_cast<PhaseSmem *>(smem + L.phase);
 
-    skim_let_next_kernel_start();
+    if (!sorts_refused_rows(THREADS)) skim_let_next_kernel_start();        // (the list kernel; the Lloyd kernel starts as the blocks leave)
     skim_wait_for_previous_kernel();
     const int64_t row = a.row0 + blockIdx.x;
     const uint16_t *Wr = a.W + row * a.ld;
@@ -648,19 +686,24 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) skim_sort_bucket16_ke
     if (tid == 0) {
         ps.misc[0] = 0;
         ps.misc[1] = 0;
+        ps.misc[2] = 0;
+        ps.misc[3] = 0;
     }
     Spread sp = spread_row16<THREADS, ITEMS, false>(Wr, Gr, m, a.status);
     bool apart = false;                    // the zeros lie between the negative and the positive buckets
     if (!sp.done && sp.zeros_only) {
         __syncthreads();
-        if (tid == 0) ps.misc[0] = 0;
+        if (tid == 0) ps.misc[0] = ps.misc[3] = 0;
         sp = spread_row16_zeros_apart<THREADS, ITEMS>(Wr, Gr, m, a.status);
         apart = true;
     }
     if (sp.bad) atomicOr(a.status, (unsigned long long)sp.bad);
     if (!sp.done) {
-        // not a row for buckets: the kernel after this one takes it
-        if (tid == 0) {
+        // not a row for buckets
+        if constexpr (sorts_refused_rows(THREADS)) {
+            __syncthreads();
+            sort_refused_row<THREADS, ITEMS>(a);
+        } else if (tid == 0) {
             const int at = atomicAdd(a.sort_count, 1);
             if (SKIM_IDX(at, a.chunk_rows, a.status)) a.sort_list[at] = (int)blockIdx.x;
         }
@@ -731,13 +774,15 @@ const BucketVariant kVariantsBucket[] = {
 
 }  // namespace
 
-int skim_launch_sort_bucket(skim_ctx *ctx, const ClusterArgs &args, int64_t rows)
+int skim_launch_sort_bucket(skim_ctx *ctx, const ClusterArgs &args, int64_t rows, bool *lists)
 {
     for (const BucketVariant &v : kVariantsBucket) {
         if (v.cap < args.m) continue;
         void (*kernel)(ClusterArgs) = args.rscale ? v.scaled : v.unscaled;
         if (!kernel) return SKIM_ERR_SHAPE;
-        const size_t smem = args.rscale ? bucket_layout(args.m, v.threads).total : bucket16_layout(args.m, v.threads).total;
+        *lists = args.rscale || !sorts_refused_rows(v.threads);
+        size_t smem = args.rscale ? bucket_layout(args.m, v.threads).total : bucket16_layout(args.m, v.threads).total;
+        if (!*lists) smem = std::max(smem, layout16(args.m, v.threads).total);
         if (smem > (size_t)ctx->max_smem_optin) return SKIM_ERR_SHAPE;
         // set on every launch: a host-side call of microseconds, and no state shared between contexts
         SKIM_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));

@@ -25,9 +25,9 @@ namespace {
 using namespace skimk;
 
 // Unscaled rows up to this length go to the bucket kernel too.  The fp16-key kernel clears and scans its counters twice whatever
-// the row length, and places every element twice: us for 4096 rows there and in buckets, 700 columns 70 and 33, 4096 129.6 and 107.2, 5600 161.4
-// and 154.1, 8192 238.8 and 222.1.  Behind it the buckets' counters leave fewer blocks on an SM: 11 008 columns 289.4 and 308.1, 2000 rows of 22 016
-// 334 and 365 (of 16 000 263 and 255).
+// the row length, and places every element twice: us for 4096 rows there and in buckets, 700 columns 70 and 33, 4096 129.6 and 102, 8192 238.8 and
+// 215 (rows that the buckets refuse: skim_bucket.cu).  Beyond, the buckets' counters leave fewer blocks on an SM: 11 008 columns 289.4 and
+// 308.1, 2000 rows of 22 016 334 and 365 (of 16 000 263 and 255).
 constexpr int BUCKET_UNSCALED_COLS = 8192;
 constexpr int RADIX_BITS = 8;
 constexpr int RADIX = 1 << RADIX_BITS;
@@ -282,9 +282,10 @@ int skim_launch_cluster(skim_ctx *ctx, const uint16_t *W, const float *importanc
         cudaEvent_t *tev = (ctx->timing && ctx->timing_used < SKIM_TIMING_SLOTS) ? ctx->timing_ev[ctx->timing_used] : nullptr;
         if (tev) SKIM_CUDA_OK(cudaEventRecord(tev[0], ctx->stream));
         a.chunk_rows = (int)n;
-        int rc = bucket ? skim_launch_sort_bucket(ctx, a, n) : skim_launch_sort16(ctx, a, n);
+        bool lists = false;
+        int rc = bucket ? skim_launch_sort_bucket(ctx, a, n, &lists) : skim_launch_sort16(ctx, a, n);
         if (rc) return rc;
-        if (bucket) {
+        if (lists) {
             // the rows the buckets could not spread: usually none
             if (scaled) rc = skim_launch_dependent(ctx, v->kernel, dim3(skim_list_blocks(ctx, v->threads, n)), v->threads, smem, a);
             else rc = skim_launch_sort16(ctx, a, n, true);

@@ -556,8 +556,8 @@ static inline unsigned skim_list_blocks(const skim_ctx *ctx, int threads, int64_
     const int64_t blocks = (int64_t)ctx->sm_count * (1024 / threads);
     return (unsigned)(rows < blocks ? rows : blocks);
 }
-// Bucket sort kernel (skim_bucket.cu): writes the row records of a chunk, or puts rows on args.sort_list.
-int skim_launch_sort_bucket(skim_ctx *ctx, const skimk::ClusterArgs &args, int64_t rows);
+// Bucket sort kernel (skim_bucket.cu): writes the row records of a chunk, or puts rows on args.sort_list (if it is one that `lists`).
+int skim_launch_sort_bucket(skim_ctx *ctx, const skimk::ClusterArgs &args, int64_t rows, bool *lists);
 // fp16-key sort kernel (skim_cluster16.cu): writes the row records of a chunk, or of the rows on args.sort_list; no scale vector
 // installed.
 int skim_launch_sort16(skim_ctx *ctx, const skimk::ClusterArgs &args, int64_t rows, bool listed = false);
