@@ -786,6 +786,16 @@ int skim_launch_sort_bucket(skim_ctx *ctx, const ClusterArgs &args, int64_t rows
         if (smem > (size_t)ctx->max_smem_optin) return SKIM_ERR_SHAPE;
         // set on every launch: a host-side call of microseconds, and no state shared between contexts
         SKIM_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        // Scaled rows whose blocks leave much of the chip free: an ordinary launch.  Blocks that may start beside the Lloyd kernel of the call before seem to crowd on the
+        // SMs that have none of its blocks.  Calls one after another, us, dependent and ordinary: 400 x 1500 37.5 and 33.5, 500 x 2000 41.0 and 37.3, 500 x 900 31.7
+        // and 29.9, 800 x 1500 39.2 and 38.6, 1000 x 2000 of refused rows 71.3 and 66.3; but 256 x 512 25.9 and 26.7, 300 x 1500 33.5 and 33.6, 1150 x 1200 38.6 and 39.5.
+        // Larger blocks, more rows and unscaled rows (whose Lloyd kernel takes shared memory itself): dependent 1 us less.
+        if (args.rscale && v.threads == 128 && rows > ctx->sm_count * 2 && rows < ctx->sm_count * 7) {
+            kernel<<<(unsigned)rows, v.threads, smem, ctx->stream>>>(args);
+            SKIM_CUDA_OK(cudaGetLastError());
+            ctx->launches += 1;
+            return SKIM_OK;
+        }
         return skim_launch_dependent(ctx, kernel, dim3((unsigned)rows), v.threads, smem, args);
     }
     return SKIM_ERR_SHAPE;
