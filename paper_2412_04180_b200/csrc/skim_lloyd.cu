@@ -539,16 +539,16 @@ int skim_launch_lloyd(skim_ctx *ctx, const ClusterArgs &args, int64_t rows)
     size_t smem = (size_t)LLOYD_WARPS * lloyd_warp_bytes(args.m, args.rec_half != 0);
     // Few rows: the compact records fit into shared memory with the launch still one wave, and an iteration then waits for no load from
     // L2.  Lloyd kernel, us, without and with: 1000 x 3001 55.7 and 49.8, 500 x 4096 55.8 and 47.6, 1000 x 1000 38.4 and 37.2; where
-    // a second wave would follow (8192 x 300, 14 us a wave) it costs 2 %, and short rows (2000 x 700 38.5 and 38.9) are in L1 anyway.  (Full
-    // records are half as long again: not tried.)
+    // a second wave would follow (8192 x 300, 14 us a wave) it costs 2 %, and short rows (2000 x 700 38.5 and 38.9) are in L1 anyway.  (From
+    // some 6900 columns on four rows do not fit: rows in order, beyond the buckets, have no such form.  Full records are half as long again: not tried.)
     const size_t near = smem + (size_t)LLOYD_WARPS * lloyd_near_bytes(args.m);
     const int64_t beside = (int64_t)((size_t)ctx->max_smem_optin / (near + LLOYD_BESIDE));       // blocks of an SM
-    const bool local = args.rec_half && args.m >= LLOYD_LOCAL_COLS && (int64_t)blocks <= ctx->sm_count * (beside < LLOYD_BLOCKS ? beside : LLOYD_BLOCKS);
+    const bool local = args.rec_half && args.unordered && args.m >= LLOYD_LOCAL_COLS && (int64_t)blocks <= ctx->sm_count * (beside < LLOYD_BLOCKS ? beside : LLOYD_BLOCKS);
     if (local) smem = near;
     // set on every launch: a host-side call of microseconds, and no state shared between contexts
     void (*kernel)(ClusterArgs, int) = !args.rec_half ? skim_lloyd_kernel<false, true, false>
-                                     : local ? (args.unordered ? skim_lloyd_kernel<true, true, true> : skim_lloyd_kernel<true, false, true>)
-                                             : (args.unordered ? skim_lloyd_kernel<true, true, false> : skim_lloyd_kernel<true, false, false>);
+                                     : local ? skim_lloyd_kernel<true, true, true>
+                                             : args.unordered ? skim_lloyd_kernel<true, true, false> : skim_lloyd_kernel<true, false, false>;
     SKIM_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     // A programmatic dependent where that is faster (with the sort kernel one too, a pipeline of 256 x 512 47.1 -> 43.0 us, 1000 x 3001 90.9 -> 86.7).
     // Many rows: blocks that move in beside the last blocks of a sort find those blocks' split of shared memory and L1, with next to no L1 for the
