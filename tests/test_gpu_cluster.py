@@ -509,14 +509,27 @@ def test_scaled_rows_are_the_same_on_every_run(ctx, rows, cols):
     assert ctx.get_status() == 0
 
 
-@pytest.mark.parametrize("rows,cols", [(1184, 3001), (592, 4096), (1036, 8), (148, 12000), (4144, 512)])
-def test_records_in_shared_memory_change_nothing(ctx, oracle, rows, cols):
-    """The Lloyd kernel reads a call's records from shared memory where they fit in one wave (the row counts here are the last ones
-    that do, or near them on other SM counts): the same rows within a larger call, which reads them from L2, come out bit for bit."""
-    w, g = inputs.make_rows(rows + 4, cols, 3000 + cols)
+def _rows_with_copies(cols):
+    """The last row count whose compact records the Lloyd kernel copies to shared memory: seven blocks of four rows an SM, or as many as fit."""
+    props = torch.cuda.get_device_properties(0)
+    groups = (cols + 7) // 8
+    index = ((groups + 7) // 8 * 8 + 16) * 2
+    row = (index + 15) // 16 * 16 + ((groups + 31) // 32 + 1) * 16 + groups * 64
+    return 4 * props.multi_processor_count * min(7, props.shared_memory_per_block_optin // (4 * row + 3072))
+
+
+@pytest.mark.parametrize("cols", [1024, 1031, 2049, 3001, 4096, 6880])
+def test_records_in_shared_memory_change_nothing(ctx, oracle, cols):
+    """The Lloyd kernel reads a call's records from shared memory where they fit in one wave, from 1024 columns on: the same rows within a larger call,
+    which reads them from L2, come out bit for bit."""
+    rows = _rows_with_copies(cols)
+    assert rows > 0
+    n = min(rows, 600)                                                 # different rows; the others repeat them
+    w, g = inputs.make_rows(n, cols, 3000 + cols)
     ctx.reserve(rows + 4, cols)
     ctx.apply_scale(None)
-    W, G = torch.from_numpy(w).cuda(), torch.from_numpy(g).cuda()
+    at = torch.arange(rows + 4, device="cuda") % n
+    W, G = torch.from_numpy(w).cuda()[at], torch.from_numpy(g).cuda()[at]
     small = ctx.cluster_rows(W[:rows].contiguous(), G[:rows].contiguous(), [1, 2, 3, 4], 20, want_codes=True)
     large = ctx.cluster_rows(W, G, [1, 2, 3, 4], 20, want_codes=True)
     few = ctx.cluster_rows(W[:5].contiguous(), G[:5].contiguous(), [1, 2, 3, 4], 20, want_codes=True)
@@ -526,3 +539,11 @@ def test_records_in_shared_memory_change_nothing(ctx, oracle, rows, cols):
         assert torch.equal(a[0], b[0][:n]) and torch.equal(a[1], b[1][:, :n])
         # (the row total of g x^2 of unscaled rows may differ in its last bit between runs)
         assert bool((a[2] - b[2][:n]).abs().le(1e-6 * b[2][:n].abs()).all())
+
+
+def test_no_copies_of_rows_that_do_not_fit(ctx, oracle):
+    """6920 columns: the copies of four rows are longer than the shared memory of a block."""
+    assert _rows_with_copies(6920) == 0 < _rows_with_copies(6880)
+    w, g = inputs.make_rows(6, 6920, 3)
+    cent, err, codes = _gpu_cluster(ctx, w, g, BITS, 10)
+    check_cluster(oracle.cluster_rows(w, g, BITS, 10), cent, err, codes, _values(w, None), BITS, label="6920")

@@ -1,11 +1,14 @@
 """GPU parity of the L-full error (Section 3.4; Section 4.2; Algorithm 3): skim_residual is bit-exact against
 the oracle; skim_err_lfull (tcgen05 GEMM with the row-wise dot fused in) is within the bound its binary32
 accumulation allows, (2 cols + 600) * 2^-24 * sum |d_j H_jk d_k|, and in practice two orders closer."""
+import ctypes as C
+
 import numpy as np
 import pytest
 import torch
 
 from paper_2412_04180_b200 import inputs
+from paper_2412_04180_b200.skim import lib
 
 pytestmark = pytest.mark.gpu
 BITS = [1, 2, 3, 4]
@@ -95,6 +98,56 @@ def test_lfull_special_matrices(ctx, oracle):
     got2 = ctx.err_lfull(torch.from_numpy((D.astype(np.float32) * 4).astype(np.float16)).cuda(), torch.from_numpy(Hx).cuda(), exp2=2)
     got3 = ctx.err_lfull(torch.from_numpy(D).cuda(), torch.from_numpy(Hx).cuda(), exp2=0)
     assert torch.equal(got2, got3)
+
+
+@pytest.mark.parametrize("rows,cols", [(130, 224), (130, 256), (300, 1056), (300, 1064)])
+def test_lfull_error_of_rows_within_sectors(ctx, oracle, rows, cols):
+    """The epilogue reads whole 32-byte sectors where all rows start at one and cols is a multiple of 32, half sectors otherwise: the residuals at 16
+    modulo 32, or every second row there, give the same bits."""
+    rng = np.random.default_rng(cols)
+    ctx.reserve(rows, cols)
+    D = (rng.standard_normal((rows, cols)) * 0.25).astype(np.float16)
+    H = inputs.make_gram(cols, 70 + cols)
+    want = _check_err(ctx, oracle, D, H, 3, label=f"{rows}x{cols}")
+    Hg = torch.from_numpy(H).cuda()
+    scratch = torch.empty(ctx.err_lfull_bytes(rows, cols), dtype=torch.uint8, device="cuda")
+    for first in (0, 8):
+        for pad in (0, 8, 16):
+            buf = torch.full((first + rows * (cols + pad),), float("nan"), dtype=torch.float16, device="cuda")
+            assert buf.data_ptr() % 32 == 0
+            view = buf[first:].view(rows, cols + pad)[:, :cols]
+            view.copy_(torch.from_numpy(D))
+            got = torch.empty(rows, device="cuda")
+            rc = lib().skim_err_lfull(ctx._h, C.c_void_p(view.data_ptr()), C.c_int64(rows), C.c_int64(cols), C.c_int64(cols + pad), C.c_void_p(Hg.data_ptr()),
+                                      C.c_int64(cols), C.c_int(3), C.c_void_p(scratch.data_ptr()), C.c_size_t(scratch.numel()),
+                                      C.c_void_p(got.data_ptr()), C.c_int64(1))
+            assert rc == 0
+            np.testing.assert_array_equal(got.cpu().numpy().astype(np.float64), want)
+    assert ctx.get_status() == 0
+
+
+@pytest.mark.parametrize("cols", [256, 264])
+def test_lfull_update_with_labels_within_sectors(ctx, cols):
+    """The same for the labels, which the epilogue of the update's contraction reads along."""
+    rows = 300
+    w, g = inputs.make_rows(rows, cols, 80 + cols)
+    H = torch.from_numpy(inputs.make_gram(cols, 90 + cols)).cuda()
+    ctx.reserve(rows, cols)
+    W, G = torch.from_numpy(w).cuda(), torch.from_numpy(g).cuda()
+    alpha = torch.from_numpy(inputs.make_scale(cols, 5)).cuda()
+    bits = torch.from_numpy((np.arange(rows) % 4 + 1).astype(np.uint8)).cuda()
+    ctx.apply_scale(alpha)
+    _, labels, _ = ctx.cluster_rows_at(W, G, bits, BITS, 10)
+    results = []
+    for first in (0, 16, 32):
+        buf = torch.zeros(first + rows * cols, dtype=torch.uint8, device="cuda")
+        at = buf[first:].view(rows, cols)
+        at.copy_(labels)
+        a = alpha.clone()
+        ctx.scale_update_lfull(W, G, at, a, H, steps=6)
+        results.append(a)
+    assert ctx.get_status() == 0
+    assert torch.equal(results[0], results[1]) and torch.equal(results[0], results[2]) and not torch.equal(results[0], alpha)
 
 
 @pytest.mark.parametrize("cols", [968, 1160, 2560])
