@@ -326,9 +326,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) skim_sort_bucket_kern
     // ---------------------------------------------------------------- order where it matters
     // The Lloyd kernel asks for groups of 8 in order, not for order inside a group: only a bucket that reaches from one
     // group into the next has to be sorted.  A row with few distinct values is sorted in full (they are counted below), and so
-    // are all rows for the exact kernel.  Scaled rows come out the same on every run (the record pass orders their groups).  An
-    // unscaled value has 11 bits, so a group's sums of g and g x are exact unless its importances spread over 2^15, whatever
-    // their order; the row total of g x^2 may differ in its last bit between runs, as it does from the fp16-key kernel.
+    // are all rows for the exact kernel.  The rows come out the same on every run (the record pass orders their groups).
     int nd = ps.misc[0];                     // more than 16 occupied words: more than 16 distinct values
     auto bucket_end = [&](int b) { return b + 1 < Bk::N ? bucket_base(cnt, b + 1) - (apart && b + 1 == Bk::HALF ? (int)bucket_zeros(ps)[NW] : 0) : m; };
     const bool full = a.full_order || nd <= 16;
@@ -374,15 +372,15 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) skim_sort_bucket_kern
 // ---------------------------------------------------------------- unscaled rows
 //
 // A value is a binary16 number, so the row lies in shared memory as 16-bit keys and importances, and a register holds an element's key
-// and bucket: the bucket is found once.  The shared-memory pipe bounds this kernel (44 wavefronts per 32 elements: an atomic, a lookup and
+// and bucket: the bucket is found once.  The shared-memory pipe bounds this kernel (42 wavefronts per 32 elements: an atomic, a lookup and
 // two stores at random addresses, the scans), then the latency of its phases, so
 //   - the buckets' first positions are 16-bit numbers of their own, read as they are used, and written without bank conflicts (4 % of
 //     the kernel);
 //   - importances are requested a batch before they are placed, the first before the scan of the counters is over (8 %);
 //   - elements past the row's end go to counters of their own behind the buckets', one per lane, so that nothing branches on them;
 //   - the record pass takes the keys as they lie (compact records hold binary16 values).
-// us for 4096 rows, the fp16-key kernel (to 3000 columns: the binary32 form of this one, before) and now: 3000 columns 92.9 -> 84.6, 4096
-// 129.6 -> 107.2, 5600 161.4 -> 154.1, 8192 238.8 -> 222.1; at 11 008, where two blocks of 512 threads fill an SM either way, 289.4 and 308.1.
+// us for 4096 rows, the fp16-key kernel (to 3000 columns: the binary32 form of this one, before) and now: 3000 columns 92.9 -> 83.3, 4096
+// 129.6 -> 103.5, 5600 161.4 -> 150.5, 8192 238.8 -> 215.8; at 11 008, where two blocks of 512 threads fill an SM either way, 289.4 and 308.1.
 struct Bucket16Layout {
     size_t keys, gs, base, phase, total;
 };
@@ -712,7 +710,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) skim_sort_bucket16_ke
     const Bk bucket{sp.inv_s};
     __syncthreads();
 
-    // ---------------------------------------------------------------- order where it matters (as for scaled rows, below)
+    // ---------------------------------------------------------------- order where it matters (as for scaled rows, above)
     // An unscaled value has 11 bits, so a group's sums of g and g x are exact unless its importances spread over 2^15, whatever
     // their order; the row total of g x^2 may differ in its last bit between runs, as it does from the fp16-key kernel.
     int nd = ps.misc[0];                     // more than 16 occupied words: more than 16 distinct values
@@ -766,8 +764,8 @@ struct BucketVariant {
 #define SKIM_BV(T, I) {T * I, T, skim_sort_bucket_kernel<T, I>, nullptr}
 #define SKIM_BV2(T, I) {T * I, T, skim_sort_bucket_kernel<T, I>, skim_sort_bucket16_kernel<T, I>}
 
-// An SM holds 1024 threads; many small blocks wait for their own barriers only (5600 columns: 256 x 22 takes 0.174 ms where
-// 512 x 16 takes 0.217 ms, 4096: 256 x 16 0.132 ms, 512 x 8 0.147 ms), as far as registers hold the row.
+// An SM holds 1024 threads; many small blocks wait for their own barriers only, as far as registers hold the row.  Sort and Lloyd kernel, us for 4096
+// rows, unscaled and scaled: 5600 columns 256 x 22 188 and 227, 512 x 16 205 and 254; 4096 columns 256 x 16 136 and 173, 512 x 8 163 and 193.
 const BucketVariant kVariantsBucket[] = {
     SKIM_BV2(128, 4), SKIM_BV2(128, 8), SKIM_BV2(128, 16), SKIM_BV2(256, 12), SKIM_BV2(256, 16), SKIM_BV2(256, 22), SKIM_BV2(512, 16), SKIM_BV(512, 22), SKIM_BV(1024, 16), SKIM_BV(1024, 22),
 };
