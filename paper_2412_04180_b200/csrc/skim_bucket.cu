@@ -410,9 +410,9 @@ __host__ __device__ inline Bucket16Layout bucket16_layout(int m, int threads)
 // The block sorts a refused row itself where it has 256 threads or more: that takes no more shared memory than the buckets (44 KB each at 4096
 // columns), the failed attempt's waits are covered by the SM's other blocks, and no other kernel has to look for such rows (2.8 us).
 // Smaller blocks would lose an eighth of their number by it; their rows go on a list.
-// us for 4096 rows of a clump (in brackets: values about 0.3), by the fp16-key kernel alone, by buckets and a list, and now: 3700 columns 229 308 231 (173 219
-// 187), 4096 243 331 242 (178 224 190), 5000 273 459 291 (190 247 235), 8192 444 590 449 (310 372 341).  Bell-shaped rows: 160 132 128, 163 139 135, 187 177 172,
-// 280 262 254.
+// us for 4096 rows of a clump (in brackets: values about 0.3), by the fp16-key kernel alone, by buckets and a list, and now: 3700 columns 229 308
+// 231 (173 219 187), 4096 243 331 242 (178 224 190), 5000 273 459 291 (190 247 235), 8192 444 590 449 (310 372 341).  Bell-shaped rows: 160 132
+// 128, 163 139 135, 187 177 172, 280 262 254.
 constexpr uint32_t BUCKET16_SLOTS = 32, EARLY_SLOTS = 12;
 __host__ __device__ constexpr bool sorts_refused_rows(int threads) { return threads >= 256; }
 template <int THREADS> constexpr int CROWDED = sorts_refused_rows(THREADS) ? THREADS / 64 : 0;
@@ -784,10 +784,11 @@ int skim_launch_sort_bucket(skim_ctx *ctx, const ClusterArgs &args, int64_t rows
         if (smem > (size_t)ctx->max_smem_optin) return SKIM_ERR_SHAPE;
         // set on every launch: a host-side call of microseconds, and no state shared between contexts
         SKIM_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        // Scaled rows whose blocks leave much of the chip free: an ordinary launch.  Blocks that may start beside the Lloyd kernel of the call before seem to crowd on the
-        // SMs that have none of its blocks.  Calls one after another, us, dependent and ordinary: 400 x 1500 37.5 and 33.5, 500 x 2000 41.0 and 37.3, 500 x 900 31.7
-        // and 29.9, 800 x 1500 39.2 and 38.6, 1000 x 2000 of refused rows 71.3 and 66.3; but 256 x 512 25.9 and 26.7, 300 x 1500 33.5 and 33.6, 1150 x 1200 38.6 and 39.5.
-        // Larger blocks, more rows and unscaled rows (whose Lloyd kernel takes shared memory itself): dependent 1 us less.
+        // Scaled rows whose blocks leave much of the chip free: an ordinary launch.  Blocks that may start beside the Lloyd kernel of the call
+        // before seem to crowd on the SMs that have none of its blocks.  Calls one after another, us, dependent and ordinary: 400 x 1500 37.5 and
+        // 33.5, 500 x 2000 41.0 and 37.3, 500 x 900 31.7 and 29.9, 800 x 1500 39.2 and 38.6, 1000 x 2000 of refused rows 71.3 and 66.3; but 256 x
+        // 512 25.9 and 26.7, 300 x 1500 33.5 and 33.6, 1150 x 1200 38.6 and 39.5. Larger blocks, more rows and unscaled rows (whose Lloyd kernel
+        // takes shared memory itself): dependent 1 us less.
         if (args.rscale && v.threads == 128 && rows > ctx->sm_count * 2 && rows < ctx->sm_count * 7) {
             kernel<<<(unsigned)rows, v.threads, smem, ctx->stream>>>(args);
             SKIM_CUDA_OK(cudaGetLastError());

@@ -554,9 +554,9 @@ int skim_launch_lloyd(skim_ctx *ctx, const ClusterArgs &args, int64_t rows)
     // Many rows: blocks that move in beside the last blocks of a sort find those blocks' split of shared memory and L1, with next to no L1 for the
     // records.  Pipeline, us, ordinary and dependent: 1184 x 4096 88.5 and 86.2, 1776 x 4096 114.5 and 116.1, 2368 x 3001 120.2 and 122.4, 4096 x
     // 11008 405 and 457; up to 1000 columns the dependent gains 1 to 2 us for any number of rows.
-    // Directly behind the fp16-key kernel (rows beyond the buckets), which lets its dependent start at once: only where the blocks have SMs of their own
-    // (16 x 11008 to 118 x 11008 and 110 x 22016 2 us less).  Others wait through all of the sort beside its blocks: 1000 x 11008 151 and 198, 592 x 22016 177 and
-    // 261, 148 x 22016 95 and 132.
+    // Directly behind the fp16-key kernel (rows beyond the buckets), which lets its dependent start at once: only where the blocks have SMs of
+    // their own (16 x 11008 to 118 x 11008 and 110 x 22016 2 us less).  Others wait through all of the sort beside its blocks: 1000 x 11008 151 and
+    // 198, 592 x 22016 177 and 261, 148 x 22016 95 and 132.
     if (args.unordered ? (int64_t)blocks <= ctx->sm_count * 2 : rows + (int64_t)blocks <= ctx->sm_count) {
         const int rc = skim_launch_dependent(ctx, kernel, dim3(blocks), LLOYD_WARPS * 32, smem, args, (int)rows);
         if (rc) return rc;

@@ -11,12 +11,13 @@
 // in shared memory.  What a warp needs of its first row is on its way while that vector is staged.
 // Both kernels are programmatic dependents of whatever runs before them.  us, call after call, with codebooks in shared memory / in registers / and as
 // a dependent, on one packed matrix (in L2) and, in brackets, on ten in turn (165 MB, more than L2 holds):
-//   mat-vec      4096 x 11008 at 3.0 bits 19.7 / 17.5 / 14.5 (18.9 / 16.8 / 14.3), 22016 x 8192 54 and now 43 either way.  Bound by the integer pipe (16 lanes a
-//                clock and scheduler: about 3 operations per element there), then by its start and end
-//   dequantiser  4096 x 11008 scaled 26.6 / 27.4 / 24.9 (25.9 / 26.9 / 24.9), unscaled 23.2 and now 21.4.  b/8 B in and 2 B out per element, 1.6 times as long as a plain fill of the
-//                output: issue is 59 % busy, and a warp has one row, eleven batches of codes one after another, with every eighth warp
-//                idle.  Lanes that own 32 columns and walk rows, the codes brought by bulk copies: 24.7 unscaled where this took 23.7, and 22.6 for the mat-vec
-//                (too few warps for the chain of a row).  Requesting whole rows into L2 first: slower by 5 % at 22016 x 8192
+//   mat-vec      4096 x 11008 at 3.0 bits 19.7 / 17.5 / 14.5 (18.9 / 16.8 / 14.3), 22016 x 8192 54 and now 43 either way.  Bound by the integer
+//                pipe (16 lanes a clock and scheduler: about 3 operations per element there), then by its start and end
+//   dequantiser  4096 x 11008 scaled 26.6 / 27.4 / 24.9 (25.9 / 26.9 / 24.9), unscaled 23.2 and now 21.4.  b/8 B in and 2 B out per element, 1.6
+//                times as long as a plain fill of the output: issue is 59 % busy, and a warp has one row, eleven batches of codes one
+//                after another, with every eighth warp idle
+// Lanes that own 32 columns and walk rows, the codes brought by bulk copies: 24.7 us for the unscaled dequantiser where this took 23.7, and 22.6 for the
+// mat-vec (too few warps for the chain of a row).  Requesting whole rows into L2 first: slower by 5 % at 22016 x 8192.
 #include "skim_internal.cuh"
 #include "skim_lane_words.h"
 
