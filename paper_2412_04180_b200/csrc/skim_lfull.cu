@@ -529,7 +529,10 @@ skim_lfull_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
     const int ntiles = a.mt * a.nt;
     int nunits = a.full_tiles + (ntiles - a.full_tiles) * a.split;
     HalfList half = {0, 0, HALF ? half_pieces(0, nkb, a.piece_kb) : 1};
-    if (!a.Y) skim_let_next_kernel_start();
+    // Behind the half form the full one lets its reduction start as it ends: usually it has nothing to do and ends at once, and where H is not symmetric,
+    // reduction blocks that wait beside it cost more than the launch (a table, us, let in at once and now: 4096 x 4096 symmetric 366 and 358, not
+    // symmetric 633 and 614, 4096 x 2048 153 and 148, 289 and 276; with ordinary launches 410, 596, 185 and 313).
+    if (!a.Y && (HALF || !a.asym)) skim_let_next_kernel_start();
     if (!HALF && a.asym) skim_wait_for_previous_kernel();
     if (HALF) {
         nunits = 0;
